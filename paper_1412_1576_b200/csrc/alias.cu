@@ -14,6 +14,8 @@
 //     heavy m+1 (or is full).
 // This is the closed form of "fill lights in order from the current heavy item; an
 // exhausted heavy item becomes a bin topped up by the next heavy item".
+#include <cooperative_groups.h>
+
 #include "lda_device.cuh"
 #include "lda_internal.cuh"
 
@@ -26,28 +28,74 @@ typedef unsigned long long ull;
 #endif
 constexpr int ALIAS_BINS_AT_ONCE = LDA_ALIAS_BINS_AT_ONCE;  // bins a thread finishes side by side
 
-template <bool BLOCK>
+// The threads that build one row together: a warp, a CTA, or a cluster of CTAs.
+enum GroupKind { WARP, CTA, CLUSTER };
+constexpr int GROUP_SMEM = 99 + 6;  // 64-bit words of shared memory a CTA of a group needs (none for WARP)
+
+template <GroupKind KIND>
 struct Group {
-    ull* smem;  // CTA groups only: >= 99 entries
-    __device__ __forceinline__ int rank() const { return BLOCK ? (int)threadIdx.x : (int)(threadIdx.x & 31); }
-    __device__ __forceinline__ int size() const { return BLOCK ? (int)blockDim.x : 32; }
+    ull* smem;  // [GROUP_SMEM]
+    __device__ __forceinline__ int cluster_rank() const
+    {
+        return KIND == CLUSTER ? (int)cooperative_groups::this_cluster().block_rank() : 0;
+    }
+    __device__ __forceinline__ int cluster_size() const
+    {
+        return KIND == CLUSTER ? (int)cooperative_groups::this_cluster().num_blocks() : 1;
+    }
+    __device__ __forceinline__ int rank() const
+    {
+        return KIND == WARP ? (int)(threadIdx.x & 31) : cluster_rank() * (int)blockDim.x + (int)threadIdx.x;
+    }
+    __device__ __forceinline__ int size() const { return KIND == WARP ? 32 : cluster_size() * (int)blockDim.x; }
     __device__ __forceinline__ void sync() const
     {
-        if (BLOCK) __syncthreads(); else __syncwarp();
+        if (KIND == WARP) __syncwarp();
+        else if (KIND == CTA) __syncthreads();
+        else cooperative_groups::this_cluster().sync();  // orders global memory between the CTAs too
+    }
+    // Sums of three values over the CTAs of the cluster (each thread holds its CTA's values), and over
+    // the CTAs of lower rank.  Through the CTAs' shared memory.
+    __device__ __forceinline__ void cluster_sums(const ull (&mine)[3], ull (&all)[3], ull (&lower)[3]) const
+    {
+        ull* slot = smem + 99;
+        if (threadIdx.x == 0) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) slot[q] = mine[q];
+        }
+        cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+        cl.sync();
+#pragma unroll
+        for (int q = 0; q < 3; ++q) all[q] = lower[q] = 0;
+        for (unsigned r = 0; r < cl.num_blocks(); ++r) {
+            const ull* other = cl.map_shared_rank(slot, r);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const ull x = other[q];
+                all[q] += x;
+                if (r < cl.block_rank()) lower[q] += x;
+            }
+        }
+        cl.sync();  // the slots may be written again
     }
     __device__ __forceinline__ ull reduce(ull v) const
     {
-        if (BLOCK) return block_reduce_sum<ull>(v, smem);
-        return warp_reduce_sum<ull>(v);
+        if (KIND == WARP) return warp_reduce_sum<ull>(v);
+        const ull t = block_reduce_sum<ull>(v, smem);
+        if (KIND == CTA) return t;
+        const ull mine[3] = {t, 0, 0};
+        ull all[3], lower[3];
+        cluster_sums(mine, all, lower);
+        return all[0];
     }
     // Exclusive scans of three values at once (one pass, one set of barriers); v[] in, prefixes
-    // out in v[], totals in tot[].  CTA groups need 99 entries of `smem`.
+    // out in v[], totals in tot[].
     __device__ __forceinline__ void scan_excl3(ull (&v)[3], ull (&tot)[3]) const
     {
         ull incl[3];
 #pragma unroll
         for (int q = 0; q < 3; ++q) incl[q] = warp_scan_incl<ull>(v[q]);
-        if (!BLOCK) {
+        if (KIND == WARP) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
                 tot[q] = __shfl_sync(0xffffffffu, incl[q], 31);
@@ -77,16 +125,15 @@ struct Group {
             tot[q] = smem[33 * q + 32];
             v[q] = smem[33 * q + warp] + incl[q] - v[q];
         }
+        if (KIND == CLUSTER) {
+            const ull mine[3] = {tot[0], tot[1], tot[2]};
+            ull lower[3];
+            cluster_sums(mine, tot, lower);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) v[q] += lower[q];
+        }
     }
 };
-
-__device__ __forceinline__ uint32_t to_frac32(ull part, ull whole)
-{
-    int sh = bit_length(whole) - 32;
-    if (sh < 0) sh = 0;
-    const ull q = ((part >> sh) << 32) / (whole >> sh);
-    return q > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)q;
-}
 
 // to_frac32(part, whole) for many parts <= whole of one whole: the quotient from a double
 // reciprocal of the (shifted) whole, then set right with the exact integer remainder.  The
@@ -129,8 +176,8 @@ __device__ __forceinline__ void store_packed_bin(uint2* out_pk, const uint32_t* 
 // sc_w, sc_de, sc_item: scratch of n entries each, private to this row.
 // out_pk (may be null) receives the packed form of every bin, see store_packed_bin().
 // Returns W44 (the sum of the fixed-point weights) to every thread of the group.
-template <bool BLOCK, class Weight>
-__device__ ull build_alias_row(const Group<BLOCK>& g, int32_t n, Weight weight, ull* __restrict__ sc_w,
+template <GroupKind KIND, class Weight>
+__device__ ull build_alias_row(const Group<KIND>& g, int32_t n, Weight weight, ull* __restrict__ sc_w,
                                ull* __restrict__ sc_de, uint32_t* __restrict__ sc_item,
                                uint32_t* __restrict__ out_thr, uint32_t* __restrict__ out_idx,
                                uint2* __restrict__ out_pk, const uint32_t* __restrict__ pk_topic, int* err)
@@ -307,21 +354,68 @@ struct SparseWeight {
     }
 };
 
+// First kernel of a sweep: the dense smoothing table.  Also moves the device's sweep counter on and
+// clears the n_k buffer the sweep's rebuild will add into (nothing else of this sweep touches either).
+// One CTA builds a table of up to DENSE_CTA_MAX_K topics; a larger one takes a cluster of DENSE_CLUSTER
+// CTAs, whose passes over the table meet at cluster barriers: what bounds the kernel is the
+// latency of a few dependent passes over K items, so threads, not bytes, are what it is short of.
+constexpr int DENSE_CTA_MAX_K = 2048;
+constexpr int DENSE_CLUSTER = 8;
+template <GroupKind KIND>
 __global__ void __launch_bounds__(1024) k_alias_dense(View v, ull* sc)
 {
-    __shared__ ull smem[99];
-    Group<true> g{smem};
+    __shared__ ull smem[GROUP_SMEM];
+    Group<KIND> g{smem};
     const int32_t K = v.K;
+    if (v.state && g.rank() == 0) {
+        SweepState& st = *v.state;
+        const uint32_t slot = st.next_slot;
+        st.sweep = st.next;
+        st.next += 1;
+        st.slot = slot;
+        st.next_slot = slot + 1;
+        st.stamps[slot][STAMP_DENSE] = global_timer();
+    }
+    if (v.nk_next)
+        for (int32_t k = g.rank(); k < v.dense_stride; k += g.size()) v.nk_next[k] = 0;
     DenseWeight wf{v.nk, v.beta, v.Vbeta};
-    const ull B = build_alias_row<true>(g, K, wf, sc, sc + K, (uint32_t*)(sc + 2 * (size_t)K), v.dn_thr,
+    const ull B = build_alias_row<KIND>(g, K, wf, sc, sc + K, (uint32_t*)(sc + 2 * (size_t)K), v.dn_thr,
                                         v.dn_idx, v.dn_pk, nullptr, v.err);
-    if (threadIdx.x == 0) *v.dense_mass = B;
+    if (g.rank() == 0) {
+        *v.dense_mass = B;
+        if (v.state) v.state->stamps[v.state->slot][STAMP_DENSE_END] = global_timer();
+    }
 }
 
-__device__ __forceinline__ uint32_t mixture_threshold(ull S, ull B)
+static cudaError_t run_alias_dense(const View& v, ull* scratch, cudaStream_t stream)
 {
-    if (S == 0) return 0;
-    return to_frac32(S, S + B);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    const int ctas = v.K > DENSE_CTA_MAX_K ? DENSE_CLUSTER : 1;
+    int threads = 64;  // about an item per thread
+    while (threads < 1024 && threads * ctas < v.K) threads <<= 1;
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = stream;
+    if (ctas == 1) return cudaLaunchKernelEx(&cfg, k_alias_dense<CTA>, v, scratch);
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = DENSE_CLUSTER;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_alias_dense<CLUSTER>, v, scratch);
+}
+
+// Mixture thresholds as lda_get_tables() reports them (the proposal pass works its tiles' out itself).
+__global__ void __launch_bounds__(256) k_mix_thresholds(View v, uint32_t* __restrict__ mix32)
+{
+    const int32_t w = blockIdx.x * blockDim.x + threadIdx.x;
+    if (w < v.V) mix32[w] = mixture_threshold(v.sp_mass[w], *v.dense_mass);
+}
+
+void launch_mix_thresholds(Ctx& c, uint32_t* mix32)
+{
+    k_mix_thresholds<<<(c.V + 255) / 256, 256, 0, c.stream>>>(c.v, mix32);
 }
 
 // One warp per word, rows of at most ALIAS_WARP_MAX items.  The two scratch arrays the binary
@@ -330,25 +424,24 @@ __device__ __forceinline__ uint32_t mixture_threshold(ull S, ull B)
 __global__ void __launch_bounds__(256) k_alias_sparse_warp(View v, ull* sc_w, int32_t w_lo, int32_t w_hi)
 {
     extern __shared__ __align__(16) unsigned char alias_scratch[];
-    Group<false> g{nullptr};
+    Group<WARP> g{nullptr};
     const int warps = (gridDim.x * blockDim.x) >> 5;
     const int wic = threadIdx.x >> 5;
     ull* de_s = reinterpret_cast<ull*>(alias_scratch) + (size_t)wic * ALIAS_WARP_MAX;
     uint32_t* item_s = reinterpret_cast<uint32_t*>(reinterpret_cast<ull*>(alias_scratch) + 8 * ALIAS_WARP_MAX) +
                        (size_t)wic * ALIAS_WARP_MAX;
-    const ull B = *v.dense_mass;
     for (int32_t w = w_lo + ((blockIdx.x * blockDim.x + threadIdx.x) >> 5); w < w_hi; w += warps) {
         const int32_t n = v.wk_nnz[w];
         if (n > ALIAS_WARP_MAX) continue;
         if (n == 0) {
-            if ((threadIdx.x & 31) == 0) v.mix32[w] = 0;
+            if ((threadIdx.x & 31) == 0) v.sp_mass[w] = 0;
             continue;
         }
         const int32_t r0 = v.row_start[w];
         SparseWeight wf{v.wk_topic + r0, v.wk_count + r0, v.nk, v.Vbeta};
-        const ull S = build_alias_row<false>(g, n, wf, sc_w + r0, de_s, item_s, v.al_thr + r0, v.al_idx + r0,
+        const ull S = build_alias_row<WARP>(g, n, wf, sc_w + r0, de_s, item_s, v.al_thr + r0, v.al_idx + r0,
                                              v.al_pk ? v.al_pk + r0 : nullptr, v.wk_topic + r0, v.err);
-        if ((threadIdx.x & 31) == 0) v.mix32[w] = mixture_threshold(S, B);
+        if ((threadIdx.x & 31) == 0) v.sp_mass[w] = S;
         __syncwarp();
     }
 }
@@ -367,8 +460,8 @@ k_alias_sparse_block(View v, const int32_t* __restrict__ words, ull* sc_w, ull* 
                      int32_t smem_items)
 {
     extern __shared__ __align__(16) unsigned char alias_scratch[];
-    __shared__ ull smem[99];
-    Group<true> g{smem};
+    __shared__ ull smem[GROUP_SMEM];
+    Group<CTA> g{smem};
     const int32_t w = words[blockIdx.x];
     const int32_t n = v.wk_nnz[w];
     if (n <= ALIAS_WARP_MAX) return;
@@ -380,20 +473,25 @@ k_alias_sparse_block(View v, const int32_t* __restrict__ words, ull* sc_w, ull* 
         ull* w_s = reinterpret_cast<ull*>(alias_scratch);
         ull* de_s = w_s + smem_items;
         uint32_t* item_s = reinterpret_cast<uint32_t*>(de_s + smem_items);
-        S = build_alias_row<true>(g, n, wf, w_s, de_s, item_s, v.al_thr + r0, v.al_idx + r0, pk, v.wk_topic + r0, v.err);
+        S = build_alias_row<CTA>(g, n, wf, w_s, de_s, item_s, v.al_thr + r0, v.al_idx + r0, pk, v.wk_topic + r0, v.err);
     } else if ((int64_t)n * 8 <= (int64_t)smem_items * ALIAS_SCRATCH_PER_ITEM) {
-        S = build_alias_row<true>(g, n, wf, sc_w + r0, reinterpret_cast<ull*>(alias_scratch), sc_item + r0,
+        S = build_alias_row<CTA>(g, n, wf, sc_w + r0, reinterpret_cast<ull*>(alias_scratch), sc_item + r0,
                                   v.al_thr + r0, v.al_idx + r0, pk, v.wk_topic + r0, v.err);
     } else {
-        S = build_alias_row<true>(g, n, wf, sc_w + r0, sc_de + r0, sc_item + r0, v.al_thr + r0, v.al_idx + r0, pk,
+        S = build_alias_row<CTA>(g, n, wf, sc_w + r0, sc_de + r0, sc_item + r0, v.al_thr + r0, v.al_idx + r0, pk,
                                   v.wk_topic + r0, v.err);
     }
-    if (threadIdx.x == 0) v.mix32[w] = mixture_threshold(S, *v.dense_mass);
+    if (threadIdx.x == 0) v.sp_mass[w] = S;
 }
 
-int launch_alias_dense(Ctx& c)
+int launch_alias_dense(Ctx& c, bool in_sweep)
 {
-    k_alias_dense<<<1, 1024, 0, c.stream>>>(c.v, c.sc_dense);
+    View v = c.v;
+    if (!in_sweep) {  // the table alone: no sweep begins
+        v.state = nullptr;
+        v.nk_next = nullptr;
+    }
+    run_alias_dense(v, c.sc_dense, c.stream);
     return 1;
 }
 
@@ -513,7 +611,9 @@ extern "C" int lda_dense_table_noalloc(const int32_t* n_k_dev, int32_t K, int32_
     v.dn_idx = (uint32_t*)dn_alias_dev;
     v.dense_mass = (unsigned long long*)dense_mass_dev;
     v.err = status;
-    k_alias_dense<<<1, 1024, 0, st>>>(v, addr->scratch);
-    if (cudaGetLastError() != cudaSuccess) return LDA_ECUDA;
+    if (run_alias_dense(v, addr->scratch, st) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
+        cudaGetLastError();
+        return LDA_ECUDA;
+    }
     return LDA_OK;
 }

@@ -2,6 +2,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include "lda_internal.cuh"
@@ -72,6 +73,92 @@ void dev_free_all(Ctx& c)
     c.device_bytes = 0;
 }
 
+// Host memory the device writes sweep reports to.  Blocks are handed from one context to the next (a
+// new one costs tens of microseconds of driver time); at most REPORTS_KEPT idle ones are kept.
+struct ReportPool {
+    static constexpr size_t REPORTS_KEPT = 4;
+    std::mutex lock;
+    std::vector<SweepReport*> idle;
+    SweepReport* take()
+    {
+        {
+            std::lock_guard<std::mutex> g(lock);
+            if (!idle.empty()) {
+                SweepReport* r = idle.back();
+                idle.pop_back();
+                return r;
+            }
+        }
+        void* p = nullptr;
+        if (cudaHostAlloc(&p, sizeof(SweepReport), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return static_cast<SweepReport*>(p);
+    }
+    void give(SweepReport* r)
+    {
+        if (!r) return;
+        {
+            std::lock_guard<std::mutex> g(lock);
+            if (idle.size() < REPORTS_KEPT) {
+                idle.push_back(r);
+                return;
+            }
+        }
+        cudaFreeHost(r);
+    }
+};
+static ReportPool& report_pool()
+{
+    static ReportPool* pool = new ReportPool;  // never destroyed: contexts may outlive static objects
+    return *pool;
+}
+
+__global__ void k_set_state(SweepState* st, uint32_t sweep)
+{
+    unsigned long long* stamps = &st->stamps[0][0];
+    for (int i = threadIdx.x; i < STAMP_RING * STAMPS; i += blockDim.x) stamps[i] = 0;
+    if (threadIdx.x == 0) {
+        st->moves[0] = st->moves[1] = 0;
+        st->next = sweep;
+        st->next_slot = 0;
+    }
+}
+
+// After a batch of sweeps: what the host wants to know goes to host memory, the rest is made ready
+// for the next batch.  One CTA; runs after the batch's last kernel.
+__global__ void k_report(SweepState* st, SweepReport* rep)
+{
+    const uint32_t n = st->next_slot;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        rep->end = global_timer();
+        rep->moves[0] = st->moves[0];
+        rep->moves[1] = st->moves[1];
+        rep->err = st->err;
+        st->moves[0] = st->moves[1] = 0;
+        st->err = 0;
+        st->next_slot = 0;
+    }
+    for (uint32_t i = threadIdx.x; i < n * STAMPS; i += blockDim.x) {
+        (&rep->stamps[0][0])[i] = (&st->stamps[0][0])[i];
+        (&st->stamps[0][0])[i] = 0;
+    }
+}
+
+void launch_set_state(Ctx& c) { k_set_state<<<1, 128, 0, c.stream>>>(c.v.state, c.sweep); }
+void launch_report(Ctx& c) { k_report<<<1, 128, 0, c.stream>>>(c.v.state, c.report); }
+
+static void drop_graphs(Ctx& c)
+{
+    for (cudaGraphExec_t& g : c.graph) {
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
+    }
+    c.plain_sweeps = 0;
+}
+
 static int fail(Ctx* c, int code, const char* msg)
 {
     if (c) c->err = msg;
@@ -138,19 +225,19 @@ static void free_corpus(Ctx& c)
 {
     if (c.copy) cudaStreamSynchronize(c.copy);  // an export may still read the staging buffer
     c.export_pending = false;
-    int* err = c.v.err;
-    // the error word is allocated in lda_create and outlives corpora
+    drop_graphs(c);
+    // the sweep state is allocated in lda_create and outlives corpora
     std::vector<void*> drop;
     for (void* p : c.allocs)
-        if (p != (void*)err) drop.push_back(p);
+        if (p != (void*)c.v.state) drop.push_back(p);
     for (void* p : drop) dev_free(c, p);
     View nv{};
     nv.V = c.V; nv.K = c.K; nv.alpha = c.alpha; nv.beta = c.beta;
     nv.Vbeta = (double)c.V * c.beta;
     nv.Kalpha = (double)c.K * c.alpha;
     nv.dense_stride = (c.K + 3) & ~3;
-    nv.err = err;
-    nv.moves = c.v.moves;
+    nv.state = c.v.state;
+    nv.err = &nv.state->err;
     c.v = nv;
     c.loaded = c.inited = c.tables_valid = false;
     c.N = c.D = 0;
@@ -210,6 +297,7 @@ int lda::ensure_exchange(Ctx& c, int mh_steps)
         return LDA_OK;
     }
     cudaStreamSynchronize(c.stream);
+    drop_graphs(c);
     dev_free(c, c.v.prop);
     dev_free(c, c.v.dside);
     dev_free(c, c.v.ua_w);
@@ -233,19 +321,103 @@ int lda::ensure_exchange(Ctx& c, int mh_steps)
 
 namespace lda {
 
-static int rebuild_counts(Ctx& c, int64_t* launches)
+void rebuild_counts(Ctx& c)
 {
-    int n = launch_count_wk(c);
-    n += launch_count_k(c);
-    if (launches) *launches += n;
+    cudaMemsetAsync(c.v.nk_next, 0, (size_t)c.v.dense_stride * 4, c.stream);
+    launch_count_wk(c);
+    launch_count_k(c);
+    exchange_nk(c);
     c.tables_valid = false;
-    return LDA_OK;
+}
+
+// One sweep, kernel by kernel.  Returns the number of kernels.
+static int queue_sweep(Ctx& c, int mh_steps)
+{
+    int n = launch_alias_dense(c, true);
+    if (c.slices.size() == 1) n += launch_alias_sparse(c);  // else slice by slice inside pass 1
+    n += launch_sample(c, mh_steps);
+    n += launch_count_wk(c);
+    n += launch_count_k(c);
+    return n;
+}
+
+// The same as a graph: the launches of a sweep and the waits between its streams are worked out once
+// and cost the host one call.  Worth it from the third sweep of a configuration on (building it takes
+// as long as launching a handful of sweeps kernel by kernel).  False: launch it kernel by kernel.
+constexpr int GRAPH_AFTER = 2;
+static bool replay_sweep(Ctx& c, int mh_steps)
+{
+    if (c.graph_refused) return false;
+    if (c.graph_steps != mh_steps || c.graph_mode != c.proposals || c.graph_seed != c.seed) {
+        drop_graphs(c);
+        c.graph_steps = mh_steps;
+        c.graph_mode = c.proposals;
+        c.graph_seed = c.seed;
+    }
+    if (c.plain_sweeps < GRAPH_AFTER) {
+        ++c.plain_sweeps;
+        return false;
+    }
+    cudaGraphExec_t& exec = c.graph[c.v.nk < c.v.nk_next ? 0 : 1];
+    if (!exec) {
+        cudaGraph_t graph = nullptr;
+        if (!c.capture && cudaStreamCreateWithFlags(&c.capture, cudaStreamNonBlocking) != cudaSuccess) c.capture = nullptr;
+        bool ok = c.capture && cudaStreamBeginCapture(c.capture, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+        if (ok) {
+            const cudaStream_t stream = c.stream;
+            c.stream = c.capture;
+            c.graph_launches = queue_sweep(c, mh_steps);
+            c.stream = stream;
+            ok = cudaStreamEndCapture(c.capture, &graph) == cudaSuccess && graph &&
+                 cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess;
+        }
+        if (graph) cudaGraphDestroy(graph);
+        if (!ok) {
+            cudaGetLastError();
+            exec = nullptr;
+            c.graph_refused = true;
+            return false;
+        }
+    }
+    return cudaGraphLaunch(exec, c.stream) == cudaSuccess;
+}
+
+// Phase times of a batch of sweeps from the start stamps of their kernels.
+static void add_phase_times(const Ctx& c, const SweepReport& r, int batch, lda_stats& s)
+{
+    auto first_of = [](unsigned long long a, unsigned long long b, unsigned long long otherwise) {
+        if (!a || (b && b < a)) a = b;
+        return a ? a : otherwise;
+    };
+    for (int b = 0; b < batch; ++b) {
+        const unsigned long long* t = r.stamps[b];
+        const unsigned long long end = b + 1 < batch ? r.stamps[b + 1][STAMP_DENSE] : r.end;
+        const unsigned long long begin = t[STAMP_DENSE];
+        const unsigned long long nk = first_of(t[STAMP_NK_DENSE], t[STAMP_NK_SPARSE], end);
+        const unsigned long long wk = first_of(first_of(t[STAMP_ROWS], t[STAMP_WARM_ROWS], 0), t[STAMP_HIST], nk);
+        const unsigned long long acc = first_of(first_of(t[STAMP_ACCEPT_HOT], t[STAMP_ACCEPT_WARM], 0), t[STAMP_ACCEPT_COLD], wk);
+        const unsigned long long doc = first_of(t[STAMP_DOC_TILES], t[STAMP_DOC_LONG], acc);
+        const unsigned long long pro = first_of(t[STAMP_PROPOSE_HOT], t[STAMP_PROPOSE_COLD],
+                                                c.slices.size() > 1 ? t[STAMP_DENSE_END] : doc);
+        auto ms = [](unsigned long long from, unsigned long long to) { return to > from ? 1e-6f * (float)(to - from) : 0.f; };
+        // the sparse tables are built beside the dense one
+        const unsigned long long dense_end = std::min(t[STAMP_DENSE_END], pro);
+        s.ms_alias_dense += ms(begin, dense_end);
+        s.ms_alias_sparse += ms(dense_end, pro);
+        s.ms_propose += ms(pro, doc);
+        s.ms_doc_side += ms(doc, acc);
+        s.ms_accept += ms(acc, wk);
+        s.ms_sample += ms(pro, wk);
+        s.ms_count_wk += ms(wk, nk);
+        s.ms_count_k += ms(nk, end);
+        s.ms_total += ms(begin, end);
+    }
 }
 
 static int ensure_tables(Ctx& c)
 {
     if (c.tables_valid) return LDA_OK;
-    launch_alias_dense(c);
+    launch_alias_dense(c, false);
     launch_alias_sparse(c);  // the running slice's (lda_get_tables walks the slices itself)
     int bits = 0;
     int rc = read_err(c, &bits);
@@ -517,11 +689,13 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.al_idx0 = (uint32_t*)A(cap_alias * 4);
     c.al_pk0 = c.wide_topics ? nullptr : (uint2*)A(cap_alias * 8);
     v.dn_pk = (uint2*)A((size_t)K * 8);
-    v.mix32 = (uint32_t*)A((size_t)V * 4);
+    v.sp_mass = (unsigned long long*)A((size_t)V * 8);
+    c.mix32 = (uint32_t*)A((size_t)V * 4);
     v.dn_thr = (uint32_t*)A((size_t)K * 4);
     v.dn_idx = (uint32_t*)A((size_t)K * 4);
     v.dense_mass = (unsigned long long*)A(8);
-    v.nk = (int32_t*)A((size_t)v.dense_stride * 4);  // padded like a dense row: copied in 16-byte units
+    v.nk = (int32_t*)A((size_t)v.dense_stride * 8);  // two, padded like a dense row: copied in 16-byte units
+    v.nk_next = v.nk ? v.nk + v.dense_stride : nullptr;
     // scratch tables of the documents longer than a tile: four slots per token, one document after the other
     std::vector<long long> long_slot_off(long_docs.size() + 1, 0);
     for (size_t i = 0; i < long_docs.size(); ++i)
@@ -542,8 +716,8 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     if (!ok) { free_corpus(c); return fail(&c, LDA_ENOMEM, "device allocation failed"); }
     set_slice(c, 0);
     cudaMemsetAsync(v.wk_nnz, 0, (size_t)V * 4, c.stream);
-    cudaMemsetAsync(v.mix32, 0, (size_t)V * 4, c.stream);
-    cudaMemsetAsync(v.nk, 0, (size_t)K * 4, c.stream);
+    cudaMemsetAsync(v.sp_mass, 0, (size_t)V * 8, c.stream);
+    cudaMemsetAsync(v.nk, 0, (size_t)v.dense_stride * 8, c.stream);
     if (cudaStreamSynchronize(c.stream) != cudaSuccess) { free_corpus(c); return cuda_fail(&c, "load"); }
     c.stats = lda_stats{};
     c.stats.n_tokens = N;
@@ -597,23 +771,16 @@ int lda_create(int32_t V, int32_t K, double alpha, double beta, lda_ctx** out)
     c.v.Vbeta = (double)V * beta;
     c.v.Kalpha = (double)K * alpha;
     c.v.dense_stride = (K + 3) & ~3;
-    c.v.err = (int*)dev_alloc(c, 32);  // the error word and, 16 bytes on, the two move counters
-    c.v.moves = c.v.err ? reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(c.v.err) + 16) : nullptr;
-    if (!c.v.err || cudaMemset(c.v.err, 0, 32) != cudaSuccess) {
+    c.v.state = (SweepState*)dev_alloc(c, sizeof(SweepState));
+    c.v.err = c.v.state ? &c.v.state->err : nullptr;
+    c.report = report_pool().take();
+    if (!c.v.state || !c.report || cudaMemset(c.v.state, 0, sizeof(SweepState)) != cudaSuccess) {
+        report_pool().give(c.report);
         dev_free_all(c);
         delete h;
         cudaGetLastError();
         return LDA_ECUDA;
     }
-    for (int i = 0; i < Ctx::EV_RING * 10; ++i)
-        if (cudaEventCreate(&c.ev_ring[i / 10][i % 10]) != cudaSuccess) {
-            for (int j = 0; j < i; ++j) cudaEventDestroy(c.ev_ring[j / 10][j % 10]);
-            dev_free_all(c);
-            delete h;
-            cudaGetLastError();
-            return LDA_ECUDA;
-        }
-    c.have_events = true;
     {
         bool ok = cudaEventCreateWithFlags(&c.ev_fork, cudaEventDisableTiming) == cudaSuccess;
         for (int i = 0; i < 2 && ok; ++i)
@@ -661,8 +828,9 @@ void lda_destroy(lda_ctx* h)
         if (c.ev_chunk) cudaEventDestroy(c.ev_chunk);
         if (c.ev_export) cudaEventDestroy(c.ev_export);
     }
-    if (c.have_events)
-        for (int i = 0; i < Ctx::EV_RING * 10; ++i) cudaEventDestroy(c.ev_ring[i / 10][i % 10]);
+    drop_graphs(c);
+    if (c.capture) cudaStreamDestroy(c.capture);
+    report_pool().give(c.report);
     dev_free_all(c);
     cudaGetLastError();
     delete h;
@@ -784,8 +952,9 @@ int lda_init(lda_ctx* h, uint64_t seed)
     order_after_export(c);
     c.seed = seed;
     c.sweep = 0;
+    launch_set_state(c);
     launch_init(c);
-    rebuild_counts(c, nullptr);
+    rebuild_counts(c);
     int bits = 0;
     if ((rc = read_err(c, &bits))) return rc;
     if (bits) return fail(&c, LDA_EINTERNAL, "count rebuild raised the device error word");
@@ -827,7 +996,8 @@ static int set_assignments(lda_ctx* h, const void* z, bool narrow, uint64_t seed
     if (bits & ERR_TOPIC_RANGE) { c.inited = false; return fail(&c, LDA_ERANGE, "assignment outside [0,K)"); }
     c.seed = seed;
     c.sweep = sweep;
-    rebuild_counts(c, nullptr);
+    launch_set_state(c);
+    rebuild_counts(c);
     if ((rc = read_err(c, &bits))) return rc;
     if (bits) return fail(&c, LDA_EINTERNAL, "count rebuild raised the device error word");
     c.inited = true;
@@ -861,69 +1031,42 @@ int lda_sweep(lda_ctx* h, int32_t iters, int32_t mh_steps)
     s.kernel_launches = 0;
     s.iters = iters;
     s.word_proposed = s.word_accepted = s.doc_proposed = s.doc_accepted = 0;
-    if (cudaMemsetAsync(c.v.moves, 0, 16, c.stream) != cudaSuccess) return cuda_fail(&c, "clearing the move counters");
-    // Iterations are queued without waiting for each other; the host waits once per EV_RING of them
-    // (and after the last) to read the error word, the move counters and the phase timings.
-    for (int32_t it0 = 0; it0 < iters; it0 += Ctx::EV_RING) {
-        const int32_t batch = std::min<int32_t>(Ctx::EV_RING, iters - it0);
+    // Iterations are queued without waiting for each other; the host waits once per STAMP_RING of them
+    // (and after the last) for the error word, the move counters and the phase times.
+    for (int32_t it0 = 0; it0 < iters; it0 += STAMP_RING) {
+        const int32_t batch = std::min<int32_t>(STAMP_RING, iters - it0);
         for (int32_t b = 0; b < batch; ++b) {
-            c.ev = c.ev_ring[b];
-            int64_t n = 0;
-            cudaEventRecord(c.ev[0], c.stream);
-            n += launch_alias_dense(c);
-            cudaEventRecord(c.ev[1], c.stream);
-            if (c.slices.size() == 1) n += launch_alias_sparse(c);  // else slice by slice inside pass 1
-            cudaEventRecord(c.ev[2], c.stream);
-            n += launch_sample(c, mh_steps);
-            cudaEventRecord(c.ev[3], c.stream);
-            n += launch_count_wk(c);
-            cudaEventRecord(c.ev[4], c.stream);
-            n += launch_count_k(c);
-            cudaEventRecord(c.ev[5], c.stream);
-            cudaEventRecord(c.ev[6], c.stream);  // n_kd is rebuilt inside the next MH step, per tile
+            s.kernel_launches += replay_sweep(c, mh_steps) ? c.graph_launches : queue_sweep(c, mh_steps);
+            exchange_nk(c);
             c.tables_valid = false;
             c.sweep += 1;
-            s.kernel_launches += n;
         }
-        c.ev = c.ev_ring[0];
-        int bits = 0;
-        if ((rc = read_err(c, &bits))) { c.inited = false; return rc; }
-        if (bits) {
+        launch_report(c);
+        ++s.kernel_launches;
+        cudaError_t e = cudaStreamSynchronize(c.stream);
+        if (e == cudaSuccess) e = cudaGetLastError();
+        if (e != cudaSuccess) {
+            c.inited = false;
+            c.err = std::string("sweep: ") + cudaGetErrorString(e);
+            return LDA_ECUDA;
+        }
+        const SweepReport& r = *c.report;
+        if (r.err) {
             // some iteration of this batch met inconsistent tables: the state is not to be trusted
             c.inited = false;
-            c.err = "a kernel raised the device error word: " + std::to_string(bits) +
+            c.err = "a kernel raised the device error word: " + std::to_string(r.err) +
                     " (call lda_init or lda_set_assignments again)";
             return LDA_EINTERNAL;
         }
-        for (int32_t b = 0; b < batch; ++b) {
-            cudaEvent_t* ev = c.ev_ring[b];
-            float ms[7] = {0};
-            for (int i = 0; i < 6; ++i) cudaEventElapsedTime(&ms[i], ev[i], ev[i + 1]);
-            cudaEventElapsedTime(&ms[6], ev[0], ev[6]);
-            if (c.N > 0) {
-                float a = 0.f, bb = 0.f, d = 0.f;
-                cudaEventElapsedTime(&a, ev[2], ev[8]);
-                cudaEventElapsedTime(&bb, ev[8], ev[9]);
-                cudaEventElapsedTime(&d, ev[9], ev[3]);
-                s.ms_propose += a; s.ms_doc_side += bb; s.ms_accept += d;
-            }
-            s.ms_alias_dense += ms[0]; s.ms_alias_sparse += ms[1]; s.ms_sample += ms[2];
-            s.ms_count_wk += ms[3]; s.ms_count_k += ms[4]; s.ms_count_dk += ms[5]; s.ms_total += ms[6];
-        }
+        add_phase_times(c, r, batch, s);
+        s.word_accepted += (int64_t)r.moves[0];
+        s.doc_accepted += (int64_t)r.moves[1];
     }
-    {
-        unsigned long long moves[2] = {0, 0};
-        if (cudaMemcpyAsync(moves, c.v.moves, 16, cudaMemcpyDeviceToHost, c.stream) != cudaSuccess ||
-            cudaStreamSynchronize(c.stream) != cudaSuccess)
-            return cuda_fail(&c, "reading the move counters");
-        const int64_t n_word = c.proposals == LDA_PROPOSALS_CYCLE  ? (mh_steps + 1) / 2
-                               : c.proposals == LDA_PROPOSALS_WORD ? mh_steps
-                                                                   : 0;
-        s.word_proposed = (int64_t)iters * c.N * n_word;
-        s.doc_proposed = (int64_t)iters * c.N * (mh_steps - n_word);
-        s.word_accepted = (int64_t)moves[0];
-        s.doc_accepted = (int64_t)moves[1];
-    }
+    const int64_t n_word = c.proposals == LDA_PROPOSALS_CYCLE  ? (mh_steps + 1) / 2
+                           : c.proposals == LDA_PROPOSALS_WORD ? mh_steps
+                                                               : 0;
+    s.word_proposed = (int64_t)iters * c.N * n_word;
+    s.doc_proposed = (int64_t)iters * c.N * (mh_steps - n_word);
     return LDA_OK;
 }
 
@@ -1167,7 +1310,7 @@ int lda_get_tables(lda_ctx* h, uint32_t* sp_thr32, int32_t* sp_alias, int64_t ca
         if ((rc = ensure_tables(c))) return rc;
     } else {
         c.tables_valid = false;
-        launch_alias_dense(c);
+        launch_alias_dense(c, false);
     }
     for (size_t sl = 0; sl < c.slices.size(); ++sl) {
         const Ctx::Slice& q = c.slices[sl];
@@ -1183,7 +1326,12 @@ int lda_get_tables(lda_ctx* h, uint32_t* sp_thr32, int32_t* sp_alias, int64_t ca
              cudaMemcpy(b.data() + q.row_lo, c.al_idx0, (size_t)q.row_n * 4, cudaMemcpyDeviceToHost) != cudaSuccess))
             return cuda_fail(&c, "copy");
     }
-    if (mix32 && cudaMemcpy(mix32, v.mix32, V * 4, cudaMemcpyDeviceToHost) != cudaSuccess) return cuda_fail(&c, "copy");
+    if (mix32) {
+        launch_mix_thresholds(c, c.mix32);
+        if (cudaStreamSynchronize(c.stream) != cudaSuccess ||
+            cudaMemcpy(mix32, c.mix32, V * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
+            return cuda_fail(&c, "copy");
+    }
     if (dn_thr32 && cudaMemcpy(dn_thr32, v.dn_thr, K * 4, cudaMemcpyDeviceToHost) != cudaSuccess) return cuda_fail(&c, "copy");
     if (dn_alias && cudaMemcpy(dn_alias, v.dn_idx, K * 4, cudaMemcpyDeviceToHost) != cudaSuccess) return cuda_fail(&c, "copy");
     if (dense_mass && cudaMemcpy(dense_mass, v.dense_mass, 8, cudaMemcpyDeviceToHost) != cudaSuccess) return cuda_fail(&c, "copy");

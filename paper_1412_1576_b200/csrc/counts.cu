@@ -41,8 +41,10 @@ struct EmitWord {
 template <typename T, class Emit>
 __global__ void __launch_bounds__(256)
 k_seg_count_sorted(const int32_t* __restrict__ tiles, const int32_t* __restrict__ seg_off,
-                   const T* __restrict__ z, int topic_bits, int32_t K, Emit emit, int* err)
+                   const T* __restrict__ z, int topic_bits, int32_t K, Emit emit, SweepState* state, int stamp_id)
 {
+    stamp(state, stamp_id);
+    int* const err = &state->err;
     __shared__ uint32_t keys[SORT_TILE];
     __shared__ int32_t soff[SORT_TILE + 1];
     __shared__ int32_t hidx[SORT_TILE + 1];
@@ -132,8 +134,10 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 k_word_rows(const int32_t* __restrict__ tiles, const int32_t* __restrict__ word_off, const T* __restrict__ z,
             const int32_t* __restrict__ row_start, uint32_t* __restrict__ wk_topic, uint32_t* __restrict__ wk_count,
-            int32_t* __restrict__ wk_nnz, int32_t K, int* err)
+            int32_t* __restrict__ wk_nnz, int32_t K, SweepState* state)
 {
+    stamp(state, STAMP_ROWS);
+    int* const err = &state->err;
     constexpr int CB = 12;  // count bits of a table entry: a tail word has at most SORT_TILE = 2048 tokens
     static_assert(SORT_TILE < (1 << CB), "count bits");
     extern __shared__ uint32_t word_smem[];
@@ -223,8 +227,10 @@ template <typename T>
 __global__ void __launch_bounds__(512)
 k_warm_rows(const int32_t* __restrict__ words, const int32_t* __restrict__ word_off, const T* __restrict__ z,
             const int32_t* __restrict__ row_start, uint32_t* __restrict__ wk_topic, uint32_t* __restrict__ wk_count,
-            int32_t* __restrict__ wk_nnz, int32_t K, int32_t window, int* err)
+            int32_t* __restrict__ wk_nnz, int32_t K, int32_t window, SweepState* state)
 {
+    stamp(state, STAMP_WARM_ROWS);
+    int* const err = &state->err;
     extern __shared__ __align__(16) uint32_t bins2[];
     __shared__ int32_t warp_total[17];
     const int32_t w = words[blockIdx.x];
@@ -298,8 +304,10 @@ template <typename T>
 __global__ void __launch_bounds__(512)
 k_hist_chunks(const int32_t* __restrict__ chunks, const T* __restrict__ z,
               const int32_t* __restrict__ dense_slot, int32_t* __restrict__ dense_rows, int32_t K,
-              int32_t stride, int32_t window, int* err)
+              int32_t stride, int32_t window, SweepState* state)
 {
+    stamp(state, STAMP_HIST);
+    int* const err = &state->err;
     extern __shared__ __align__(16) int32_t hist_bins[];
     const int32_t w = chunks[4 * blockIdx.x], first = chunks[4 * blockIdx.x + 1],
                   cnt = chunks[4 * blockIdx.x + 2];
@@ -393,8 +401,9 @@ k_compact_dense(const int32_t* __restrict__ dense_words, const int32_t* __restri
 //     of words, flushed with one global add per nonzero bin.
 __global__ void __launch_bounds__(256)
 k_nk_from_dense(const int32_t* __restrict__ dense_rows, int32_t n_dense, int32_t K, int32_t stride,
-                int32_t* __restrict__ nk)
+                int32_t* __restrict__ nk, SweepState* state)
 {
+    stamp(state, STAMP_NK_DENSE);
     // four consecutive topics per thread (rows are padded to a multiple of four and 16-byte aligned;
     // the padding is never written, so it reads as zero), a slice of the rows per blockIdx.y
     const int32_t k = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -415,8 +424,9 @@ __global__ void __launch_bounds__(512)
 k_nk_from_sparse(const int32_t* __restrict__ row_start, const int32_t* __restrict__ wk_nnz,
                  const uint32_t* __restrict__ wk_topic, const uint32_t* __restrict__ wk_count,
                  const int32_t* __restrict__ dense_slot, int32_t V, int32_t* __restrict__ nk, int32_t K,
-                 int32_t window)
+                 int32_t window, SweepState* state)
 {
+    stamp(state, STAMP_NK_SPARSE);
     extern __shared__ int32_t bins[];
     const int32_t per = (V + gridDim.x - 1) / gridDim.x;
     const int32_t w_lo = per * blockIdx.x, w_hi = min(V, w_lo + per);
@@ -447,8 +457,9 @@ k_nk_from_sparse(const int32_t* __restrict__ row_start, const int32_t* __restric
 __global__ void __launch_bounds__(256)
 k_nk_from_sparse_direct(const int32_t* __restrict__ row_start, const int32_t* __restrict__ wk_nnz,
                         const uint32_t* __restrict__ wk_topic, const uint32_t* __restrict__ wk_count,
-                        const int32_t* __restrict__ dense_slot, int32_t V, int32_t* __restrict__ nk)
+                        const int32_t* __restrict__ dense_slot, int32_t V, int32_t* __restrict__ nk, SweepState* state)
 {
+    stamp(state, STAMP_NK_SPARSE);
     const int lane = threadIdx.x & 31;
     const int32_t warps = (gridDim.x * blockDim.x) >> 5;
     for (int32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < V; w += warps) {
@@ -485,10 +496,10 @@ void launch_doc_rows(Ctx& c, const int32_t* tiles, int32_t n_tiles, const T* z, 
 {
     if (nnz)
         k_seg_count_sorted<T, EmitRowSizes><<<n_tiles, 256, 0, c.stream>>>(tiles, c.v.doc_off, z, c.v.topic_bits, c.K,
-                                                                            EmitRowSizes{nnz}, c.v.err);
+                                                                            EmitRowSizes{nnz}, c.v.state, -1);
     else
         k_seg_count_sorted<T, EmitRowEntries><<<n_tiles, 256, 0, c.stream>>>(
-            tiles, c.v.doc_off, z, c.v.topic_bits, c.K, EmitRowEntries{row_off, topic, count}, c.v.err);
+            tiles, c.v.doc_off, z, c.v.topic_bits, c.K, EmitRowEntries{row_off, topic, count}, c.v.state, -1);
 }
 template void launch_doc_rows<uint16_t>(Ctx&, const int32_t*, int32_t, const uint16_t*, int32_t*, const long long*, int32_t*, int32_t*);
 template void launch_doc_rows<int32_t>(Ctx&, const int32_t*, int32_t, const int32_t*, int32_t*, const long long*, int32_t*, int32_t*);
@@ -507,25 +518,25 @@ static int count_wk_t(Ctx& c)
         if (c.K <= WORD_ROWS_BITMAP_MAX_K) {
             const size_t smem = 2 * (size_t)((c.K + 31) / 32) * 4;
             k_word_rows<T><<<c.n_word_tiles, 256, smem, c.side[0]>>>(c.word_tiles, v.word_off, z, v.row_start,
-                                                                    v.wk_topic, v.wk_count, v.wk_nnz, c.K, v.err);
+                                                                    v.wk_topic, v.wk_count, v.wk_nnz, c.K, v.state);
         } else {
             EmitWord e{v.row_start, v.wk_topic, v.wk_count, v.wk_nnz};
             k_seg_count_sorted<T, EmitWord><<<c.n_word_tiles, 256, 0, c.side[0]>>>(
-                c.word_tiles, v.word_off, z, v.topic_bits, c.K, e, v.err);
+                c.word_tiles, v.word_off, z, v.topic_bits, c.K, e, v.state, STAMP_ROWS);
         }
         ++launches;
     }
     if (c.n_warm) {
         const int win = c.K < HIST16_BINS ? c.K : HIST16_BINS;
         k_warm_rows<T><<<c.n_warm, 512, (size_t)((win + 7) / 8) * 16, c.side[1]>>>(
-            c.warm_words, v.word_off, z, v.row_start, v.wk_topic, v.wk_count, v.wk_nnz, c.K, win, v.err);
+            c.warm_words, v.word_off, z, v.row_start, v.wk_topic, v.wk_count, v.wk_nnz, c.K, win, v.state);
         ++launches;
     }
     if (c.n_dense) {
         cudaMemsetAsync(v.dense_rows, 0, (size_t)c.n_dense * v.dense_stride * 4, c.stream);
         const int win = c.K < HIST32_BINS ? c.K : HIST32_BINS;
         k_hist_chunks<T><<<c.n_hist_chunks, 512, (size_t)((win + 3) / 4) * 16, c.stream>>>(
-            c.hist_chunks, z, v.dense_slot, v.dense_rows, c.K, v.dense_stride, win, v.err);
+            c.hist_chunks, z, v.dense_slot, v.dense_rows, c.K, v.dense_stride, win, v.state);
         k_compact_dense<<<c.n_dense, 256, 0, c.stream>>>(c.dense_words, v.dense_slot, v.dense_rows,
                                                          v.row_start, v.wk_topic, v.wk_count,
                                                          v.wk_nnz, c.K, v.dense_stride, v.err);
@@ -535,18 +546,18 @@ static int count_wk_t(Ctx& c)
     return launches;
 }
 
-// Must follow launch_count_wk(): reads the rows it wrote.
+// Must follow launch_count_wk(): reads the rows it wrote and adds into View::nk_next, which the sweep's
+// first kernel (or the caller) has cleared.
 static int count_k(Ctx& c)
 {
     View& v = c.v;
-    cudaMemsetAsync(v.nk, 0, (size_t)c.K * 4, c.stream);
     if (c.N == 0) return 0;
     int launches = 0;
     // both kernels add into n_k (integer adds: any order gives the same sums)
     fork_streams(c);
     if (c.n_dense) {
         const dim3 grid((unsigned)((v.dense_stride / 4 + 255) / 256), (unsigned)std::min(c.n_dense, 256));
-        k_nk_from_dense<<<grid, 256, 0, c.stream>>>(v.dense_rows, c.n_dense, c.K, v.dense_stride, v.nk);
+        k_nk_from_dense<<<grid, 256, 0, c.stream>>>(v.dense_rows, c.n_dense, c.K, v.dense_stride, v.nk_next, v.state);
         ++launches;
     }
     if (c.n_dense < c.V) {
@@ -554,11 +565,11 @@ static int count_k(Ctx& c)
             const int win = hist_window(c);
             const int grid = std::min(148 * 4, (int)((c.V + 255) / 256));
             k_nk_from_sparse<<<grid, 512, (size_t)win * 4, c.side[0]>>>(v.row_start, v.wk_nnz, v.wk_topic, v.wk_count,
-                                                                       v.dense_slot, c.V, v.nk, c.K, win);
+                                                                       v.dense_slot, c.V, v.nk_next, c.K, win, v.state);
         } else {
             const int grid = (int)std::min<int64_t>(148 * 16, ((int64_t)c.V * 32 + 255) / 256);
             k_nk_from_sparse_direct<<<grid, 256, 0, c.side[0]>>>(v.row_start, v.wk_nnz, v.wk_topic, v.wk_count,
-                                                                v.dense_slot, c.V, v.nk);
+                                                                v.dense_slot, c.V, v.nk_next, v.state);
         }
         ++launches;
     }

@@ -44,7 +44,7 @@ __device__ __forceinline__ void load_topic_pair(const int32_t* zbm, uint32_t bm,
 template <typename T, int MODE, int FIXED, int SLOTS, class SlotAt>
 __device__ __forceinline__ void doc_side_token(const View& v, const uint32_t* tab, uint32_t tok, uint32_t doc_len,
                                                uint32_t own, uint32_t t_first, uint32_t bm, const SlotAt& slot_at,
-                                               uint2 key, uint32_t sweep, int32_t mh_steps)
+                                               uint2 key, int32_t mh_steps)
 {
     const uint32_t cap = SLOTS * doc_len;
     const int cb = v.count_bits;
@@ -77,7 +77,7 @@ __device__ __forceinline__ void doc_side_token(const View& v, const uint32_t* ta
     };
     // doc-proposal of step st, the di-th of its kind
     auto doc_step = [&](int32_t st, int32_t di) {
-        const uint4 r = philox4x32_10(make_uint4(v.tok_base + tok, sweep, (uint32_t)st, 0u), key);
+        const uint4 r = philox4x32_10(make_uint4(v.tok_base + tok, running_sweep(v), (uint32_t)st, 0u), key);
         const double uu = __dmul_rn((double)r.x, INV_2_32);
         uint32_t o2;
         if (__dmul_rn(uu, __dadd_rn(n_d, v.Kalpha)) < n_d) {
@@ -119,8 +119,9 @@ __host__ __device__ constexpr int doc_resident_threads(int mode, int fixed)
 }
 template <typename T, int THREADS, int MODE, int FIXED>
 __global__ void __launch_bounds__(THREADS, doc_resident_threads(MODE, FIXED) / THREADS)
-k_doc_tile(View v, const int32_t* __restrict__ tiles, uint2 key, uint32_t sweep, int32_t mh_steps_arg)
+k_doc_tile(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_steps_arg)
 {
+    stamp(v, STAMP_DOC_TILES);
     const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
     constexpr int cap = DOC_TILE_ROUNDS * THREADS;
     extern __shared__ __align__(16) uint32_t doc_smem[];
@@ -184,8 +185,7 @@ k_doc_tile(View v, const int32_t* __restrict__ tiles, uint2 key, uint32_t sweep,
             const uint32_t* tab = slots + TILE_SLOTS * first[r];
             const uint32_t* slot_of = slot_s + first[r];
             auto slot_at = [slot_of](uint32_t jj) { return slot_of[jj]; };
-            doc_side_token<T, MODE, FIXED, TILE_SLOTS>(v, tab, (uint32_t)(base + j), (uint32_t)len[r], tab[z[r]], t1[r], bm[r], slot_at, key,
-                              sweep, mh_steps);
+            doc_side_token<T, MODE, FIXED, TILE_SLOTS>(v, tab, (uint32_t)(base + j), (uint32_t)len[r], tab[z[r]], t1[r], bm[r], slot_at, key, mh_steps);
         }
     }
 }
@@ -195,8 +195,9 @@ k_doc_tile(View v, const int32_t* __restrict__ tiles, uint2 key, uint32_t sweep,
 // one after the other) and the slot indices in its range of the record array.
 template <typename T, int MODE, int FIXED>
 __global__ void __launch_bounds__(512)
-k_long_doc_tile(View v, const int32_t* __restrict__ long_docs, uint2 key, uint32_t sweep, int32_t mh_steps_arg)
+k_long_doc_tile(View v, const int32_t* __restrict__ long_docs, uint2 key, int32_t mh_steps_arg)
 {
+    stamp(v, STAMP_DOC_LONG);
     const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
     const int32_t d = long_docs[blockIdx.x];
     const int32_t first = v.doc_off[d], cnt = v.doc_off[d + 1] - first;
@@ -221,7 +222,7 @@ k_long_doc_tile(View v, const int32_t* __restrict__ long_docs, uint2 key, uint32
     for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
         const uint32_t bm = v.bm_of_tok[first + j];
         doc_side_token<T, MODE, FIXED, DK_SLOTS_PER_TOKEN>(v, tab, (uint32_t)(first + j), (uint32_t)cnt, tab[slot_of[j]], (uint32_t)zbm[2 * (size_t)bm + 1], bm,
-                          slot_at, key, sweep, mh_steps);
+                          slot_at, key, mh_steps);
     }
 }
 
@@ -260,15 +261,15 @@ static int doc_side_tm(Ctx& c, int mh_steps)
     if (c.n_doc_tiles) {
         const size_t smem = doc_tile_smem_bytes(c.doc_tile);
         switch (c.doc_threads) {
-            case 128: k_doc_tile<T, 128, MODE, FIXED><<<c.n_doc_tiles, 128, smem, c.stream>>>(c.v, c.doc_tiles, key, c.sweep, mh_steps); break;
-            case 256: k_doc_tile<T, 256, MODE, FIXED><<<c.n_doc_tiles, 256, smem, c.stream>>>(c.v, c.doc_tiles, key, c.sweep, mh_steps); break;
-            case 512: k_doc_tile<T, 512, MODE, FIXED><<<c.n_doc_tiles, 512, smem, c.stream>>>(c.v, c.doc_tiles, key, c.sweep, mh_steps); break;
-            default: k_doc_tile<T, 1024, MODE, FIXED><<<c.n_doc_tiles, 1024, smem, c.stream>>>(c.v, c.doc_tiles, key, c.sweep, mh_steps); break;
+            case 128: k_doc_tile<T, 128, MODE, FIXED><<<c.n_doc_tiles, 128, smem, c.stream>>>(c.v, c.doc_tiles, key, mh_steps); break;
+            case 256: k_doc_tile<T, 256, MODE, FIXED><<<c.n_doc_tiles, 256, smem, c.stream>>>(c.v, c.doc_tiles, key, mh_steps); break;
+            case 512: k_doc_tile<T, 512, MODE, FIXED><<<c.n_doc_tiles, 512, smem, c.stream>>>(c.v, c.doc_tiles, key, mh_steps); break;
+            default: k_doc_tile<T, 1024, MODE, FIXED><<<c.n_doc_tiles, 1024, smem, c.stream>>>(c.v, c.doc_tiles, key, mh_steps); break;
         }
         ++launches;
     }
     if (c.n_long_docs) {
-        k_long_doc_tile<T, MODE, FIXED><<<c.n_long_docs, 512, 0, c.stream>>>(c.v, c.long_docs, key, c.sweep, mh_steps);
+        k_long_doc_tile<T, MODE, FIXED><<<c.n_long_docs, 512, 0, c.stream>>>(c.v, c.long_docs, key, mh_steps);
         ++launches;
     }
     return launches;

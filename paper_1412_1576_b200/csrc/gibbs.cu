@@ -168,14 +168,13 @@ int lda::gibbs_sweep(Ctx& c, int32_t iters)
             k_gibbs_tokens<uint16_t><<<grid, 256, 0, c.stream>>>(v, (const uint16_t*)v.rec, word_of, r.row_off, r.topic,
                                                                 r.count, prefix, z_new, key, c.sweep);
         launch_spread_assignments(c, z_new, false);
-        launch_count_wk(c);
-        launch_count_k(c);
-        c.tables_valid = false;
-            c.sweep += 1;
+        rebuild_counts(c);
+        c.sweep += 1;
         if (cudaStreamSynchronize(c.stream) != cudaSuccess) rc = LDA_ECUDA;
         free_dk_csr(c, r);
     }
     if (iters > 0 && c.N == 0) c.sweep += (uint32_t)iters;
+    launch_set_state(c);  // the device's sweep counter follows
     cudaStreamSynchronize(c.stream);
     raw_free(c, word_of);
     raw_free(c, z_new);

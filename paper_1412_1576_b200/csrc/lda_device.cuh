@@ -32,6 +32,21 @@ __device__ __forceinline__ uint32_t scale_to_range(uint32_t r, uint32_t n) { ret
 
 __device__ __forceinline__ int bit_length(unsigned long long x) { return 64 - __clzll((long long)x); }
 
+// A quotient part/whole <= 1 as a 32-bit fraction (Section 4.2 tables: split points, mixture thresholds).
+__device__ __forceinline__ uint32_t to_frac32(unsigned long long part, unsigned long long whole)
+{
+    int sh = bit_length(whole) - 32;
+    if (sh < 0) sh = 0;
+    const unsigned long long q = ((part >> sh) << 32) / (whole >> sh);
+    return q > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)q;
+}
+
+// Share of a word's sparse term (mass S) in its proposal, the dense term having mass B.
+__device__ __forceinline__ uint32_t mixture_threshold(unsigned long long S, unsigned long long B)
+{
+    return S == 0 ? 0u : to_frac32(S, S + B);
+}
+
 // --- n_kd tables --------------------------------------------------------------------------------
 // Section 5's hashed rows (fn. 5 asks for at least twice as many slots as entries), one table per
 // document: `cap` = 4 * (document length) slots, so the load factor stays <= 0.25.  A slot is

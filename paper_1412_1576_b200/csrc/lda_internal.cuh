@@ -101,6 +101,32 @@ constexpr int ALIAS_SCRATCH_PER_ITEM = 20;   // bytes of construction scratch pe
 constexpr int ALIAS_SMEM_ITEMS_MID = LDA_ALIAS_SMEM_ITEMS_MID;   // rows a 256-thread CTA builds entirely in shared memory
 constexpr int ALIAS_SMEM_ITEMS_BIG = 4096;   // ... and a 512-thread CTA
 
+// Start times (nanoseconds of the device's global timer) a sweep's kernels leave for lda_stats.
+enum : int {
+    STAMP_DENSE = 0, STAMP_DENSE_END, STAMP_PROPOSE_HOT, STAMP_PROPOSE_COLD, STAMP_DOC_TILES, STAMP_DOC_LONG,
+    STAMP_ACCEPT_HOT, STAMP_ACCEPT_WARM, STAMP_ACCEPT_COLD, STAMP_ROWS, STAMP_WARM_ROWS, STAMP_HIST,
+    STAMP_NK_DENSE, STAMP_NK_SPARSE, STAMPS
+};
+constexpr int STAMP_RING = 32;  // sweeps queued before the host waits and reads their stamps
+
+// What changes from sweep to sweep lives in device memory, so that a sweep is the same sequence of
+// launches with the same arguments every time (and can be replayed as a CUDA graph).  One per context.
+struct SweepState {
+    unsigned long long moves[2];  // steps of the running lda_sweep() that moved a chain: word-, doc-proposals
+    int32_t err;                  // device error word
+    uint32_t sweep, next;         // Philox sweep counter of the running sweep; of the one after it
+    uint32_t slot, next_slot;     // their rows of `stamps`
+    uint32_t pad;
+    unsigned long long stamps[STAMP_RING][STAMPS];
+};
+// The part of it the host reads after a batch of sweeps, in host memory the device writes to.
+struct SweepReport {
+    unsigned long long moves[2];
+    unsigned long long end;  // time after the batch
+    int32_t err, pad;
+    unsigned long long stamps[STAMP_RING][STAMPS];
+};
+
 // Everything a kernel needs, passed by value.
 struct View {
     int32_t V, K, N, D;
@@ -143,19 +169,20 @@ struct View {
     uint32_t* al_idx;  // alias item of each sparse bin
     uint2* al_pk;      // 16-bit topics only: bin as (split point, topic of the bin's item | topic of
                        // its alias item << 16), so a draw costs one read
-    uint32_t* mix32;   // [V] share of the sparse term
+    unsigned long long* sp_mass;  // [V] fixed-point mass of the word's sparse term
     uint32_t* dn_thr;  // [K]
     uint32_t* dn_idx;  // [K]
     uint2* dn_pk;      // [K] (split point, alias) of the dense table in one word pair
     unsigned long long* dense_mass;
-    int32_t* nk;  // [K]
+    int32_t* nk;       // [K] column sums of n_kw: the counts frozen at sweep start
+    int32_t* nk_next;  // [K] ... of the rebuild in progress; the host exchanges the two after a rebuild
     // n_kd of the documents longer than a tile (the others' tables only ever live in shared memory):
     // the i-th long document owns the open-addressing table dk_slots[long_slot_off[i] .. long_slot_off[i+1])
     // (four slots per token, load <= 0.25); layout and probe order: dk_insert in lda_device.cuh.
     uint32_t* dk_slots;
     const long long* long_slot_off;
-    int* err;
-    unsigned long long* moves;  // [2] steps of the running lda_sweep() that moved a chain: word-, doc-proposals
+    int* err;           // = &state->err
+    SweepState* state;  // sweep counter, move counters, stamps
 };
 
 struct Ctx {
@@ -226,6 +253,7 @@ struct Ctx {
     unsigned long long* sc_de = nullptr;  // deficits prefix (front) / surpluses prefix (back)
     uint32_t* sc_item = nullptr;          // light items (front) / heavy items (back)
     unsigned long long* sc_dense = nullptr;  // same three for the dense table, [3*K]
+    uint32_t* mix32 = nullptr;               // [V] mixture thresholds, for lda_get_tables()
     double* ll_tab = nullptr;        // [2 * 512] lgamma tables of the log-likelihood's document part
     double* ll_tile_part = nullptr;  // [n_doc_tiles] its partial sums, one per tile of documents
     uint32_t* ll_tile_nnz = nullptr; // [n_doc_tiles] filled table slots of the tile: its share of nnz(n_kd)
@@ -242,12 +270,17 @@ struct Ctx {
     int64_t device_bytes = 0;
     lda_stats stats{};
     int64_t launches = 0;
-    // Events of up to EV_RING iterations of a sweep call (per iteration: 0..6 bracket the phases, 8 and
-    // 9 the passes of the MH step); the host waits and reads them once per EV_RING iterations.
-    static constexpr int EV_RING = 8;
-    cudaEvent_t ev_ring[EV_RING][10] = {};
-    cudaEvent_t* ev = ev_ring[0];  // the running iteration's
-    bool have_events = false;
+    SweepReport* report = nullptr;  // host memory the device writes (one block of the process-wide pool)
+    // A sweep as a CUDA graph, one per parity of the sweep counter (the two n_k buffers take turns).
+    // Built once a configuration has run a few sweeps launch by launch; dropped whenever an argument of
+    // its kernels changes.
+    cudaGraphExec_t graph[2] = {};
+    int graph_launches = 0;      // kernels in it
+    int graph_steps = 0, graph_mode = 0;
+    uint64_t graph_seed = 0;
+    int plain_sweeps = 0;        // sweeps launched one kernel at a time since the last change
+    bool graph_refused = false;  // capture failed once: this context launches kernel by kernel
+    cudaStream_t capture = nullptr;
     // Two more streams for kernels of one phase that touch different words: fork_streams() makes them
     // wait for the work queued on `stream` so far, join_streams() makes `stream` wait for theirs.
     cudaStream_t side[2] = {};
@@ -263,6 +296,30 @@ struct Ctx {
     bool export_pending = false;
     std::string err;
 };
+
+// The running sweep's counter.  Read where it is used (a cache hit after a CTA's first read): kept in a
+// register across a kernel it costs the register-bound passes a spill.  Constant while its readers run.
+__device__ __forceinline__ uint32_t running_sweep(const View& v)
+{
+    uint32_t s;
+    asm volatile("ld.global.ca.u32 %0, [%1];" : "=r"(s) : "l"(&v.state->sweep));
+    return s;
+}
+
+__device__ __forceinline__ unsigned long long global_timer()
+{
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+
+// First instruction of a kernel: one thread of the grid notes the time (`id` < 0: not noted).
+__device__ __forceinline__ void stamp(SweepState* state, int id)
+{
+    if (id >= 0 && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
+        state->stamps[state->slot][id] = global_timer();
+}
+__device__ __forceinline__ void stamp(const View& v, int id) { stamp(v.state, id); }
 
 inline void fork_streams(Ctx& c)
 {
@@ -280,14 +337,19 @@ inline void join_streams(Ctx& c)
 
 // --- launchers (each returns the number of kernels it launched) -----------------
 int launch_init(Ctx& c);
+void launch_set_state(Ctx& c);   // the device's copy of the sweep counter := the host's; move counters and stamps cleared
+void launch_report(Ctx& c);      // state -> c.report, move counters and stamps cleared
 int launch_spread_assignments(Ctx& c, const void* z_dev, bool narrow);  // z (doc order; u16 if narrow, else i32) -> both layouts
 int launch_spread_chunk(Ctx& c, const void* z_dev, bool narrow, int64_t first, int64_t count);  // ... tokens [first, first+count) -> block-major
 int launch_word_order_topics(Ctx& c);                                  // block-major -> word order, all tokens
 int launch_export_assignments(Ctx& c, void* z_dev, bool narrow);
 int launch_export_chunk(Ctx& c, void* z_dev, bool narrow, int64_t first, int64_t count);
 int launch_count_wk(Ctx& c);
-int launch_count_k(Ctx& c);
-int launch_alias_dense(Ctx& c);
+int launch_count_k(Ctx& c);      // n_k of the rows just rebuilt, added to View::nk_next (cleared before)
+void rebuild_counts(Ctx& c);     // n_kw and n_k from the assignments, outside a sweep
+inline void exchange_nk(Ctx& c) { int32_t* t = c.v.nk; c.v.nk = c.v.nk_next; c.v.nk_next = t; }
+int launch_alias_dense(Ctx& c, bool in_sweep);  // in_sweep: as the first kernel of a sweep, see there
+void launch_mix_thresholds(Ctx& c, uint32_t* mix32);  // of the tables last built
 int launch_alias_sparse(Ctx& c);            // the running slice's tables
 void set_slice(Ctx& c, int slice);          // makes `slice` the running one (moves the table pointers)
 int launch_sample(Ctx& c, int mh_steps);   // all passes of the MH step; needs ensure_exchange()

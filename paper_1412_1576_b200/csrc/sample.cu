@@ -264,7 +264,7 @@ struct WarmTile {
 template <typename T, int MODE, int FIXED, class Tile>
 __device__ __forceinline__ void propose_tokens(const View& v, const Tile& tile, const int32_t p_begin,
                                                const int32_t p_end, const int32_t nthreads, const uint2 key,
-                                               const uint32_t sweep, const int32_t mh_steps)
+                                               const int32_t mh_steps)
 {
     T* prop = reinterpret_cast<T*>(v.prop);
     if (FIXED == 2 && MODE == LDA_PROPOSALS_CYCLE) {
@@ -274,6 +274,7 @@ __device__ __forceinline__ void propose_tokens(const View& v, const Tile& tile, 
         for (int32_t p0 = p_begin + (int32_t)threadIdx.x; p0 < p_end; p0 += U * nthreads) {
             uint32_t tok[U], at[U], ua[U];
             Draw d[U];
+            const uint32_t sweep = running_sweep(v);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int32_t p = p0 + u * nthreads;
@@ -307,7 +308,7 @@ __device__ __forceinline__ void propose_tokens(const View& v, const Tile& tile, 
             const typename Tile::Ref w = tile.ref(p - p_begin);
             for (int32_t m = 0; m < mh_steps; m += (MODE == LDA_PROPOSALS_CYCLE ? 2 : 1)) {
                 const int32_t wi = step_kind_index<MODE>(m);
-                const uint4 r = philox4x32_10(make_uint4(tok, sweep, (uint32_t)m, 0u), key);
+                const uint4 r = philox4x32_10(make_uint4(tok, running_sweep(v), (uint32_t)m, 0u), key);
                 const Draw d = tile.draw_issue(w, v, r);
                 uint32_t t;
                 int32_t n_tw;
@@ -338,8 +339,7 @@ __device__ __forceinline__ void store_topic_pair(int32_t* zbm, uint32_t at, uint
 // gathered by pass 2, the word side comes from the tile's staged rows.
 template <typename T, int CH, int MODE, int FIXED, class Tile>
 __device__ __forceinline__ void accept_tokens(const View& v, Tile& tile, const int32_t p_begin, const int32_t p_end,
-                                              const int32_t nthreads, const uint2 key, const uint32_t sweep,
-                                              const int32_t mh_steps)
+                                              const int32_t nthreads, const int32_t mh_steps)
 {
     const int cb = v.count_bits;
     const uint32_t cmask = (1u << cb) - 1u;
@@ -467,8 +467,8 @@ __device__ __forceinline__ void accept_tokens(const View& v, Tile& tile, const i
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        if (moved_s[0]) atomicAdd(v.moves + 0, (unsigned long long)moved_s[0]);
-        if (moved_s[1]) atomicAdd(v.moves + 1, (unsigned long long)moved_s[1]);
+        if (moved_s[0]) atomicAdd(&v.state->moves[0], (unsigned long long)moved_s[0]);
+        if (moved_s[1]) atomicAdd(&v.state->moves[1], (unsigned long long)moved_s[1]);
     }
 }
 
@@ -480,8 +480,9 @@ __global__ void __launch_bounds__(ACCEPT ? accept_threads(FIXED) : PROPOSE_THREA
                                   ACCEPT      ? LDA_ACCEPT_MIN_CTAS
                                   : FIXED > 0 ? LDA_PROPOSE_FIXED_MIN_CTAS
                                               : LDA_PROPOSE_MIN_CTAS)
-k_word_hot(View v, const int32_t* __restrict__ tiles, uint2 key, uint32_t sweep, int32_t mh_steps_arg)
+k_word_hot(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_steps_arg, int stamp_id)
 {
+    stamp(v, stamp_id);
     const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
     extern __shared__ __align__(128) unsigned char dyn_smem[];
     __shared__ __align__(8) unsigned long long bar;
@@ -490,6 +491,11 @@ k_word_hot(View v, const int32_t* __restrict__ tiles, uint2 key, uint32_t sweep,
     const int32_t* row_g = v.dense_rows + (size_t)__ldg(v.dense_slot + w) * v.dense_stride;
     int32_t* row_s = reinterpret_cast<int32_t*>(dyn_smem);
     int32_t* nk_s = row_s + v.dense_stride;
+    __shared__ uint32_t mix_s;
+    if (!ACCEPT) {
+        if (threadIdx.x == 0) mix_s = mixture_threshold(__ldg(v.sp_mass + w), __ldg(v.dense_mass));
+        __syncthreads();
+    }
     if (STAGED && ACCEPT) {
         if (threadIdx.x == 0) {
             // the word's dense n_kw row and n_k, one bulk copy each, both signalling the same barrier
@@ -510,12 +516,12 @@ k_word_hot(View v, const int32_t* __restrict__ tiles, uint2 key, uint32_t sweep,
     tile.idx = v.al_idx + r0;
     tile.topic = v.wk_topic + r0;
     tile.nnz = __ldg(v.wk_nnz + w);
-    tile.mix = __ldg(v.mix32 + w);
+    tile.mix = ACCEPT ? 0u : mix_s;
     tile.bar = &bar;
     tile.ready = !(STAGED && ACCEPT);
     tile.gave_up = false;
-    if (ACCEPT) accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, accept_threads(FIXED), key, sweep, mh_steps);
-    else propose_tokens<T, MODE, FIXED>(v, tile, p0, p0 + cnt, PROPOSE_THREADS, key, sweep, mh_steps);
+    if (ACCEPT) accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, accept_threads(FIXED), mh_steps);
+    else propose_tokens<T, MODE, FIXED>(v, tile, p0, p0 + cnt, PROPOSE_THREADS, key, mh_steps);
     // ACCEPT: every thread that had a token waited for the copy; thread 0 always has one.  A thread
     // whose wait ran out waits once more (bounded again) before the CTA may retire: a bulk copy still
     // in flight must not land in shared memory that belongs to the next CTA.
@@ -526,8 +532,9 @@ k_word_hot(View v, const int32_t* __restrict__ tiles, uint2 key, uint32_t sweep,
 // instead of a dense one.
 template <typename T, int CH, int MODE, int FIXED>
 __global__ void __launch_bounds__(accept_threads(FIXED), LDA_ACCEPT_MIN_CTAS)
-k_word_warm(View v, const int32_t* __restrict__ tiles, uint2 key, uint32_t sweep, int32_t mh_steps_arg)
+k_word_warm(View v, const int32_t* __restrict__ tiles, int32_t mh_steps_arg, int stamp_id)
 {
+    stamp(v, stamp_id);
     const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
     extern __shared__ __align__(16) uint32_t warm_smem[];  // [2 * WARM_MAX_TF] topics, counts
     __shared__ uint32_t start_s[WARM_BUCKETS + 1];
@@ -554,14 +561,15 @@ k_word_warm(View v, const int32_t* __restrict__ tiles, uint2 key, uint32_t sweep
     }
     __syncthreads();
     WarmTile tile{topic_s, count_s, v.nk, start_s, shift};
-    accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, accept_threads(FIXED), key, sweep, mh_steps);
+    accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, accept_threads(FIXED), mh_steps);
 }
 
 // Tail words: tile = range of whole words [w0, w1) with at most COLD_TILE tokens.
 template <typename T, int CH, bool ACCEPT, int MODE, int FIXED>
 __global__ void __launch_bounds__(COLD_THREADS)
-k_word_cold(View v, const int32_t* __restrict__ tiles, uint2 key, uint32_t sweep, int32_t mh_steps_arg)
+k_word_cold(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_steps_arg, int stamp_id)
 {
+    stamp(v, stamp_id);
     const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
     __shared__ int32_t woff_s[COLD_WORDS + 1];  // first token of each word, relative to the tile
     __shared__ int32_t rs_s[COLD_WORDS + 1];    // first row slot of each word, relative to the tile
@@ -580,7 +588,7 @@ k_word_cold(View v, const int32_t* __restrict__ tiles, uint2 key, uint32_t sweep
     }
     for (int j = tid; j < nw; j += COLD_THREADS) {
         nnz_s[j] = __ldg(v.wk_nnz + w0 + j);
-        mix_s[j] = __ldg(v.mix32 + w0 + j);
+        if (!ACCEPT) mix_s[j] = mixture_threshold(__ldg(v.sp_mass + w0 + j), __ldg(v.dense_mass));
     }
     for (int j = tid; j < ne; j += COLD_THREADS) {
         topic_s[j] = __ldcs(v.wk_topic + e0 + j);
@@ -593,8 +601,8 @@ k_word_cold(View v, const int32_t* __restrict__ tiles, uint2 key, uint32_t sweep
     }
     __syncthreads();
     ColdTile tile{woff_s, rs_s, nnz_s, mix_s, topic_s, count_s, thr_s, idx_s, nw, v.nk};
-    if (ACCEPT) accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, COLD_THREADS, key, sweep, mh_steps);
-    else propose_tokens<T, MODE, FIXED>(v, tile, p0, p0 + cnt, COLD_THREADS, key, sweep, mh_steps);
+    if (ACCEPT) accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, COLD_THREADS, mh_steps);
+    else propose_tokens<T, MODE, FIXED>(v, tile, p0, p0 + cnt, COLD_THREADS, key, mh_steps);
 }
 
 // z_i uniform on {0..K-1}: Philox counter (token, 0, 0, 1), word 0.
@@ -666,21 +674,21 @@ static int launch_accept(Ctx& c, uint2 key, int mh_steps)
     if (c.n_hot_tiles) {
         if (c.K <= HOT_STAGE_MAX_K)
             k_word_hot<T, CH, true, true, MODE, FIXED>
-                <<<c.n_hot_tiles, accept_threads(FIXED), (size_t)v.dense_stride * 8, c.stream>>>(v, c.hot_tiles, key, c.sweep,
-                                                                                          mh_steps);
+                <<<c.n_hot_tiles, accept_threads(FIXED), (size_t)v.dense_stride * 8, c.stream>>>(v, c.hot_tiles, key, mh_steps,
+                                                                                          STAMP_ACCEPT_HOT);
         else
             k_word_hot<T, CH, false, true, MODE, FIXED>
-                <<<c.n_hot_tiles, accept_threads(FIXED), 0, c.stream>>>(v, c.hot_tiles, key, c.sweep, mh_steps);
+                <<<c.n_hot_tiles, accept_threads(FIXED), 0, c.stream>>>(v, c.hot_tiles, key, mh_steps, STAMP_ACCEPT_HOT);
         ++launches;
     }
     if (c.n_hot_tiles_warm) {
         k_word_warm<T, CH, MODE, FIXED><<<c.n_hot_tiles_warm, accept_threads(FIXED), WARM_MAX_TF * 8, c.stream>>>(
-            v, c.hot_tiles_warm, key, c.sweep, mh_steps);
+            v, c.hot_tiles_warm, mh_steps, STAMP_ACCEPT_WARM);
         ++launches;
     }
     if (c.n_cold_tiles) {
-        k_word_cold<T, CH, true, MODE, FIXED><<<c.n_cold_tiles, COLD_THREADS, 0, c.stream>>>(v, c.cold_tiles, key,
-                                                                                           c.sweep, mh_steps);
+        k_word_cold<T, CH, true, MODE, FIXED><<<c.n_cold_tiles, COLD_THREADS, 0, c.stream>>>(v, c.cold_tiles, key, mh_steps,
+                                                                                           STAMP_ACCEPT_COLD);
         ++launches;
     }
     return launches;
@@ -692,15 +700,16 @@ static int launch_propose(Ctx& c, uint2 key, int mh_steps)
     // the running vocabulary slice's tokens (its tables are the ones in memory)
     const View& v = c.v;
     const Ctx::Slice& q = c.slices[(size_t)c.cur_slice];
+    const bool noted = c.slices.size() == 1;  // several slices: the pass starts with the first slice's tables
     int launches = 0;
     if (q.hotp_n) {
         k_word_hot<T, CH, false, false, MODE, FIXED><<<q.hotp_n, PROPOSE_THREADS, 0, c.stream>>>(
-            v, c.hot_tiles_propose + 3 * (size_t)q.hotp_lo, key, c.sweep, mh_steps);
+            v, c.hot_tiles_propose + 3 * (size_t)q.hotp_lo, key, mh_steps, noted ? STAMP_PROPOSE_HOT : -1);
         ++launches;
     }
     if (q.cold_n) {
         k_word_cold<T, CH, false, MODE, FIXED><<<q.cold_n, COLD_THREADS, 0, c.stream>>>(
-            v, c.cold_tiles + 2 * (size_t)q.cold_lo, key, c.sweep, mh_steps);
+            v, c.cold_tiles + 2 * (size_t)q.cold_lo, key, mh_steps, noted ? STAMP_PROPOSE_COLD : -1);
         ++launches;
     }
     return launches;
@@ -728,10 +737,8 @@ static int sample_tc(Ctx& c, int mh_steps)
         }
     }
     // pass 2: document side
-    cudaEventRecord(c.ev[8], c.stream);
     launches += launch_doc_side(c, mh_steps);
     // pass 3: accept / reject; chains of two steps (and the cycle with four) have kernels of their own
-    cudaEventRecord(c.ev[9], c.stream);
     if (CH == 2 && mh_steps == 2)
         launches += launch_accept<T, 2, MODE, 2>(c, key, mh_steps);
     else if (CH == 4 && MODE == LDA_PROPOSALS_CYCLE && mh_steps == 4)

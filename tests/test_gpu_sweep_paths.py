@@ -1,0 +1,58 @@
+"""Branches of the sweep that depend on sizes: the oracle's assignments, counts and tables on both sides of
+each of them."""
+import numpy as np
+import pytest
+
+from oracle import ldaref
+from paper_1412_1576_b200 import binding, synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _pair(c, seed=77):
+    w, off = c.word_ids.numpy(), c.doc_offsets.numpy()
+    g = binding.LightLDA(c.V, c.K, c.alpha, c.beta)
+    o = ldaref.Oracle(c.V, c.K, c.alpha, c.beta)
+    for e in (g, o):
+        e.load_corpus(w, off)
+        e.init(seed)
+    return g, o
+
+
+def _same(g, o):
+    assert np.array_equal(g.get_assignments(), o.get_assignments())
+    assert np.array_equal(g.get_nk(), o.get_nk())
+    for which in (binding.LDA_NWK, binding.LDA_NDK):
+        for a, b in zip(g.get_csr(which), o.get_csr(which)):
+            assert np.array_equal(a, b)
+    a, b = g.get_tables(), o.get_tables()
+    for k in a:
+        assert np.array_equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("K", [1, 63, 65, 2048, 2049, 8193, 100_003])
+def test_dense_table_by_one_cta_and_by_a_cluster(K):
+    c = synth.generate(V=300, K=K, D=150, length=("poisson", 40.0), zipf_s=1.1, alpha=0.05, beta=0.01, seed=5)
+    g, o = _pair(c)
+    _same(g, o)
+    g.sweep(4, 2)  # the last ones replayed as a graph
+    o.sweep(4, 2)
+    _same(g, o)
+
+
+def test_replayed_sweeps_follow_changes_of_their_arguments(tiny_corpus):
+    """Step count, schedule, seed and state change between sweeps that are otherwise replayed."""
+    g, o = _pair(tiny_corpus)
+    z = None
+    for iters, steps, mode, seed in ((5, 2, 0, None), (1, 2, 0, None), (4, 4, 0, None), (4, 2, 1, None), (35, 2, 0, None),
+                                     (4, 2, 0, 123), (3, 2, 2, 124)):
+        if seed is not None:
+            z = o.get_assignments()
+            g.set_assignments(z, seed, 9)
+            o.set_assignments(z, seed, 9)
+        g.set_proposals(mode)
+        o.set_proposals(mode)
+        g.sweep(iters, steps)
+        o.sweep(iters, steps)
+        assert np.array_equal(g.get_assignments(), o.get_assignments()), (iters, steps, mode, seed)
+    _same(g, o)
