@@ -488,9 +488,39 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     // others with more tokens than a tail tile holds a sorted row built by a CTA of their own
     const bool warm_class = K > HOT_STAGE_MAX_K;
     std::vector<int32_t> warm_words;
-    std::vector<int32_t> dense_slot((size_t)V, -1), dense_words, row_start((size_t)V + 1), alias_big, alias_mid;
-    std::vector<int32_t> hist_chunks, word_tiles;
+    // How the words' tokens are cut into runs.  A run is staged, or counted, by one CTA, so long runs
+    // cost the least work -- but the pass lasts as long as its longest CTA, and a corpus of a few million
+    // tokens in the longest runs occupies a handful of multiprocessors.  So: the longest run that
+    // still gives every multiprocessor `per_sm` CTAs, and no shorter than what its staging is worth
+    // (measured on 2 M tokens, K = 100: histograms 56 -> 8 us, accept pass of the hot words 40 -> 9 us).
+    const auto run_for = [&](int64_t tokens, int64_t per_sm, int32_t longest, int32_t shortest) {
+        int32_t r = longest;
+        while (r > shortest && tokens / r < per_sm * c.n_sm) r /= 2;
+        return std::max(r, shortest);
+    };
+    const auto is_hot = [&](int32_t w) { return tf[w] > COLD_TILE; };
+    const auto has_dense_row = [&](int32_t w) {
+        return !(warm_class && tf[w] > SORT_TILE && tf[w] <= WARM_MAX_TF) && (tf[w] > SORT_TILE || (tf[w] > 0 && tf[w] >= tf_cut));
+    };
+    int64_t t_hot = 0, t_cold = 0, t_dense = 0;
+    for (int32_t w = 0; w < V; ++w) {
+        (is_hot(w) ? t_hot : t_cold) += tf_here[w];
+        if (has_dense_row(w)) t_dense += tf_here[w];
+    }
+    int32_t k_pow2 = 1;  // a row of K counters: staged by the accept pass, added up by the histograms
+    while (k_pow2 < K) k_pow2 *= 2;
+    const int32_t hist_run = run_for(t_dense, 8, HIST_RUN_MAX, std::min(std::max(4 * k_pow2, 4096), HIST_RUN_MAX));
+    const int32_t hot_tile = run_for(t_hot, 4, HOT_TILE_MAX, std::min(std::max(k_pow2, 2048), 8192));
+    int32_t propose_tile = run_for(t_hot, 4, HOT_TILE_PROPOSE_MAX, 2048);
+    if (propose_tile == 2048) propose_tile = 1536;  // one turn of the two-step kernel
+    const int32_t cold_tile = run_for(t_cold, 4, COLD_TILE, 256);
+    const bool sorted_rows = K > WORD_ROWS_BITMAP_MAX_K;
+    const int32_t row_tile = run_for(N - t_dense, 4, SORT_TILE, 256), row_tile_words = sorted_rows ? SORT_TILE : ROW_TILE_WORDS;
+
+    std::vector<int32_t> dense_slot((size_t)V, -1), row_start((size_t)V + 1), alias_big, alias_mid;
+    std::vector<int32_t> hot_runs, acc_runs, word_tiles;
     int64_t cap_total = 0;
+    c.n_dense = 0;
     for (int32_t w = 0; w < V; ++w) {
         row_start[w] = (int32_t)cap_total;
         const int32_t cap = std::min(tf[w], K);
@@ -499,15 +529,15 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
         else if (cap > ALIAS_WARP_MAX) alias_mid.push_back(w);
         if (warm_class && tf[w] > SORT_TILE && tf[w] <= WARM_MAX_TF) {
             warm_words.push_back(w);
-        } else if (tf[w] > SORT_TILE || (tf[w] > 0 && tf[w] >= tf_cut)) {
-            dense_slot[w] = (int32_t)dense_words.size();
-            dense_words.push_back(w);
-            for (int32_t o = 0; o < tf_here[w]; o += HIST_CHUNK) {
-                hist_chunks.push_back(w);
-                hist_chunks.push_back(word_off[w] + o);
-                hist_chunks.push_back(std::min(HIST_CHUNK, tf_here[w] - o));
-                hist_chunks.push_back(tf_here[w] <= HIST_CHUNK ? 1 : 0);
+        } else if (has_dense_row(w)) {
+            dense_slot[w] = c.n_dense++;
+            const int32_t runs = std::max(1, (tf_here[w] + hist_run - 1) / hist_run);
+            for (int32_t i = 0; i < runs; ++i) {
+                const int32_t o = i * hist_run;
+                hot_runs.insert(hot_runs.end(), {w, word_off[w] + o, std::min(hist_run, tf_here[w] - o),
+                                                 runs > 1 ? (int32_t)acc_runs.size() : -1});
             }
+            if (runs > 1) acc_runs.push_back(runs);
         }
     }
     row_start[V] = (int32_t)cap_total;
@@ -521,7 +551,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     }
     std::vector<char> slice_starts((size_t)V + 1, 0);
     for (int sl = 1; sl < n_slices; ++sl) slice_starts[(size_t)slice_w[sl]] = 1;
-    // tiles of consecutive sparse words: <= SORT_TILE tokens and <= SORT_TILE words each
+    // tiles of consecutive sparse words: <= row_tile tokens (or one longer word) and <= row_tile_words words each
     {
         int32_t s0 = 0, tok = 0;
         auto close = [&](int32_t s1) {
@@ -529,38 +559,40 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
         };
         for (int32_t w = 0; w < V; ++w) {
             if (dense_slot[w] >= 0 || tf[w] > SORT_TILE) { close(w); s0 = w + 1; tok = 0; continue; }
-            if (tok + tf[w] > SORT_TILE || w - s0 >= SORT_TILE) { close(w); s0 = w; tok = 0; }
+            if (tok + tf[w] > row_tile || w - s0 >= row_tile_words) { close(w); s0 = w; tok = 0; }
             tok += tf[w];
         }
         close(V);
     }
     // MH kernel work lists: a hot word (more tokens than a tail tile holds; it has a dense row by
-    // the rule above) is cut into runs of HOT_TILE tokens, tail words are packed whole into tiles
+    // the rule above) is cut into runs, tail words are packed whole into tiles, one longer than a tile cut
     std::vector<int32_t> hot_tiles, hot_tiles_warm, hot_tiles_propose, cold_tiles;
     {
         static_assert(COLD_TILE >= SORT_TILE, "every word longer than a tail tile must have a dense row or a warm one");
         int32_t s0 = 0, tok = 0;
         auto close = [&](int32_t s1) {
-            if (s1 > s0 && tok > 0) { cold_tiles.push_back(s0); cold_tiles.push_back(s1); }
+            if (s1 > s0 && word_off[s1] > word_off[s0])
+                cold_tiles.insert(cold_tiles.end(), {s0, s1, word_off[s0], word_off[s1] - word_off[s0]});
+        };
+        auto cut = [&](std::vector<int32_t>& list, int32_t w, int32_t run) {
+            for (int32_t o = 0; o < tf_here[w]; o += run)
+                list.insert(list.end(), {w, word_off[w] + o, std::min(run, tf_here[w] - o)});
         };
         for (int32_t w = 0; w < V; ++w) {
             if (slice_starts[w]) { close(w); s0 = w; tok = 0; }  // no tile reaches across two slices
-            if (tf[w] > COLD_TILE) {
+            if (is_hot(w)) {
                 close(w); s0 = w + 1; tok = 0;
-                std::vector<int32_t>& runs = dense_slot[w] >= 0 ? hot_tiles : hot_tiles_warm;
-                for (int32_t o = 0; o < tf_here[w]; o += HOT_TILE) {
-                    runs.push_back(w);
-                    runs.push_back(word_off[w] + o);
-                    runs.push_back(std::min(HOT_TILE, tf_here[w] - o));
-                }
-                for (int32_t o = 0; o < tf_here[w]; o += HOT_TILE_PROPOSE) {
-                    hot_tiles_propose.push_back(w);
-                    hot_tiles_propose.push_back(word_off[w] + o);
-                    hot_tiles_propose.push_back(std::min(HOT_TILE_PROPOSE, tf_here[w] - o));
-                }
+                cut(dense_slot[w] >= 0 ? hot_tiles : hot_tiles_warm, w, hot_tile);
+                cut(hot_tiles_propose, w, propose_tile);
                 continue;
             }
-            if (tok + tf[w] > COLD_TILE || w - s0 >= COLD_WORDS) { close(w); s0 = w; tok = 0; }
+            if (tf[w] > cold_tile) {
+                close(w); s0 = w + 1; tok = 0;
+                for (int32_t o = 0; o < tf_here[w]; o += cold_tile)
+                    cold_tiles.insert(cold_tiles.end(), {w, w + 1, word_off[w] + o, std::min(cold_tile, tf_here[w] - o)});
+                continue;
+            }
+            if (tok + tf[w] > cold_tile || w - s0 >= COLD_WORDS) { close(w); s0 = w; tok = 0; }
             tok += tf[w];
         }
         close(V);
@@ -614,8 +646,8 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.n_doc_sort_long = (int32_t)doc_sort_long.size();
     c.n_word_tiles = (int32_t)(word_tiles.size() / 2);
     c.n_doc_tiles = (int32_t)(doc_tiles.size() / 2);
-    c.n_dense = (int32_t)dense_words.size();
-    c.n_hist_chunks = (int32_t)(hist_chunks.size() / 4);
+    c.n_hot_runs = (int32_t)(hot_runs.size() / 4);
+    c.nk_with_rows = K <= NK_WITH_ROWS_MAX_K && c.n_hot_runs + c.n_word_tiles <= NK_WITH_ROWS_MAX_CTAS;
     c.n_long_docs = (int32_t)long_docs.size();
     c.n_alias_mid = (int32_t)alias_mid.size();
     alias_big.insert(alias_big.begin(), alias_mid.begin(), alias_mid.end());
@@ -624,7 +656,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.n_hot_tiles_warm = (int32_t)(hot_tiles_warm.size() / 3);
     c.n_warm = (int32_t)warm_words.size();
     c.n_hot_tiles_propose = (int32_t)(hot_tiles_propose.size() / 3);
-    c.n_cold_tiles = (int32_t)(cold_tiles.size() / 2);
+    c.n_cold_tiles = (int32_t)(cold_tiles.size() / 4);
     c.slices.assign((size_t)n_slices, Ctx::Slice{});
     int64_t slice_rows_max = 1;
     {
@@ -651,8 +683,8 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
             q.big_n = first_at(alias_big, n_mid, n_big, 1, q.w_hi) - (int32_t)n_mid - q.big_lo;
             q.hotp_lo = first_at(hot_tiles_propose, 0, (size_t)c.n_hot_tiles_propose, 3, q.w_lo);
             q.hotp_n = first_at(hot_tiles_propose, 0, (size_t)c.n_hot_tiles_propose, 3, q.w_hi) - q.hotp_lo;
-            q.cold_lo = first_at(cold_tiles, 0, (size_t)c.n_cold_tiles, 2, q.w_lo);
-            q.cold_n = first_at(cold_tiles, 0, (size_t)c.n_cold_tiles, 2, q.w_hi) - q.cold_lo;
+            q.cold_lo = first_at(cold_tiles, 0, (size_t)c.n_cold_tiles, 4, q.w_lo);
+            q.cold_n = first_at(cold_tiles, 0, (size_t)c.n_cold_tiles, 4, q.w_hi) - q.cold_lo;
         }
     }
     const size_t cap_alias = (size_t)slice_rows_max;
@@ -668,8 +700,10 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     v.dense_slot = upload(c, dense_slot);
     c.word_tiles = upload(c, word_tiles);
     c.doc_tiles = upload(c, doc_tiles);
-    c.dense_words = upload(c, dense_words);
-    c.hist_chunks = upload(c, hist_chunks);
+    c.hot_runs = upload(c, hot_runs);
+    c.acc_runs = upload(c, acc_runs);
+    c.acc = (int32_t*)A(acc_runs.size() * (size_t)v.dense_stride * 4);
+    c.acc_done = (int32_t*)A(acc_runs.size() * 4);
     c.long_docs = upload(c, long_docs);
     c.doc_sort_tiles = upload(c, doc_sort_tiles);
     c.doc_sort_long = upload(c, doc_sort_long);
@@ -679,8 +713,8 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.warm_words = upload(c, warm_words);
     c.hot_tiles_propose = upload(c, hot_tiles_propose);
     c.cold_tiles = upload(c, cold_tiles);
-    ok = ok && v.row_start && v.dense_slot && c.word_tiles && c.doc_tiles && c.dense_words &&
-         c.hist_chunks && c.long_docs && c.doc_sort_tiles && c.doc_sort_long && c.alias_big && c.hot_tiles && c.hot_tiles_warm && c.warm_words && c.hot_tiles_propose && c.cold_tiles;
+    ok = ok && v.row_start && v.dense_slot && c.word_tiles && c.doc_tiles && c.hot_runs && c.acc_runs &&
+         c.long_docs && c.doc_sort_tiles && c.doc_sort_long && c.alias_big && c.hot_tiles && c.hot_tiles_warm && c.warm_words && c.hot_tiles_propose && c.cold_tiles;
     v.wk_nnz = (int32_t*)A((size_t)V * 4);
     v.wk_topic = (uint32_t*)A(cap1 * 4);
     v.wk_count = (uint32_t*)A(cap1 * 4);
@@ -717,6 +751,9 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     set_slice(c, 0);
     cudaMemsetAsync(v.wk_nnz, 0, (size_t)V * 4, c.stream);
     cudaMemsetAsync(v.sp_mass, 0, (size_t)V * 8, c.stream);
+    cudaMemsetAsync(c.acc, 0, acc_runs.size() * (size_t)v.dense_stride * 4, c.stream);
+    cudaMemsetAsync(c.acc_done, 0, acc_runs.size() * 4, c.stream);
+    cudaMemsetAsync(v.dense_rows, 0, (size_t)c.n_dense * v.dense_stride * 4, c.stream);  // the rows' padding stays zero
     cudaMemsetAsync(v.nk, 0, (size_t)v.dense_stride * 8, c.stream);
     if (cudaStreamSynchronize(c.stream) != cudaSuccess) { free_corpus(c); return cuda_fail(&c, "load"); }
     c.stats = lda_stats{};

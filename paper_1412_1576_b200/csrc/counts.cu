@@ -2,13 +2,14 @@
 //
 // n_kw (segments = words over the word-sorted z): per word, the sorted list of
 // (topic, count).  Two paths, chosen per word at load time:
-//   - tail words: whole words are packed into tiles of <= SORT_TILE tokens; one
-//     CTA counts each word's topics in a shared-memory hash table and reads them
-//     back in topic order through a bitmap over the topics (K <= 16384), or sorts
+//   - tail words: whole words are packed into tiles of <= SORT_TILE tokens; the
+//     warps of a CTA count each word's topics in shared-memory hash tables and read them
+//     back in topic order through a bitmap over the topics (K <= 16384), or the CTA sorts
 //     the tile's (word, topic) keys (larger K);
-//   - hot words: shared-memory histogram over a window of topics, merged into
-//     the word's dense row, then compacted into the sorted row.
-// n_k: column sums of the rows just written.
+//   - hot words: shared-memory histogram over a window of topics, written out as
+//     dense row and sorted row.
+// n_k: column sums, added up by the kernels that write the rows when K and the number of CTAs are small
+// enough for that (nk_with_rows), else taken from the rows just written.
 // n_kd (segments = documents): the MH step builds every document's table itself, per tile, in
 // shared memory (docside.cu), and so does the log-likelihood (loglik.cu); lda_get_counts gets
 // sorted rows from export.cu.
@@ -126,95 +127,188 @@ k_seg_count_sorted(const int32_t* __restrict__ tiles, const int32_t* __restrict_
     for (int j = tid; j < nseg; j += blockDim.x) emit.rows(s0 + j, hidx[soff[j + 1]] - hidx[soff[j]]);
 }
 
-// Tail words: one CTA per tile of whole words [s0, s1) holding <= SORT_TILE tokens; the words are
-// taken one after the other.  A word's tokens are counted in a shared-memory hash table (same
-// tables as n_kd: 4 slots per token) and marked in a bitmap over the K topics; the bitmap, read in
-// order, gives the sorted row: the rank of a topic is the number of set bits before it.
-template <typename T>
+// Tail words (K <= WORD_ROWS_BITMAP_MAX_K): one CTA per tile of whole words [s0, s1) holding at most
+// SORT_TILE tokens and ROW_TILE_WORDS words.  The tile's topics are read once, into shared memory; the
+// words are then handed to the CTA's warps one at a time, without a barrier between them:
+//   - up to 32 tokens: a lane holds a token, lanes with the same topic find each other, the lowest of
+//     them writes the entry at the rank of its topic among the word's distinct topics;
+//   - up to ROW_WARP_TOKENS: counted in a hash table of the warp's own (load <= 1/2) and marked in its
+//     bitmap over the topics; the bitmap, read in order, gives the sorted row;
+//   - longer words are left for the whole CTA at the end (the same with four slots per token).
+// What bounds it is latency (a word is a chain of a dozen dependent shared-memory steps), so the
+// point of the split is many words in flight per multiprocessor and no CTA-wide steps for short ones.
+// NK: the tile's column sums go to n_k too, through bins in shared memory.
+constexpr int ROW_WARP_TOKENS = 256;
+constexpr int ROW_WARP_SLOTS = 512;
+constexpr int ROW_COUNT_BITS = 12;  // of a table entry: a tail word has at most SORT_TILE = 2048 tokens
+static_assert(SORT_TILE < (1 << ROW_COUNT_BITS), "count bits");
+
+struct RowTables {
+    const int32_t* row_start;
+    uint32_t* topic;
+    uint32_t* count;
+    int32_t* nnz;
+    int32_t* nk;  // column sums are added here (NK kernels)
+    SweepState* state;
+};
+
+// Words of 32 bits of a bitmap over K topics such that each lane of a warp owns an odd number of them (no
+// two lanes on the same shared-memory bank).
+__host__ __device__ constexpr int row_bitmap_lane_words(int K) { return (((K + 31) / 32 + 31) / 32) | 1; }
+static size_t row_area_bytes(int K)
+{
+    const size_t warps = 8 * (ROW_WARP_SLOTS * 4 + (size_t)row_bitmap_lane_words(K) * 32 * 4);
+    const size_t cta = (size_t)DK_SLOTS_PER_TOKEN_HOST * SORT_TILE * 4 + 2 * (size_t)((K + 31) / 32) * 4;
+    return ((warps > cta ? warps : cta) + 15) / 16 * 16;
+}
+
+template <typename T, bool NK>
 __global__ void __launch_bounds__(256)
 k_word_rows(const int32_t* __restrict__ tiles, const int32_t* __restrict__ word_off, const T* __restrict__ z,
-            const int32_t* __restrict__ row_start, uint32_t* __restrict__ wk_topic, uint32_t* __restrict__ wk_count,
-            int32_t* __restrict__ wk_nnz, int32_t K, SweepState* state)
+            RowTables out, int32_t K, int32_t area_words)
 {
-    stamp(state, STAMP_ROWS);
-    int* const err = &state->err;
-    constexpr int CB = 12;  // count bits of a table entry: a tail word has at most SORT_TILE = 2048 tokens
-    static_assert(SORT_TILE < (1 << CB), "count bits");
-    extern __shared__ uint32_t word_smem[];
-    __shared__ uint32_t table[DK_SLOTS_PER_TOKEN * SORT_TILE];
+    stamp(out.state, STAMP_ROWS);
+    extern __shared__ __align__(16) uint32_t row_area[];  // the warps' tables and bitmaps, then the CTA's; NK: bins behind
+    __shared__ int32_t soff[ROW_TILE_WORDS + 1];
+    __shared__ T zs[SORT_TILE];
+    __shared__ int32_t long_words[ROW_TILE_WORDS];
     __shared__ int32_t scan_tmp[33];
-    const int32_t bw = (K + 31) >> 5;
-    uint32_t* bitmap = word_smem;  // [bw] topics present in the word
-    uint32_t* before = word_smem + bw;  // [bw] set bits before each bitmap word
-    const int tid = threadIdx.x;
-    const int32_t s0 = tiles[2 * blockIdx.x], s1 = tiles[2 * blockIdx.x + 1];
-    // Words of at most 32 tokens (most of the vocabulary) take one warp each and no barrier: a lane
-    // holds a token, lanes with the same topic find each other, the lowest of them writes the entry at
-    // the rank of its topic among the word's distinct topics.
-    {
-        const int lane = tid & 31;
-        for (int32_t w = s0 + (tid >> 5); w < s1; w += (int32_t)(blockDim.x >> 5)) {
-            const int32_t first = word_off[w], n = word_off[w + 1] - first;
-            if (n > 32) continue;
-            uint32_t k = 0xFFFFFFFFu;
-            if (lane < n) {
-                k = (uint32_t)__ldcs(z + first + lane);
-                if (k >= (uint32_t)K) { atomicOr(err, ERR_TOPIC_RANGE); k = 0xFFFFFFFFu; }
-            }
+    __shared__ int32_t next_word, n_long;
+    int* const err = &out.state->err;
+    int32_t* bins = reinterpret_cast<int32_t*>(row_area + area_words);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int32_t s0 = tiles[2 * blockIdx.x], nw = tiles[2 * blockIdx.x + 1] - s0;
+    const int32_t base = __ldg(word_off + s0), cnt = __ldg(word_off + s0 + nw) - base;
+    if (tid == 0) {
+        next_word = 0;
+        n_long = 0;
+    }
+    for (int32_t j = tid; j <= nw; j += 256) soff[j] = __ldg(word_off + s0 + j) - base;
+    for (int32_t j = tid; j < cnt; j += 256) {
+        const T k = __ldcs(z + base + j);
+        if ((uint32_t)k >= (uint32_t)K) atomicOr(err, ERR_TOPIC_RANGE);
+        zs[j] = (uint32_t)k < (uint32_t)K ? k : (T)0;
+    }
+    if (NK)
+        for (int32_t k = tid; k < K; k += 256) bins[k] = 0;
+    __syncthreads();
+    auto emit = [&](int32_t at, uint32_t k, uint32_t n) {
+        out.topic[at] = k;
+        out.count[at] = n;
+        if (NK) atomicAdd(&bins[k], (int32_t)n);
+    };
+    const int32_t lane_words = row_bitmap_lane_words(K);
+    uint32_t* table = row_area + warp * ROW_WARP_SLOTS;
+    uint32_t* bitmap = row_area + 8 * ROW_WARP_SLOTS + warp * 32 * lane_words;
+    for (;;) {
+        int32_t w = 0;
+        if (lane == 0) w = atomicAdd(&next_word, 1);
+        w = __shfl_sync(0xFFFFFFFFu, w, 0);
+        if (w >= nw) break;
+        const int32_t first = soff[w], n = soff[w + 1] - first;
+        const int32_t out0 = __ldg(out.row_start + s0 + w);
+        if (n <= 32) {
+            const uint32_t k = lane < n ? (uint32_t)zs[first + lane] : 0xFFFFFFFFu;
             const uint32_t same = __match_any_sync(0xFFFFFFFFu, k);
-            const bool lead = k != 0xFFFFFFFFu && (uint32_t)(__ffs((int)same) - 1) == (uint32_t)lane;
+            const bool lead = lane < n && (uint32_t)(__ffs((int)same) - 1) == (uint32_t)lane;
             const uint32_t leaders = __ballot_sync(0xFFFFFFFFu, lead);
             int32_t rank = 0;
             for (uint32_t m = leaders; m; m &= m - 1u) {
                 const uint32_t other = __shfl_sync(0xFFFFFFFFu, k, __ffs((int)m) - 1);
                 rank += other < k ? 1 : 0;
             }
-            if (lead) {
-                const int32_t r = row_start[w] + rank;
-                wk_topic[r] = k;
-                wk_count[r] = (uint32_t)__popc(same);
+            if (lead) emit(out0 + rank, k, (uint32_t)__popc(same));
+            if (lane == 0) out.nnz[s0 + w] = __popc(leaders);
+        } else if (n <= ROW_WARP_TOKENS) {
+            const int log2_slots = n <= ROW_WARP_TOKENS / 2 ? 8 : 9;
+            const uint32_t slots = 1u << log2_slots;
+            const uint4 empty = make_uint4(DK_EMPTY, DK_EMPTY, DK_EMPTY, DK_EMPTY), zero = make_uint4(0u, 0u, 0u, 0u);
+            for (uint32_t i = lane; i < slots / 4; i += 32) reinterpret_cast<uint4*>(table)[i] = empty;
+            for (int32_t i = lane; i < 8 * lane_words; i += 32) reinterpret_cast<uint4*>(bitmap)[i] = zero;
+            __syncwarp();
+            for (int32_t j = lane; j < n; j += 32) {
+                const uint32_t k = (uint32_t)zs[first + j], fresh = (k << ROW_COUNT_BITS) | 1u;
+                uint32_t h = (k * DK_HASH_MULT) >> (32 - log2_slots);
+                for (uint32_t tries = 0; tries < slots; ++tries, h = (h + 1) & (slots - 1)) {
+                    const uint32_t prev = atomicCAS(&table[h], DK_EMPTY, fresh);
+                    if (prev == DK_EMPTY) {
+                        atomicOr(&bitmap[k >> 5], 1u << (k & 31u));
+                        break;
+                    }
+                    if ((prev >> ROW_COUNT_BITS) == k) {
+                        atomicAdd(&table[h], 1u);
+                        break;
+                    }
+                }
             }
-            if (lane == 0) wk_nnz[w] = __popc(leaders);
+            __syncwarp();
+            const uint32_t* mine = bitmap + lane * lane_words;
+            int32_t c = 0;
+            for (int32_t i = 0; i < lane_words; ++i) c += __popc(mine[i]);
+            const int32_t incl = warp_scan_incl<int32_t>(c);
+            int32_t at = out0 + incl - c;
+            for (int32_t i = 0; i < lane_words; ++i) {
+                for (uint32_t m = mine[i]; m; m &= m - 1u) {
+                    const uint32_t k = 32u * (uint32_t)(lane * lane_words + i) + (uint32_t)(__ffs((int)m) - 1);
+                    uint32_t h = (k * DK_HASH_MULT) >> (32 - log2_slots);
+                    uint32_t e = table[h];
+                    for (uint32_t tries = 0; tries < slots && (e >> ROW_COUNT_BITS) != k; ++tries) {
+                        h = (h + 1) & (slots - 1);
+                        e = table[h];
+                    }
+                    emit(at++, k, e & ((1u << ROW_COUNT_BITS) - 1u));
+                }
+            }
+            if (lane == 31) out.nnz[s0 + w] = incl;
+            __syncwarp();
+        } else if (lane == 0) {
+            long_words[atomicAdd(&n_long, 1)] = w;
         }
     }
-    for (int32_t w = s0; w < s1; ++w) {
-        const int32_t first = word_off[w], n = word_off[w + 1] - first;
-        if (n <= 32) continue;  // done above
+    __syncthreads();
+    const int32_t bw = (K + 31) >> 5;
+    uint32_t* cta_table = row_area;
+    uint32_t* cta_bitmap = row_area + DK_SLOTS_PER_TOKEN * SORT_TILE;  // [bw] topics present in the word
+    uint32_t* before = cta_bitmap + bw;                                // [bw] set bits before each bitmap word
+    for (int32_t q = 0; q < n_long; ++q) {
+        const int32_t w = long_words[q], first = soff[w], n = soff[w + 1] - first;
+        const int32_t out0 = __ldg(out.row_start + s0 + w);
         const uint32_t cap = DK_SLOTS_PER_TOKEN * (uint32_t)n;
-        for (int32_t i = tid; i < bw; i += blockDim.x) bitmap[i] = 0;
-        for (uint32_t i = tid; i < cap; i += blockDim.x) table[i] = DK_EMPTY;
+        for (int32_t i = tid; i < bw; i += 256) cta_bitmap[i] = 0;
+        for (uint32_t i = tid; i < cap; i += 256) cta_table[i] = DK_EMPTY;
         __syncthreads();
-        for (int32_t j = tid; j < n; j += blockDim.x) {
-            const uint32_t k = (uint32_t)__ldcs(z + first + j);
-            if (k >= (uint32_t)K) { atomicOr(err, ERR_TOPIC_RANGE); continue; }
-            atomicOr(&bitmap[k >> 5], 1u << (k & 31u));
-            if (dk_insert(table, cap, k, CB) == DK_EMPTY) atomicOr(err, ERR_ROW_OVERFLOW);
+        for (int32_t j = tid; j < n; j += 256) {
+            const uint32_t k = (uint32_t)zs[first + j];
+            atomicOr(&cta_bitmap[k >> 5], 1u << (k & 31u));
+            if (dk_insert(cta_table, cap, k, ROW_COUNT_BITS) == DK_EMPTY) atomicOr(err, ERR_ROW_OVERFLOW);
         }
         __syncthreads();
         int32_t running = 0;
-        for (int32_t i0 = 0; i0 < bw; i0 += blockDim.x) {
+        for (int32_t i0 = 0; i0 < bw; i0 += 256) {
             const int32_t i = i0 + tid;
-            const int32_t c = i < bw ? __popc(bitmap[i]) : 0;
+            const int32_t c = i < bw ? __popc(cta_bitmap[i]) : 0;
             int32_t total;
             const int32_t pos = block_scan_excl<int32_t>(c, scan_tmp, total);
             if (i < bw) before[i] = (uint32_t)(running + pos);
             running += total;
         }
         __syncthreads();
-        const int32_t out0 = row_start[w];
-        for (int32_t i = tid; i < bw; i += blockDim.x) {
-            uint32_t m = bitmap[i];
+        for (int32_t i = tid; i < bw; i += 256) {
             int32_t r = out0 + (int32_t)before[i];
-            while (m) {
+            for (uint32_t m = cta_bitmap[i]; m; m &= m - 1u, ++r) {
                 const uint32_t k = 32u * (uint32_t)i + (uint32_t)(__ffs((int)m) - 1);
-                m &= m - 1u;
-                wk_topic[r] = k;
-                wk_count[r] = dk_lookup(table, cap, k, CB) & ((1u << CB) - 1u);
-                ++r;
+                emit(r, k, dk_lookup(cta_table, cap, k, ROW_COUNT_BITS) & ((1u << ROW_COUNT_BITS) - 1u));
             }
         }
-        if (tid == 0) wk_nnz[w] = running;
+        if (tid == 0) out.nnz[s0 + w] = running;
         __syncthreads();
+    }
+    if (NK) {
+        __syncthreads();
+        for (int32_t k = tid; k < K; k += 256) {
+            const int32_t n = bins[k];
+            if (n) atomicAdd(&out.nk[k], n);
+        }
     }
 }
 
@@ -296,23 +390,72 @@ k_warm_rows(const int32_t* __restrict__ words, const int32_t* __restrict__ word_
     if (threadIdx.x == 0) wk_nnz[w] = done;
 }
 
-// Hot words: one CTA per run of a word's tokens (up to HIST_CHUNK of them); histogram of a window
-// of topics in shared memory (32-bit bins), merged into the word's dense row.  A word that fits
-// one run owns its row: its nonzero bins are stored.  A longer word's runs add theirs, one global
-// add per nonzero bin and run -- a few runs per word, so a row takes few adds per bin.
-template <typename T>
-__global__ void __launch_bounds__(512)
-k_hist_chunks(const int32_t* __restrict__ chunks, const T* __restrict__ z,
-              const int32_t* __restrict__ dense_slot, int32_t* __restrict__ dense_rows, int32_t K,
-              int32_t stride, int32_t window, SweepState* state)
+// Hot words: one CTA per run of a word's tokens; histogram of a window of topics in shared memory
+// (32-bit bins).  A word of one run (nearly all of them: runs are long) has its whole row in the bins, and the
+// CTA writes it out in both forms -- the dense row, zeros included, and the sorted one -- and, NK, adds it to
+// n_k.  The runs of a longer word add their nonzero bins to the word's line of `acc`; the last of them to
+// finish takes the line's contents the same way and leaves it zero for the next rebuild.
+// How the tokens are cut: load_common() in api.cu.
+struct HotRuns {
+    const int4* runs;      // (word, first token, tokens, index of the word among those with several runs or -1)
+    const int32_t* dense_slot;
+    int32_t* dense_rows;
+    int32_t stride;
+    int32_t* acc;          // [words with several runs][stride], all zero between rebuilds
+    int32_t* acc_done;     // [...] runs that have added theirs
+    const int32_t* acc_runs;  // [...] runs in all
+};
+
+// Bins [0, nb) of topics k0.. -> dense row and sorted entries from position `done` of the word's row on;
+// returns how many there were.  Every warp owns a run of bins: one walk to count, one to write.
+template <bool NK, class Bin>
+__device__ __forceinline__ int32_t emit_bins(const Bin& bin, int32_t k0, int32_t nb, int32_t* dense, int32_t out0,
+                                             int32_t cap, int32_t done, const RowTables& out, int32_t* warp_total)
 {
-    stamp(state, STAMP_HIST);
-    int* const err = &state->err;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int32_t per_warp = ((nb + nwarps - 1) / nwarps + 31) & ~31;
+    const int32_t q0 = min(nb, warp * per_warp), q1 = min(nb, q0 + per_warp);
+    int32_t mine = 0;
+    for (int32_t q = q0 + lane; q - lane < q1; q += 32) mine += __popc(__ballot_sync(0xFFFFFFFFu, q < q1 && bin(q) != 0));
+    if (lane == 0) warp_total[warp] = mine;
+    __syncthreads();
+    const int32_t t = lane < nwarps ? warp_total[lane] : 0;
+    const int32_t incl = warp_scan_incl<int32_t>(t);
+    const int32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    int32_t at = done + __shfl_sync(0xFFFFFFFFu, incl - t, warp);
+    const bool fits = done + total <= cap;
+    if (!fits && threadIdx.x == 0) atomicOr(&out.state->err, ERR_ROW_OVERFLOW);
+    for (int32_t q = q0 + lane; q - lane < q1; q += 32) {
+        const int32_t n = q < q1 ? bin(q) : 0;
+        const uint32_t some = __ballot_sync(0xFFFFFFFFu, n != 0);
+        if (q < q1) dense[k0 + q] = n;
+        if (n && fits) {
+            const int32_t slot = out0 + at + __popc(some & ((1u << lane) - 1u));
+            out.topic[slot] = (uint32_t)(k0 + q);
+            out.count[slot] = (uint32_t)n;
+            if (NK) atomicAdd(&out.nk[k0 + q], n);
+        }
+        at += __popc(some);
+    }
+    __syncthreads();
+    return total;
+}
+
+template <typename T, bool NK>
+__global__ void __launch_bounds__(512)
+k_hot_rows(HotRuns h, const T* __restrict__ z, RowTables out, int32_t K, int32_t window)
+{
+    stamp(out.state, STAMP_HIST);
     extern __shared__ __align__(16) int32_t hist_bins[];
-    const int32_t w = chunks[4 * blockIdx.x], first = chunks[4 * blockIdx.x + 1],
-                  cnt = chunks[4 * blockIdx.x + 2];
-    const bool alone = chunks[4 * blockIdx.x + 3] != 0;  // the word's only run
-    int32_t* row = dense_rows + (size_t)dense_slot[w] * stride;
+    __shared__ int32_t warp_total[16];
+    __shared__ bool last;
+    int* const err = &out.state->err;
+    const int4 run = h.runs[blockIdx.x];
+    const int32_t w = run.x, first = run.y, cnt = run.z, multi = run.w;
+    int32_t* dense = h.dense_rows + (size_t)h.dense_slot[w] * h.stride;
+    int32_t* acc = h.acc + (size_t)max(multi, 0) * h.stride;
+    const int32_t out0 = out.row_start[w], cap = out.row_start[w + 1] - out0;
+    int32_t done = 0;
     for (int32_t k0 = 0; k0 < K; k0 += window) {
         const int32_t nb = min(window, K - k0);
         for (int b = threadIdx.x; b < (nb + 3) / 4; b += blockDim.x)
@@ -345,53 +488,28 @@ k_hist_chunks(const int32_t* __restrict__ chunks, const T* __restrict__ z,
         for (int j = threadIdx.x; j < cnt - nvec * E; j += blockDim.x)
             add((uint32_t)z[first + (j < head ? j : nvec * E + j)]);
         __syncthreads();
-        for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-            const int32_t n = hist_bins[b];
-            if (n) {
-                if (alone) row[k0 + b] = n;  // the row was cleared before the launch
-                else atomicAdd(&row[k0 + b], n);
-            }
-        }
-        __syncthreads();
-    }
-}
-
-// Dense row -> sorted (topic, count) row, one CTA per dense word.
-__global__ void __launch_bounds__(256)
-k_compact_dense(const int32_t* __restrict__ dense_words, const int32_t* __restrict__ dense_slot,
-                const int32_t* __restrict__ dense_rows, const int32_t* __restrict__ row_start,
-                uint32_t* __restrict__ wk_topic, uint32_t* __restrict__ wk_count,
-                int32_t* __restrict__ wk_nnz, int32_t K, int32_t stride, int* err)
-{
-    __shared__ int32_t scan_tmp[33];
-    const int32_t w = dense_words[blockIdx.x];
-    const int32_t* row = dense_rows + (size_t)dense_slot[w] * stride;
-    const int32_t out0 = row_start[w], cap = row_start[w + 1] - out0;
-    // four consecutive topics per thread and step (rows are padded to a multiple of four and start
-    // 16-byte aligned; the padding is never written, so it reads as zero)
-    int32_t done = 0;
-    for (int32_t k0 = 0; k0 < stride; k0 += 4 * blockDim.x) {
-        const int32_t k = k0 + 4 * (int32_t)threadIdx.x;
-        int4 n = make_int4(0, 0, 0, 0);
-        if (k < stride) n = __ldcs(reinterpret_cast<const int4*>(row + k));
-        const int32_t mine = (n.x > 0) + (n.y > 0) + (n.z > 0) + (n.w > 0);
-        int32_t total;
-        int32_t pos = done + block_scan_excl<int32_t>(mine, scan_tmp, total);
-        if (pos + mine > cap) {
-            atomicOr(err, ERR_ROW_OVERFLOW);
+        if (multi < 0) {
+            done += emit_bins<NK>([](int32_t q) { return hist_bins[q]; }, k0, nb, dense, out0, cap, done, out, warp_total);
         } else {
-            const int32_t nv[4] = {n.x, n.y, n.z, n.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (nv[q] > 0) {
-                    wk_topic[out0 + pos] = (uint32_t)(k + q);
-                    wk_count[out0 + pos] = (uint32_t)nv[q];
-                    ++pos;
-                }
+            for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+                const int32_t n = hist_bins[b];
+                if (n) atomicAdd(&acc[k0 + b], n);
+            }
+            __syncthreads();
         }
-        done += total;
     }
-    if (threadIdx.x == 0) wk_nnz[w] = done;
+    if (multi >= 0) {
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(&h.acc_done[multi], 1) == h.acc_runs[multi] - 1;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        done = emit_bins<NK>([acc](int32_t q) { return __ldcg(acc + q); }, 0, K, dense, out0, cap, 0, out, warp_total);
+        for (int k = threadIdx.x; k < K; k += blockDim.x) acc[k] = 0;
+        if (threadIdx.x == 0) h.acc_done[multi] = 0;
+    }
+    if (threadIdx.x == 0) out.nnz[w] = done;
 }
 
 // n_k = sum over words of n_kw (Section 3), taken from the rows the n_kw rebuild has just written
@@ -506,19 +624,27 @@ template void launch_doc_rows<int32_t>(Ctx&, const int32_t*, int32_t, const int3
 
 static int hist_window(const Ctx& c) { return c.K < HIST_BINS ? c.K : HIST_BINS; }
 
-template <typename T>
+template <typename T, bool NK>
 static int count_wk_t(Ctx& c)
 {
     View& v = c.v;
     int launches = 0;
     const T* z = (const T*)v.zw;
+    const RowTables out{v.row_start, v.wk_topic, v.wk_count, v.wk_nnz, v.nk_next, v.state};
     // the tail words' rows and the hot words' rows are built side by side
     fork_streams(c);
+    if (c.n_hot_runs) {
+        const HotRuns h{reinterpret_cast<const int4*>(c.hot_runs), v.dense_slot, v.dense_rows, v.dense_stride, c.acc,
+                        c.acc_done, c.acc_runs};
+        const int win = c.K < HIST32_BINS ? c.K : HIST32_BINS;
+        k_hot_rows<T, NK><<<c.n_hot_runs, 512, (size_t)((win + 3) / 4) * 16, c.stream>>>(h, z, out, c.K, win);
+        ++launches;
+    }
     if (c.n_word_tiles) {
         if (c.K <= WORD_ROWS_BITMAP_MAX_K) {
-            const size_t smem = 2 * (size_t)((c.K + 31) / 32) * 4;
-            k_word_rows<T><<<c.n_word_tiles, 256, smem, c.side[0]>>>(c.word_tiles, v.word_off, z, v.row_start,
-                                                                    v.wk_topic, v.wk_count, v.wk_nnz, c.K, v.state);
+            const size_t area = row_area_bytes(c.K);
+            k_word_rows<T, NK><<<c.n_word_tiles, 256, area + (NK ? (size_t)c.K * 4 : 0), c.side[0]>>>(
+                c.word_tiles, v.word_off, z, out, c.K, (int32_t)(area / 4));
         } else {
             EmitWord e{v.row_start, v.wk_topic, v.wk_count, v.wk_nnz};
             k_seg_count_sorted<T, EmitWord><<<c.n_word_tiles, 256, 0, c.side[0]>>>(
@@ -532,23 +658,13 @@ static int count_wk_t(Ctx& c)
             c.warm_words, v.word_off, z, v.row_start, v.wk_topic, v.wk_count, v.wk_nnz, c.K, win, v.state);
         ++launches;
     }
-    if (c.n_dense) {
-        cudaMemsetAsync(v.dense_rows, 0, (size_t)c.n_dense * v.dense_stride * 4, c.stream);
-        const int win = c.K < HIST32_BINS ? c.K : HIST32_BINS;
-        k_hist_chunks<T><<<c.n_hist_chunks, 512, (size_t)((win + 3) / 4) * 16, c.stream>>>(
-            c.hist_chunks, z, v.dense_slot, v.dense_rows, c.K, v.dense_stride, win, v.state);
-        k_compact_dense<<<c.n_dense, 256, 0, c.stream>>>(c.dense_words, v.dense_slot, v.dense_rows,
-                                                         v.row_start, v.wk_topic, v.wk_count,
-                                                         v.wk_nnz, c.K, v.dense_stride, v.err);
-        launches += 2;
-    }
     join_streams(c);
     return launches;
 }
 
 // Must follow launch_count_wk(): reads the rows it wrote and adds into View::nk_next, which the sweep's
 // first kernel (or the caller) has cleared.
-static int count_k(Ctx& c)
+int launch_count_k_from_rows(Ctx& c)
 {
     View& v = c.v;
     if (c.N == 0) return 0;
@@ -577,15 +693,24 @@ static int count_k(Ctx& c)
     return launches;
 }
 
-int launch_count_wk(Ctx& c) { return c.wide_topics ? count_wk_t<int32_t>(c) : count_wk_t<uint16_t>(c); }
-int launch_count_k(Ctx& c) { return count_k(c); }
+int launch_count_wk(Ctx& c)
+{
+    if (c.wide_topics) return count_wk_t<int32_t, false>(c);
+    return c.nk_with_rows ? count_wk_t<uint16_t, true>(c) : count_wk_t<uint16_t, false>(c);
+}
+int launch_count_k(Ctx& c) { return c.nk_with_rows ? 0 : launch_count_k_from_rows(c); }
 
 void set_hist_smem_limits()
 {
     cudaFuncSetAttribute(k_warm_rows<uint16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST16_BINS * 2 + 16);
     cudaFuncSetAttribute(k_warm_rows<int32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST16_BINS * 2 + 16);
-    cudaFuncSetAttribute(k_hist_chunks<uint16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST32_BINS * 4);
-    cudaFuncSetAttribute(k_hist_chunks<int32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST32_BINS * 4);
+    cudaFuncSetAttribute(k_hot_rows<uint16_t, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST32_BINS * 4);
+    cudaFuncSetAttribute(k_hot_rows<uint16_t, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST32_BINS * 4);
+    cudaFuncSetAttribute(k_hot_rows<int32_t, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST32_BINS * 4);
+    cudaFuncSetAttribute(k_word_rows<uint16_t, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)row_area_bytes(WORD_ROWS_BITMAP_MAX_K));
+    cudaFuncSetAttribute(k_word_rows<uint16_t, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)row_area_bytes(NK_WITH_ROWS_MAX_K) + NK_WITH_ROWS_MAX_K * 4);
     cudaFuncSetAttribute(k_nk_from_sparse, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST_BINS * 4);
 }
 

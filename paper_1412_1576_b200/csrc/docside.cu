@@ -257,19 +257,20 @@ template <typename T, int MODE, int FIXED>
 static int doc_side_tm(Ctx& c, int mh_steps)
 {
     const uint2 key = make_uint2((uint32_t)c.seed, (uint32_t)(c.seed >> 32));
+    const PassStreams on(c, (c.n_doc_tiles > 0) + (c.n_long_docs > 0));
     int launches = 0;
     if (c.n_doc_tiles) {
         const size_t smem = doc_tile_smem_bytes(c.doc_tile);
         switch (c.doc_threads) {
-            case 128: k_doc_tile<T, 128, MODE, FIXED><<<c.n_doc_tiles, 128, smem, c.stream>>>(c.v, c.doc_tiles, key, mh_steps); break;
-            case 256: k_doc_tile<T, 256, MODE, FIXED><<<c.n_doc_tiles, 256, smem, c.stream>>>(c.v, c.doc_tiles, key, mh_steps); break;
-            case 512: k_doc_tile<T, 512, MODE, FIXED><<<c.n_doc_tiles, 512, smem, c.stream>>>(c.v, c.doc_tiles, key, mh_steps); break;
-            default: k_doc_tile<T, 1024, MODE, FIXED><<<c.n_doc_tiles, 1024, smem, c.stream>>>(c.v, c.doc_tiles, key, mh_steps); break;
+            case 128: k_doc_tile<T, 128, MODE, FIXED><<<c.n_doc_tiles, 128, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
+            case 256: k_doc_tile<T, 256, MODE, FIXED><<<c.n_doc_tiles, 256, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
+            case 512: k_doc_tile<T, 512, MODE, FIXED><<<c.n_doc_tiles, 512, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
+            default: k_doc_tile<T, 1024, MODE, FIXED><<<c.n_doc_tiles, 1024, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
         }
         ++launches;
     }
     if (c.n_long_docs) {
-        k_long_doc_tile<T, MODE, FIXED><<<c.n_long_docs, 512, 0, c.stream>>>(c.v, c.long_docs, key, mh_steps);
+        k_long_doc_tile<T, MODE, FIXED><<<c.n_long_docs, 512, 0, on[0]>>>(c.v, c.long_docs, key, mh_steps);
         ++launches;
     }
     return launches;

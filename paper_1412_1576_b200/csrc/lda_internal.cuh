@@ -69,19 +69,15 @@ constexpr int HIST_BINS = 32768;     // shared-memory histogram window (32-bit b
 constexpr int WORD_ROWS_BITMAP_MAX_K = 16384;  // tail rows: topic bitmap up to this K, key sort above
 constexpr int HIST16_BINS = 106496;  // window of a warm word's n_kw histogram (16-bit bins, 208 KB)
 constexpr int HIST32_BINS = 49152;   // window of a hot word's n_kw histogram (32-bit bins, 192 KB)
-#ifndef LDA_HIST_CHUNK
-#define LDA_HIST_CHUNK 262144
-#endif
-constexpr int HIST_CHUNK = LDA_HIST_CHUNK;    // tokens per CTA (one run of a word) in the histogram path
-#ifndef LDA_HOT_TILE
-#define LDA_HOT_TILE 32768
-#endif
-#ifndef LDA_HOT_TILE_PROPOSE
-#define LDA_HOT_TILE_PROPOSE 8192
-#endif
-constexpr int HOT_TILE = LDA_HOT_TILE;  // accept pass: tokens of one hot word per CTA (the word's row is staged once per CTA)
-constexpr int HOT_TILE_PROPOSE = LDA_HOT_TILE_PROPOSE;  // propose pass: nothing is staged, shorter runs balance better
-constexpr int COLD_TILE = 2048;      // MH kernel: tokens of a tile of whole tail words
+constexpr int HIST_RUN_MAX = 262144;  // tokens per CTA (one run of a word) in the histogram path, at most
+constexpr int ROW_TILE_WORDS = 512;   // words per tile of the tail words' row kernel
+// n_k is added up by the row kernels themselves up to this K (bins in shared memory) ...
+constexpr int NK_WITH_ROWS_MAX_K = 4096;
+// ... and this many CTAs: each adds to every topic's counter once, and the adds to one counter queue
+constexpr int NK_WITH_ROWS_MAX_CTAS = 16384;
+constexpr int HOT_TILE_MAX = 32768;  // accept pass: tokens of one hot word per CTA (the word's row is staged once per CTA), at most
+constexpr int HOT_TILE_PROPOSE_MAX = 8192;  // propose pass: nothing is staged, shorter runs balance better
+constexpr int COLD_TILE = 2048;      // MH kernel: tokens of a tile of tail words, at most
 constexpr int COLD_WORDS = 512;      // MH kernel: words per tail tile
 constexpr int HOT_STAGE_MAX_K = 16384;  // dense rows up to this many topics are staged in shared memory
 // Beyond that K a dense row (4 K bytes) only pays for frequent words.  Words with more tokens than
@@ -209,12 +205,15 @@ struct Ctx {
     int64_t N = 0, D = 0;
     View v{};
     // host-side work lists (device copies below)
-    int32_t n_word_tiles = 0, n_doc_tiles = 0, n_dense = 0, n_hist_chunks = 0, n_long_docs = 0,
+    int32_t n_word_tiles = 0, n_doc_tiles = 0, n_dense = 0, n_hot_runs = 0, n_long_docs = 0,
             n_alias_big = 0, n_alias_mid = 0, n_hot_tiles = 0, n_hot_tiles_propose = 0, n_cold_tiles = 0;
     int32_t* word_tiles = nullptr;   // [n_word_tiles*2] word ranges sorted per CTA
     int32_t* doc_tiles = nullptr;    // [n_doc_tiles*2]
-    int32_t* dense_words = nullptr;  // [n_dense]
-    int32_t* hist_chunks = nullptr;  // [n_hist_chunks*4] (word, first token, count, 1 if the word's only run)
+    int32_t* hot_runs = nullptr;     // [n_hot_runs*4] (word, first token, count, index of a word with several runs or -1)
+    int32_t* acc = nullptr;          // [words with several runs][dense_stride], zero between rebuilds
+    int32_t* acc_done = nullptr;     // [...] runs of the word that are done, zero between rebuilds
+    int32_t* acc_runs = nullptr;     // [...] runs of the word
+    bool nk_with_rows = false;       // the row kernels add up n_k too
     int32_t* long_docs = nullptr;    // [n_long_docs]
     // sorted n_kd rows (export.cu): tiles of whole documents of at most SORT_TILE tokens, and the longer documents
     int32_t n_doc_sort_tiles = 0, n_doc_sort_long = 0;
@@ -227,7 +226,8 @@ struct Ctx {
     int32_t* hot_tiles_warm = nullptr;  // [n_hot_tiles_warm*3] their runs for the accept pass
     int32_t* hot_tiles = nullptr;    // [n_hot_tiles*3] (word, first token, count): MH kernel, words with a dense row (accept pass)
     int32_t* hot_tiles_propose = nullptr;  // the same cut into the shorter runs of the propose passs
-    int32_t* cold_tiles = nullptr;   // [n_cold_tiles*2] word ranges of whole tail words: MH kernel
+    int32_t* cold_tiles = nullptr;   // [n_cold_tiles*4] (first word, end word, first token, count): MH kernel, whole tail
+                                     // words or a run of one
     // Vocabulary slices (Section 3, Fig. 1: the model is visited slice by slice): the words are cut into
     // runs of about equal row capacity; the sparse alias tables and their construction scratch hold one
     // slice at a time (entry of row slot r of the running slice: r - row_lo), so pass 1 goes slice by
@@ -335,6 +335,24 @@ inline void join_streams(Ctx& c)
     }
 }
 
+// The kernels of one pass of the MH step touch different tokens and could always run side by side.  With
+// few tokens none of them fills the GPU and the pass lasts as long as the slower one; with many
+// (738 M tokens: accept pass 6.7 ms side by side, 6.1 one after the other) they only compete for L2.
+constexpr int64_t SIDE_BY_SIDE_MAX_TOKENS = (int64_t)1 << 24;
+struct PassStreams {
+    Ctx& c;
+    bool side;
+    PassStreams(Ctx& ctx, int kernels) : c(ctx), side(kernels > 1 && ctx.N <= SIDE_BY_SIDE_MAX_TOKENS)
+    {
+        if (side) fork_streams(c);
+    }
+    ~PassStreams()
+    {
+        if (side) join_streams(c);
+    }
+    cudaStream_t operator[](int i) const { return side && i > 0 ? c.side[i - 1] : c.stream; }
+};
+
 // --- launchers (each returns the number of kernels it launched) -----------------
 int launch_init(Ctx& c);
 void launch_set_state(Ctx& c);   // the device's copy of the sweep counter := the host's; move counters and stamps cleared
@@ -345,7 +363,9 @@ int launch_word_order_topics(Ctx& c);                                  // block-
 int launch_export_assignments(Ctx& c, void* z_dev, bool narrow);
 int launch_export_chunk(Ctx& c, void* z_dev, bool narrow, int64_t first, int64_t count);
 int launch_count_wk(Ctx& c);
-int launch_count_k(Ctx& c);      // n_k of the rows just rebuilt, added to View::nk_next (cleared before)
+int launch_count_k(Ctx& c);      // n_k of the rows just rebuilt, added to View::nk_next (cleared before), unless the
+                                 // row kernels have done it
+int launch_count_k_from_rows(Ctx& c);  // ... in any case
 void rebuild_counts(Ctx& c);     // n_kw and n_k from the assignments, outside a sweep
 inline void exchange_nk(Ctx& c) { int32_t* t = c.v.nk; c.v.nk = c.v.nk_next; c.v.nk_next = t; }
 int launch_alias_dense(Ctx& c, bool in_sweep);  // in_sweep: as the first kernel of a sweep, see there

@@ -564,10 +564,11 @@ k_word_warm(View v, const int32_t* __restrict__ tiles, int32_t mh_steps_arg, int
     accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, accept_threads(FIXED), mh_steps);
 }
 
-// Tail words: tile = range of whole words [w0, w1) with at most COLD_TILE tokens.
+// Tail words: tile = (first word, end word, first token, count): whole words with at most COLD_TILE tokens
+// between them, or a run of one word's tokens (small corpora: see load_common() for where the cuts lie).
 template <typename T, int CH, bool ACCEPT, int MODE, int FIXED>
 __global__ void __launch_bounds__(COLD_THREADS)
-k_word_cold(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_steps_arg, int stamp_id)
+k_word_cold(View v, const int4* __restrict__ tiles, uint2 key, int32_t mh_steps_arg, int stamp_id)
 {
     stamp(v, stamp_id);
     const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
@@ -577,11 +578,11 @@ k_word_cold(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_ste
     __shared__ uint32_t mix_s[COLD_WORDS];
     __shared__ uint32_t topic_s[COLD_TILE], count_s[COLD_TILE], thr_s[COLD_TILE], idx_s[COLD_TILE];
     const int tid = threadIdx.x;
-    const int32_t w0 = tiles[2 * blockIdx.x], w1 = tiles[2 * blockIdx.x + 1];
+    const int4 t4 = __ldg(tiles + blockIdx.x);
+    const int32_t w0 = t4.x, w1 = t4.y, p0 = t4.z, cnt = t4.w;
     const int32_t nw = w1 - w0;
-    const int32_t p0 = __ldg(v.word_off + w0), cnt = __ldg(v.word_off + w1) - p0;
-    const int32_t e0 = __ldg(v.row_start + w0), ne = __ldg(v.row_start + w1) - e0;
-    if (cnt == 0) return;
+    const int32_t e0 = __ldg(v.row_start + w0);
+    const int32_t ne = nw == 1 ? __ldg(v.wk_nnz + w0) : __ldg(v.row_start + w1) - e0;
     for (int j = tid; j <= nw; j += COLD_THREADS) {
         woff_s[j] = __ldg(v.word_off + w0 + j) - p0;
         rs_s[j] = __ldg(v.row_start + w0 + j) - e0;
@@ -670,24 +671,25 @@ template <typename T, int CH, int MODE, int FIXED>
 static int launch_accept(Ctx& c, uint2 key, int mh_steps)
 {
     const View& v = c.v;
+    const PassStreams on(c, (c.n_hot_tiles > 0) + (c.n_hot_tiles_warm > 0) + (c.n_cold_tiles > 0));
     int launches = 0;
     if (c.n_hot_tiles) {
         if (c.K <= HOT_STAGE_MAX_K)
             k_word_hot<T, CH, true, true, MODE, FIXED>
-                <<<c.n_hot_tiles, accept_threads(FIXED), (size_t)v.dense_stride * 8, c.stream>>>(v, c.hot_tiles, key, mh_steps,
+                <<<c.n_hot_tiles, accept_threads(FIXED), (size_t)v.dense_stride * 8, on[0]>>>(v, c.hot_tiles, key, mh_steps,
                                                                                           STAMP_ACCEPT_HOT);
         else
             k_word_hot<T, CH, false, true, MODE, FIXED>
-                <<<c.n_hot_tiles, accept_threads(FIXED), 0, c.stream>>>(v, c.hot_tiles, key, mh_steps, STAMP_ACCEPT_HOT);
+                <<<c.n_hot_tiles, accept_threads(FIXED), 0, on[0]>>>(v, c.hot_tiles, key, mh_steps, STAMP_ACCEPT_HOT);
         ++launches;
     }
     if (c.n_hot_tiles_warm) {
-        k_word_warm<T, CH, MODE, FIXED><<<c.n_hot_tiles_warm, accept_threads(FIXED), WARM_MAX_TF * 8, c.stream>>>(
+        k_word_warm<T, CH, MODE, FIXED><<<c.n_hot_tiles_warm, accept_threads(FIXED), WARM_MAX_TF * 8, on[2]>>>(
             v, c.hot_tiles_warm, mh_steps, STAMP_ACCEPT_WARM);
         ++launches;
     }
     if (c.n_cold_tiles) {
-        k_word_cold<T, CH, true, MODE, FIXED><<<c.n_cold_tiles, COLD_THREADS, 0, c.stream>>>(v, c.cold_tiles, key, mh_steps,
+        k_word_cold<T, CH, true, MODE, FIXED><<<c.n_cold_tiles, COLD_THREADS, 0, on[1]>>>(v, reinterpret_cast<const int4*>(c.cold_tiles), key, mh_steps,
                                                                                            STAMP_ACCEPT_COLD);
         ++launches;
     }
@@ -700,16 +702,17 @@ static int launch_propose(Ctx& c, uint2 key, int mh_steps)
     // the running vocabulary slice's tokens (its tables are the ones in memory)
     const View& v = c.v;
     const Ctx::Slice& q = c.slices[(size_t)c.cur_slice];
+    const PassStreams on(c, (q.hotp_n > 0) + (q.cold_n > 0));
     const bool noted = c.slices.size() == 1;  // several slices: the pass starts with the first slice's tables
     int launches = 0;
     if (q.hotp_n) {
-        k_word_hot<T, CH, false, false, MODE, FIXED><<<q.hotp_n, PROPOSE_THREADS, 0, c.stream>>>(
+        k_word_hot<T, CH, false, false, MODE, FIXED><<<q.hotp_n, PROPOSE_THREADS, 0, on[0]>>>(
             v, c.hot_tiles_propose + 3 * (size_t)q.hotp_lo, key, mh_steps, noted ? STAMP_PROPOSE_HOT : -1);
         ++launches;
     }
     if (q.cold_n) {
-        k_word_cold<T, CH, false, MODE, FIXED><<<q.cold_n, COLD_THREADS, 0, c.stream>>>(
-            v, c.cold_tiles + 2 * (size_t)q.cold_lo, key, mh_steps, noted ? STAMP_PROPOSE_COLD : -1);
+        k_word_cold<T, CH, false, MODE, FIXED><<<q.cold_n, COLD_THREADS, 0, on[1]>>>(
+            v, reinterpret_cast<const int4*>(c.cold_tiles) + q.cold_lo, key, mh_steps, noted ? STAMP_PROPOSE_COLD : -1);
         ++launches;
     }
     return launches;

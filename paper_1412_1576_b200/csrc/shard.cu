@@ -72,7 +72,7 @@ int launch_word_counts_from_dense(Ctx& c, const int32_t* nwk_dev)
 {
     k_rows_from_dense<<<c.V, 256, 0, c.stream>>>(c.v, nwk_dev);
     cudaMemsetAsync(c.v.nk_next, 0, (size_t)c.v.dense_stride * 4, c.stream);
-    const int launches = 1 + launch_count_k(c);  // n_k = column sums of the rows just written
+    const int launches = 1 + launch_count_k_from_rows(c);  // n_k = column sums of the rows just written
     exchange_nk(c);
     return launches;
 }
