@@ -3,7 +3,7 @@
 // table per word, O(K_w) to build) and a dense term beta/(n_k + V*beta) whose alias
 // table is shared by all words.
 //
-// Alias construction is cooperative (a warp for short rows, a CTA for long ones)
+// Alias construction is cooperative (a few lanes to a cluster of CTAs per row)
 // and exact in integers, so the table is a function of the counts alone:
 //   - fixed-point weights wt_i = floor(weight_i * 2^44), W44 = sum wt_i;
 //   - pre-shift sh = max(0, bitlen(W44) + bitlen(n) - 62), w_i = wt_i >> sh, W = sum w_i;
@@ -16,17 +16,15 @@
 // exhausted heavy item becomes a bin topped up by the next heavy item".
 #include <cooperative_groups.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "lda_device.cuh"
 #include "lda_internal.cuh"
 
 namespace lda {
 
 typedef unsigned long long ull;
-
-#ifndef LDA_ALIAS_BINS_AT_ONCE
-#define LDA_ALIAS_BINS_AT_ONCE 2
-#endif
-constexpr int ALIAS_BINS_AT_ONCE = LDA_ALIAS_BINS_AT_ONCE;  // bins a thread finishes side by side
 
 // The threads that build one row together: a warp, a CTA, or a cluster of CTAs.
 enum GroupKind { WARP, CTA, CLUSTER };
@@ -135,52 +133,13 @@ struct Group {
     }
 };
 
-// to_frac32(part, whole) for many parts <= whole of one whole: the quotient from a double
-// reciprocal of the (shifted) whole, then set right with the exact integer remainder.  The
-// estimate is within 2^-20 of the true quotient (two roundings of 2^-53 on a value <= 2^32), so
-// its integer part is off by one at most.
-struct Frac32 {
-    int sh;
-    uint32_t w;  // whole >> sh, < 2^32
-    double inv;  // 1 / w
-    __device__ __forceinline__ explicit Frac32(ull whole)
-    {
-        sh = bit_length(whole) - 32;
-        if (sh < 0) sh = 0;
-        w = (uint32_t)(whole >> sh);
-        inv = __ddiv_rn(1.0, u32_to_double(w));
-    }
-    __device__ __forceinline__ uint32_t operator()(ull part) const
-    {
-        const uint32_t p = (uint32_t)(part >> sh);  // part <= whole
-        const ull x = (ull)p << 32;
-        ull q = __double2ull_rz(__dmul_rn(__dmul_rn(u32_to_double(p), 4294967296.0), inv));
-        const long long r = (long long)(x - q * (ull)w);
-        if (r < 0) --q;
-        else if (r >= (long long)w) ++q;
-        return q > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)q;
-    }
-};
-
-// One bin in the form the MH kernel reads with a single load.  With `topic` (a word's sorted
-// row) the second word holds the topics of the bin's own item and of its alias item, 16 bits
-// each; without it (the dense table, whose items are the topics) it holds the alias.
-__device__ __forceinline__ void store_packed_bin(uint2* out_pk, const uint32_t* topic, uint32_t i, uint32_t thr32,
-                                                 uint32_t al)
-{
-    if (!out_pk) return;
-    out_pk[i] = make_uint2(thr32, topic ? (topic[i] | (topic[al] << 16)) : al);
-}
-
 // Builds one table of n items.  weight(i) gives the fixed-point weight of item i.
 // sc_w, sc_de, sc_item: scratch of n entries each, private to this row.
-// out_pk (may be null) receives the packed form of every bin, see store_packed_bin().
+// out.bin(i, split point, alias item) receives every bin.
 // Returns W44 (the sum of the fixed-point weights) to every thread of the group.
-template <GroupKind KIND, class Weight>
-__device__ ull build_alias_row(const Group<KIND>& g, int32_t n, Weight weight, ull* __restrict__ sc_w,
-                               ull* __restrict__ sc_de, uint32_t* __restrict__ sc_item,
-                               uint32_t* __restrict__ out_thr, uint32_t* __restrict__ out_idx,
-                               uint2* __restrict__ out_pk, const uint32_t* __restrict__ pk_topic, int* err)
+template <GroupKind KIND, class Weight, class Item, class Out>
+__device__ ull build_alias_row(const Group<KIND>& g, int32_t n, Weight weight, ull* __restrict__ sc_w, ull* __restrict__ sc_de,
+                               Item* __restrict__ sc_item, const Out& out, int* err)
 {
     const int r = g.rank(), gs = g.size();
     // Items are taken four (weights) or two (bins) at a time per thread, their loads issued side by
@@ -236,13 +195,13 @@ __device__ ull build_alias_row(const Group<KIND>& g, int32_t n, Weight weight, u
             sc_w[i] = a;
             if (a <= W) {
                 sc_de[l] = d_at;  // deficits of the lights before this one
-                sc_item[l] = (uint32_t)i;
+                sc_item[l] = (Item)i;
                 ++l;
                 d_at += W - a;
             } else {
                 e_at += a - W;
                 sc_de[n - 1 - m] = e_at;  // surpluses of the heavies up to and including this one
-                sc_item[n - 1 - m] = (uint32_t)i;
+                sc_item[n - 1 - m] = (Item)i;
                 ++m;
             }
         }
@@ -252,9 +211,9 @@ __device__ ull build_alias_row(const Group<KIND>& g, int32_t n, Weight weight, u
     g.sync();
     const Frac32 frac(W);
     // The searches below count the entries of a sorted prefix array under a bound, one bit of the
-    // answer per step from the top: the same number of steps for every item, so two items' searches
-    // run in one loop.
-    constexpr int U = ALIAS_BINS_AT_ONCE;
+    // answer per step from the top: the same number of steps for every item, so several items' searches
+    // run in one loop (a CTA has more barriers to make up for than a warp, and fewer neighbours on its SM).
+    constexpr int U = KIND == WARP ? 2 : 4;
     const uint32_t top_h = H ? 1u << (31 - __clz((int)H)) : 0u;
     const uint32_t top_l = L ? 1u << (31 - __clz((int)L)) : 0u;
     for (uint32_t l0 = r; l0 < L; l0 += U * gs) {
@@ -287,9 +246,7 @@ __device__ ull build_alias_row(const Group<KIND>& g, int32_t n, Weight weight, u
                 al = H ? sc_item[n - 1 - lo] : i;
             }
             const uint32_t thr32 = frac(a[u]);
-            out_thr[i] = thr32;
-            out_idx[i] = al;
-            store_packed_bin(out_pk, pk_topic, i, thr32, al);
+            out.bin(i, thr32, al);
         }
     }
     for (uint32_t m0 = r; m0 < H; m0 += U * gs) {
@@ -322,9 +279,7 @@ __device__ ull build_alias_row(const Group<KIND>& g, int32_t n, Weight weight, u
                 else al = sc_item[n - 1 - (m + 1)];
             }
             const uint32_t thr32 = frac(thr);
-            out_thr[i] = thr32;
-            out_idx[i] = al;
-            store_packed_bin(out_pk, pk_topic, i, thr32, al);
+            out.bin(i, thr32, al);
         }
     }
     return W44;
@@ -354,6 +309,18 @@ struct SparseWeight {
     }
 };
 
+struct DenseOut {
+    uint32_t* thr;
+    uint32_t* idx;
+    uint2* pk;  // both in one word pair, for the proposal pass; may be null
+    __device__ __forceinline__ void bin(uint32_t i, uint32_t thr32, uint32_t al) const
+    {
+        thr[i] = thr32;
+        idx[i] = al;
+        if (pk) pk[i] = make_uint2(thr32, al);
+    }
+};
+
 // First kernel of a sweep: the dense smoothing table.  Also moves the device's sweep counter on and
 // clears the n_k buffer the sweep's rebuild will add into (nothing else of this sweep touches either).
 // One CTA builds a table of up to DENSE_CTA_MAX_K topics; a larger one takes a cluster of DENSE_CLUSTER
@@ -379,8 +346,8 @@ __global__ void __launch_bounds__(1024) k_alias_dense(View v, ull* sc)
     if (v.nk_next)
         for (int32_t k = g.rank(); k < v.dense_stride; k += g.size()) v.nk_next[k] = 0;
     DenseWeight wf{v.nk, v.beta, v.Vbeta};
-    const ull B = build_alias_row<KIND>(g, K, wf, sc, sc + K, (uint32_t*)(sc + 2 * (size_t)K), v.dn_thr,
-                                        v.dn_idx, v.dn_pk, nullptr, v.err);
+    const ull B = build_alias_row<KIND>(g, K, wf, sc, sc + K, (uint32_t*)(sc + 2 * (size_t)K),
+                                        DenseOut{v.dn_thr, v.dn_idx, v.dn_pk}, v.err);
     if (g.rank() == 0) {
         *v.dense_mass = B;
         if (v.state) v.state->stamps[v.state->slot][STAMP_DENSE_END] = global_timer();
@@ -418,70 +385,225 @@ void launch_mix_thresholds(Ctx& c, uint32_t* mix32)
     k_mix_thresholds<<<(c.V + 255) / 256, 256, 0, c.stream>>>(c.v, mix32);
 }
 
-// One warp per word, rows of at most ALIAS_WARP_MAX items.  The two scratch arrays the binary
-// searches run over live in shared memory (12 bytes per item and warp), the third in the row's
-// range of the scratch array in device memory.
-__global__ void __launch_bounds__(256) k_alias_sparse_warp(View v, ull* sc_w, int32_t w_lo, int32_t w_hi)
-{
-    extern __shared__ __align__(16) unsigned char alias_scratch[];
-    Group<WARP> g{nullptr};
-    const int warps = (gridDim.x * blockDim.x) >> 5;
-    const int wic = threadIdx.x >> 5;
-    ull* de_s = reinterpret_cast<ull*>(alias_scratch) + (size_t)wic * ALIAS_WARP_MAX;
-    uint32_t* item_s = reinterpret_cast<uint32_t*>(reinterpret_cast<ull*>(alias_scratch) + 8 * ALIAS_WARP_MAX) +
-                       (size_t)wic * ALIAS_WARP_MAX;
-    for (int32_t w = w_lo + ((blockIdx.x * blockDim.x + threadIdx.x) >> 5); w < w_hi; w += warps) {
-        const int32_t n = v.wk_nnz[w];
-        if (n > ALIAS_WARP_MAX) continue;
-        if (n == 0) {
-            if ((threadIdx.x & 31) == 0) v.sp_mass[w] = 0;
-            continue;
+// ---- per-word sparse tables ----------------------------------------------------------------------
+// Rows differ in length by four orders of magnitude, and what a row costs is the latency of its chain
+// of dependent steps (weights, two sums, one scan, one search per item), so a row gets as many threads as
+// it has work for: a few lanes (up to 32 items, everything in registers), a warp (256, 512), a CTA of 256 threads (2048),
+// one of 1024 (ALIAS_BIG_MAX), a cluster (longer).  Which kernel looks at a word depends on the
+// row's capacity, which one builds it on its length in this sweep.
+//
+// Who reads a table decides what is written: hot words (with 16-bit topics) are drawn from through packed bins,
+// all others through split points and alias items (lda_get_tables() wants those of all words: `all`).
+struct RowOut {
+    uint32_t* thr;
+    uint32_t* idx;
+    uint2* pk;               // null: not wanted
+    const uint32_t* topic;   // of the row's items
+    bool plain;              // thr, idx wanted
+    __device__ __forceinline__ RowOut(const View& v, int32_t w, int32_t r0, bool all)
+    {
+        const bool hot = __ldg(v.hot_word + w) != 0;
+        thr = v.al_thr + r0;
+        idx = v.al_idx + r0;
+        pk = (v.al_pk && (hot || all)) ? v.al_pk + r0 : nullptr;
+        topic = v.wk_topic + r0;
+        plain = all || !hot || !v.al_pk;
+    }
+    __device__ __forceinline__ void bin(int32_t i, uint32_t thr32, uint32_t al) const
+    {
+        if (plain) {
+            thr[i] = thr32;
+            idx[i] = al;
         }
-        const int32_t r0 = v.row_start[w];
-        SparseWeight wf{v.wk_topic + r0, v.wk_count + r0, v.nk, v.Vbeta};
-        const ull S = build_alias_row<WARP>(g, n, wf, sc_w + r0, de_s, item_s, v.al_thr + r0, v.al_idx + r0,
-                                             v.al_pk ? v.al_pk + r0 : nullptr, v.wk_topic + r0, v.err);
-        if ((threadIdx.x & 31) == 0) v.sp_mass[w] = S;
-        __syncwarp();
+        if (pk) pk[i] = make_uint2(thr32, topic[i] | (topic[al] << 16));
+    }
+};
+
+__device__ __forceinline__ ull sparse_weight(uint32_t count, int32_t nk, double Vbeta)
+{
+    const double den = __dadd_rn(u32_to_double((uint32_t)nk), Vbeta);
+    return __double2ull_rz(__dmul_rn(__ddiv_rn(u32_to_double(count), den), FIXED_ONE));
+}
+
+// Rows of at most WD items, one lane per item, 32 / WD rows per warp.  Every lane of the warp calls it
+// (n = 0: no row).
+template <int WD>
+__device__ __forceinline__ void alias_row_lanes(const View& v, int32_t w, int32_t n, int32_t r0, bool all)
+{
+    constexpr uint32_t FULL = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31, l = lane & (WD - 1);
+    const bool live = l < n;
+    uint32_t k = 0;
+    ull a = 0;
+    if (live) {
+        k = __ldg(v.wk_topic + r0 + l);
+        a = sparse_weight(__ldg(v.wk_count + r0 + l), __ldg(v.nk + k), v.Vbeta);
+    }
+    ull W44 = a;
+#pragma unroll
+    for (int o = WD / 2; o > 0; o >>= 1) W44 += __shfl_xor_sync(FULL, W44, o);
+    const int sh = max(0, bit_length(W44) + bit_length((ull)n) - 62);
+    a >>= sh;
+    ull W = a;
+#pragma unroll
+    for (int o = WD / 2; o > 0; o >>= 1) W += __shfl_xor_sync(FULL, W, o);
+    a *= (ull)n;
+    const bool heavy = live && a > W;
+    const ull d = live && !heavy ? W - a : 0, e = heavy ? a - W : 0;
+    ull D = d, E = e;  // inclusive prefixes over the row's lanes
+#pragma unroll
+    for (int o = 1; o < WD; o <<= 1) {
+        const ull x = __shfl_up_sync(FULL, D, o, WD), y = __shfl_up_sync(FULL, E, o, WD);
+        if (l >= o) {
+            D += x;
+            E += y;
+        }
+    }
+    const ull d_sum = __shfl_sync(FULL, D, WD - 1, WD);
+    D -= d;  // deficits of the lights before this lane
+    // a light item looks for the first lane whose surpluses exceed D, a heavy one for the first lane with
+    // deficits of at least E before it; both prefixes ascend over the lanes
+    int pos = 0;
+#pragma unroll
+    for (int step = WD / 2; step > 0; step >>= 1) {
+        const int q = pos + step;
+        const ull x = __shfl_sync(FULL, E, q - 1, WD), y = __shfl_sync(FULL, D, q - 1, WD);
+        if (heavy ? y < E : x <= D) pos = q;
+    }
+    {
+        const ull x = __shfl_sync(FULL, E, pos, WD), y = __shfl_sync(FULL, D, pos, WD);
+        if (heavy ? y < E : x <= D) ++pos;
+    }
+    const ull D_at = __shfl_sync(FULL, D, min(pos, WD - 1), WD);
+    const uint32_t heavies = (__ballot_sync(FULL, heavy) >> (lane & ~(WD - 1))) & (WD == 32 ? FULL : (1u << WD) - 1u);
+    const uint32_t above = heavies & ~((2u << l) - 1u);
+    ull part = a;
+    int al = l;
+    bool bad = live && W == 0;
+    if (heavy) {
+        part = W + E - (pos < WD ? D_at : d_sum);
+        if (part != W) {
+            bad = bad || !above;
+            if (above) al = __ffs((int)above) - 1;
+        }
+    } else if (live && a != W) {
+        bad = bad || pos >= n;
+        if (pos < n) al = pos;
+    }
+    if (bad) atomicOr(v.err, ERR_ALIAS);
+    const uint32_t k_al = __shfl_sync(FULL, k, al, WD);
+    if (live) {
+        const uint32_t thr32 = Frac32(W)(part);
+        const RowOut out(v, w, r0, all);
+        if (out.plain) {
+            out.thr[l] = thr32;
+            out.idx[l] = (uint32_t)al;
+        }
+        if (out.pk) out.pk[l] = make_uint2(thr32, k | (k_al << 16));
+        if (l == 0) v.sp_mass[w] = W44;
     }
 }
 
-// One CTA per word whose row can be longer than ALIAS_WARP_MAX.  The construction's scratch
-// (20 bytes per item) lives in shared memory when the row has at most `smem_items` items; a longer
-// row keeps the array its binary searches run over (8 bytes per item) there as long as that fits,
-// and the rest -- or, beyond that, everything -- in the row's range of the scratch arrays in
-// device memory.
-#ifndef LDA_ALIAS_MID_MIN_CTAS
-#define LDA_ALIAS_MID_MIN_CTAS 1
-#endif
-template <int THREADS>
-__global__ void __launch_bounds__(THREADS, THREADS == 256 ? LDA_ALIAS_MID_MIN_CTAS : 1)
-k_alias_sparse_block(View v, const int32_t* __restrict__ words, ull* sc_w, ull* sc_de, uint32_t* sc_item,
-                     int32_t smem_items)
+constexpr int ALIAS_WARP_THREADS = 256;
+constexpr int ALIAS_WARP_SMEM = ALIAS_WARP_THREADS / 32 * ALIAS_WARP_MAX * ALIAS_SCRATCH_PER_ITEM;
+// Rows of up to ALIAS_WARP_MAX items: a warp takes `per_warp` consecutive words, the short rows several at a time.
+__global__ void __launch_bounds__(ALIAS_WARP_THREADS) k_alias_sparse_warp(View v, int32_t w_lo, int32_t w_hi, int32_t per_warp, bool all)
+{
+    extern __shared__ __align__(16) unsigned char alias_scratch[];
+    constexpr int WARPS = ALIAS_WARP_THREADS / 32;
+    constexpr uint32_t FULL = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31, wic = threadIdx.x >> 5;
+    const Group<WARP> g{nullptr};
+    const int32_t stride = (int32_t)((gridDim.x * blockDim.x) >> 5) * per_warp;
+    for (int32_t wb = w_lo + (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per_warp; wb < w_hi; wb += stride) {
+        const int32_t mine = wb + lane;
+        int32_t n_mine = -1, r_mine = 0;
+        if (lane < per_warp && mine < w_hi) {
+            n_mine = v.wk_nnz[mine];
+            r_mine = v.row_start[mine];
+            if (n_mine == 0) v.sp_mass[mine] = 0;
+        }
+        // the lanes of `words` that hold a row of the class; `rows` of them are built at once
+        auto several = [&](uint32_t words, auto width) {
+            constexpr int WD = decltype(width)::value;
+            while (words) {
+                uint32_t rest = words;
+                for (int i = 0; i < lane / WD; ++i) rest &= rest - 1;  // this lane's group takes the (lane / WD)-th
+                const int src = rest ? __ffs((int)rest) - 1 : 0;
+                const int32_t n = __shfl_sync(FULL, n_mine, src), r0 = __shfl_sync(FULL, r_mine, src);
+                alias_row_lanes<WD>(v, wb + src, rest ? n : 0, r0, all);
+                for (int i = 0; i < 32 / WD; ++i) words &= words - 1;
+            }
+        };
+        several(__ballot_sync(FULL, n_mine > 0 && n_mine <= 8), std::integral_constant<int, 8>{});
+        several(__ballot_sync(FULL, n_mine > 8 && n_mine <= 16), std::integral_constant<int, 16>{});
+        several(__ballot_sync(FULL, n_mine > 16 && n_mine <= 32), std::integral_constant<int, 32>{});
+        for (uint32_t words = __ballot_sync(FULL, n_mine > 32 && n_mine <= ALIAS_WARP_MAX); words; words &= words - 1) {
+            const int src = __ffs((int)words) - 1;
+            const int32_t n = __shfl_sync(FULL, n_mine, src), r0 = __shfl_sync(FULL, r_mine, src);
+            const int32_t w = wb + src;
+            ull* de = reinterpret_cast<ull*>(alias_scratch) + (size_t)wic * ALIAS_WARP_MAX;
+            ull* wt = de + WARPS * ALIAS_WARP_MAX;
+            uint16_t* item = reinterpret_cast<uint16_t*>(reinterpret_cast<ull*>(alias_scratch) + 2 * WARPS * ALIAS_WARP_MAX) +
+                             (size_t)wic * ALIAS_WARP_MAX;
+            const SparseWeight wf{v.wk_topic + r0, v.wk_count + r0, v.nk, v.Vbeta};
+            const ull S = build_alias_row<WARP>(g, n, wf, wt, de, item, RowOut(v, w, r0, all), v.err);
+            if (lane == 0) v.sp_mass[w] = S;
+            __syncwarp();
+        }
+    }
+}
+
+// One warp per word of the list: rows of ALIAS_WARP_MAX < n <= ALIAS_LONG_WARP_MAX items.  Their weights stay in
+// device memory: 18 bytes of shared memory per item would leave too few warps per multiprocessor (738 M tokens,
+// K = 10 000, all kernels together: 1.6 ms so, 1.8 with these rows on CTAs of 256 threads).
+__global__ void __launch_bounds__(128) k_alias_sparse_long_warp(View v, const int32_t* __restrict__ words, int32_t n_words, bool all,
+                                                                ull* sc_w)
+{
+    __shared__ ull de_s[4][ALIAS_LONG_WARP_MAX];
+    __shared__ uint16_t item_s[4][ALIAS_LONG_WARP_MAX];
+    const int wic = threadIdx.x >> 5;
+    const int32_t i = blockIdx.x * 4 + wic;
+    if (i >= n_words) return;
+    const int32_t w = words[i], n = v.wk_nnz[w];
+    if (n <= ALIAS_WARP_MAX || n > ALIAS_LONG_WARP_MAX) return;
+    const int32_t r0 = v.row_start[w];
+    const SparseWeight wf{v.wk_topic + r0, v.wk_count + r0, v.nk, v.Vbeta};
+    const ull S = build_alias_row<WARP>(Group<WARP>{nullptr}, n, wf, sc_w + r0, de_s[wic], item_s[wic], RowOut(v, w, r0, all), v.err);
+    if ((threadIdx.x & 31) == 0) v.sp_mass[w] = S;
+}
+
+// One CTA per word: rows of LO < n <= HI items.
+template <int THREADS, int LO, int HI>
+__global__ void __launch_bounds__(THREADS)
+k_alias_sparse_cta(View v, const int32_t* __restrict__ words, bool all)
 {
     extern __shared__ __align__(16) unsigned char alias_scratch[];
     __shared__ ull smem[GROUP_SMEM];
-    Group<CTA> g{smem};
+    const Group<CTA> g{smem};
     const int32_t w = words[blockIdx.x];
     const int32_t n = v.wk_nnz[w];
-    if (n <= ALIAS_WARP_MAX) return;
+    if (n <= LO || n > HI) return;
     const int32_t r0 = v.row_start[w];
-    SparseWeight wf{v.wk_topic + r0, v.wk_count + r0, v.nk, v.Vbeta};
-    uint2* pk = v.al_pk ? v.al_pk + r0 : nullptr;
-    ull S;
-    if (n <= smem_items) {
-        ull* w_s = reinterpret_cast<ull*>(alias_scratch);
-        ull* de_s = w_s + smem_items;
-        uint32_t* item_s = reinterpret_cast<uint32_t*>(de_s + smem_items);
-        S = build_alias_row<CTA>(g, n, wf, w_s, de_s, item_s, v.al_thr + r0, v.al_idx + r0, pk, v.wk_topic + r0, v.err);
-    } else if ((int64_t)n * 8 <= (int64_t)smem_items * ALIAS_SCRATCH_PER_ITEM) {
-        S = build_alias_row<CTA>(g, n, wf, sc_w + r0, reinterpret_cast<ull*>(alias_scratch), sc_item + r0,
-                                  v.al_thr + r0, v.al_idx + r0, pk, v.wk_topic + r0, v.err);
-    } else {
-        S = build_alias_row<CTA>(g, n, wf, sc_w + r0, sc_de + r0, sc_item + r0, v.al_thr + r0, v.al_idx + r0, pk,
-                                  v.wk_topic + r0, v.err);
-    }
+    ull* wt = reinterpret_cast<ull*>(alias_scratch);
+    const SparseWeight wf{v.wk_topic + r0, v.wk_count + r0, v.nk, v.Vbeta};
+    const ull S = build_alias_row<CTA>(g, n, wf, wt, wt + HI, reinterpret_cast<uint16_t*>(wt + 2 * HI), RowOut(v, w, r0, all), v.err);
     if (threadIdx.x == 0) v.sp_mass[w] = S;
+}
+
+// Rows longer than ALIAS_BIG_MAX: a cluster of CTAs per word, scratch in the row's range of the arrays in device memory.
+__global__ void __cluster_dims__(ALIAS_ROW_CLUSTER) __launch_bounds__(512)
+k_alias_sparse_cluster(View v, const int32_t* __restrict__ words, ull* sc_w, ull* sc_de, uint32_t* sc_item, bool all)
+{
+    __shared__ ull smem[GROUP_SMEM];
+    const Group<CLUSTER> g{smem};
+    const int32_t w = words[blockIdx.x / ALIAS_ROW_CLUSTER];
+    const int32_t n = v.wk_nnz[w];
+    if (n <= ALIAS_BIG_MAX) return;
+    const int32_t r0 = v.row_start[w];
+    const SparseWeight wf{v.wk_topic + r0, v.wk_count + r0, v.nk, v.Vbeta};
+    const ull S = build_alias_row<CLUSTER>(g, n, wf, sc_w + r0, sc_de + r0, sc_item + r0, RowOut(v, w, r0, all), v.err);
+    if (g.rank() == 0) v.sp_mass[w] = S;
 }
 
 int launch_alias_dense(Ctx& c, bool in_sweep)
@@ -495,28 +617,40 @@ int launch_alias_dense(Ctx& c, bool in_sweep)
     return 1;
 }
 
-// The three kernels build the tables of different words: they run side by side, the one with the
-// longest rows (and the longest tail) first.
-int launch_alias_sparse(Ctx& c)
+// The kernels build the tables of different words: they run side by side, the ones with the longest rows
+// (and the longest tail) first.
+int launch_alias_sparse(Ctx& c, bool all)
 {
     const Ctx::Slice& q = c.slices[(size_t)c.cur_slice];
     if (q.w_hi <= q.w_lo) return 0;
     int launches = 0;
     fork_streams(c);
-    // words whose row cannot exceed ALIAS_SMEM_ITEMS_MID come first in the list
-    if (q.big_n) {
-        k_alias_sparse_block<512><<<q.big_n, 512, ALIAS_SMEM_ITEMS_BIG * ALIAS_SCRATCH_PER_ITEM, c.stream>>>(
-            c.v, c.alias_big + c.n_alias_mid + q.big_lo, c.sc_w, c.sc_de, c.sc_item, ALIAS_SMEM_ITEMS_BIG);
+    const auto words = [&](int cls) { return c.alias_words[cls] + q.alias_lo[cls]; };
+    if (q.alias_n[3]) {
+        k_alias_sparse_cluster<<<q.alias_n[3] * ALIAS_ROW_CLUSTER, 512, 0, c.stream>>>(c.v, words(3), c.sc_w, c.sc_de, c.sc_item, all);
         ++launches;
     }
-    if (q.mid_n) {
-        k_alias_sparse_block<256><<<q.mid_n, 256, ALIAS_SMEM_ITEMS_MID * ALIAS_SCRATCH_PER_ITEM, c.side[0]>>>(
-            c.v, c.alias_big + q.mid_lo, c.sc_w, c.sc_de, c.sc_item, ALIAS_SMEM_ITEMS_MID);
+    if (q.alias_n[2]) {
+        k_alias_sparse_cta<1024, ALIAS_MID_MAX, ALIAS_BIG_MAX>
+            <<<q.alias_n[2], 1024, ALIAS_BIG_MAX * ALIAS_SCRATCH_PER_ITEM, c.stream>>>(c.v, words(2), all);
         ++launches;
     }
-    int grid = (int)(((int64_t)(q.w_hi - q.w_lo) * 32 + 255) / 256);
-    if (grid > 148 * 16) grid = 148 * 16;
-    k_alias_sparse_warp<<<grid, 256, ALIAS_WARP_SMEM, c.side[1]>>>(c.v, c.sc_w, q.w_lo, q.w_hi);
+    if (q.alias_n[1]) {
+        k_alias_sparse_cta<256, ALIAS_LONG_WARP_MAX, ALIAS_MID_MAX>
+            <<<q.alias_n[1], 256, ALIAS_MID_MAX * ALIAS_SCRATCH_PER_ITEM, c.side[0]>>>(c.v, words(1), all);
+        ++launches;
+    }
+    if (q.alias_n[0]) {
+        k_alias_sparse_long_warp<<<(q.alias_n[0] + 3) / 4, 128, 0, c.side[0]>>>(c.v, words(0), q.alias_n[0], all, c.sc_w);
+        ++launches;
+    }
+    // words per warp: as many as fill a warp's lanes with the words' sizes, as long as every multiprocessor gets two CTAs
+    int per_warp = 32;
+    while (per_warp > 4 && (int64_t)(q.w_hi - q.w_lo) / per_warp < (int64_t)c.n_sm * 16) per_warp /= 2;
+    const int64_t warps = ((int64_t)(q.w_hi - q.w_lo) + per_warp - 1) / per_warp;
+    constexpr int WARPS = ALIAS_WARP_THREADS / 32;
+    k_alias_sparse_warp<<<(int)std::min<int64_t>((warps + WARPS - 1) / WARPS, (int64_t)c.n_sm * 16), ALIAS_WARP_THREADS,
+                          ALIAS_WARP_SMEM, c.side[1]>>>(c.v, q.w_lo, q.w_hi, per_warp, all);
     ++launches;
     join_streams(c);
     return launches;
@@ -525,10 +659,10 @@ int launch_alias_sparse(Ctx& c)
 void set_alias_smem_limits()
 {
     cudaFuncSetAttribute(k_alias_sparse_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, ALIAS_WARP_SMEM);
-    cudaFuncSetAttribute(k_alias_sparse_block<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         ALIAS_SMEM_ITEMS_MID * ALIAS_SCRATCH_PER_ITEM);
-    cudaFuncSetAttribute(k_alias_sparse_block<512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         ALIAS_SMEM_ITEMS_BIG * ALIAS_SCRATCH_PER_ITEM);
+    cudaFuncSetAttribute(k_alias_sparse_cta<256, ALIAS_LONG_WARP_MAX, ALIAS_MID_MAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         ALIAS_MID_MAX * ALIAS_SCRATCH_PER_ITEM);
+    cudaFuncSetAttribute(k_alias_sparse_cta<1024, ALIAS_MID_MAX, ALIAS_BIG_MAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         ALIAS_BIG_MAX * ALIAS_SCRATCH_PER_ITEM);
 }
 
 }  // namespace lda

@@ -334,7 +334,7 @@ void rebuild_counts(Ctx& c)
 static int queue_sweep(Ctx& c, int mh_steps)
 {
     int n = launch_alias_dense(c, true);
-    if (c.slices.size() == 1) n += launch_alias_sparse(c);  // else slice by slice inside pass 1
+    if (c.slices.size() == 1) n += launch_alias_sparse(c, false);  // else slice by slice inside pass 1
     n += launch_sample(c, mh_steps);
     n += launch_count_wk(c);
     n += launch_count_k(c);
@@ -418,7 +418,7 @@ static int ensure_tables(Ctx& c)
 {
     if (c.tables_valid) return LDA_OK;
     launch_alias_dense(c, false);
-    launch_alias_sparse(c);  // the running slice's (lda_get_tables walks the slices itself)
+    launch_alias_sparse(c, true);  // the running slice's (lda_get_tables walks the slices itself)
     int bits = 0;
     int rc = read_err(c, &bits);
     if (rc) return rc;
@@ -514,10 +514,15 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     int32_t propose_tile = run_for(t_hot, 4, HOT_TILE_PROPOSE_MAX, 2048);
     if (propose_tile == 2048) propose_tile = 1536;  // one turn of the two-step kernel
     const int32_t cold_tile = run_for(t_cold, 4, COLD_TILE, 256);
+    // tail tiles of few enough words for a counter per word and topic, if they still hold a fair number of tokens
+    const int32_t direct_words = std::min(COLD_DIRECT / K, COLD_WORDS);
+    c.cold_direct = direct_words > 0 && t_cold / std::max(1, V) * direct_words >= cold_tile / 2;
+    const int32_t cold_words = c.cold_direct ? direct_words : COLD_WORDS;
     const bool sorted_rows = K > WORD_ROWS_BITMAP_MAX_K;
     const int32_t row_tile = run_for(N - t_dense, 4, SORT_TILE, 256), row_tile_words = sorted_rows ? SORT_TILE : ROW_TILE_WORDS;
 
-    std::vector<int32_t> dense_slot((size_t)V, -1), row_start((size_t)V + 1), alias_big, alias_mid;
+    std::vector<int32_t> dense_slot((size_t)V, -1), row_start((size_t)V + 1), alias_words[ALIAS_CLASSES];
+    std::vector<uint8_t> hot_word((size_t)V);
     std::vector<int32_t> hot_runs, acc_runs, word_tiles;
     int64_t cap_total = 0;
     c.n_dense = 0;
@@ -525,8 +530,8 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
         row_start[w] = (int32_t)cap_total;
         const int32_t cap = std::min(tf[w], K);
         cap_total += cap;
-        if (cap > ALIAS_SMEM_ITEMS_MID) alias_big.push_back(w);
-        else if (cap > ALIAS_WARP_MAX) alias_mid.push_back(w);
+        hot_word[w] = is_hot(w);
+        for (int i = 0; i < ALIAS_CLASSES && cap > ALIAS_CLASS_MAX[i]; ++i) alias_words[i].push_back(w);
         if (warm_class && tf[w] > SORT_TILE && tf[w] <= WARM_MAX_TF) {
             warm_words.push_back(w);
         } else if (has_dense_row(w)) {
@@ -592,7 +597,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
                     cold_tiles.insert(cold_tiles.end(), {w, w + 1, word_off[w] + o, std::min(cold_tile, tf_here[w] - o)});
                 continue;
             }
-            if (tok + tf[w] > cold_tile || w - s0 >= COLD_WORDS) { close(w); s0 = w; tok = 0; }
+            if (tok + tf[w] > cold_tile || w - s0 >= cold_words) { close(w); s0 = w; tok = 0; }
             tok += tf[w];
         }
         close(V);
@@ -649,9 +654,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.n_hot_runs = (int32_t)(hot_runs.size() / 4);
     c.nk_with_rows = K <= NK_WITH_ROWS_MAX_K && c.n_hot_runs + c.n_word_tiles <= NK_WITH_ROWS_MAX_CTAS;
     c.n_long_docs = (int32_t)long_docs.size();
-    c.n_alias_mid = (int32_t)alias_mid.size();
-    alias_big.insert(alias_big.begin(), alias_mid.begin(), alias_mid.end());
-    c.n_alias_big = (int32_t)alias_big.size();
+    for (int i = 0; i < ALIAS_CLASSES; ++i) c.n_alias_words[i] = (int32_t)alias_words[i].size();
     c.n_hot_tiles = (int32_t)(hot_tiles.size() / 3);
     c.n_hot_tiles_warm = (int32_t)(hot_tiles_warm.size() / 3);
     c.n_warm = (int32_t)warm_words.size();
@@ -669,7 +672,6 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
             }
             return (int32_t)a;
         };
-        const size_t n_mid = (size_t)c.n_alias_mid, n_big = (size_t)c.n_alias_big;
         for (int sl = 0; sl < n_slices; ++sl) {
             Ctx::Slice& q = c.slices[(size_t)sl];
             q.w_lo = slice_w[(size_t)sl];
@@ -677,10 +679,10 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
             q.row_lo = row_start[(size_t)q.w_lo];
             q.row_n = row_start[(size_t)q.w_hi] - q.row_lo;
             slice_rows_max = std::max(slice_rows_max, q.row_n);
-            q.mid_lo = first_at(alias_big, 0, n_mid, 1, q.w_lo);
-            q.mid_n = first_at(alias_big, 0, n_mid, 1, q.w_hi) - q.mid_lo;
-            q.big_lo = first_at(alias_big, n_mid, n_big, 1, q.w_lo) - (int32_t)n_mid;
-            q.big_n = first_at(alias_big, n_mid, n_big, 1, q.w_hi) - (int32_t)n_mid - q.big_lo;
+            for (int i = 0; i < ALIAS_CLASSES; ++i) {
+                q.alias_lo[i] = first_at(alias_words[i], 0, alias_words[i].size(), 1, q.w_lo);
+                q.alias_n[i] = first_at(alias_words[i], 0, alias_words[i].size(), 1, q.w_hi) - q.alias_lo[i];
+            }
             q.hotp_lo = first_at(hot_tiles_propose, 0, (size_t)c.n_hot_tiles_propose, 3, q.w_lo);
             q.hotp_n = first_at(hot_tiles_propose, 0, (size_t)c.n_hot_tiles_propose, 3, q.w_hi) - q.hotp_lo;
             q.cold_lo = first_at(cold_tiles, 0, (size_t)c.n_cold_tiles, 4, q.w_lo);
@@ -707,14 +709,15 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.long_docs = upload(c, long_docs);
     c.doc_sort_tiles = upload(c, doc_sort_tiles);
     c.doc_sort_long = upload(c, doc_sort_long);
-    c.alias_big = upload(c, alias_big);
+    v.hot_word = upload(c, hot_word);
+    for (int i = 0; i < ALIAS_CLASSES; ++i) ok = (c.alias_words[i] = upload(c, alias_words[i])) && ok;
     c.hot_tiles = upload(c, hot_tiles);
     c.hot_tiles_warm = upload(c, hot_tiles_warm);
     c.warm_words = upload(c, warm_words);
     c.hot_tiles_propose = upload(c, hot_tiles_propose);
     c.cold_tiles = upload(c, cold_tiles);
     ok = ok && v.row_start && v.dense_slot && c.word_tiles && c.doc_tiles && c.hot_runs && c.acc_runs &&
-         c.long_docs && c.doc_sort_tiles && c.doc_sort_long && c.alias_big && c.hot_tiles && c.hot_tiles_warm && c.warm_words && c.hot_tiles_propose && c.cold_tiles;
+         c.long_docs && c.doc_sort_tiles && c.doc_sort_long && v.hot_word && c.hot_tiles && c.hot_tiles_warm && c.warm_words && c.hot_tiles_propose && c.cold_tiles;
     v.wk_nnz = (int32_t*)A((size_t)V * 4);
     v.wk_topic = (uint32_t*)A(cap1 * 4);
     v.wk_count = (uint32_t*)A(cap1 * 4);
@@ -1353,7 +1356,7 @@ int lda_get_tables(lda_ctx* h, uint32_t* sp_thr32, int32_t* sp_alias, int64_t ca
         const Ctx::Slice& q = c.slices[sl];
         if (!one) {
             set_slice(c, (int)sl);
-            launch_alias_sparse(c);
+            launch_alias_sparse(c, true);
             int bits = 0;
             if ((rc = read_err(c, &bits))) return rc;
             if (bits) return fail(&c, LDA_EINTERNAL, "alias construction raised the device error word");

@@ -128,18 +128,20 @@ k_seg_count_sorted(const int32_t* __restrict__ tiles, const int32_t* __restrict_
 }
 
 // Tail words (K <= WORD_ROWS_BITMAP_MAX_K): one CTA per tile of whole words [s0, s1) holding at most
-// SORT_TILE tokens and ROW_TILE_WORDS words.  The tile's topics are read once, into shared memory; the
-// words are then handed to the CTA's warps one at a time, without a barrier between them:
+// SORT_TILE tokens and ROW_TILE_WORDS words.  The tile's topics are read once, into shared memory; words of
+// up to ROW_WARP_TOKENS are then handed to the CTA's warps one at a time, without a barrier between them:
 //   - up to 32 tokens: a lane holds a token, lanes with the same topic find each other, the lowest of
 //     them writes the entry at the rank of its topic among the word's distinct topics;
-//   - up to ROW_WARP_TOKENS: counted in a hash table of the warp's own (load <= 1/2) and marked in its
-//     bitmap over the topics; the bitmap, read in order, gives the sorted row;
-//   - longer words are left for the whole CTA at the end (the same with four slots per token).
-// What bounds it is latency (a word is a chain of a dozen dependent shared-memory steps), so the
-// point of the split is many words in flight per multiprocessor and no CTA-wide steps for short ones.
+//   - longer: counted in a hash table of the warp's own (load <= 1/2); the token that claims a topic's
+//     slot marks the topic in a bitmap, and writes its entry once the bitmap's running popcounts tell the
+//     topic's rank.
+// Words longer than that take the whole CTA, one after the other, in the same way.
+// What bounds it is latency (a word is a chain of a dozen dependent shared-memory steps): hence many words in
+// flight per multiprocessor, little shared memory per CTA, and no CTA-wide steps for short words.
 // NK: the tile's column sums go to n_k too, through bins in shared memory.
-constexpr int ROW_WARP_TOKENS = 256;
-constexpr int ROW_WARP_SLOTS = 512;
+constexpr int ROW_WARP_TOKENS = 128;
+constexpr int ROW_WARP_SLOTS = 2 * ROW_WARP_TOKENS;
+constexpr int ROW_CTA_SLOTS = 2 * SORT_TILE;
 constexpr int ROW_COUNT_BITS = 12;  // of a table entry: a tail word has at most SORT_TILE = 2048 tokens
 static_assert(SORT_TILE < (1 << ROW_COUNT_BITS), "count bits");
 
@@ -155,15 +157,33 @@ struct RowTables {
 // Words of 32 bits of a bitmap over K topics such that each lane of a warp owns an odd number of them (no
 // two lanes on the same shared-memory bank).
 __host__ __device__ constexpr int row_bitmap_lane_words(int K) { return (((K + 31) / 32 + 31) / 32) | 1; }
+// Bytes of a warp's (table, bitmap, running popcounts) times eight, or of the CTA's, whichever is more.
 static size_t row_area_bytes(int K)
 {
-    const size_t warps = 8 * (ROW_WARP_SLOTS * 4 + (size_t)row_bitmap_lane_words(K) * 32 * 4);
-    const size_t cta = (size_t)DK_SLOTS_PER_TOKEN_HOST * SORT_TILE * 4 + 2 * (size_t)((K + 31) / 32) * 4;
+    const size_t bitmap = (size_t)row_bitmap_lane_words(K) * 32;
+    const size_t warps = 8 * (ROW_WARP_SLOTS * 4 + bitmap * 6), cta = ROW_CTA_SLOTS * 4 + bitmap * 6;
     return ((warps > cta ? warps : cta) + 15) / 16 * 16;
 }
 
+// Counts one token of topic k in a table of 2^log2_slots slots (never full: load <= 1/2).  Returns the slot
+// if this token claimed it, else ~0.
+__device__ __forceinline__ uint32_t row_count(uint32_t* table, int log2_slots, uint32_t k)
+{
+    const uint32_t mask = (1u << log2_slots) - 1u, fresh = (k << ROW_COUNT_BITS) | 1u;
+    uint32_t h = (k * DK_HASH_MULT) >> (32 - log2_slots);
+    for (uint32_t tries = 0; tries <= mask; ++tries, h = (h + 1) & mask) {
+        const uint32_t prev = atomicCAS(&table[h], DK_EMPTY, fresh);
+        if (prev == DK_EMPTY) return h;
+        if ((prev >> ROW_COUNT_BITS) == k) {
+            atomicAdd(&table[h], 1u);
+            break;
+        }
+    }
+    return 0xFFFFFFFFu;
+}
+
 template <typename T, bool NK>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 6)
 k_word_rows(const int32_t* __restrict__ tiles, const int32_t* __restrict__ word_off, const T* __restrict__ z,
             RowTables out, int32_t K, int32_t area_words)
 {
@@ -171,8 +191,8 @@ k_word_rows(const int32_t* __restrict__ tiles, const int32_t* __restrict__ word_
     extern __shared__ __align__(16) uint32_t row_area[];  // the warps' tables and bitmaps, then the CTA's; NK: bins behind
     __shared__ int32_t soff[ROW_TILE_WORDS + 1];
     __shared__ T zs[SORT_TILE];
-    __shared__ int32_t long_words[ROW_TILE_WORDS];
-    __shared__ int32_t scan_tmp[33];
+    __shared__ uint16_t long_words[SORT_TILE / ROW_WARP_TOKENS];
+    __shared__ int32_t warp_total[8];
     __shared__ int32_t next_word, n_long;
     int* const err = &out.state->err;
     int32_t* bins = reinterpret_cast<int32_t*>(row_area + area_words);
@@ -198,109 +218,122 @@ k_word_rows(const int32_t* __restrict__ tiles, const int32_t* __restrict__ word_
         if (NK) atomicAdd(&bins[k], (int32_t)n);
     };
     const int32_t lane_words = row_bitmap_lane_words(K);
-    uint32_t* table = row_area + warp * ROW_WARP_SLOTS;
-    uint32_t* bitmap = row_area + 8 * ROW_WARP_SLOTS + warp * 32 * lane_words;
-    for (;;) {
-        int32_t w = 0;
-        if (lane == 0) w = atomicAdd(&next_word, 1);
-        w = __shfl_sync(0xFFFFFFFFu, w, 0);
-        if (w >= nw) break;
-        const int32_t first = soff[w], n = soff[w + 1] - first;
-        const int32_t out0 = __ldg(out.row_start + s0 + w);
-        if (n <= 32) {
-            const uint32_t k = lane < n ? (uint32_t)zs[first + lane] : 0xFFFFFFFFu;
-            const uint32_t same = __match_any_sync(0xFFFFFFFFu, k);
-            const bool lead = lane < n && (uint32_t)(__ffs((int)same) - 1) == (uint32_t)lane;
-            const uint32_t leaders = __ballot_sync(0xFFFFFFFFu, lead);
-            int32_t rank = 0;
-            for (uint32_t m = leaders; m; m &= m - 1u) {
-                const uint32_t other = __shfl_sync(0xFFFFFFFFu, k, __ffs((int)m) - 1);
-                rank += other < k ? 1 : 0;
-            }
-            if (lead) emit(out0 + rank, k, (uint32_t)__popc(same));
-            if (lane == 0) out.nnz[s0 + w] = __popc(leaders);
-        } else if (n <= ROW_WARP_TOKENS) {
-            const int log2_slots = n <= ROW_WARP_TOKENS / 2 ? 8 : 9;
-            const uint32_t slots = 1u << log2_slots;
-            const uint4 empty = make_uint4(DK_EMPTY, DK_EMPTY, DK_EMPTY, DK_EMPTY), zero = make_uint4(0u, 0u, 0u, 0u);
-            for (uint32_t i = lane; i < slots / 4; i += 32) reinterpret_cast<uint4*>(table)[i] = empty;
-            for (int32_t i = lane; i < 8 * lane_words; i += 32) reinterpret_cast<uint4*>(bitmap)[i] = zero;
-            __syncwarp();
-            for (int32_t j = lane; j < n; j += 32) {
-                const uint32_t k = (uint32_t)zs[first + j], fresh = (k << ROW_COUNT_BITS) | 1u;
-                uint32_t h = (k * DK_HASH_MULT) >> (32 - log2_slots);
-                for (uint32_t tries = 0; tries < slots; ++tries, h = (h + 1) & (slots - 1)) {
-                    const uint32_t prev = atomicCAS(&table[h], DK_EMPTY, fresh);
-                    if (prev == DK_EMPTY) {
-                        atomicOr(&bitmap[k >> 5], 1u << (k & 31u));
-                        break;
-                    }
-                    if ((prev >> ROW_COUNT_BITS) == k) {
-                        atomicAdd(&table[h], 1u);
-                        break;
+    const uint4 empty = make_uint4(DK_EMPTY, DK_EMPTY, DK_EMPTY, DK_EMPTY), zero = make_uint4(0u, 0u, 0u, 0u);
+    {
+        uint32_t* table = row_area + warp * ROW_WARP_SLOTS;
+        uint32_t* bitmap = row_area + 8 * ROW_WARP_SLOTS + warp * 32 * lane_words;
+        uint16_t* before = reinterpret_cast<uint16_t*>(row_area + 8 * ROW_WARP_SLOTS + 8 * 32 * lane_words) + warp * 32 * lane_words;
+        for (;;) {
+            int32_t w = 0;
+            if (lane == 0) w = atomicAdd(&next_word, 1);
+            w = __shfl_sync(0xFFFFFFFFu, w, 0);
+            if (w >= nw) break;
+            const int32_t first = soff[w], n = soff[w + 1] - first;
+            const int32_t out0 = __ldg(out.row_start + s0 + w);
+            if (n <= 32) {
+                const uint32_t k = lane < n ? (uint32_t)zs[first + lane] : 0xFFFFFFFFu;
+                const uint32_t same = __match_any_sync(0xFFFFFFFFu, k);
+                const bool lead = lane < n && (uint32_t)(__ffs((int)same) - 1) == (uint32_t)lane;
+                const uint32_t leaders = __ballot_sync(0xFFFFFFFFu, lead);
+                int32_t rank = 0;
+                for (uint32_t m = leaders; m; m &= m - 1u) {
+                    const uint32_t other = __shfl_sync(0xFFFFFFFFu, k, __ffs((int)m) - 1);
+                    rank += other < k ? 1 : 0;
+                }
+                if (lead) emit(out0 + rank, k, (uint32_t)__popc(same));
+                if (lane == 0) out.nnz[s0 + w] = __popc(leaders);
+            } else if (n <= ROW_WARP_TOKENS) {
+                const int log2_slots = n <= 64 ? 7 : 8;
+                static_assert(ROW_WARP_SLOTS == 256, "table sizes above");
+                for (uint32_t i = lane; i < (1u << log2_slots) / 4; i += 32) reinterpret_cast<uint4*>(table)[i] = empty;
+                for (int32_t i = lane; i < 8 * lane_words; i += 32) reinterpret_cast<uint4*>(bitmap)[i] = zero;
+                __syncwarp();
+                uint32_t slot[ROW_WARP_TOKENS / 32], topic[ROW_WARP_TOKENS / 32];
+#pragma unroll
+                for (int r = 0; r < ROW_WARP_TOKENS / 32; ++r) {
+                    const int32_t j = lane + 32 * r;
+                    slot[r] = 0xFFFFFFFFu;
+                    topic[r] = 0;
+                    if (j < n) {
+                        topic[r] = (uint32_t)zs[first + j];
+                        slot[r] = row_count(table, log2_slots, topic[r]);
+                        if (slot[r] != 0xFFFFFFFFu) atomicOr(&bitmap[topic[r] >> 5], 1u << (topic[r] & 31u));
                     }
                 }
-            }
-            __syncwarp();
-            const uint32_t* mine = bitmap + lane * lane_words;
-            int32_t c = 0;
-            for (int32_t i = 0; i < lane_words; ++i) c += __popc(mine[i]);
-            const int32_t incl = warp_scan_incl<int32_t>(c);
-            int32_t at = out0 + incl - c;
-            for (int32_t i = 0; i < lane_words; ++i) {
-                for (uint32_t m = mine[i]; m; m &= m - 1u) {
-                    const uint32_t k = 32u * (uint32_t)(lane * lane_words + i) + (uint32_t)(__ffs((int)m) - 1);
-                    uint32_t h = (k * DK_HASH_MULT) >> (32 - log2_slots);
-                    uint32_t e = table[h];
-                    for (uint32_t tries = 0; tries < slots && (e >> ROW_COUNT_BITS) != k; ++tries) {
-                        h = (h + 1) & (slots - 1);
-                        e = table[h];
-                    }
-                    emit(at++, k, e & ((1u << ROW_COUNT_BITS) - 1u));
+                __syncwarp();
+                int32_t c = 0;
+                for (int32_t i = lane * lane_words; i < (lane + 1) * lane_words; ++i) {
+                    before[i] = (uint16_t)c;
+                    c += __popc(bitmap[i]);
                 }
+                const int32_t incl = warp_scan_incl<int32_t>(c);
+                for (int32_t i = lane * lane_words; i < (lane + 1) * lane_words; ++i) before[i] += (uint16_t)(incl - c);
+                __syncwarp();
+#pragma unroll
+                for (int r = 0; r < ROW_WARP_TOKENS / 32; ++r) {
+                    if (slot[r] == 0xFFFFFFFFu) continue;
+                    const uint32_t k = topic[r], below = (1u << (k & 31u)) - 1u;
+                    emit(out0 + (int32_t)before[k >> 5] + __popc(bitmap[k >> 5] & below), k,
+                         table[slot[r]] & ((1u << ROW_COUNT_BITS) - 1u));
+                }
+                if (lane == 31) out.nnz[s0 + w] = incl;
+                __syncwarp();
+            } else if (lane == 0) {
+                long_words[atomicAdd(&n_long, 1)] = (uint16_t)w;  // at most SORT_TILE / ROW_WARP_TOKENS of them
             }
-            if (lane == 31) out.nnz[s0 + w] = incl;
-            __syncwarp();
-        } else if (lane == 0) {
-            long_words[atomicAdd(&n_long, 1)] = w;
         }
     }
     __syncthreads();
-    const int32_t bw = (K + 31) >> 5;
-    uint32_t* cta_table = row_area;
-    uint32_t* cta_bitmap = row_area + DK_SLOTS_PER_TOKEN * SORT_TILE;  // [bw] topics present in the word
-    uint32_t* before = cta_bitmap + bw;                                // [bw] set bits before each bitmap word
+    uint32_t* table = row_area;
+    uint32_t* bitmap = row_area + ROW_CTA_SLOTS;
+    uint16_t* before = reinterpret_cast<uint16_t*>(bitmap + 32 * lane_words);
+    const int32_t per = (32 * lane_words + 255) / 256;  // bitmap words per thread
     for (int32_t q = 0; q < n_long; ++q) {
         const int32_t w = long_words[q], first = soff[w], n = soff[w + 1] - first;
         const int32_t out0 = __ldg(out.row_start + s0 + w);
-        const uint32_t cap = DK_SLOTS_PER_TOKEN * (uint32_t)n;
-        for (int32_t i = tid; i < bw; i += 256) cta_bitmap[i] = 0;
-        for (uint32_t i = tid; i < cap; i += 256) cta_table[i] = DK_EMPTY;
+        const int log2_slots = 33 - __clz(n - 1);  // at least 2 n slots
+        for (uint32_t i = tid; i < (1u << log2_slots) / 4; i += 256) reinterpret_cast<uint4*>(table)[i] = empty;
+        for (int32_t i = tid; i < 8 * lane_words; i += 256) reinterpret_cast<uint4*>(bitmap)[i] = zero;
         __syncthreads();
-        for (int32_t j = tid; j < n; j += 256) {
-            const uint32_t k = (uint32_t)zs[first + j];
-            atomicOr(&cta_bitmap[k >> 5], 1u << (k & 31u));
-            if (dk_insert(cta_table, cap, k, ROW_COUNT_BITS) == DK_EMPTY) atomicOr(err, ERR_ROW_OVERFLOW);
-        }
-        __syncthreads();
-        int32_t running = 0;
-        for (int32_t i0 = 0; i0 < bw; i0 += 256) {
-            const int32_t i = i0 + tid;
-            const int32_t c = i < bw ? __popc(cta_bitmap[i]) : 0;
-            int32_t total;
-            const int32_t pos = block_scan_excl<int32_t>(c, scan_tmp, total);
-            if (i < bw) before[i] = (uint32_t)(running + pos);
-            running += total;
-        }
-        __syncthreads();
-        for (int32_t i = tid; i < bw; i += 256) {
-            int32_t r = out0 + (int32_t)before[i];
-            for (uint32_t m = cta_bitmap[i]; m; m &= m - 1u, ++r) {
-                const uint32_t k = 32u * (uint32_t)i + (uint32_t)(__ffs((int)m) - 1);
-                emit(r, k, dk_lookup(cta_table, cap, k, ROW_COUNT_BITS) & ((1u << ROW_COUNT_BITS) - 1u));
+        uint32_t slot[SORT_TILE / 256];
+#pragma unroll
+        for (int r = 0; r < SORT_TILE / 256; ++r) {
+            const int32_t j = tid + 256 * r;
+            slot[r] = 0xFFFFFFFFu;
+            if (j < n) {
+                const uint32_t k = (uint32_t)zs[first + j];
+                slot[r] = row_count(table, log2_slots, k);
+                if (slot[r] != 0xFFFFFFFFu) atomicOr(&bitmap[k >> 5], 1u << (k & 31u));
             }
         }
-        if (tid == 0) out.nnz[s0 + w] = running;
+        __syncthreads();
+        const int32_t i0 = min(32 * lane_words, tid * per), i1 = min(32 * lane_words, i0 + per);
+        int32_t c = 0;
+        for (int32_t i = i0; i < i1; ++i) c += __popc(bitmap[i]);
+        const int32_t incl = warp_scan_incl<int32_t>(c);
+        if (lane == 31) warp_total[warp] = incl;
+        __syncthreads();
+        int32_t lower = 0, all = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int32_t t = warp_total[i];
+            if (i < warp) lower += t;
+            all += t;
+        }
+        c = lower + incl - c;
+        for (int32_t i = i0; i < i1; ++i) {
+            before[i] = (uint16_t)c;
+            c += __popc(bitmap[i]);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < SORT_TILE / 256; ++r) {
+            if (slot[r] == 0xFFFFFFFFu) continue;
+            const uint32_t k = (uint32_t)zs[first + tid + 256 * r], below = (1u << (k & 31u)) - 1u;
+            emit(out0 + (int32_t)before[k >> 5] + __popc(bitmap[k >> 5] & below), k,
+                 table[slot[r]] & ((1u << ROW_COUNT_BITS) - 1u));
+        }
+        if (tid == 0) out.nnz[s0 + w] = all;
         __syncthreads();
     }
     if (NK) {

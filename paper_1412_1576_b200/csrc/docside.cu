@@ -44,7 +44,7 @@ __device__ __forceinline__ void load_topic_pair(const int32_t* zbm, uint32_t bm,
 template <typename T, int MODE, int FIXED, int SLOTS, class SlotAt>
 __device__ __forceinline__ void doc_side_token(const View& v, const uint32_t* tab, uint32_t tok, uint32_t doc_len,
                                                uint32_t own, uint32_t t_first, uint32_t bm, const SlotAt& slot_at,
-                                               uint2 key, int32_t mh_steps)
+                                               uint2 key, uint32_t sweep, int32_t mh_steps)
 {
     const uint32_t cap = SLOTS * doc_len;
     const int cb = v.count_bits;
@@ -77,7 +77,7 @@ __device__ __forceinline__ void doc_side_token(const View& v, const uint32_t* ta
     };
     // doc-proposal of step st, the di-th of its kind
     auto doc_step = [&](int32_t st, int32_t di) {
-        const uint4 r = philox4x32_10(make_uint4(v.tok_base + tok, running_sweep(v), (uint32_t)st, 0u), key);
+        const uint4 r = philox4x32_10(make_uint4(v.tok_base + tok, sweep, (uint32_t)st, 0u), key);
         const double uu = __dmul_rn((double)r.x, INV_2_32);
         uint32_t o2;
         if (__dmul_rn(uu, __dadd_rn(n_d, v.Kalpha)) < n_d) {
@@ -178,6 +178,7 @@ k_doc_tile(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_step
     }
     __syncthreads();
     // the tables are complete: every token gathers its share
+    const uint32_t sweep = running_sweep(v);
 #pragma unroll
     for (int r = 0; r < DOC_TILE_ROUNDS; ++r) {
         const int j = tid + r * THREADS;
@@ -185,7 +186,7 @@ k_doc_tile(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_step
             const uint32_t* tab = slots + TILE_SLOTS * first[r];
             const uint32_t* slot_of = slot_s + first[r];
             auto slot_at = [slot_of](uint32_t jj) { return slot_of[jj]; };
-            doc_side_token<T, MODE, FIXED, TILE_SLOTS>(v, tab, (uint32_t)(base + j), (uint32_t)len[r], tab[z[r]], t1[r], bm[r], slot_at, key, mh_steps);
+            doc_side_token<T, MODE, FIXED, TILE_SLOTS>(v, tab, (uint32_t)(base + j), (uint32_t)len[r], tab[z[r]], t1[r], bm[r], slot_at, key, sweep, mh_steps);
         }
     }
 }
@@ -218,11 +219,12 @@ k_long_doc_tile(View v, const int32_t* __restrict__ long_docs, uint2 key, int32_
         slot_of[j] = at;
     }
     __syncthreads();
+    const uint32_t sweep = running_sweep(v);
     auto slot_at = [slot_of](uint32_t j) { return slot_of[j]; };
     for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
         const uint32_t bm = v.bm_of_tok[first + j];
         doc_side_token<T, MODE, FIXED, DK_SLOTS_PER_TOKEN>(v, tab, (uint32_t)(first + j), (uint32_t)cnt, tab[slot_of[j]], (uint32_t)zbm[2 * (size_t)bm + 1], bm,
-                          slot_at, key, mh_steps);
+                          slot_at, key, sweep, mh_steps);
     }
 }
 

@@ -32,19 +32,38 @@ __device__ __forceinline__ uint32_t scale_to_range(uint32_t r, uint32_t n) { ret
 
 __device__ __forceinline__ int bit_length(unsigned long long x) { return 64 - __clzll((long long)x); }
 
-// A quotient part/whole <= 1 as a 32-bit fraction (Section 4.2 tables: split points, mixture thresholds).
-__device__ __forceinline__ uint32_t to_frac32(unsigned long long part, unsigned long long whole)
-{
-    int sh = bit_length(whole) - 32;
-    if (sh < 0) sh = 0;
-    const unsigned long long q = ((part >> sh) << 32) / (whole >> sh);
-    return q > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)q;
-}
+// Quotients part/whole <= 1 as 32-bit fractions (split points and mixture thresholds of Section 4.2),
+// min(2^32 - 1, floor((part >> sh) * 2^32 / (whole >> sh))) with whole >> sh < 2^32, for many parts of one
+// whole: from a double reciprocal of the (shifted) whole, set right with the exact integer remainder.  The
+// estimate is within 2^-20 of the true quotient (two roundings of 2^-53 on a value <= 2^32), so
+// its integer part is off by one at most.  A 64-bit integer division costs several times as much.
+struct Frac32 {
+    int sh;
+    uint32_t w;  // whole >> sh, < 2^32
+    double inv;  // 1 / w
+    __device__ __forceinline__ explicit Frac32(unsigned long long whole)
+    {
+        sh = bit_length(whole) - 32;
+        if (sh < 0) sh = 0;
+        w = (uint32_t)(whole >> sh);
+        inv = __ddiv_rn(1.0, u32_to_double(w));
+    }
+    __device__ __forceinline__ uint32_t operator()(unsigned long long part) const
+    {
+        const uint32_t p = (uint32_t)(part >> sh);  // part <= whole
+        const unsigned long long x = (unsigned long long)p << 32;
+        unsigned long long q = __double2ull_rz(__dmul_rn(__dmul_rn(u32_to_double(p), 4294967296.0), inv));
+        const long long r = (long long)(x - q * (unsigned long long)w);
+        if (r < 0) --q;
+        else if (r >= (long long)w) ++q;
+        return q > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)q;
+    }
+};
 
 // Share of a word's sparse term (mass S) in its proposal, the dense term having mass B.
 __device__ __forceinline__ uint32_t mixture_threshold(unsigned long long S, unsigned long long B)
 {
-    return S == 0 ? 0u : to_frac32(S, S + B);
+    return S == 0 ? 0u : Frac32(S + B)(S);
 }
 
 // --- n_kd tables --------------------------------------------------------------------------------

@@ -79,23 +79,19 @@ constexpr int HOT_TILE_MAX = 32768;  // accept pass: tokens of one hot word per 
 constexpr int HOT_TILE_PROPOSE_MAX = 8192;  // propose pass: nothing is staged, shorter runs balance better
 constexpr int COLD_TILE = 2048;      // MH kernel: tokens of a tile of tail words, at most
 constexpr int COLD_WORDS = 512;      // MH kernel: words per tail tile
+constexpr int COLD_DIRECT = 12288;   // MH kernel: 16-bit counters of a tail tile in shared memory
 constexpr int HOT_STAGE_MAX_K = 16384;  // dense rows up to this many topics are staged in shared memory
 // Beyond that K a dense row (4 K bytes) only pays for frequent words.  Words with more tokens than
 // a tail tile holds but at most WARM_MAX_TF keep a sorted sparse row only ("warm" words): rebuilt by
 // one CTA per word from a 16-bit histogram over the topics, and staged whole in shared memory by
 // the accept pass (a row has at most as many entries as the word has tokens).
 constexpr int WARM_MAX_TF = 12288;
-#ifndef LDA_ALIAS_WARP_MAX
-#define LDA_ALIAS_WARP_MAX 512
-#endif
-constexpr int ALIAS_WARP_MAX = LDA_ALIAS_WARP_MAX;  // rows up to this many items are built by one warp
-constexpr int ALIAS_WARP_SMEM = 8 * ALIAS_WARP_MAX * 12;  // eight warps per CTA, 12 bytes of scratch per item
-constexpr int ALIAS_SCRATCH_PER_ITEM = 20;   // bytes of construction scratch per item
-#ifndef LDA_ALIAS_SMEM_ITEMS_MID
-#define LDA_ALIAS_SMEM_ITEMS_MID 2048
-#endif
-constexpr int ALIAS_SMEM_ITEMS_MID = LDA_ALIAS_SMEM_ITEMS_MID;   // rows a 256-thread CTA builds entirely in shared memory
-constexpr int ALIAS_SMEM_ITEMS_BIG = 4096;   // ... and a 512-thread CTA
+// longest sparse alias row built by a warp (of either kernel), by a CTA of 256 and of 1024 threads; longer: a cluster
+constexpr int ALIAS_WARP_MAX = 256, ALIAS_LONG_WARP_MAX = 512, ALIAS_MID_MAX = 2048, ALIAS_BIG_MAX = 10240;
+constexpr int ALIAS_CLASSES = 4;
+constexpr int ALIAS_CLASS_MAX[ALIAS_CLASSES] = {ALIAS_WARP_MAX, ALIAS_LONG_WARP_MAX, ALIAS_MID_MAX, ALIAS_BIG_MAX};
+constexpr int ALIAS_ROW_CLUSTER = 8;         // CTAs of that cluster
+constexpr int ALIAS_SCRATCH_PER_ITEM = 18;   // bytes of construction scratch per item
 
 // Start times (nanoseconds of the device's global timer) a sweep's kernels leave for lda_stats.
 enum : int {
@@ -150,6 +146,7 @@ struct View {
     // One word per token in document order: scratch (slot indices of long documents during the MH
     // step, staging of assignments on their way in and out, z in document order for export.cu).
     uint32_t* rec;
+    const uint8_t* hot_word;  // [V] 1: the MH step treats the word as hot (more than COLD_TILE tokens)
     const int32_t* word_off;  // [V+1] token range of each word in word-sorted order
     const int32_t* doc_off;   // [D+1]
     // n_kw: every word has a sorted (topic, count) row of fixed capacity; hot words also a dense row
@@ -206,21 +203,23 @@ struct Ctx {
     View v{};
     // host-side work lists (device copies below)
     int32_t n_word_tiles = 0, n_doc_tiles = 0, n_dense = 0, n_hot_runs = 0, n_long_docs = 0,
-            n_alias_big = 0, n_alias_mid = 0, n_hot_tiles = 0, n_hot_tiles_propose = 0, n_cold_tiles = 0;
+            n_hot_tiles = 0, n_hot_tiles_propose = 0, n_cold_tiles = 0;
     int32_t* word_tiles = nullptr;   // [n_word_tiles*2] word ranges sorted per CTA
     int32_t* doc_tiles = nullptr;    // [n_doc_tiles*2]
     int32_t* hot_runs = nullptr;     // [n_hot_runs*4] (word, first token, count, index of a word with several runs or -1)
     int32_t* acc = nullptr;          // [words with several runs][dense_stride], zero between rebuilds
     int32_t* acc_done = nullptr;     // [...] runs of the word that are done, zero between rebuilds
     int32_t* acc_runs = nullptr;     // [...] runs of the word
+    bool cold_direct = false;        // the accept pass keeps the tail tiles' rows as counters
     bool nk_with_rows = false;       // the row kernels add up n_k too
     int32_t* long_docs = nullptr;    // [n_long_docs]
     // sorted n_kd rows (export.cu): tiles of whole documents of at most SORT_TILE tokens, and the longer documents
     int32_t n_doc_sort_tiles = 0, n_doc_sort_long = 0;
     int32_t* doc_sort_tiles = nullptr;
     int32_t* doc_sort_long = nullptr;
-    int32_t* alias_big = nullptr;    // [n_alias_big] words whose row can exceed ALIAS_WARP_MAX; the first
-                                     // n_alias_mid of them cannot exceed ALIAS_SMEM_ITEMS_MID
+    // words whose row can exceed ALIAS_CLASS_MAX[i] (each list is part of the one before it)
+    int32_t n_alias_words[ALIAS_CLASSES] = {};
+    int32_t* alias_words[ALIAS_CLASSES] = {};
     int32_t n_warm = 0, n_hot_tiles_warm = 0;
     int32_t* warm_words = nullptr;      // [n_warm] words with a sorted row and more tokens than a tail tile holds
     int32_t* hot_tiles_warm = nullptr;  // [n_hot_tiles_warm*3] their runs for the accept pass
@@ -235,8 +234,7 @@ struct Ctx {
     struct Slice {
         int32_t w_lo = 0, w_hi = 0;        // words [w_lo, w_hi)
         int64_t row_lo = 0, row_n = 0;     // their row slots [row_lo, row_lo + row_n)
-        int32_t mid_lo = 0, mid_n = 0;     // their part of alias_big[0 .. n_alias_mid)
-        int32_t big_lo = 0, big_n = 0;     // ... of alias_big[n_alias_mid .. n_alias_big), relative to n_alias_mid
+        int32_t alias_lo[ALIAS_CLASSES] = {}, alias_n[ALIAS_CLASSES] = {};  // their part of the lists alias_words
         int32_t hotp_lo = 0, hotp_n = 0;   // ... of hot_tiles_propose
         int32_t cold_lo = 0, cold_n = 0;   // ... of cold_tiles
     };
@@ -370,7 +368,7 @@ void rebuild_counts(Ctx& c);     // n_kw and n_k from the assignments, outside a
 inline void exchange_nk(Ctx& c) { int32_t* t = c.v.nk; c.v.nk = c.v.nk_next; c.v.nk_next = t; }
 int launch_alias_dense(Ctx& c, bool in_sweep);  // in_sweep: as the first kernel of a sweep, see there
 void launch_mix_thresholds(Ctx& c, uint32_t* mix32);  // of the tables last built
-int launch_alias_sparse(Ctx& c);            // the running slice's tables
+int launch_alias_sparse(Ctx& c, bool all);  // the running slice's tables (all: in every form, for lda_get_tables)
 void set_slice(Ctx& c, int slice);          // makes `slice` the running one (moves the table pointers)
 int launch_sample(Ctx& c, int mh_steps);   // all passes of the MH step; needs ensure_exchange()
 int launch_doc_side(Ctx& c, int mh_steps);  // pass 2 of the MH step

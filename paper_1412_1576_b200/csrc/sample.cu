@@ -30,9 +30,6 @@ constexpr double INV_2_32 = 1.0 / 4294967296.0;
 #ifndef LDA_PROPOSE_MIN_CTAS
 #define LDA_PROPOSE_MIN_CTAS 2
 #endif
-#ifndef LDA_PROPOSE_FIXED_MIN_CTAS
-#define LDA_PROPOSE_FIXED_MIN_CTAS 4
-#endif
 #ifndef LDA_PROPOSE_TOKENS
 #define LDA_PROPOSE_TOKENS 3
 #endif
@@ -167,42 +164,23 @@ struct HotTile {
     }
 };
 
-// A tile of tail words: sorted n_kw rows and alias bins in shared memory.
-struct ColdTile {
+// A tile of tail words, pass 1: alias bins in shared memory.
+struct ColdBins {
     struct Ref {
         int32_t rs, nnz;  // the word's row inside the tile's arrays
         uint32_t mix;
     };
-    const int32_t* woff;  // [nw+1] first token of each word, relative to the tile
-    const int32_t* rs;    // [nw+1] first row slot of each word, relative to the tile
+    const uint16_t* word;  // word of each of the tile's tokens
+    const int32_t* rs;     // first row slot of each word, relative to the tile
     const int32_t* nnz;
     const uint32_t* mix;
     const uint32_t* topic;
-    const uint32_t* cnt;
     const uint32_t* thr;
     const uint32_t* idx;
-    int32_t nw;
-    const int32_t* nk_tab;  // n_k in global memory
-    static constexpr bool gave_up = false;
-    __device__ __forceinline__ int32_t nk(uint32_t k) const { return __ldg(nk_tab + k); }
     __device__ __forceinline__ Ref ref(int32_t q) const
     {
-        int32_t lo = 0, hi = nw;  // last word with woff[word] <= q
-        while (hi - lo > 1) {
-            const int32_t mid = (lo + hi) >> 1;
-            if (woff[mid] <= q) lo = mid; else hi = mid;
-        }
-        return Ref{rs[lo], nnz[lo], mix[lo]};
-    }
-    __device__ __forceinline__ bool prepare(const View&) { return true; }
-    __device__ __forceinline__ int32_t count(const Ref& w, uint32_t k) const
-    {
-        int32_t lo = 0, hi = w.nnz;
-        while (lo < hi) {
-            const int32_t mid = (lo + hi) >> 1;
-            if (topic[w.rs + mid] < k) lo = mid + 1; else hi = mid;
-        }
-        return (lo < w.nnz && topic[w.rs + lo] == k) ? (int32_t)cnt[w.rs + lo] : 0;
+        const uint32_t w = word[q];
+        return Ref{rs[w], nnz[w], mix[w]};
     }
     __device__ __forceinline__ Draw draw_issue(const Ref& w, const View& v, const uint4& r) const
     {
@@ -220,11 +198,50 @@ struct ColdTile {
             const uint32_t al = idx[w.rs + d.b];
             const uint32_t item = (al == d.b || d.rz < thr[w.rs + d.b]) ? d.b : al;
             t = topic[w.rs + item];
-            n_tw = (int32_t)cnt[w.rs + item];
         } else {
             t = (d.e.y == d.b || d.rz < d.e.x) ? d.b : d.e.y;
-            n_tw = -1;
         }
+        n_tw = -1;
+    }
+};
+
+// A tile of tail words, pass 3.  The words' n_kw rows lie in shared memory in one of two forms:
+//   - DIRECT, corpora of few topics (every tile's words x K <= COLD_DIRECT): a 16-bit counter per word and topic, so a lookup
+//     is one read (99 M tokens, K = 1000: the pass over the tail words 350 -> 290 us);
+//   - otherwise the sorted rows, searched by bisection.  Hashed rows were measured too: what the lookups
+//     gain (2 probes for 5 to 11 steps) the tables' construction costs again, a row of these words having
+//     about as many entries as three tokens have lookups (738 M tokens, K = 10 000: 1.43 against 1.39 ms).
+static_assert(COLD_TILE < 65536, "a tail word's counts fit 16 bits");
+template <bool DIRECT>
+struct ColdRows {
+    static constexpr bool direct = DIRECT;
+    struct Ref {
+        int32_t base;  // counters: the word's first; sorted: first row slot of the word, relative to the tile
+        int32_t nnz;   // sorted: entries
+    };
+    const uint16_t* word;  // word of each of the tile's tokens
+    const int32_t* rs;     // first row slot of each word, relative to the tile
+    const int32_t* nnz;
+    const uint32_t* row;   // counters, or COLD_TILE topics and COLD_TILE counts
+    int32_t K;
+    const int32_t* nk_tab;  // n_k in global memory
+    static constexpr bool gave_up = false;
+    __device__ __forceinline__ bool prepare(const View&) { return true; }
+    __device__ __forceinline__ int32_t nk(uint32_t k) const { return __ldg(nk_tab + k); }
+    __device__ __forceinline__ Ref ref(int32_t q) const
+    {
+        const int32_t w = word[q];
+        return direct ? Ref{w * K, 0} : Ref{rs[w], nnz[w]};
+    }
+    __device__ __forceinline__ int32_t count(const Ref& w, uint32_t k) const
+    {
+        if (direct) return reinterpret_cast<const uint16_t*>(row)[w.base + (int32_t)k];
+        int32_t lo = 0, hi = w.nnz;
+        while (lo < hi) {
+            const int32_t mid = (lo + hi) >> 1;
+            if (row[w.base + mid] < k) lo = mid + 1; else hi = mid;
+        }
+        return (lo < w.nnz && row[w.base + lo] == k) ? (int32_t)row[COLD_TILE + w.base + lo] : 0;
     }
 };
 
@@ -478,7 +495,7 @@ __device__ __forceinline__ void accept_tokens(const View& v, Tile& tile, const i
 template <typename T, int CH, bool STAGED, bool ACCEPT, int MODE, int FIXED>
 __global__ void __launch_bounds__(ACCEPT ? accept_threads(FIXED) : PROPOSE_THREADS,
                                   ACCEPT      ? LDA_ACCEPT_MIN_CTAS
-                                  : FIXED > 0 ? LDA_PROPOSE_FIXED_MIN_CTAS
+                                  : FIXED > 0 ? (sizeof(T) == 2 ? 4 : 3)  // 32-bit topics: three table reads per draw, more registers
                                               : LDA_PROPOSE_MIN_CTAS)
 k_word_hot(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_steps_arg, int stamp_id)
 {
@@ -564,46 +581,143 @@ k_word_warm(View v, const int32_t* __restrict__ tiles, int32_t mh_steps_arg, int
     accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, accept_threads(FIXED), mh_steps);
 }
 
+// `a` holds ascending nonzero marks in some places and zeros elsewhere: every place becomes the last mark at or
+// before it.  Called by all COLD_THREADS threads after a barrier; ends with one.
+__device__ __forceinline__ void fill_from_marks(uint16_t* a, uint32_t* warp_last)
+{
+    constexpr int PER = COLD_TILE / COLD_THREADS;
+    static_assert(PER == 8, "a thread's places are one 16-byte word");
+    const int tid = threadIdx.x, lane = tid & 31;
+    const uint4 mine = reinterpret_cast<const uint4*>(a)[tid];
+    uint32_t at[PER] = {mine.x & 0xFFFFu, mine.x >> 16, mine.y & 0xFFFFu, mine.y >> 16,
+                        mine.z & 0xFFFFu, mine.z >> 16, mine.w & 0xFFFFu, mine.w >> 16};
+#pragma unroll
+    for (int i = 1; i < PER; ++i) at[i] = max(at[i], at[i - 1]);
+    uint32_t top = at[PER - 1];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, top, o);
+        if (lane >= o) top = max(top, u);
+    }
+    if (lane == 31) warp_last[tid >> 5] = top;
+    uint32_t before = __shfl_up_sync(0xFFFFFFFFu, top, 1);
+    if (lane == 0) before = 0;
+    __syncthreads();
+    for (int i = 0; i < (tid >> 5); ++i) before = max(before, warp_last[i]);
+#pragma unroll
+    for (int i = 0; i < PER; ++i) at[i] = max(at[i], before);
+    reinterpret_cast<uint4*>(a)[tid] =
+        make_uint4(at[0] | at[1] << 16, at[2] | at[3] << 16, at[4] | at[5] << 16, at[6] | at[7] << 16);
+    __syncthreads();
+}
+
 // Tail words: tile = (first word, end word, first token, count): whole words with at most COLD_TILE tokens
 // between them, or a run of one word's tokens (small corpora: see load_common() for where the cuts lie).
-template <typename T, int CH, bool ACCEPT, int MODE, int FIXED>
-__global__ void __launch_bounds__(COLD_THREADS)
-k_word_cold(View v, const int4* __restrict__ tiles, uint2 key, int32_t mh_steps_arg, int stamp_id)
+template <typename T, int CH, int MODE, int FIXED>
+__global__ void __launch_bounds__(COLD_THREADS, 5)
+k_word_cold_propose(View v, const int4* __restrict__ tiles, uint2 key, int32_t mh_steps_arg, int stamp_id)
 {
     stamp(v, stamp_id);
     const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
-    __shared__ int32_t woff_s[COLD_WORDS + 1];  // first token of each word, relative to the tile
-    __shared__ int32_t rs_s[COLD_WORDS + 1];    // first row slot of each word, relative to the tile
+    __shared__ int32_t rs_s[COLD_WORDS];
     __shared__ int32_t nnz_s[COLD_WORDS];
     __shared__ uint32_t mix_s[COLD_WORDS];
-    __shared__ uint32_t topic_s[COLD_TILE], count_s[COLD_TILE], thr_s[COLD_TILE], idx_s[COLD_TILE];
+    __shared__ uint32_t topic_s[COLD_TILE], thr_s[COLD_TILE], idx_s[COLD_TILE];
+    __shared__ __align__(16) uint16_t word_s[COLD_TILE];
+    __shared__ uint32_t warp_last[COLD_THREADS / 32];
+    static_assert(COLD_WORDS <= 65536, "a word's number in the tile fits 16 bits");
     const int tid = threadIdx.x;
     const int4 t4 = __ldg(tiles + blockIdx.x);
     const int32_t w0 = t4.x, w1 = t4.y, p0 = t4.z, cnt = t4.w;
     const int32_t nw = w1 - w0;
     const int32_t e0 = __ldg(v.row_start + w0);
     const int32_t ne = nw == 1 ? __ldg(v.wk_nnz + w0) : __ldg(v.row_start + w1) - e0;
-    for (int j = tid; j <= nw; j += COLD_THREADS) {
-        woff_s[j] = __ldg(v.word_off + w0 + j) - p0;
-        rs_s[j] = __ldg(v.row_start + w0 + j) - e0;
-    }
-    for (int j = tid; j < nw; j += COLD_THREADS) {
-        nnz_s[j] = __ldg(v.wk_nnz + w0 + j);
-        if (!ACCEPT) mix_s[j] = mixture_threshold(__ldg(v.sp_mass + w0 + j), __ldg(v.dense_mass));
-    }
+    reinterpret_cast<uint4*>(word_s)[tid] = make_uint4(0u, 0u, 0u, 0u);
     for (int j = tid; j < ne; j += COLD_THREADS) {
         topic_s[j] = __ldcs(v.wk_topic + e0 + j);
-        if (ACCEPT) {
-            count_s[j] = __ldcs(v.wk_count + e0 + j);
-        } else {
-            thr_s[j] = __ldcs(v.al_thr + e0 + j);
-            idx_s[j] = __ldcs(v.al_idx + e0 + j);
-        }
+        thr_s[j] = __ldcs(v.al_thr + e0 + j);
+        idx_s[j] = __ldcs(v.al_idx + e0 + j);
     }
     __syncthreads();
-    ColdTile tile{woff_s, rs_s, nnz_s, mix_s, topic_s, count_s, thr_s, idx_s, nw, v.nk};
-    if (ACCEPT) accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, COLD_THREADS, mh_steps);
-    else propose_tokens<T, MODE, FIXED>(v, tile, p0, p0 + cnt, COLD_THREADS, key, mh_steps);
+    for (int j = tid; j < nw; j += COLD_THREADS) {
+        rs_s[j] = __ldg(v.row_start + w0 + j) - e0;
+        nnz_s[j] = __ldg(v.wk_nnz + w0 + j);
+        mix_s[j] = mixture_threshold(__ldg(v.sp_mass + w0 + j), __ldg(v.dense_mass));
+        const int32_t first = __ldg(v.word_off + w0 + j), end = __ldg(v.word_off + w0 + j + 1);
+        if (j > 0 && end > first) word_s[first - p0] = (uint16_t)j;  // the word's first token carries its number
+    }
+    __syncthreads();
+    if (nw > 1) fill_from_marks(word_s, warp_last);
+    const ColdBins tile{word_s, rs_s, nnz_s, mix_s, topic_s, thr_s, idx_s};
+    propose_tokens<T, MODE, FIXED>(v, tile, p0, p0 + cnt, COLD_THREADS, key, mh_steps);
+}
+
+template <typename T, int CH, int MODE, int FIXED, bool DIRECT>
+__global__ void __launch_bounds__(COLD_THREADS, FIXED == 2 ? 5 : 4)
+k_word_cold_accept(View v, const int4* __restrict__ tiles, int32_t mh_steps_arg, int stamp_id)
+{
+    stamp(v, stamp_id);
+    const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
+    constexpr int PER = COLD_TILE / COLD_THREADS;
+    __shared__ int32_t rs_s[COLD_WORDS];
+    __shared__ int32_t nnz_s[COLD_WORDS];
+    __shared__ __align__(16) uint32_t row_s[DIRECT ? COLD_DIRECT / 2 : 2 * COLD_TILE];
+    __shared__ __align__(16) uint16_t word_s[COLD_TILE];   // word of each token
+    __shared__ __align__(16) uint16_t owner_s[DIRECT ? COLD_TILE : 8];  // word of each row slot
+    __shared__ uint32_t warp_last[COLD_THREADS / 32];
+    const int tid = threadIdx.x;
+    const int4 t4 = __ldg(tiles + blockIdx.x);
+    const int32_t w0 = t4.x, w1 = t4.y, p0 = t4.z, cnt = t4.w;
+    const int32_t nw = w1 - w0;
+    constexpr bool direct = DIRECT;  // every tile of the corpus (load_common())
+    const int32_t e0 = __ldg(v.row_start + w0);
+    const int32_t ne = nw == 1 ? __ldg(v.wk_nnz + w0) : __ldg(v.row_start + w1) - e0;
+    uint32_t entry[PER];  // counters: row slots tid, tid + COLD_THREADS, ... as topic << 16 | count
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int32_t j = tid + i * COLD_THREADS;
+        entry[i] = 0;
+        if (j >= ne) continue;
+        const uint32_t k = __ldcs(v.wk_topic + e0 + j), n = __ldcs(v.wk_count + e0 + j);
+        if (direct) {
+            entry[i] = k << 16 | n;
+        } else {
+            row_s[j] = k;
+            row_s[COLD_TILE + j] = n;
+        }
+    }
+    reinterpret_cast<uint4*>(word_s)[tid] = make_uint4(0u, 0u, 0u, 0u);
+    if (direct) {
+        reinterpret_cast<uint4*>(owner_s)[tid] = make_uint4(0u, 0u, 0u, 0u);
+        for (int j = tid; j < (nw * v.K + 7) / 8; j += COLD_THREADS) reinterpret_cast<uint4*>(row_s)[j] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    __syncthreads();
+    for (int j = tid; j < nw; j += COLD_THREADS) {
+        const int32_t rs = __ldg(v.row_start + w0 + j) - e0, nnz = __ldg(v.wk_nnz + w0 + j);
+        rs_s[j] = rs;
+        nnz_s[j] = nnz;
+        const int32_t first = __ldg(v.word_off + w0 + j), end = __ldg(v.word_off + w0 + j + 1);
+        if (j > 0 && end > first) word_s[first - p0] = (uint16_t)j;  // the word's first token carries its number
+        if (direct && j > 0 && nnz > 0) owner_s[rs] = (uint16_t)j;   // ... and its first row slot
+    }
+    __syncthreads();
+    if (nw > 1) {
+        fill_from_marks(word_s, warp_last);
+        if (direct) fill_from_marks(owner_s, warp_last);
+    }
+    if (direct) {
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int32_t j = tid + i * COLD_THREADS;
+            if (j >= ne) continue;
+            const int32_t w = owner_s[j];
+            // slots behind a row's entries are never written by the rebuild
+            if (j - rs_s[w] < nnz_s[w]) reinterpret_cast<uint16_t*>(row_s)[w * v.K + (int32_t)(entry[i] >> 16)] = (uint16_t)entry[i];
+        }
+        __syncthreads();
+    }
+    ColdRows<DIRECT> tile{word_s, rs_s, nnz_s, row_s, v.K, v.nk};
+    accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, COLD_THREADS, mh_steps);
 }
 
 // z_i uniform on {0..K-1}: Philox counter (token, 0, 0, 1), word 0.
@@ -689,8 +803,8 @@ static int launch_accept(Ctx& c, uint2 key, int mh_steps)
         ++launches;
     }
     if (c.n_cold_tiles) {
-        k_word_cold<T, CH, true, MODE, FIXED><<<c.n_cold_tiles, COLD_THREADS, 0, on[1]>>>(v, reinterpret_cast<const int4*>(c.cold_tiles), key, mh_steps,
-                                                                                           STAMP_ACCEPT_COLD);
+        const auto kernel = c.cold_direct ? k_word_cold_accept<T, CH, MODE, FIXED, true> : k_word_cold_accept<T, CH, MODE, FIXED, false>;
+        kernel<<<c.n_cold_tiles, COLD_THREADS, 0, on[1]>>>(v, reinterpret_cast<const int4*>(c.cold_tiles), mh_steps, STAMP_ACCEPT_COLD);
         ++launches;
     }
     return launches;
@@ -711,7 +825,7 @@ static int launch_propose(Ctx& c, uint2 key, int mh_steps)
         ++launches;
     }
     if (q.cold_n) {
-        k_word_cold<T, CH, false, MODE, FIXED><<<q.cold_n, COLD_THREADS, 0, on[1]>>>(
+        k_word_cold_propose<T, CH, MODE, FIXED><<<q.cold_n, COLD_THREADS, 0, on[1]>>>(
             v, reinterpret_cast<const int4*>(c.cold_tiles) + q.cold_lo, key, mh_steps, noted ? STAMP_PROPOSE_COLD : -1);
         ++launches;
     }
@@ -731,7 +845,7 @@ static int sample_tc(Ctx& c, int mh_steps)
         for (int sl = 0; sl < n_slices; ++sl) {
             if (n_slices > 1) {
                 set_slice(c, sl);
-                launches += launch_alias_sparse(c);
+                launches += launch_alias_sparse(c, false);
             }
             if (CH == 2 && mh_steps == 2)
                 launches += launch_propose<T, 2, MODE, 2>(c, key, mh_steps);

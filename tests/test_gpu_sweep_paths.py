@@ -56,3 +56,27 @@ def test_replayed_sweeps_follow_changes_of_their_arguments(tiny_corpus):
         o.sweep(iters, steps)
         assert np.array_equal(g.get_assignments(), o.get_assignments()), (iters, steps, mode, seed)
     _same(g, o)
+
+
+@pytest.mark.parametrize("K,V", [(10_500, 3), (2_500, 40), (600, 400), (40, 3_000)])
+def test_rows_of_every_length(K, V):
+    """Alias rows, count rows and runs on both sides of every class border: words from one token to a few
+    thousand (lengths around powers of two among them), rows from one topic to K."""
+    rng = np.random.default_rng(K)
+    edges = [1, 2, 7, 8, 9, 15, 16, 17, 31, 32, 33, 63, 64, 65, 96, 97, 127, 128, 129, 255, 256, 257, 511, 512, 513, 1023, 2047,
+             2048, 2049, 4095, 6000]
+    tf = np.array([edges[i % len(edges)] if V > 3 else [11_500, 10_241, 2_100][i] for i in range(V)])
+    while tf.sum() > 150_000:
+        tf[rng.integers(V)] = 3
+    words = rng.permutation(np.repeat(np.arange(V), tf)).astype(np.int32)
+    cuts = np.sort(rng.integers(0, words.size + 1, words.size // 60))
+    offsets = np.concatenate([[0], cuts, [words.size]]).astype(np.int64)
+    g = binding.LightLDA(V, K, 0.05, 0.01)
+    o = ldaref.Oracle(V, K, 0.05, 0.01)
+    for e in (g, o):
+        e.load_corpus(words, offsets)
+        e.init(3)
+    _same(g, o)
+    g.sweep(3, 2)
+    o.sweep(3, 2)
+    _same(g, o)
