@@ -602,18 +602,33 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
         }
         close(V);
     }
-    // document tiles: the smallest tile shape that leaves at most 5 % of the tokens in documents
-    // too long for a tile (those get a CTA of their own and a table in device memory)
+    // document tiles
     std::vector<int32_t> doc_tiles, long_docs;
     {
-        int shape = DOC_TILE_SHAPES - 1;
-        for (int sft = 0; sft < DOC_TILE_SHAPES; ++sft) {
-            int64_t over = 0;
-            for (int32_t d = 0; d < D; ++d) {
-                const int64_t len = doc_off[d + 1] - doc_off[d];
-                if (len > DOC_TILE_TOKENS[sft]) over += len;
+        // A document that does not fit a tile takes the long documents' kernels; the shape with the least
+        // estimated time is taken, relative costs per token as measured (12 M tokens of 4000-token documents at
+        // K = 777, 99 M of 330 at K = 1000, 200 M of log-normal ones at K = 100 000): a tile of the largest shape leaves few
+        // CTAs per multiprocessor, a table in device memory is the slower the less of it shared memory can stand in for.
+        constexpr double TILE_COST[DOC_TILE_SHAPES] = {1.0, 1.0, 1.02, 1.6};
+        int64_t over[DOC_TILE_SHAPES] = {};
+        double over_cost[DOC_TILE_SHAPES] = {};
+        for (int32_t d = 0; d < D; ++d) {
+            const int64_t len = doc_off[d + 1] - doc_off[d];
+            if (len <= DOC_TILE_TOKENS[0]) continue;
+            const double cost = (K > DK_SLOTS_PER_TOKEN_HOST * len ? 3.7 : K > LONG_STAGE_MAX_K ? 2.5 : 1.0) * (double)len;
+            for (int sft = 0; sft < DOC_TILE_SHAPES && len > DOC_TILE_TOKENS[sft]; ++sft) {
+                over[sft] += len;
+                over_cost[sft] += cost;
             }
-            if (over * 20 <= (int64_t)N) { shape = sft; break; }
+        }
+        int shape = 0;
+        double best = 0;
+        for (int sft = 0; sft < DOC_TILE_SHAPES; ++sft) {
+            const double cost = over_cost[sft] + TILE_COST[sft] * (double)(N - over[sft]);
+            if (sft == 0 || cost < best) {
+                best = cost;
+                shape = sft;
+            }
         }
         c.doc_tile = DOC_TILE_TOKENS[shape];
         c.doc_threads = DOC_TILE_THREADS[shape];
@@ -706,7 +721,6 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.acc_runs = upload(c, acc_runs);
     c.acc = (int32_t*)A(acc_runs.size() * (size_t)v.dense_stride * 4);
     c.acc_done = (int32_t*)A(acc_runs.size() * 4);
-    c.long_docs = upload(c, long_docs);
     c.doc_sort_tiles = upload(c, doc_sort_tiles);
     c.doc_sort_long = upload(c, doc_sort_long);
     v.hot_word = upload(c, hot_word);
@@ -717,7 +731,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.hot_tiles_propose = upload(c, hot_tiles_propose);
     c.cold_tiles = upload(c, cold_tiles);
     ok = ok && v.row_start && v.dense_slot && c.word_tiles && c.doc_tiles && c.hot_runs && c.acc_runs &&
-         c.long_docs && c.doc_sort_tiles && c.doc_sort_long && v.hot_word && c.hot_tiles && c.hot_tiles_warm && c.warm_words && c.hot_tiles_propose && c.cold_tiles;
+         c.doc_sort_tiles && c.doc_sort_long && v.hot_word && c.hot_tiles && c.hot_tiles_warm && c.warm_words && c.hot_tiles_propose && c.cold_tiles;
     v.wk_nnz = (int32_t*)A((size_t)V * 4);
     v.wk_topic = (uint32_t*)A(cap1 * 4);
     v.wk_count = (uint32_t*)A(cap1 * 4);
@@ -733,13 +747,27 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     v.dense_mass = (unsigned long long*)A(8);
     v.nk = (int32_t*)A((size_t)v.dense_stride * 8);  // two, padded like a dense row: copied in 16-byte units
     v.nk_next = v.nk ? v.nk + v.dense_stride : nullptr;
-    // scratch tables of the documents longer than a tile: four slots per token, one document after the other
-    std::vector<long long> long_slot_off(long_docs.size() + 1, 0);
-    for (size_t i = 0; i < long_docs.size(); ++i)
-        long_slot_off[i + 1] = long_slot_off[i] + 4ll * (doc_off[long_docs[i] + 1] - doc_off[long_docs[i]]);
-    v.dk_slots = (uint32_t*)A((size_t)long_slot_off.back() * 4 + 32);
-    v.long_slot_off = upload(c, long_slot_off);
-    ok = ok && v.long_slot_off;
+    // tables of the documents longer than a tile (hashed ones first), and their chunks
+    std::vector<LongDoc> long_list;
+    std::vector<int32_t> long_chunks;
+    long long slots = 0;
+    for (const bool dense : {false, true}) {
+        for (const int32_t d : long_docs) {
+            const int32_t first = (int32_t)doc_off[d], len = (int32_t)(doc_off[d + 1] - doc_off[d]);
+            if ((K <= DK_SLOTS_PER_TOKEN_HOST * (int64_t)len) != dense) continue;
+            for (int32_t o = 0; o < len; o += LONG_CHUNK)
+                long_chunks.insert(long_chunks.end(), {(int32_t)long_list.size(), first + o, std::min(LONG_CHUNK, len - o), 0});
+            long_list.push_back(LongDoc{slots, first, len, dense, 0});
+            slots += dense ? (K + 3) / 4 * 4 : (long long)DK_SLOTS_PER_TOKEN_HOST * len;
+        }
+        if (!dense) c.long_hashed_slots = slots;
+    }
+    c.long_slots = slots;
+    c.n_long_chunks = (int32_t)(long_chunks.size() / 4);
+    v.dk_slots = (uint32_t*)A((size_t)slots * 4 + 32);
+    v.long_docs = upload(c, long_list);
+    c.long_chunks = upload(c, long_chunks);
+    ok = ok && v.long_docs && c.long_chunks;
     c.sc_w0 = (unsigned long long*)A(cap_alias * 8);
     c.sc_de0 = (unsigned long long*)A(cap_alias * 8);
     c.sc_item0 = (uint32_t*)A(cap_alias * 4);

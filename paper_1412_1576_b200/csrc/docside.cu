@@ -37,17 +37,44 @@ __device__ __forceinline__ void load_topic_pair(const int32_t* zbm, uint32_t bm,
     t1 = w.y;
 }
 
+// The n_kd table of a document in a tile: hashed, in shared memory.
+struct TileTable {
+    const uint32_t* tab;      // TILE_SLOTS * doc_len slots
+    const uint32_t* slot_of;  // slot holding the topic of the document's j-th token
+    uint32_t cap;
+    int cb;
+    // (topic << count_bits) | n_kd of topic k, and of the j-th token's topic
+    __device__ __forceinline__ uint32_t of_topic(uint32_t k) const
+    {
+        const uint32_t e = dk_lookup(tab, cap, k, cb);
+        return e ? e : k << cb;
+    }
+    __device__ __forceinline__ uint32_t of_token(uint32_t j) const { return tab[slot_of[j]]; }
+};
+
+// The table of a document longer than a tile, in device memory or staged: a counter per topic (DENSE) or hashed.
+template <bool DENSE>
+struct LongTable {
+    const uint32_t* tab;
+    const uint32_t* topic_of;  // topics of the document's tokens, in document order
+    uint32_t cap;
+    int cb;
+    __device__ __forceinline__ uint32_t of_topic(uint32_t k) const
+    {
+        if (DENSE) return k << cb | tab[k];
+        const uint32_t e = dk_lookup(tab, cap, k, cb);
+        return e ? e : k << cb;
+    }
+    __device__ __forceinline__ uint32_t of_token(uint32_t j) const { return of_topic(topic_of[j]); }
+};
+
 // Everything pass 3 needs from the document side for one token, written at the token's
 // block-major index `bm`.
-//   tab     : the document's table, 4 * doc_len slots
-//   slot_at : slot holding the topic of the document's j-th token
-template <typename T, int MODE, int FIXED, int SLOTS, class SlotAt>
-__device__ __forceinline__ void doc_side_token(const View& v, const uint32_t* tab, uint32_t tok, uint32_t doc_len,
-                                               uint32_t own, uint32_t t_first, uint32_t bm, const SlotAt& slot_at,
+template <typename T, int MODE, int FIXED, class Table>
+__device__ __forceinline__ void doc_side_token(const View& v, const Table& table, uint32_t tok, uint32_t doc_len,
+                                               uint32_t own, uint32_t t_first, uint32_t bm,
                                                uint2 key, uint32_t sweep, int32_t mh_steps)
 {
-    const uint32_t cap = SLOTS * doc_len;
-    const int cb = v.count_bits;
     const T* prop = reinterpret_cast<const T*>(v.prop);
     const size_t N = (size_t)v.N;
     uint32_t* out = v.dside + (size_t)bm * v.side_stride;
@@ -72,8 +99,7 @@ __device__ __forceinline__ void doc_side_token(const View& v, const uint32_t* ta
     // word-proposal of step st, the wi-th of its kind: n_kd at the topic pass 1 drew
     auto word_step = [&](int32_t st, int32_t wi) {
         const uint32_t t1 = wi == 0 ? t_first : (uint32_t)__ldcg(prop + (size_t)wi * N + bm);
-        const uint32_t e1 = dk_lookup(tab, cap, t1, cb);
-        put(1 + st, e1 ? e1 : t1 << cb);
+        put(1 + st, table.of_topic(t1));
     };
     // doc-proposal of step st, the di-th of its kind
     auto doc_step = [&](int32_t st, int32_t di) {
@@ -81,11 +107,9 @@ __device__ __forceinline__ void doc_side_token(const View& v, const uint32_t* ta
         const double uu = __dmul_rn((double)r.x, INV_2_32);
         uint32_t o2;
         if (__dmul_rn(uu, __dadd_rn(n_d, v.Kalpha)) < n_d) {
-            o2 = tab[slot_at(scale_to_range(r.y, doc_len))];
+            o2 = table.of_token(scale_to_range(r.y, doc_len));
         } else {
-            const uint32_t t2 = scale_to_range(r.y, (uint32_t)v.K);
-            const uint32_t e2 = dk_lookup(tab, cap, t2, cb);
-            o2 = e2 ? e2 : t2 << cb;
+            o2 = table.of_topic(scale_to_range(r.y, (uint32_t)v.K));
         }
         put(1 + st, o2);
         put(1 + mh_steps + di, r.w);  // the step's acceptance uniform
@@ -183,49 +207,117 @@ k_doc_tile(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_step
     for (int r = 0; r < DOC_TILE_ROUNDS; ++r) {
         const int j = tid + r * THREADS;
         if (j < cnt) {
-            const uint32_t* tab = slots + TILE_SLOTS * first[r];
-            const uint32_t* slot_of = slot_s + first[r];
-            auto slot_at = [slot_of](uint32_t jj) { return slot_of[jj]; };
-            doc_side_token<T, MODE, FIXED, TILE_SLOTS>(v, tab, (uint32_t)(base + j), (uint32_t)len[r], tab[z[r]], t1[r], bm[r], slot_at, key, sweep, mh_steps);
+            const TileTable table{slots + TILE_SLOTS * first[r], slot_s + first[r], TILE_SLOTS * (uint32_t)len[r], v.count_bits};
+            doc_side_token<T, MODE, FIXED>(v, table, (uint32_t)(base + j), (uint32_t)len[r], table.tab[z[r]], t1[r], bm[r], key,
+                                           sweep, mh_steps);
         }
     }
 }
 
-// Documents longer than a tile: one CTA per document; the table lives in the document's range of
-// the scratch slots in device memory (long_slot_off: four slots per token of the long documents,
-// one after the other) and the slot indices in its range of the record array.
-template <typename T, int MODE, int FIXED>
-__global__ void __launch_bounds__(512)
-k_long_doc_tile(View v, const int32_t* __restrict__ long_docs, uint2 key, int32_t mh_steps_arg)
+// Documents longer than a tile are cut into chunks of LONG_CHUNK tokens, a CTA each, in two kernels: the first
+// adds the chunk's topics to the document's table in device memory (cleared before) and leaves them in document order, the
+// second gathers the tokens' records.  A table is a counter per topic where that takes no more room than
+// hashing, else hashed like a tile's; counters of up to LONG_STAGE_MAX_K topics go through shared memory.
+// (One CTA per document, as the tiles have it, lasts as long as the longest document: 12 M tokens in
+// 3000 documents of log-normal length, K = 777, took 523 us per sweep, the two kernels take 230.)
+template <typename T, bool DENSE>
+__device__ __forceinline__ void long_count(const View& v, uint32_t* tab, uint32_t cap, int32_t first, int32_t cnt, uint32_t* bins,
+                                           bool keep_topics)
 {
-    stamp(v, STAMP_DOC_LONG);
-    const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
-    const int32_t d = long_docs[blockIdx.x];
-    const int32_t first = v.doc_off[d], cnt = v.doc_off[d + 1] - first;
-    const uint32_t cap = DK_SLOTS_PER_TOKEN * (uint32_t)cnt;
     const T* zbm = reinterpret_cast<const T*>(v.zbm);
-    uint32_t* tab = v.dk_slots + v.long_slot_off[blockIdx.x];
-    uint32_t* slot_of = v.rec + first;
-    for (uint32_t j = threadIdx.x; j < cap; j += blockDim.x) tab[j] = DK_EMPTY;
-    __syncthreads();
-    for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
-        const uint32_t k = (uint32_t)zbm[2 * (size_t)v.bm_of_tok[first + j]];
-        uint32_t at = 0xFFFFFFFFu;
-        if (k < (uint32_t)v.K) at = dk_insert(tab, cap, k, v.count_bits);
-        if (at == 0xFFFFFFFFu) {
-            atomicOr(v.err, k < (uint32_t)v.K ? ERR_ROW_OVERFLOW : ERR_TOPIC_RANGE);
-            at = 0;
+    const bool staged = DENSE && v.K <= LONG_STAGE_MAX_K;
+    if (staged) {
+        for (int32_t k = threadIdx.x; k < v.K; k += LONG_THREADS) bins[k] = 0;
+        __syncthreads();
+    }
+    for (int32_t j = threadIdx.x; j < cnt; j += LONG_THREADS) {
+        const uint32_t k = (uint32_t)__ldcg(zbm + 2 * (size_t)__ldcs(v.bm_of_tok + first + j));
+        if (keep_topics) v.rec[first + j] = min(k, (uint32_t)v.K - 1u);
+        if (k >= (uint32_t)v.K) {
+            atomicOr(v.err, ERR_TOPIC_RANGE);
+        } else if (staged) {
+            atomicAdd(&bins[k], 1u);
+        } else if (DENSE) {
+            atomicAdd(&tab[k], 1u);
+        } else if (dk_insert(tab, cap, k, v.count_bits) == 0xFFFFFFFFu) {
+            atomicOr(v.err, ERR_ROW_OVERFLOW);
         }
-        slot_of[j] = at;
     }
-    __syncthreads();
+    if (staged) {
+        __syncthreads();
+        for (int32_t k = threadIdx.x; k < v.K; k += LONG_THREADS) {
+            const uint32_t n = bins[k];
+            if (n) atomicAdd(&tab[k], n);
+        }
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(LONG_THREADS)
+k_long_count(View v, const int4* __restrict__ chunks, bool keep_topics, int stamp_id)
+{
+    stamp(v, stamp_id);
+    extern __shared__ __align__(16) uint32_t long_bins[];
+    const int4 c = __ldg(chunks + blockIdx.x);
+    const LongDoc d = v.long_docs[c.x];
+    uint32_t* tab = v.dk_slots + d.slot;
+    if (d.dense) long_count<T, true>(v, tab, 0u, c.y, c.z, long_bins, keep_topics);
+    else long_count<T, false>(v, tab, DK_SLOTS_PER_TOKEN * (uint32_t)d.len, c.y, c.z, long_bins, keep_topics);
+}
+
+template <typename T, int MODE, int FIXED, bool DENSE>
+__device__ __forceinline__ void long_gather(const View& v, const LongDoc& d, const uint32_t* tab, int32_t first, int32_t cnt,
+                                            uint2 key, int32_t mh_steps)
+{
+    const T* zbm = reinterpret_cast<const T*>(v.zbm);
     const uint32_t sweep = running_sweep(v);
-    auto slot_at = [slot_of](uint32_t j) { return slot_of[j]; };
-    for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
-        const uint32_t bm = v.bm_of_tok[first + j];
-        doc_side_token<T, MODE, FIXED, DK_SLOTS_PER_TOKEN>(v, tab, (uint32_t)(first + j), (uint32_t)cnt, tab[slot_of[j]], (uint32_t)zbm[2 * (size_t)bm + 1], bm,
-                          slot_at, key, sweep, mh_steps);
+    const LongTable<DENSE> table{tab, v.rec + d.first, DK_SLOTS_PER_TOKEN * (uint32_t)d.len, v.count_bits};
+    for (int32_t j = threadIdx.x; j < cnt; j += LONG_THREADS) {
+        const uint32_t bm = __ldcs(v.bm_of_tok + first + j);
+        uint32_t z, t1;
+        load_topic_pair(zbm, bm, z, t1);
+        doc_side_token<T, MODE, FIXED>(v, table, (uint32_t)(first + j), (uint32_t)d.len, table.of_topic(z), t1, bm, key, sweep,
+                                       mh_steps);
     }
+}
+
+template <typename T, int MODE, int FIXED>
+__global__ void __launch_bounds__(LONG_THREADS)
+k_long_gather(View v, const int4* __restrict__ chunks, uint2 key, int32_t mh_steps_arg)
+{
+    const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
+    extern __shared__ __align__(16) uint32_t long_bins[];
+    const int4 c = __ldg(chunks + blockIdx.x);
+    const LongDoc d = v.long_docs[c.x];
+    const uint32_t* tab = v.dk_slots + d.slot;
+    if (!d.dense) {
+        long_gather<T, MODE, FIXED, false>(v, d, tab, c.y, c.z, key, mh_steps);
+        return;
+    }
+    if (v.K <= LONG_STAGE_MAX_K) {
+        for (int32_t k = threadIdx.x; k < v.K; k += LONG_THREADS) long_bins[k] = __ldcg(tab + k);
+        __syncthreads();
+        tab = long_bins;
+    }
+    long_gather<T, MODE, FIXED, true>(v, d, tab, c.y, c.z, key, mh_steps);
+}
+
+static size_t long_smem_bytes(const Ctx& c) { return c.K <= LONG_STAGE_MAX_K ? (size_t)c.K * 4 : 0; }
+
+// Tables of the documents longer than a tile; keep_topics: and their topics in document order in View::rec
+// (which an export in flight may be reading).
+int launch_long_tables(Ctx& c, cudaStream_t stream, bool keep_topics, int stamp_id)
+{
+    if (!c.n_long_chunks) return 0;
+    if (c.long_hashed_slots) cudaMemsetAsync(c.v.dk_slots, 0xFF, (size_t)c.long_hashed_slots * 4, stream);
+    if (c.long_slots > c.long_hashed_slots)
+        cudaMemsetAsync(c.v.dk_slots + c.long_hashed_slots, 0, (size_t)(c.long_slots - c.long_hashed_slots) * 4, stream);
+    const int4* chunks = reinterpret_cast<const int4*>(c.long_chunks);
+    if (c.wide_topics)
+        k_long_count<int32_t><<<c.n_long_chunks, LONG_THREADS, long_smem_bytes(c), stream>>>(c.v, chunks, keep_topics, stamp_id);
+    else
+        k_long_count<uint16_t><<<c.n_long_chunks, LONG_THREADS, long_smem_bytes(c), stream>>>(c.v, chunks, keep_topics, stamp_id);
+    return 1;
 }
 
 size_t doc_tile_smem_bytes(int tile_tokens) { return (size_t)tile_tokens * DOC_TILE_SMEM_PER_TOKEN + 16; }
@@ -259,7 +351,7 @@ template <typename T, int MODE, int FIXED>
 static int doc_side_tm(Ctx& c, int mh_steps)
 {
     const uint2 key = make_uint2((uint32_t)c.seed, (uint32_t)(c.seed >> 32));
-    const PassStreams on(c, (c.n_doc_tiles > 0) + (c.n_long_docs > 0));
+    const PassStreams on(c, (c.n_doc_tiles > 0) + (c.n_long_chunks > 0));
     int launches = 0;
     if (c.n_doc_tiles) {
         const size_t smem = doc_tile_smem_bytes(c.doc_tile);
@@ -271,8 +363,10 @@ static int doc_side_tm(Ctx& c, int mh_steps)
         }
         ++launches;
     }
-    if (c.n_long_docs) {
-        k_long_doc_tile<T, MODE, FIXED><<<c.n_long_docs, 512, 0, on[0]>>>(c.v, c.long_docs, key, mh_steps);
+    if (c.n_long_chunks) {
+        launches += launch_long_tables(c, on[0], true, STAMP_DOC_LONG);
+        k_long_gather<T, MODE, FIXED><<<c.n_long_chunks, LONG_THREADS, long_smem_bytes(c), on[0]>>>(
+            c.v, reinterpret_cast<const int4*>(c.long_chunks), key, mh_steps);
         ++launches;
     }
     return launches;

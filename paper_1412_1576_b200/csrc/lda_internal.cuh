@@ -119,6 +119,16 @@ struct SweepReport {
     unsigned long long stamps[STAMP_RING][STAMPS];
 };
 
+// A document longer than a tile: its tokens [first, first + len) and its table in View::dk_slots, from
+// `slot` on -- K counters (dense) or 4 * len slots, probed as dk_insert in lda_device.cuh has it.
+struct LongDoc {
+    long long slot;
+    int32_t first, len;
+    int32_t dense, pad;
+};
+constexpr int LONG_CHUNK = 2048, LONG_THREADS = 256;
+constexpr int LONG_STAGE_MAX_K = 4096;  // counters of a long document staged in shared memory up to this K
+
 // Everything a kernel needs, passed by value.
 struct View {
     int32_t V, K, N, D;
@@ -169,11 +179,10 @@ struct View {
     unsigned long long* dense_mass;
     int32_t* nk;       // [K] column sums of n_kw: the counts frozen at sweep start
     int32_t* nk_next;  // [K] ... of the rebuild in progress; the host exchanges the two after a rebuild
-    // n_kd of the documents longer than a tile (the others' tables only ever live in shared memory):
-    // the i-th long document owns the open-addressing table dk_slots[long_slot_off[i] .. long_slot_off[i+1])
-    // (four slots per token, load <= 0.25); layout and probe order: dk_insert in lda_device.cuh.
+    // n_kd of the documents longer than a tile (the others' tables only ever live in shared memory), built
+    // by k_long_count: hashed ones first, then the ones with a counter per topic
     uint32_t* dk_slots;
-    const long long* long_slot_off;
+    const LongDoc* long_docs;
     int* err;           // = &state->err
     SweepState* state;  // sweep counter, move counters, stamps
 };
@@ -212,7 +221,9 @@ struct Ctx {
     int32_t* acc_runs = nullptr;     // [...] runs of the word
     bool cold_direct = false;        // the accept pass keeps the tail tiles' rows as counters
     bool nk_with_rows = false;       // the row kernels add up n_k too
-    int32_t* long_docs = nullptr;    // [n_long_docs]
+    int32_t n_long_chunks = 0;
+    int32_t* long_chunks = nullptr;  // [n_long_chunks*4] (index into View::long_docs, first token, count, 0)
+    int64_t long_slots = 0, long_hashed_slots = 0;  // of View::dk_slots: in all, of the hashed tables
     // sorted n_kd rows (export.cu): tiles of whole documents of at most SORT_TILE tokens, and the longer documents
     int32_t n_doc_sort_tiles = 0, n_doc_sort_long = 0;
     int32_t* doc_sort_tiles = nullptr;
@@ -372,6 +383,7 @@ int launch_alias_sparse(Ctx& c, bool all);  // the running slice's tables (all: 
 void set_slice(Ctx& c, int slice);          // makes `slice` the running one (moves the table pointers)
 int launch_sample(Ctx& c, int mh_steps);   // all passes of the MH step; needs ensure_exchange()
 int launch_doc_side(Ctx& c, int mh_steps);  // pass 2 of the MH step
+int launch_long_tables(Ctx& c, cudaStream_t stream, bool keep_topics, int stamp_id);  // n_kd tables of the documents longer than a tile
 size_t doc_tile_smem_bytes(int tile_tokens);  // dynamic shared memory of the document-tile kernels
 int ensure_exchange(Ctx& c, int mh_steps);  // (re)allocates View::prop / View::dside; LDA_* status
 int launch_loglik(Ctx& c, double* out3_host);

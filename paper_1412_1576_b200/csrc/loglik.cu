@@ -163,43 +163,31 @@ __global__ void __launch_bounds__(256) k_ll_sum_tiles(const double* __restrict__
     if (threadIdx.x == 0 && filled) atomicAdd(nnz_out, filled);
 }
 
-// Documents longer than a tile: a CTA takes them in turns, with the table in the document's range
-// of the scratch slots in device memory (the same scratch the MH step uses for these documents).
-template <typename T>
+// Documents longer than a tile, from their tables in device memory (launch_long_tables()): CTAs take them in turns.
 __global__ void __launch_bounds__(512)
-k_ll_doc_long(View v, const int32_t* __restrict__ long_docs, int32_t n_long, double lg_alpha,
-              double* __restrict__ out, unsigned long long* __restrict__ nnz_out)
+k_ll_doc_long(View v, int32_t n_long, double lg_alpha, double* __restrict__ out, unsigned long long* __restrict__ nnz_out)
 {
     __shared__ double tmp[32];
     __shared__ double small[LL_TABLE];
     fill_ll_table(small, v.alpha, lg_alpha);
-    const T* zbm = reinterpret_cast<const T*>(v.zbm);
     const uint32_t cmask = (1u << v.count_bits) - 1u;
     double s = 0.0;
     unsigned long long filled = 0;
     for (int32_t i = blockIdx.x; i < n_long; i += gridDim.x) {
-        const int32_t d = long_docs[i];
-        const int32_t first = v.doc_off[d], cnt = v.doc_off[d + 1] - first;
-        const uint32_t cap = DK_SLOTS_PER_TOKEN * (uint32_t)cnt;
-        uint32_t* tab = v.dk_slots + v.long_slot_off[i];
-        for (uint32_t j = threadIdx.x; j < cap; j += blockDim.x) tab[j] = DK_EMPTY;
-        __syncthreads();
-        for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
-            const uint32_t k = (uint32_t)zbm[2 * (size_t)v.bm_of_tok[first + j]];
-            if (k >= (uint32_t)v.K) atomicOr(v.err, ERR_TOPIC_RANGE);
-            else if (dk_insert(tab, cap, k, v.count_bits) == DK_EMPTY) atomicOr(v.err, ERR_ROW_OVERFLOW);
-        }
-        __syncthreads();
-        for (uint32_t j = threadIdx.x; j < cap; j += blockDim.x) {
-            const uint32_t e = tab[j];
-            if (e != DK_EMPTY) {
-                const uint32_t c = e & cmask;
+        const LongDoc d = v.long_docs[i];
+        const uint32_t* tab = v.dk_slots + d.slot;
+        const uint32_t slots = d.dense ? (uint32_t)v.K : DK_SLOTS_PER_TOKEN * (uint32_t)d.len;
+        const uint32_t none = d.dense ? 0u : DK_EMPTY, mask = d.dense ? 0xFFFFFFFFu : cmask;
+#pragma unroll 4
+        for (uint32_t j = threadIdx.x; j < slots; j += blockDim.x) {
+            const uint32_t e = __ldcg(tab + j);
+            if (e != none) {
+                const uint32_t c = e & mask;
                 s += c < (uint32_t)LL_TABLE ? small[c] : lgamma((double)c + v.alpha) - lg_alpha;
                 ++filled;
             }
         }
-        if (threadIdx.x == 0) s -= lgamma((double)cnt + v.Kalpha);
-        __syncthreads();
+        if (threadIdx.x == 0) s -= lgamma((double)d.len + v.Kalpha);
     }
     s = block_reduce_sum<double>(s, tmp);
     if (threadIdx.x == 0) out[blockIdx.x] = s;
@@ -248,10 +236,8 @@ static int queue_doc_part(Ctx& c, double* part, unsigned long long* nnz_dev)
     }
     if (c.n_long_docs) {
         const int g = long_ll_grid(c);
-        if (c.wide_topics)
-            k_ll_doc_long<int32_t><<<g, 512, 0, c.stream>>>(c.v, c.long_docs, c.n_long_docs, lg_alpha, part + n, nnz_dev);
-        else
-            k_ll_doc_long<uint16_t><<<g, 512, 0, c.stream>>>(c.v, c.long_docs, c.n_long_docs, lg_alpha, part + n, nnz_dev);
+        launch_long_tables(c, c.stream, false, -1);
+        k_ll_doc_long<<<g, 512, 0, c.stream>>>(c.v, c.n_long_docs, lg_alpha, part + n, nnz_dev);
         n += g;
     }
     return n;

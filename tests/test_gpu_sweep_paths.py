@@ -80,3 +80,25 @@ def test_rows_of_every_length(K, V):
     g.sweep(3, 2)
     o.sweep(3, 2)
     _same(g, o)
+
+
+@pytest.mark.parametrize("K", [37, 3_000, 4_096, 4_097, 20_000])
+@pytest.mark.parametrize("mode", [0, 2])
+def test_long_documents_by_chunks(K, mode):
+    """Documents around the tile sizes and the chunk size, long ones with a counter per topic (staged or not) and
+    hashed ones, beside short ones."""
+    lengths = np.array([1, 383, 384, 385, 768, 769, 1537, 2047, 2048, 2049, 4097, 0, 9_001, 30, 30, 0, 3_073, 5_200])
+    rng = np.random.default_rng(K + mode)
+    words = rng.integers(0, 700, lengths.sum()).astype(np.int32)
+    offsets = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
+    g = binding.LightLDA(700, K, 0.05, 0.01)
+    o = ldaref.Oracle(700, K, 0.05, 0.01)
+    for e in (g, o):
+        e.load_corpus(words, offsets)
+        e.init(11)
+        e.set_proposals(mode)
+        e.sweep(4, 2)
+    _same(g, o)
+    for a, b in zip(g.loglik(), o.loglik()):
+        assert a == pytest.approx(b, rel=1e-10)
+    assert g.stats()["nnz_dk"] == g.get_csr(binding.LDA_NDK)[1].size
