@@ -646,7 +646,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
         }
         close(D);
     }
-    // tiles of whole documents for the sorted n_kd rows: <= SORT_TILE tokens and <= SORT_TILE documents each
+    // tiles of whole documents for the sorted n_kd rows: <= SORT_TILE tokens and <= ROW_TILE_WORDS documents each
     std::vector<int32_t> doc_sort_tiles, doc_sort_long;
     {
         int32_t s0 = 0;
@@ -657,7 +657,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
         for (int32_t d = 0; d < D; ++d) {
             const int64_t len = doc_off[d + 1] - doc_off[d];
             if (len > SORT_TILE) { close(d); s0 = d + 1; tok = 0; doc_sort_long.push_back(d); continue; }
-            if (tok + len > SORT_TILE || d - s0 >= SORT_TILE) { close(d); s0 = d; tok = 0; }
+            if (tok + len > SORT_TILE || d - s0 >= ROW_TILE_WORDS) { close(d); s0 = d; tok = 0; }
             tok += len;
         }
         close(D);
@@ -732,7 +732,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.cold_tiles = upload(c, cold_tiles);
     ok = ok && v.row_start && v.dense_slot && c.word_tiles && c.doc_tiles && c.hot_runs && c.acc_runs &&
          c.doc_sort_tiles && c.doc_sort_long && v.hot_word && c.hot_tiles && c.hot_tiles_warm && c.warm_words && c.hot_tiles_propose && c.cold_tiles;
-    v.wk_nnz = (int32_t*)A((size_t)V * 4);
+    v.wk_nnz = (int32_t*)A(((size_t)V + 1) * 4);  // one past the end is read by the row offsets' scan
     v.wk_topic = (uint32_t*)A(cap1 * 4);
     v.wk_count = (uint32_t*)A(cap1 * 4);
     v.dense_rows = (int32_t*)A(std::max<size_t>((size_t)c.n_dense * v.dense_stride, 1) * 4);
@@ -780,7 +780,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.ll_tables_ready = false;
     if (!ok) { free_corpus(c); return fail(&c, LDA_ENOMEM, "device allocation failed"); }
     set_slice(c, 0);
-    cudaMemsetAsync(v.wk_nnz, 0, (size_t)V * 4, c.stream);
+    cudaMemsetAsync(v.wk_nnz, 0, ((size_t)V + 1) * 4, c.stream);
     cudaMemsetAsync(v.sp_mass, 0, (size_t)V * 8, c.stream);
     cudaMemsetAsync(c.acc, 0, acc_runs.size() * (size_t)v.dense_stride * 4, c.stream);
     cudaMemsetAsync(c.acc_done, 0, acc_runs.size() * 4, c.stream);
@@ -1265,40 +1265,31 @@ int lda_get_counts(lda_ctx* h, int which, int64_t* row_offsets, int32_t* topics,
         if (capacity < total) { free_dk_csr(c, r); return fail(&c, LDA_ERANGE, "capacity below the number of nonzeros"); }
         static_assert(sizeof(long long) == sizeof(int64_t), "row offsets are copied as they are");
         bool ok = true;
-        if (row_offsets) ok = ok && cudaMemcpy(row_offsets, r.row_off, ((size_t)c.D + 1) * 8, cudaMemcpyDeviceToHost) == cudaSuccess;
-        if (topics && total) ok = ok && cudaMemcpy(topics, r.topic, (size_t)total * 4, cudaMemcpyDeviceToHost) == cudaSuccess;
-        if (counts && total) ok = ok && cudaMemcpy(counts, r.count, (size_t)total * 4, cudaMemcpyDeviceToHost) == cudaSuccess;
+        if (row_offsets) ok = ok && copy_to_host(c, row_offsets, r.row_off, ((size_t)c.D + 1) * 8) == cudaSuccess;
+        if (topics && total) ok = ok && copy_to_host(c, topics, r.topic, (size_t)total * 4) == cudaSuccess;
+        if (counts && total) ok = ok && copy_to_host(c, counts, r.count, (size_t)total * 4) == cudaSuccess;
         free_dk_csr(c, r);
         if (!ok) return cuda_fail(&c, "copying the n_kd rows");
         return LDA_OK;
     }
     if (which != LDA_NWK) return fail(&c, LDA_EINVAL, "unknown table");
-    const int64_t rows = c.V;
-    std::vector<int32_t> nnz((size_t)rows), start((size_t)rows + 1);
-    if (cudaMemcpy(nnz.data(), v.wk_nnz, (size_t)rows * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
-        return cuda_fail(&c, "copying row sizes");
-    if (cudaMemcpy(start.data(), v.row_start, ((size_t)rows + 1) * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
-        return cuda_fail(&c, "copying row starts");
-    int64_t total = 0;
-    for (int64_t r = 0; r < rows; ++r) total += nnz[(size_t)r];
+    const bool sizes_only = !row_offsets && !topics && !counts;
+    WkCsr r;
+    if ((rc = build_wk_csr(c, r, sizes_only))) return fail(&c, rc, "building the n_kw rows failed");
+    const int64_t total = (int64_t)r.total;
     if (nnz_out) *nnz_out = total;
-    if (!row_offsets && !topics && !counts) return LDA_OK;
-    if (capacity < total) return fail(&c, LDA_ERANGE, "capacity below the number of nonzeros");
-    const size_t cap = (size_t)start[(size_t)rows];
-    std::vector<uint32_t> a(std::max<size_t>(cap, 1)), b(std::max<size_t>(cap, 1));
-    if (cap && (cudaMemcpy(a.data(), v.wk_topic, cap * 4, cudaMemcpyDeviceToHost) != cudaSuccess ||
-                cudaMemcpy(b.data(), v.wk_count, cap * 4, cudaMemcpyDeviceToHost) != cudaSuccess))
-        return cuda_fail(&c, "copying n_kw rows");
-    int64_t o = 0;
-    for (int64_t r = 0; r < rows; ++r) {
-        if (row_offsets) row_offsets[r] = o;
-        const size_t s0 = (size_t)start[(size_t)r];
-        for (int32_t j = 0; j < nnz[(size_t)r]; ++j, ++o) {
-            if (topics) topics[o] = (int32_t)a[s0 + j];
-            if (counts) counts[o] = (int32_t)b[s0 + j];
-        }
+    if (!sizes_only && capacity < total) {
+        cudaStreamSynchronize(c.stream);
+        free_wk_csr(c, r);
+        return fail(&c, LDA_ERANGE, "capacity below the number of nonzeros");
     }
-    if (row_offsets) row_offsets[rows] = o;
+    bool ok = true;
+    if (row_offsets) ok = ok && copy_to_host(c, row_offsets, r.row_off, ((size_t)c.V + 1) * 8) == cudaSuccess;
+    if (topics && total) ok = ok && copy_to_host(c, topics, r.topic, (size_t)total * 4) == cudaSuccess;
+    if (counts && total) ok = ok && copy_to_host(c, counts, r.count, (size_t)total * 4) == cudaSuccess;
+    cudaStreamSynchronize(c.stream);
+    free_wk_csr(c, r);
+    if (!ok) return cuda_fail(&c, "copying the n_kw rows");
     return LDA_OK;
 }
 

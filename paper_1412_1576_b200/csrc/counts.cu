@@ -185,9 +185,9 @@ __device__ __forceinline__ uint32_t row_count(uint32_t* table, int log2_slots, u
 template <typename T, bool NK>
 __global__ void __launch_bounds__(256, 6)
 k_word_rows(const int32_t* __restrict__ tiles, const int32_t* __restrict__ word_off, const T* __restrict__ z,
-            RowTables out, int32_t K, int32_t area_words)
+            RowTables out, int32_t K, int32_t area_words, int stamp_id)
 {
-    stamp(out.state, STAMP_ROWS);
+    stamp(out.state, stamp_id);
     extern __shared__ __align__(16) uint32_t row_area[];  // the warps' tables and bitmaps, then the CTA's; NK: bins behind
     __shared__ int32_t soff[ROW_TILE_WORDS + 1];
     __shared__ T zs[SORT_TILE];
@@ -652,6 +652,17 @@ void launch_doc_rows(Ctx& c, const int32_t* tiles, int32_t n_tiles, const T* z, 
         k_seg_count_sorted<T, EmitRowEntries><<<n_tiles, 256, 0, c.stream>>>(
             tiles, c.v.doc_off, z, c.v.topic_bits, c.K, EmitRowEntries{row_off, topic, count}, c.v.state, -1);
 }
+// The same, single pass, for K <= WORD_ROWS_BITMAP_MAX_K: sizes, and entries from the documents' first tokens on (a row
+// has at most as many entries as the document has tokens).
+template <typename T>
+void launch_doc_rows_spread(Ctx& c, const int32_t* tiles, int32_t n_tiles, const T* z, int32_t* nnz, uint32_t* topic, uint32_t* count)
+{
+    const RowTables out{c.v.doc_off, topic, count, nnz, nullptr, c.v.state};
+    const size_t area = row_area_bytes(c.K);
+    k_word_rows<T, false><<<n_tiles, 256, area, c.stream>>>(tiles, c.v.doc_off, z, out, c.K, (int32_t)(area / 4), -1);
+}
+template void launch_doc_rows_spread<uint16_t>(Ctx&, const int32_t*, int32_t, const uint16_t*, int32_t*, uint32_t*, uint32_t*);
+template void launch_doc_rows_spread<int32_t>(Ctx&, const int32_t*, int32_t, const int32_t*, int32_t*, uint32_t*, uint32_t*);
 template void launch_doc_rows<uint16_t>(Ctx&, const int32_t*, int32_t, const uint16_t*, int32_t*, const long long*, int32_t*, int32_t*);
 template void launch_doc_rows<int32_t>(Ctx&, const int32_t*, int32_t, const int32_t*, int32_t*, const long long*, int32_t*, int32_t*);
 
@@ -677,7 +688,7 @@ static int count_wk_t(Ctx& c)
         if (c.K <= WORD_ROWS_BITMAP_MAX_K) {
             const size_t area = row_area_bytes(c.K);
             k_word_rows<T, NK><<<c.n_word_tiles, 256, area + (NK ? (size_t)c.K * 4 : 0), c.side[0]>>>(
-                c.word_tiles, v.word_off, z, out, c.K, (int32_t)(area / 4));
+                c.word_tiles, v.word_off, z, out, c.K, (int32_t)(area / 4), STAMP_ROWS);
         } else {
             EmitWord e{v.row_start, v.wk_topic, v.wk_count, v.wk_nnz};
             k_seg_count_sorted<T, EmitWord><<<c.n_word_tiles, 256, 0, c.side[0]>>>(
@@ -741,6 +752,8 @@ void set_hist_smem_limits()
     cudaFuncSetAttribute(k_hot_rows<uint16_t, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST32_BINS * 4);
     cudaFuncSetAttribute(k_hot_rows<int32_t, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST32_BINS * 4);
     cudaFuncSetAttribute(k_word_rows<uint16_t, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)row_area_bytes(WORD_ROWS_BITMAP_MAX_K));
+    cudaFuncSetAttribute(k_word_rows<int32_t, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)row_area_bytes(WORD_ROWS_BITMAP_MAX_K));
     cudaFuncSetAttribute(k_word_rows<uint16_t, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)row_area_bytes(NK_WITH_ROWS_MAX_K) + NK_WITH_ROWS_MAX_K * 4);

@@ -5,6 +5,8 @@
 // SORT_TILE tokens, sorted and run-length encoded by k_seg_count_sorted (counts.cu); a longer document
 // gets a CTA of its own and a histogram over the topics.  Two passes: row sizes, a prefix sum for
 // the row offsets (CUB's device scan: this path is off the sweep), then the entries.
+#include <algorithm>
+
 #include <cub/device/device_scan.cuh>
 
 #include "lda_device.cuh"
@@ -66,6 +68,56 @@ void free_dk_csr(Ctx& c, DkCsr& r)
     r = DkCsr{};
 }
 
+// Rows from where they lie (row r at first[r]) to row_off[r], one warp per row.
+__global__ void __launch_bounds__(256)
+k_compact_rows(const int32_t* __restrict__ first, const long long* __restrict__ row_off, int32_t rows, const uint32_t* __restrict__ topic_in,
+               const uint32_t* __restrict__ count_in, int32_t* __restrict__ topic, int32_t* __restrict__ count)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < rows; r += warps) {
+        const long long o = row_off[r];
+        const int32_t n = (int32_t)(row_off[r + 1] - o), f = first[r];
+        for (int32_t j = lane; j < n; j += 32) {
+            topic[o + j] = (int32_t)__ldcs(topic_in + f + j);
+            count[o + j] = (int32_t)__ldcs(count_in + f + j);
+        }
+    }
+}
+
+static void compact_rows(Ctx& c, const int32_t* first, const long long* row_off, int64_t rows, const uint32_t* topic_in,
+                         const uint32_t* count_in, int32_t* topic, int32_t* count)
+{
+    const int grid = (int)std::min<int64_t>((int64_t)c.n_sm * 16, (rows * 32 + 255) / 256);
+    if (grid > 0) k_compact_rows<<<grid, 256, 0, c.stream>>>(first, row_off, (int32_t)rows, topic_in, count_in, topic, count);
+}
+
+// Exclusive prefix sum of nnz[0..n) into row_off[0..n], its total to the host.  nnz[n] must be there (any value).
+static int row_offsets(Ctx& c, const int32_t* nnz, long long* row_off, int64_t n, long long* total)
+{
+    void* temp = nullptr;
+    size_t temp_bytes = 0;
+    // nnz(n_kd), nnz(n_kw) <= n_tokens < 2^31: the 32-bit running sum cannot overflow
+    if (cub::DeviceScan::ExclusiveSum(nullptr, temp_bytes, nnz, row_off, (int)(n + 1), c.stream) != cudaSuccess ||
+        !tmp_alloc(c, &temp, temp_bytes)) {
+        cudaGetLastError();
+        return LDA_ENOMEM;
+    }
+    const cudaError_t e = cub::DeviceScan::ExclusiveSum(temp, temp_bytes, nnz, row_off, (int)(n + 1), c.stream);
+    int rc = LDA_OK;
+    if (e != cudaSuccess || cudaMemcpyAsync(total, row_off + n, 8, cudaMemcpyDeviceToHost, c.stream) != cudaSuccess ||
+        cudaStreamSynchronize(c.stream) != cudaSuccess) {
+        cudaGetLastError();
+        rc = LDA_ECUDA;
+    }
+    raw_free(c, temp);
+    return rc;
+}
+
+template <typename T>
+void launch_doc_rows_spread(Ctx& c, const int32_t* tiles, int32_t n_tiles, const T* z, int32_t* nnz, uint32_t* topic,
+                            uint32_t* count);  // counts.cu
+
 template <typename T>
 static int build_dk_csr_t(Ctx& c, DkCsr& r, bool sizes_only)
 {
@@ -81,44 +133,66 @@ static int build_dk_csr_t(Ctx& c, DkCsr& r, bool sizes_only)
     T* z = reinterpret_cast<T*>(v.rec);
     launch_export_assignments(c, z, sizeof(T) == 2);
     const int win = c.K < HIST_BINS ? c.K : HIST_BINS;
-    if (c.n_doc_sort_tiles)
-        launch_doc_rows<T>(c, c.doc_sort_tiles, c.n_doc_sort_tiles, z, r.nnz, nullptr, nullptr, nullptr);
+    // K small enough for the row kernel of the tail words: sizes and entries in one pass, the entries apart
+    // first; else, or without room for that, the sorting kernel twice
+    uint32_t *topic_at = nullptr, *count_at = nullptr;
+    if (c.K <= WORD_ROWS_BITMAP_MAX_K && c.n_doc_sort_tiles && !sizes_only) {
+        if (!tmp_alloc(c, &topic_at, (size_t)c.N * 4) || !tmp_alloc(c, &count_at, (size_t)c.N * 4)) {
+            raw_free(c, topic_at);
+            topic_at = nullptr;
+        }
+    }
+    if (topic_at) launch_doc_rows_spread<T>(c, c.doc_sort_tiles, c.n_doc_sort_tiles, z, r.nnz, topic_at, count_at);
+    else if (c.n_doc_sort_tiles) launch_doc_rows<T>(c, c.doc_sort_tiles, c.n_doc_sort_tiles, z, r.nnz, nullptr, nullptr, nullptr);
     if (c.n_doc_sort_long)
         k_long_doc_rows<T, false><<<c.n_doc_sort_long, 512, (size_t)win * 4, c.stream>>>(
             c.doc_sort_long, v.doc_off, z, c.K, win, r.nnz, nullptr, nullptr, nullptr, v.err);
-    void* temp = nullptr;
-    size_t temp_bytes = 0;
-    // nnz(n_kd) <= n_tokens < 2^31: the 32-bit running sum cannot overflow
-    if (cub::DeviceScan::ExclusiveSum(nullptr, temp_bytes, r.nnz, r.row_off, D + 1, c.stream) != cudaSuccess ||
-        !tmp_alloc(c, &temp, temp_bytes)) {
-        cudaGetLastError();
-        free_dk_csr(c, r);
-        return LDA_ENOMEM;
+    int rc = row_offsets(c, r.nnz, r.row_off, D, &r.total);
+    const size_t cap = (size_t)(r.total > 0 ? r.total : 1);
+    if (rc == LDA_OK && !sizes_only && (!tmp_alloc(c, &r.topic, cap * 4) || !tmp_alloc(c, &r.count, cap * 4))) rc = LDA_ENOMEM;
+    if (rc == LDA_OK && !sizes_only) {
+        if (topic_at) {
+            // the rows of the documents longer than a tile are written over below
+            compact_rows(c, v.doc_off, r.row_off, D, topic_at, count_at, r.topic, r.count);
+        } else if (c.n_doc_sort_tiles) {
+            launch_doc_rows<T>(c, c.doc_sort_tiles, c.n_doc_sort_tiles, z, nullptr, r.row_off, r.topic, r.count);
+        }
+        if (c.n_doc_sort_long)
+            k_long_doc_rows<T, true><<<c.n_doc_sort_long, 512, (size_t)win * 4, c.stream>>>(
+                c.doc_sort_long, v.doc_off, z, c.K, win, nullptr, r.row_off, r.topic, r.count, v.err);
     }
-    const cudaError_t e = cub::DeviceScan::ExclusiveSum(temp, temp_bytes, r.nnz, r.row_off, D + 1, c.stream);
-    long long total = 0;
-    if (e != cudaSuccess ||
-        cudaMemcpyAsync(&total, r.row_off + D, 8, cudaMemcpyDeviceToHost, c.stream) != cudaSuccess ||
-        cudaStreamSynchronize(c.stream) != cudaSuccess) {
-        cudaGetLastError();
-        raw_free(c, temp);
-        free_dk_csr(c, r);
-        return LDA_ECUDA;
+    if (topic_at) {
+        cudaStreamSynchronize(c.stream);
+        raw_free(c, topic_at);
+        raw_free(c, count_at);
     }
-    raw_free(c, temp);
-    r.total = total;
-    if (sizes_only) return LDA_OK;
-    const size_t cap = (size_t)(total > 0 ? total : 1);
-    if (!tmp_alloc(c, &r.topic, cap * 4) || !tmp_alloc(c, &r.count, cap * 4)) {
-        free_dk_csr(c, r);
-        return LDA_ENOMEM;
+    if (rc != LDA_OK) free_dk_csr(c, r);
+    return rc;
+}
+
+int build_wk_csr(Ctx& c, WkCsr& r, bool sizes_only)
+{
+    const View& v = c.v;
+    const int64_t V = c.V;
+    r = WkCsr{};
+    int rc = tmp_alloc(c, &r.row_off, ((size_t)V + 1) * 8) ? row_offsets(c, v.wk_nnz, r.row_off, V, &r.total) : LDA_ENOMEM;
+    const size_t cap = (size_t)(r.total > 0 ? r.total : 1);
+    if (rc == LDA_OK && !sizes_only) {
+        if (tmp_alloc(c, &r.topic, cap * 4) && tmp_alloc(c, &r.count, cap * 4))
+            compact_rows(c, v.row_start, r.row_off, V, v.wk_topic, v.wk_count, r.topic, r.count);
+        else
+            rc = LDA_ENOMEM;
     }
-    if (c.n_doc_sort_tiles)
-        launch_doc_rows<T>(c, c.doc_sort_tiles, c.n_doc_sort_tiles, z, nullptr, r.row_off, r.topic, r.count);
-    if (c.n_doc_sort_long)
-        k_long_doc_rows<T, true><<<c.n_doc_sort_long, 512, (size_t)win * 4, c.stream>>>(
-            c.doc_sort_long, v.doc_off, z, c.K, win, nullptr, r.row_off, r.topic, r.count, v.err);
-    return LDA_OK;
+    if (rc != LDA_OK) free_wk_csr(c, r);
+    return rc;
+}
+
+void free_wk_csr(Ctx& c, WkCsr& r)
+{
+    raw_free(c, r.row_off);
+    raw_free(c, r.topic);
+    raw_free(c, r.count);
+    r = WkCsr{};
 }
 
 int build_dk_csr(Ctx& c, DkCsr& r, bool sizes_only)

@@ -412,6 +412,21 @@ constexpr long long GIBBS_MAX_PREFIX_BYTES = 24ll << 30;  // V * K running sums 
 int gibbs_sweep(Ctx& c, int32_t iters);
 void set_gibbs_smem_limits();
 
+// Blocking copies that are fast for host memory that is not page-locked, too (staging.cu); after everything
+// queued on the context's stream.
+cudaError_t copy_to_host(Ctx& c, void* host, const void* dev, size_t bytes);
+cudaError_t copy_to_device(Ctx& c, void* dev, const void* host, size_t bytes);
+
+// n_kw as compact rows in device memory: row offsets [V+1] and the entries (export.cu).  LDA_* status.
+struct WkCsr {
+    long long* row_off = nullptr;
+    int32_t* topic = nullptr;
+    int32_t* count = nullptr;
+    long long total = 0;
+};
+int build_wk_csr(Ctx& c, WkCsr& r, bool sizes_only);
+void free_wk_csr(Ctx& c, WkCsr& r);
+
 // load-time layout (sort + offsets); fills c.v token arrays. Returns LDA_* status.
 int build_layout(Ctx& c, const int32_t* word_ids_dev, const int64_t* doc_off_host);
 
