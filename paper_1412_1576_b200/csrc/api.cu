@@ -773,6 +773,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.sc_item0 = (uint32_t*)A(cap_alias * 4);
     c.sc_dense = (unsigned long long*)A((size_t)K * 8 * 3);
     c.red = (double*)A(sizeof(double) * (LL_WORD_PARTIALS + LL_DOC_PARTIALS));
+    c.red_nnz = (uint32_t*)A(4 * LL_DOC_PARTIALS);
     c.red_i = (int64_t*)A(16);
     c.ll_tab = (double*)A(sizeof(double) * 2 * 512);
     c.ll_tile_part = (double*)A(sizeof(double) * std::max<size_t>((size_t)c.n_doc_tiles, 1));
@@ -1221,10 +1222,12 @@ int lda_loglik(lda_ctx* h, double* total, double* word_ll, double* doc_ll)
     int rc = check_device(c);
     if (rc) return rc;
     double out[3];
-    if (launch_loglik(c, out) < 0) return cuda_fail(&c, "log-likelihood");
-    int bits = 0;
-    if ((rc = read_err(c, &bits))) return rc;
-    if (bits) return fail(&c, LDA_EINTERNAL, "the log-likelihood kernels raised the device error word");
+    if (launch_loglik(c, out) < 0 || cudaPeekAtLastError() != cudaSuccess) return cuda_fail(&c, "log-likelihood");
+    if (c.report->err) {
+        int bits = 0;
+        if ((rc = read_err(c, &bits))) return rc;  // clears it
+        return fail(&c, LDA_EINTERNAL, "the log-likelihood kernels raised the device error word");
+    }
     if (total) *total = out[0];
     if (word_ll) *word_ll = out[1];
     if (doc_ll) *doc_ll = out[2];
@@ -1293,6 +1296,7 @@ int lda_get_counts(lda_ctx* h, int which, int64_t* row_offsets, int32_t* topics,
     return LDA_OK;
 }
 
+constexpr size_t EXPORT_ONE_STREAM_BYTES = 256 << 10;
 static int get_assignments(lda_ctx* h, void* z_out, bool narrow, bool wait)
 {
     if (!h) return LDA_EINVAL;
@@ -1308,6 +1312,13 @@ static int get_assignments(lda_ctx* h, void* z_out, bool narrow, bool wait)
     // chunk by chunk: collected into document order on the context's stream, copied out on the copy
     // stream while the next chunk is collected
     const size_t zt = narrow ? 2 : 4;
+    if ((size_t)c.N * zt <= EXPORT_ONE_STREAM_BYTES) {
+        // a copy of a few microseconds is not worth the events that would order a second stream
+        launch_export_chunk(c, zdev, narrow, 0, c.N);
+        if (cudaMemcpyAsync(z_out, zdev, (size_t)c.N * zt, cudaMemcpyDeviceToHost, c.stream) != cudaSuccess)
+            return cuda_fail(&c, "copying assignments");
+        return wait ? wait_all(c) : LDA_OK;
+    }
     for (int64_t first = 0; first < c.N; first += c.copy_chunk) {
         const int64_t count = std::min<int64_t>(c.copy_chunk, c.N - first);
         launch_export_chunk(c, zdev, narrow, first, count);

@@ -117,6 +117,9 @@ struct SweepReport {
     unsigned long long end;  // time after the batch
     int32_t err, pad;
     unsigned long long stamps[STAMP_RING][STAMPS];
+    // of the log-likelihood's last kernel (which writes `err` too)
+    double ll_word, ll_doc;
+    unsigned long long nnz_dk;
 };
 
 // A document longer than a tile: its tokens [first, first + len) and its table in View::dk_slots, from
@@ -268,6 +271,7 @@ struct Ctx {
     uint32_t* ll_tile_nnz = nullptr; // [n_doc_tiles] filled table slots of the tile: its share of nnz(n_kd)
     bool ll_tables_ready = false;
     double* red = nullptr;                   // reduction partials for the log-likelihood
+    uint32_t* red_nnz = nullptr;             // [LL_DOC_PARTIALS] nnz(n_kd) beside the document part's partials
     int64_t* red_i = nullptr;
     // device memory comes from cudaMalloc / cudaFree unless lda_set_allocator() gave other routines
     lda_alloc_fn alloc_fn = nullptr;

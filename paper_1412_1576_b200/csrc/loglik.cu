@@ -2,7 +2,7 @@
 // part and a document part (Dirichlet-multinomial closed form):
 //   word = K lgamma(V beta) + sum_{n_kw>0} [lgamma(n_kw+beta) - lgamma(beta)] - sum_k lgamma(n_k + V beta)
 //   doc  = D lgamma(K alpha) + sum_{n_kd>0} [lgamma(n_kd+alpha) - lgamma(alpha)] - sum_d lgamma(n_d + K alpha)
-// Each CTA writes one partial sum; the host adds the partials in a fixed order.
+// Each CTA writes one partial sum; a last kernel adds the partials in a fixed order.
 #include <algorithm>
 #include <cmath>
 
@@ -22,18 +22,28 @@ __device__ __forceinline__ void fill_ll_table(double* tab, double prior, double 
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(256) k_ll_word(View v, double lg_beta, double* __restrict__ out)
+__global__ void __launch_bounds__(256) k_ll_word(View v, double lg_beta, int32_t per_warp, double* __restrict__ out)
 {
     __shared__ double tmp[32];
     __shared__ double small[LL_TABLE];
     fill_ll_table(small, v.beta, lg_beta);
+    // a warp takes up to 32 consecutive words, its lanes their sizes at once; rows of a few entries (most) would
+    // otherwise cost a chain of reads each
     const int warps = (gridDim.x * blockDim.x) >> 5, lane = threadIdx.x & 31;
     double s = 0.0;
-    for (int32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < v.V; w += warps) {
-        const int32_t r0 = v.row_start[w], n = v.wk_nnz[w];
-        for (int32_t j = lane; j < n; j += 32) {
-            const uint32_t c = v.wk_count[r0 + j];
-            s += c < (uint32_t)LL_TABLE ? small[c] : lgamma((double)c + v.beta) - lg_beta;
+    for (int32_t wb = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per_warp; wb < v.V; wb += warps * per_warp) {
+        int32_t n_mine = 0, r_mine = 0;
+        if (lane < per_warp && wb + lane < v.V) {
+            n_mine = v.wk_nnz[wb + lane];
+            r_mine = v.row_start[wb + lane];
+        }
+        for (uint32_t some = __ballot_sync(0xFFFFFFFFu, n_mine > 0); some; some &= some - 1) {
+            const int src = __ffs((int)some) - 1;
+            const int32_t n = __shfl_sync(0xFFFFFFFFu, n_mine, src), r0 = __shfl_sync(0xFFFFFFFFu, r_mine, src);
+            for (int32_t j = lane; j < n; j += 32) {
+                const uint32_t c = v.wk_count[r0 + j];
+                s += c < (uint32_t)LL_TABLE ? small[c] : lgamma((double)c + v.beta) - lg_beta;
+            }
         }
     }
     for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < v.K; k += gridDim.x * blockDim.x)
@@ -146,7 +156,7 @@ k_ll_doc_tiles(View v, const int32_t* __restrict__ tiles, double lg_alpha, const
 // Adds the tiles' partial sums: CTA b takes the b-th run of `per` consecutive tiles, always in the same order.
 __global__ void __launch_bounds__(256) k_ll_sum_tiles(const double* __restrict__ tile_part,
                                                       const uint32_t* __restrict__ tile_nnz, int32_t n_tiles, int32_t per,
-                                                      double* __restrict__ out, unsigned long long* __restrict__ nnz_out)
+                                                      double* __restrict__ out, uint32_t* __restrict__ nnz_out)
 {
     __shared__ double tmp[32];
     const int32_t t0 = blockIdx.x * per, t1 = min(n_tiles, t0 + per);
@@ -160,12 +170,12 @@ __global__ void __launch_bounds__(256) k_ll_sum_tiles(const double* __restrict__
     if (threadIdx.x == 0) out[blockIdx.x] = s;
     __syncthreads();
     filled = block_reduce_sum<unsigned long long>(filled, reinterpret_cast<unsigned long long*>(tmp));
-    if (threadIdx.x == 0 && filled) atomicAdd(nnz_out, filled);
+    if (threadIdx.x == 0) nnz_out[blockIdx.x] = (uint32_t)filled;  // nnz(n_kd) <= n_tokens < 2^31
 }
 
 // Documents longer than a tile, from their tables in device memory (launch_long_tables()): CTAs take them in turns.
 __global__ void __launch_bounds__(512)
-k_ll_doc_long(View v, int32_t n_long, double lg_alpha, double* __restrict__ out, unsigned long long* __restrict__ nnz_out)
+k_ll_doc_long(View v, int32_t n_long, double lg_alpha, double* __restrict__ out, uint32_t* __restrict__ nnz_out)
 {
     __shared__ double tmp[32];
     __shared__ double small[LL_TABLE];
@@ -193,73 +203,115 @@ k_ll_doc_long(View v, int32_t n_long, double lg_alpha, double* __restrict__ out,
     if (threadIdx.x == 0) out[blockIdx.x] = s;
     __syncthreads();
     filled = block_reduce_sum<unsigned long long>(filled, reinterpret_cast<unsigned long long*>(tmp));
-    if (threadIdx.x == 0 && filled) atomicAdd(nnz_out, filled);
+    if (threadIdx.x == 0) nnz_out[blockIdx.x] = (uint32_t)filled;
+}
+
+// Last kernel: the partial sums of both parts, always in the same order, and the error word, to host memory.
+__global__ void __launch_bounds__(512) k_ll_finish(const double* __restrict__ word, int32_t n_word, const double* __restrict__ doc_a,
+                                                   const uint32_t* __restrict__ nnz_a, int32_t n_a, const double* __restrict__ doc_b,
+                                                   const uint32_t* __restrict__ nnz_b, int32_t n_b, const int* __restrict__ err,
+                                                   SweepReport* __restrict__ rep)
+{
+    __shared__ double tmp[32];
+    __shared__ unsigned long long tmp_n[32];
+    double w = 0.0, d = 0.0;
+    unsigned long long nnz = 0;
+    for (int32_t i = threadIdx.x; i < n_word; i += blockDim.x) w += word[i];
+    for (int32_t i = threadIdx.x; i < n_a; i += blockDim.x) {
+        d += doc_a[i];
+        nnz += nnz_a[i];
+    }
+    for (int32_t i = threadIdx.x; i < n_b; i += blockDim.x) {
+        d += doc_b[i];
+        nnz += nnz_b[i];
+    }
+    w = block_reduce_sum<double>(w, tmp);
+    __syncthreads();
+    d = block_reduce_sum<double>(d, tmp);
+    nnz = block_reduce_sum<unsigned long long>(nnz, tmp_n);
+    if (threadIdx.x == 0) {
+        rep->ll_word = w;
+        rep->ll_doc = d;
+        rep->nnz_dk = nnz;
+        rep->err = *err;
+    }
 }
 
 constexpr int LL_TILE_SUMS = 1024;  // partial sums the tiles' sums are folded into
+constexpr int LL_TILE_DIRECT = 4096;  // up to this many tiles the last kernel adds them up itself
 
 static int long_ll_grid(const Ctx& c) { return std::max(1, std::min<int>(c.n_long_docs, LL_BLOCKS)); }
 
 template <typename T>
-static void launch_ll_tiles_t(Ctx& c, size_t smem, double lg_alpha)
+static void launch_ll_tiles_t(Ctx& c, size_t smem, double lg_alpha, cudaStream_t stream)
 {
     switch (c.doc_threads) {
-        case 128: k_ll_doc_tiles<T, 128><<<c.n_doc_tiles, 128, smem, c.stream>>>(c.v, c.doc_tiles, lg_alpha, c.ll_tab, c.ll_tile_part, c.ll_tile_nnz); break;
-        case 256: k_ll_doc_tiles<T, 256><<<c.n_doc_tiles, 256, smem, c.stream>>>(c.v, c.doc_tiles, lg_alpha, c.ll_tab, c.ll_tile_part, c.ll_tile_nnz); break;
-        case 512: k_ll_doc_tiles<T, 512><<<c.n_doc_tiles, 512, smem, c.stream>>>(c.v, c.doc_tiles, lg_alpha, c.ll_tab, c.ll_tile_part, c.ll_tile_nnz); break;
-        default: k_ll_doc_tiles<T, 1024><<<c.n_doc_tiles, 1024, smem, c.stream>>>(c.v, c.doc_tiles, lg_alpha, c.ll_tab, c.ll_tile_part, c.ll_tile_nnz); break;
+        case 128: k_ll_doc_tiles<T, 128><<<c.n_doc_tiles, 128, smem, stream>>>(c.v, c.doc_tiles, lg_alpha, c.ll_tab, c.ll_tile_part, c.ll_tile_nnz); break;
+        case 256: k_ll_doc_tiles<T, 256><<<c.n_doc_tiles, 256, smem, stream>>>(c.v, c.doc_tiles, lg_alpha, c.ll_tab, c.ll_tile_part, c.ll_tile_nnz); break;
+        case 512: k_ll_doc_tiles<T, 512><<<c.n_doc_tiles, 512, smem, stream>>>(c.v, c.doc_tiles, lg_alpha, c.ll_tab, c.ll_tile_part, c.ll_tile_nnz); break;
+        default: k_ll_doc_tiles<T, 1024><<<c.n_doc_tiles, 1024, smem, stream>>>(c.v, c.doc_tiles, lg_alpha, c.ll_tab, c.ll_tile_part, c.ll_tile_nnz); break;
     }
 }
-static void launch_ll_tiles(Ctx& c, size_t smem, double lg_alpha)
+static void launch_ll_tiles(Ctx& c, size_t smem, double lg_alpha, cudaStream_t stream)
 {
-    if (c.wide_topics) launch_ll_tiles_t<int32_t>(c, smem, lg_alpha);
-    else launch_ll_tiles_t<uint16_t>(c, smem, lg_alpha);
+    if (c.wide_topics) launch_ll_tiles_t<int32_t>(c, smem, lg_alpha, stream);
+    else launch_ll_tiles_t<uint16_t>(c, smem, lg_alpha, stream);
 }
 
-// Queues the document part: partial sums to part[0 .. number returned), nnz(n_kd) to *nnz_dev (cleared here).
-static int queue_doc_part(Ctx& c, double* part, unsigned long long* nnz_dev)
+// Queues the word part (if asked for) and the document part, side by side, and the kernel that reports their sums.
+static void queue_loglik(Ctx& c, bool word_part)
 {
-    cudaMemsetAsync(nnz_dev, 0, 8, c.stream);
+    double* part = c.red;  // [LL_WORD_PARTIALS + LL_DOC_PARTIALS]
+    uint32_t* nnz = c.red_nnz;  // [LL_DOC_PARTIALS]
     const double lg_alpha = std::lgamma(c.alpha);
-    int n = 0;
+    int n_word = 0, n_a = 0, n_b = 0;
+    const double* doc_a = part + LL_BLOCKS;
+    const uint32_t* nnz_a = nnz;
+    double* doc_b = part + LL_BLOCKS + LL_TILE_SUMS;
+    uint32_t* nnz_b = nnz + LL_TILE_SUMS;
+    fork_streams(c);
+    if (word_part) {
+        int per_warp = 32;
+        while (per_warp > 4 && c.V / per_warp < c.n_sm * 16) per_warp /= 2;
+        n_word = (int)std::min<int64_t>(LL_BLOCKS, (c.V + 8 * (int64_t)per_warp - 1) / (8 * (int64_t)per_warp));
+        k_ll_word<<<n_word, 256, 0, c.side[0]>>>(c.v, std::lgamma(c.beta), per_warp, part);
+    }
+    if (c.n_long_docs) {
+        n_b = long_ll_grid(c);
+        launch_long_tables(c, c.side[1], false, -1);
+        k_ll_doc_long<<<n_b, 512, 0, c.side[1]>>>(c.v, c.n_long_docs, lg_alpha, doc_b, nnz_b);
+    }
     if (c.n_doc_tiles) {
         if (!c.ll_tables_ready) {
             k_ll_fill_tables<<<2, 256, 0, c.stream>>>(c.v, lg_alpha, c.ll_tab);
             c.ll_tables_ready = true;
         }
-        const size_t smem = doc_tile_smem_bytes(c.doc_tile);
-        launch_ll_tiles(c, smem, lg_alpha);
-        const int per = (c.n_doc_tiles + LL_TILE_SUMS - 1) / LL_TILE_SUMS;
-        const int g = (c.n_doc_tiles + per - 1) / per;
-        k_ll_sum_tiles<<<g, 256, 0, c.stream>>>(c.ll_tile_part, c.ll_tile_nnz, c.n_doc_tiles, per, part, nnz_dev);
-        n += g;
+        launch_ll_tiles(c, doc_tile_smem_bytes(c.doc_tile), lg_alpha, c.stream);
+        if (c.n_doc_tiles <= LL_TILE_DIRECT) {
+            doc_a = c.ll_tile_part;
+            nnz_a = c.ll_tile_nnz;
+            n_a = c.n_doc_tiles;
+        } else {
+            const int per = (c.n_doc_tiles + LL_TILE_SUMS - 1) / LL_TILE_SUMS;
+            n_a = (c.n_doc_tiles + per - 1) / per;
+            k_ll_sum_tiles<<<n_a, 256, 0, c.stream>>>(c.ll_tile_part, c.ll_tile_nnz, c.n_doc_tiles, per, part + LL_BLOCKS, nnz);
+        }
     }
-    if (c.n_long_docs) {
-        const int g = long_ll_grid(c);
-        launch_long_tables(c, c.stream, false, -1);
-        k_ll_doc_long<<<g, 512, 0, c.stream>>>(c.v, c.n_long_docs, lg_alpha, part + n, nnz_dev);
-        n += g;
-    }
-    return n;
+    join_streams(c);
+    k_ll_finish<<<1, 512, 0, c.stream>>>(part, n_word, doc_a, nnz_a, n_a, doc_b, nnz_b, n_b, c.v.err, c.report);
 }
 
 int launch_loglik(Ctx& c, double* out3_host)
 {
-    double* part = c.red;  // [LL_WORD_PARTIALS + LL_DOC_PARTIALS]
-    k_ll_word<<<LL_BLOCKS, 256, 0, c.stream>>>(c.v, std::lgamma(c.beta), part);
-    const int n_doc = queue_doc_part(c, part + LL_BLOCKS, reinterpret_cast<unsigned long long*>(c.red_i) + 1);
-    std::vector<double> h((size_t)LL_BLOCKS + n_doc);
-    if (cudaMemcpyAsync(h.data(), part, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, c.stream) != cudaSuccess ||
-        cudaStreamSynchronize(c.stream) != cudaSuccess)
-        return -1;
+    queue_loglik(c, true);
+    if (cudaStreamSynchronize(c.stream) != cudaSuccess) return -1;
     // every document with tokens contributes lgamma(K alpha) - lgamma(n_d + K alpha); an empty one nothing
-    double lw = (double)c.K * std::lgamma(c.v.Vbeta), ld = (double)c.n_nonempty_docs * std::lgamma(c.v.Kalpha);
-    for (int i = 0; i < LL_BLOCKS; ++i) lw += h[i];
-    for (int i = 0; i < n_doc; ++i) ld += h[LL_BLOCKS + i];
+    const double lw = (double)c.K * std::lgamma(c.v.Vbeta) + c.report->ll_word;
+    const double ld = (double)c.n_nonempty_docs * std::lgamma(c.v.Kalpha) + c.report->ll_doc;
     out3_host[0] = lw + ld;
     out3_host[1] = lw;
     out3_host[2] = ld;
-    return 2 + (c.n_doc_tiles ? 2 : 0) + (c.n_long_docs ? 1 : 0);
+    return 0;
 }
 
 // nnz(n_kw) and nnz(n_kd) of the current assignments (the latter by the document part's kernels).
@@ -268,12 +320,12 @@ int launch_count_nnz(Ctx& c, int64_t* nnz_wk_host, int64_t* nnz_dk_host)
     unsigned long long* acc = (unsigned long long*)c.red_i;
     cudaMemsetAsync(acc, 0, 8, c.stream);
     k_sum_nnz<<<296, 256, 0, c.stream>>>(c.v.wk_nnz, c.V, acc);
-    queue_doc_part(c, c.red + LL_BLOCKS, acc + 1);
-    unsigned long long h[2] = {0, 0};
-    cudaMemcpyAsync(h, acc, 16, cudaMemcpyDeviceToHost, c.stream);
+    queue_loglik(c, false);
+    unsigned long long h = 0;
+    cudaMemcpyAsync(&h, acc, 8, cudaMemcpyDeviceToHost, c.stream);
     cudaStreamSynchronize(c.stream);
-    *nnz_wk_host = (int64_t)h[0];
-    *nnz_dk_host = (int64_t)h[1];
+    *nnz_wk_host = (int64_t)h;
+    *nnz_dk_host = (int64_t)c.report->nnz_dk;
     return 3;
 }
 
