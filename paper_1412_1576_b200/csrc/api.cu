@@ -4,6 +4,7 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <utility>
 
 #include "lda_internal.cuh"
 
@@ -73,47 +74,88 @@ void dev_free_all(Ctx& c)
     c.device_bytes = 0;
 }
 
-// Host memory the device writes sweep reports to.  Blocks are handed from one context to the next (a
-// new one costs tens of microseconds of driver time); at most REPORTS_KEPT idle ones are kept.
-struct ReportPool {
-    static constexpr size_t REPORTS_KEPT = 4;
+// A context's sweep state (device memory) and the report the device writes for it (host memory), with the streams
+// and events a context needs.  Sets are handed from one context to the next -- a new one costs more driver time
+// than a small corpus takes to load -- and at most KEPT idle ones are kept.
+struct ContextParts {
+    int device = -1;
+    SweepState* state = nullptr;
+    SweepReport* report = nullptr;
+    cudaStream_t side[2] = {}, copy = nullptr;
+    cudaEvent_t ev[5] = {};
+};
+struct PartsPool {
+    static constexpr size_t KEPT = 4;
     std::mutex lock;
-    std::vector<SweepReport*> idle;
-    SweepReport* take()
+    std::vector<ContextParts> idle;
+    static PartsPool& pool()
     {
-        {
-            std::lock_guard<std::mutex> g(lock);
-            if (!idle.empty()) {
-                SweepReport* r = idle.back();
-                idle.pop_back();
-                return r;
-            }
-        }
-        void* p = nullptr;
-        if (cudaHostAlloc(&p, sizeof(SweepReport), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        return static_cast<SweepReport*>(p);
+        static PartsPool* p = new PartsPool;  // never destroyed: contexts may outlive static objects
+        return *p;
     }
-    void give(SweepReport* r)
+    static void release(ContextParts& b)
     {
-        if (!r) return;
+        for (cudaEvent_t e : b.ev)
+            if (e) cudaEventDestroy(e);
+        for (cudaStream_t s : {b.side[0], b.side[1], b.copy})
+            if (s) cudaStreamDestroy(s);
+        if (b.state) cudaFree(b.state);
+        if (b.report) cudaFreeHost(b.report);
+        cudaGetLastError();
+    }
+    bool take(Ctx& c)
+    {
+        ContextParts b;
         {
             std::lock_guard<std::mutex> g(lock);
-            if (idle.size() < REPORTS_KEPT) {
-                idle.push_back(r);
+            for (size_t i = 0; i < idle.size() && b.device < 0; ++i)
+                if (idle[i].device == c.device) {
+                    b = idle[i];
+                    idle.erase(idle.begin() + (long)i);
+                }
+        }
+        if (b.device < 0) {
+            bool ok = cudaMalloc(reinterpret_cast<void**>(&b.state), sizeof(SweepState)) == cudaSuccess &&
+                      cudaHostAlloc(reinterpret_cast<void**>(&b.report), sizeof(SweepReport),
+                                    cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess;
+            for (cudaEvent_t& e : b.ev) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+            for (cudaStream_t* s : {&b.side[0], &b.side[1], &b.copy})
+                ok = ok && cudaStreamCreateWithFlags(s, cudaStreamNonBlocking) == cudaSuccess;
+            if (!ok) {
+                release(b);
+                return false;
+            }
+            b.device = c.device;
+        }
+        c.v.state = b.state;
+        c.v.err = &b.state->err;
+        c.report = b.report;
+        for (int i = 0; i < 2; ++i) {
+            c.side[i] = b.side[i];
+            c.ev_join[i] = b.ev[i];
+        }
+        c.copy = b.copy;
+        c.ev_fork = b.ev[2];
+        c.ev_chunk = b.ev[3];
+        c.ev_export = b.ev[4];
+        return true;
+    }
+    void give(Ctx& c)  // nothing of the context runs any more
+    {
+        if (!c.v.state) return;
+        ContextParts b{c.device, c.v.state, c.report, {c.side[0], c.side[1]}, c.copy,
+                       {c.ev_join[0], c.ev_join[1], c.ev_fork, c.ev_chunk, c.ev_export}};
+        c.v.state = nullptr;
+        {
+            std::lock_guard<std::mutex> g(lock);
+            if (idle.size() < KEPT) {
+                idle.push_back(b);
                 return;
             }
         }
-        cudaFreeHost(r);
+        release(b);
     }
 };
-static ReportPool& report_pool()
-{
-    static ReportPool* pool = new ReportPool;  // never destroyed: contexts may outlive static objects
-    return *pool;
-}
 
 __global__ void k_set_state(SweepState* st, uint32_t sweep)
 {
@@ -211,26 +253,12 @@ static int wait_all(Ctx& c)
     return e == cudaSuccess ? LDA_OK : cuda_fail(&c, "waiting for the context's streams");
 }
 
-template <typename T>
-static T* upload(Ctx& c, const std::vector<T>& h)
-{
-    T* d = (T*)dev_alloc(c, h.size() * sizeof(T));
-    if (d && !h.empty() &&
-        cudaMemcpyAsync(d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice, c.stream) != cudaSuccess)
-        return nullptr;
-    return d;
-}
-
 static void free_corpus(Ctx& c)
 {
     if (c.copy) cudaStreamSynchronize(c.copy);  // an export may still read the staging buffer
     c.export_pending = false;
     drop_graphs(c);
-    // the sweep state is allocated in lda_create and outlives corpora
-    std::vector<void*> drop;
-    for (void* p : c.allocs)
-        if (p != (void*)c.v.state) drop.push_back(p);
-    for (void* p : drop) dev_free(c, p);
+    dev_free_all(c);
     View nv{};
     nv.V = c.V; nv.K = c.K; nv.alpha = c.alpha; nv.beta = c.beta;
     nv.Vbeta = (double)c.V * c.beta;
@@ -427,8 +455,52 @@ static int ensure_tables(Ctx& c)
     return LDA_OK;
 }
 
-static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const int64_t* doc_off,
-                       int64_t n_docs)
+// What one pass over the document offsets tells.
+struct Documents {
+    std::vector<int32_t> off;  // the offsets in 32 bits
+    int64_t longest = 0, nonempty = 0;
+};
+
+static int scan_documents(Ctx* c, int64_t n_tokens, const int64_t* doc_off, int64_t n_docs, Documents& docs)
+{
+    if (n_tokens >= 2147483648ll || n_docs >= 2147483647ll) return fail(c, LDA_ERANGE, "n_tokens and n_docs must be below 2^31");
+    if (doc_off[0] != 0 || doc_off[n_docs] != n_tokens)
+        return fail(c, LDA_ERANGE, "doc_offsets must start at 0 and end at n_tokens");
+    docs.off.resize((size_t)n_docs + 1);
+    int64_t shortest = 0;
+    for (int64_t d = 0; d < n_docs; ++d) {
+        const int64_t len = doc_off[d + 1] - doc_off[d];
+        shortest = std::min(shortest, len);
+        docs.longest = std::max(docs.longest, len);
+        docs.nonempty += len > 0;
+        docs.off[(size_t)d + 1] = (int32_t)doc_off[d + 1];
+    }
+    if (shortest < 0) return fail(c, LDA_ERANGE, "doc_offsets must be non-decreasing");
+    return LDA_OK;
+}
+
+// Work lists on their way to the device: one allocation and one copy for all of them.
+struct ListPack {
+    std::vector<char> host;
+    std::vector<std::pair<size_t, void**>> lists;
+    template <typename E, typename P>
+    void add(const std::vector<E>& list, P** target)
+    {
+        lists.emplace_back(host.size(), const_cast<void**>(reinterpret_cast<const void* const*>(target)));
+        const size_t bytes = list.size() * sizeof(E);
+        host.resize((host.size() + bytes + 15) / 16 * 16);
+        if (bytes) std::memcpy(host.data() + lists.back().first, list.data(), bytes);
+    }
+    bool send(Ctx& c)
+    {
+        char* dev = (char*)dev_alloc(c, host.size());
+        if (!dev || cudaMemcpyAsync(dev, host.data(), host.size(), cudaMemcpyHostToDevice, c.stream) != cudaSuccess) return false;
+        for (const auto& l : lists) *l.second = dev + l.first;
+        return true;
+    }
+};
+
+static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const Documents& docs, int64_t n_docs)
 {
     free_corpus(c);
     c.N = n_tokens;
@@ -438,13 +510,12 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     v.D = (int32_t)n_docs;
     const int32_t V = c.V, K = c.K;
     const int32_t N = v.N, D = v.D;
+    const std::vector<int32_t>& doc_off = docs.off;
 
-    int64_t max_len = 0;
-    for (int64_t d = 0; d < n_docs; ++d) max_len = std::max(max_len, doc_off[d + 1] - doc_off[d]);
     int tb = 1;
     while ((1ll << tb) < (long long)K) ++tb;
     int cb = 1;  // a count never has all bits set, so no entry equals the empty-slot marker
-    while ((1ll << cb) <= max_len + 1) ++cb;
+    while ((1ll << cb) <= docs.longest + 1) ++cb;
     if (tb + cb > 32) {
         free_corpus(c);
         return fail(&c, LDA_ERANGE, "bits(K-1) + bits(longest document) exceeds 32");
@@ -453,17 +524,85 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     v.count_bits = cb;
     v.tok_base = (uint32_t)c.shard_first_token;
 
-    int rc = build_layout(c, words_dev, doc_off);
-    if (rc != LDA_OK) { free_corpus(c); return fail(&c, rc, "building the word-sorted layout failed"); }
-    int bits = 0;
-    rc = read_err(c, &bits);
-    if (rc) { free_corpus(c); return rc; }
-    if (bits & ERR_WORD_RANGE) { free_corpus(c); return fail(&c, LDA_ERANGE, "word id outside [0,V)"); }
-
+    // The sorts are queued; the documents' lists are made meanwhile, the words' lists beside the second sort.
+    LayoutTemps temps;
+    struct Release {
+        Ctx& c;
+        LayoutTemps& t;
+        ~Release()
+        {
+            cudaStreamSynchronize(c.stream);
+            for (void* p : t.held) raw_free(c, p);
+        }
+    } release{c, temps};
+    int rc = build_layout(c, words_dev, doc_off, temps);
+    if (rc != LDA_OK) {
+        cudaStreamSynchronize(c.stream);
+        cudaGetLastError();
+        free_corpus(c);
+        return fail(&c, rc, "building the word-sorted layout failed");
+    }
+    // tiles of whole documents: for the MH step, and for the sorted n_kd rows (<= SORT_TILE tokens and <= ROW_TILE_WORDS
+    // documents each)
+    std::vector<int32_t> doc_tiles, long_docs, doc_sort_tiles, doc_sort_long;
+    {
+        // A document that does not fit a tile takes the long documents' kernels; the shape with the least
+        // estimated time is taken, relative costs per token as measured (12 M tokens of 4000-token documents at
+        // K = 777, 99 M of 330 at K = 1000, 200 M of log-normal ones at K = 100 000): a tile of the largest shape leaves few
+        // CTAs per multiprocessor, a table in device memory is the slower the less of it shared memory can stand in for.
+        constexpr double TILE_COST[DOC_TILE_SHAPES] = {1.0, 1.0, 1.02, 1.6};
+        int64_t over[DOC_TILE_SHAPES] = {};
+        double over_cost[DOC_TILE_SHAPES] = {};
+        for (int32_t d = 0; d < D && docs.longest > DOC_TILE_TOKENS[0]; ++d) {
+            const int32_t len = doc_off[d + 1] - doc_off[d];
+            if (len <= DOC_TILE_TOKENS[0]) continue;
+            const double cost = (K > DK_SLOTS_PER_TOKEN_HOST * (int64_t)len ? 3.7 : K > LONG_STAGE_MAX_K ? 2.5 : 1.0) * (double)len;
+            for (int sft = 0; sft < DOC_TILE_SHAPES && len > DOC_TILE_TOKENS[sft]; ++sft) {
+                over[sft] += len;
+                over_cost[sft] += cost;
+            }
+        }
+        int shape = 0;
+        double best = 0;
+        for (int sft = 0; sft < DOC_TILE_SHAPES; ++sft) {
+            const double cost = over_cost[sft] + TILE_COST[sft] * (double)(N - over[sft]);
+            if (sft == 0 || cost < best) {
+                best = cost;
+                shape = sft;
+            }
+        }
+        c.doc_tile = DOC_TILE_TOKENS[shape];
+        c.doc_threads = DOC_TILE_THREADS[shape];
+        auto pack = [&](int32_t tokens, int32_t documents, std::vector<int32_t>& tiles, std::vector<int32_t>& longer) {
+            int32_t s0 = 0, tok = 0;
+            auto close = [&](int32_t s1) {
+                if (s1 > s0) { tiles.push_back(s0); tiles.push_back(s1); }
+            };
+            for (int32_t d = 0; d < D; ++d) {
+                const int32_t len = doc_off[d + 1] - doc_off[d];
+                if (len > tokens) { close(d); s0 = d + 1; tok = 0; longer.push_back(d); continue; }
+                if (tok + len > tokens || d - s0 >= documents) { close(d); s0 = d; tok = 0; }
+                tok += len;
+            }
+            close(D);
+        };
+        pack(c.doc_tile, c.doc_tile, doc_tiles, long_docs);
+        pack(SORT_TILE, ROW_TILE_WORDS, doc_sort_tiles, doc_sort_long);
+    }
     std::vector<int32_t> word_off((size_t)V + 1);
-    if (cudaMemcpy(word_off.data(), v.word_off, ((size_t)V + 1) * 4, cudaMemcpyDeviceToHost) != cudaSuccess) {
+    int bits = 0;
+    cudaStreamWaitEvent(c.side[0], c.ev_chunk, 0);  // word_off is there
+    if (cudaMemcpyAsync(word_off.data(), v.word_off, ((size_t)V + 1) * 4, cudaMemcpyDeviceToHost, c.side[0]) != cudaSuccess ||
+        cudaMemcpyAsync(&bits, v.err, sizeof(int), cudaMemcpyDeviceToHost, c.side[0]) != cudaSuccess ||
+        cudaStreamSynchronize(c.side[0]) != cudaSuccess) {
+        cudaStreamSynchronize(c.stream);
         free_corpus(c);
         return cuda_fail(&c, "copying word offsets");
+    }
+    if (bits) {
+        read_err(c, &bits);  // waits for the stream and clears the word
+        free_corpus(c);
+        return fail(&c, LDA_ERANGE, "word id outside [0,V)");
     }
 
     // --- dense / sparse class of every word (Section 5) ---------------------------------
@@ -602,66 +741,6 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
         }
         close(V);
     }
-    // document tiles
-    std::vector<int32_t> doc_tiles, long_docs;
-    {
-        // A document that does not fit a tile takes the long documents' kernels; the shape with the least
-        // estimated time is taken, relative costs per token as measured (12 M tokens of 4000-token documents at
-        // K = 777, 99 M of 330 at K = 1000, 200 M of log-normal ones at K = 100 000): a tile of the largest shape leaves few
-        // CTAs per multiprocessor, a table in device memory is the slower the less of it shared memory can stand in for.
-        constexpr double TILE_COST[DOC_TILE_SHAPES] = {1.0, 1.0, 1.02, 1.6};
-        int64_t over[DOC_TILE_SHAPES] = {};
-        double over_cost[DOC_TILE_SHAPES] = {};
-        for (int32_t d = 0; d < D; ++d) {
-            const int64_t len = doc_off[d + 1] - doc_off[d];
-            if (len <= DOC_TILE_TOKENS[0]) continue;
-            const double cost = (K > DK_SLOTS_PER_TOKEN_HOST * len ? 3.7 : K > LONG_STAGE_MAX_K ? 2.5 : 1.0) * (double)len;
-            for (int sft = 0; sft < DOC_TILE_SHAPES && len > DOC_TILE_TOKENS[sft]; ++sft) {
-                over[sft] += len;
-                over_cost[sft] += cost;
-            }
-        }
-        int shape = 0;
-        double best = 0;
-        for (int sft = 0; sft < DOC_TILE_SHAPES; ++sft) {
-            const double cost = over_cost[sft] + TILE_COST[sft] * (double)(N - over[sft]);
-            if (sft == 0 || cost < best) {
-                best = cost;
-                shape = sft;
-            }
-        }
-        c.doc_tile = DOC_TILE_TOKENS[shape];
-        c.doc_threads = DOC_TILE_THREADS[shape];
-        const int32_t tile = c.doc_tile;
-        int32_t s0 = 0;
-        int64_t tok = 0;
-        auto close = [&](int32_t s1) {
-            if (s1 > s0) { doc_tiles.push_back(s0); doc_tiles.push_back(s1); }
-        };
-        for (int32_t d = 0; d < D; ++d) {
-            const int64_t len = doc_off[d + 1] - doc_off[d];
-            if (len > tile) { close(d); s0 = d + 1; tok = 0; long_docs.push_back(d); continue; }
-            if (tok + len > tile || d - s0 >= tile) { close(d); s0 = d; tok = 0; }
-            tok += len;
-        }
-        close(D);
-    }
-    // tiles of whole documents for the sorted n_kd rows: <= SORT_TILE tokens and <= ROW_TILE_WORDS documents each
-    std::vector<int32_t> doc_sort_tiles, doc_sort_long;
-    {
-        int32_t s0 = 0;
-        int64_t tok = 0;
-        auto close = [&](int32_t s1) {
-            if (s1 > s0) { doc_sort_tiles.push_back(s0); doc_sort_tiles.push_back(s1); }
-        };
-        for (int32_t d = 0; d < D; ++d) {
-            const int64_t len = doc_off[d + 1] - doc_off[d];
-            if (len > SORT_TILE) { close(d); s0 = d + 1; tok = 0; doc_sort_long.push_back(d); continue; }
-            if (tok + len > SORT_TILE || d - s0 >= ROW_TILE_WORDS) { close(d); s0 = d; tok = 0; }
-            tok += len;
-        }
-        close(D);
-    }
     c.n_doc_sort_tiles = (int32_t)(doc_sort_tiles.size() / 2);
     c.n_doc_sort_long = (int32_t)doc_sort_long.size();
     c.n_word_tiles = (int32_t)(word_tiles.size() / 2);
@@ -713,25 +792,24 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     v.zw = A(n1 * zt);
     v.zbm = A(2 * n1 * zt);  // (topic, first word-proposal) pairs
     v.rec = (uint32_t*)A(n1 * 4 + 16);  // + one aligned group of four words past the last record
-    v.row_start = upload(c, row_start);
-    v.dense_slot = upload(c, dense_slot);
-    c.word_tiles = upload(c, word_tiles);
-    c.doc_tiles = upload(c, doc_tiles);
-    c.hot_runs = upload(c, hot_runs);
-    c.acc_runs = upload(c, acc_runs);
+    ListPack lists;
+    lists.add(row_start, &v.row_start);
+    lists.add(dense_slot, &v.dense_slot);
+    lists.add(hot_word, &v.hot_word);
+    lists.add(word_tiles, &c.word_tiles);
+    lists.add(doc_tiles, &c.doc_tiles);
+    lists.add(hot_runs, &c.hot_runs);
+    lists.add(acc_runs, &c.acc_runs);
+    lists.add(doc_sort_tiles, &c.doc_sort_tiles);
+    lists.add(doc_sort_long, &c.doc_sort_long);
+    for (int i = 0; i < ALIAS_CLASSES; ++i) lists.add(alias_words[i], &c.alias_words[i]);
+    lists.add(hot_tiles, &c.hot_tiles);
+    lists.add(hot_tiles_warm, &c.hot_tiles_warm);
+    lists.add(warm_words, &c.warm_words);
+    lists.add(hot_tiles_propose, &c.hot_tiles_propose);
+    lists.add(cold_tiles, &c.cold_tiles);
     c.acc = (int32_t*)A(acc_runs.size() * (size_t)v.dense_stride * 4);
     c.acc_done = (int32_t*)A(acc_runs.size() * 4);
-    c.doc_sort_tiles = upload(c, doc_sort_tiles);
-    c.doc_sort_long = upload(c, doc_sort_long);
-    v.hot_word = upload(c, hot_word);
-    for (int i = 0; i < ALIAS_CLASSES; ++i) ok = (c.alias_words[i] = upload(c, alias_words[i])) && ok;
-    c.hot_tiles = upload(c, hot_tiles);
-    c.hot_tiles_warm = upload(c, hot_tiles_warm);
-    c.warm_words = upload(c, warm_words);
-    c.hot_tiles_propose = upload(c, hot_tiles_propose);
-    c.cold_tiles = upload(c, cold_tiles);
-    ok = ok && v.row_start && v.dense_slot && c.word_tiles && c.doc_tiles && c.hot_runs && c.acc_runs &&
-         c.doc_sort_tiles && c.doc_sort_long && v.hot_word && c.hot_tiles && c.hot_tiles_warm && c.warm_words && c.hot_tiles_propose && c.cold_tiles;
     v.wk_nnz = (int32_t*)A(((size_t)V + 1) * 4);  // one past the end is read by the row offsets' scan
     v.wk_topic = (uint32_t*)A(cap1 * 4);
     v.wk_count = (uint32_t*)A(cap1 * 4);
@@ -753,7 +831,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     long long slots = 0;
     for (const bool dense : {false, true}) {
         for (const int32_t d : long_docs) {
-            const int32_t first = (int32_t)doc_off[d], len = (int32_t)(doc_off[d + 1] - doc_off[d]);
+            const int32_t first = doc_off[d], len = doc_off[d + 1] - doc_off[d];
             if ((K <= DK_SLOTS_PER_TOKEN_HOST * (int64_t)len) != dense) continue;
             for (int32_t o = 0; o < len; o += LONG_CHUNK)
                 long_chunks.insert(long_chunks.end(), {(int32_t)long_list.size(), first + o, std::min(LONG_CHUNK, len - o), 0});
@@ -765,9 +843,9 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.long_slots = slots;
     c.n_long_chunks = (int32_t)(long_chunks.size() / 4);
     v.dk_slots = (uint32_t*)A((size_t)slots * 4 + 32);
-    v.long_docs = upload(c, long_list);
-    c.long_chunks = upload(c, long_chunks);
-    ok = ok && v.long_docs && c.long_chunks;
+    lists.add(long_list, &v.long_docs);
+    lists.add(long_chunks, &c.long_chunks);
+    ok = lists.send(c) && ok;
     c.sc_w0 = (unsigned long long*)A(cap_alias * 8);
     c.sc_de0 = (unsigned long long*)A(cap_alias * 8);
     c.sc_item0 = (uint32_t*)A(cap_alias * 4);
@@ -792,19 +870,8 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.stats.n_tokens = N;
     c.stats.n_docs = D;
     c.stats.n_dense_words = c.n_dense;
-    c.n_nonempty_docs = 0;
-    for (int64_t d = 0; d < n_docs; ++d) c.n_nonempty_docs += doc_off[d + 1] > doc_off[d];
+    c.n_nonempty_docs = docs.nonempty;
     c.loaded = true;
-    return LDA_OK;
-}
-
-static int validate_offsets(Ctx* c, int64_t n_tokens, const int64_t* doc_off, int64_t n_docs)
-{
-    if (n_tokens >= 2147483648ll || n_docs >= 2147483647ll) return fail(c, LDA_ERANGE, "n_tokens and n_docs must be below 2^31");
-    if (doc_off[0] != 0 || doc_off[n_docs] != n_tokens)
-        return fail(c, LDA_ERANGE, "doc_offsets must start at 0 and end at n_tokens");
-    for (int64_t d = 0; d < n_docs; ++d)
-        if (doc_off[d + 1] < doc_off[d]) return fail(c, LDA_ERANGE, "doc_offsets must be non-decreasing");
     return LDA_OK;
 }
 
@@ -840,37 +907,24 @@ int lda_create(int32_t V, int32_t K, double alpha, double beta, lda_ctx** out)
     c.v.Vbeta = (double)V * beta;
     c.v.Kalpha = (double)K * alpha;
     c.v.dense_stride = (K + 3) & ~3;
-    c.v.state = (SweepState*)dev_alloc(c, sizeof(SweepState));
-    c.v.err = c.v.state ? &c.v.state->err : nullptr;
-    c.report = report_pool().take();
-    if (!c.v.state || !c.report || cudaMemset(c.v.state, 0, sizeof(SweepState)) != cudaSuccess) {
-        report_pool().give(c.report);
-        dev_free_all(c);
+    if (!PartsPool::pool().take(c) || cudaMemset(c.v.state, 0, sizeof(SweepState)) != cudaSuccess) {
+        PartsPool::pool().give(c);
         delete h;
         cudaGetLastError();
         return LDA_ECUDA;
     }
-    {
-        bool ok = cudaEventCreateWithFlags(&c.ev_fork, cudaEventDisableTiming) == cudaSuccess;
-        for (int i = 0; i < 2 && ok; ++i)
-            ok = cudaEventCreateWithFlags(&c.ev_join[i], cudaEventDisableTiming) == cudaSuccess &&
-                 cudaStreamCreateWithFlags(&c.side[i], cudaStreamNonBlocking) == cudaSuccess;
-        ok = ok && cudaStreamCreateWithFlags(&c.copy, cudaStreamNonBlocking) == cudaSuccess &&
-             cudaEventCreateWithFlags(&c.ev_chunk, cudaEventDisableTiming) == cudaSuccess &&
-             cudaEventCreateWithFlags(&c.ev_export, cudaEventDisableTiming) == cudaSuccess;
-        c.have_side = true;  // lda_destroy() releases whatever was created
-        if (!ok) {
-            lda_destroy(h);
-            return LDA_ECUDA;
-        }
-    }
-    set_hist_smem_limits();
-    set_sample_smem_limits();
-    set_doc_smem_limits();
-    set_alias_smem_limits();
-    set_export_smem_limits();
-    set_loglik_smem_limits();
-    set_gibbs_smem_limits();
+    static std::once_flag limits_set[64];  // the kernels' limits stay with the device
+    auto set_limits = [] {
+        set_hist_smem_limits();
+        set_sample_smem_limits();
+        set_doc_smem_limits();
+        set_alias_smem_limits();
+        set_export_smem_limits();
+        set_loglik_smem_limits();
+        set_gibbs_smem_limits();
+    };
+    if (dev < 64) std::call_once(limits_set[dev], set_limits);
+    else set_limits();
     *out = h;
     return LDA_OK;
 }
@@ -881,26 +935,11 @@ void lda_destroy(lda_ctx* h)
     Ctx& c = h->c;
     cudaSetDevice(c.device);
     cudaStreamSynchronize(c.stream);
-    if (c.have_side) {
-        for (int i = 0; i < 2; ++i) {
-            if (c.side[i]) {
-                cudaStreamSynchronize(c.side[i]);
-                cudaStreamDestroy(c.side[i]);
-            }
-            if (c.ev_join[i]) cudaEventDestroy(c.ev_join[i]);
-        }
-        if (c.ev_fork) cudaEventDestroy(c.ev_fork);
-        if (c.copy) {
-            cudaStreamSynchronize(c.copy);
-            cudaStreamDestroy(c.copy);
-        }
-        if (c.ev_chunk) cudaEventDestroy(c.ev_chunk);
-        if (c.ev_export) cudaEventDestroy(c.ev_export);
-    }
+    for (cudaStream_t s : {c.side[0], c.side[1], c.copy}) cudaStreamSynchronize(s);
     drop_graphs(c);
     if (c.capture) cudaStreamDestroy(c.capture);
-    report_pool().give(c.report);
     dev_free_all(c);
+    PartsPool::pool().give(c);
     cudaGetLastError();
     delete h;
 }
@@ -978,17 +1017,17 @@ int lda_load_corpus(lda_ctx* h, const int32_t* word_ids, int64_t n_tokens, const
     Ctx& c = h->c;
     if (!doc_offsets || n_tokens < 0 || n_docs < 0 || (n_tokens > 0 && !word_ids))
         return fail(&c, LDA_EINVAL, "null pointer or negative size");
-    int rc = validate_offsets(&c, n_tokens, doc_offsets, n_docs);
+    Documents docs;
+    int rc = scan_documents(&c, n_tokens, doc_offsets, n_docs, docs);
     if (rc) return rc;
     if ((rc = check_device(c))) return rc;
     int32_t* wd = nullptr;
     if (!tmp_alloc(c, &wd, (size_t)std::max<int64_t>(n_tokens, 1) * 4)) return fail(&c, LDA_ENOMEM, "device allocation failed");
-    if (n_tokens > 0 &&
-        cudaMemcpyAsync(wd, word_ids, (size_t)n_tokens * 4, cudaMemcpyHostToDevice, c.stream) != cudaSuccess) {
+    if (copy_to_device(c, wd, word_ids, (size_t)n_tokens * 4) != cudaSuccess) {
         raw_free(c, wd);
         return cuda_fail(&c, "copying word ids");
     }
-    rc = load_common(c, wd, n_tokens, doc_offsets, n_docs);
+    rc = load_common(c, wd, n_tokens, docs, n_docs);
     cudaStreamSynchronize(c.stream);
     raw_free(c, wd);
     return rc;
@@ -1005,10 +1044,11 @@ int lda_load_corpus_device(lda_ctx* h, const int32_t* word_ids_dev, int64_t n_to
     int rc = check_device(c);
     if (rc) return rc;
     std::vector<int64_t> off((size_t)n_docs + 1);
-    if (cudaMemcpy(off.data(), doc_offsets_dev, ((size_t)n_docs + 1) * 8, cudaMemcpyDeviceToHost) != cudaSuccess)
+    if (copy_to_host(c, off.data(), doc_offsets_dev, ((size_t)n_docs + 1) * 8) != cudaSuccess)
         return cuda_fail(&c, "copying doc offsets");
-    if ((rc = validate_offsets(&c, n_tokens, off.data(), n_docs))) return rc;
-    return load_common(c, word_ids_dev, n_tokens, off.data(), n_docs);
+    Documents docs;
+    if ((rc = scan_documents(&c, n_tokens, off.data(), n_docs, docs))) return rc;
+    return load_common(c, word_ids_dev, n_tokens, docs, n_docs);
 }
 
 int lda_init(lda_ctx* h, uint64_t seed)

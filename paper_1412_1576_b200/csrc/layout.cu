@@ -58,7 +58,7 @@ __global__ void k_block_major_maps(const uint32_t* __restrict__ order, const uin
     }
 }
 
-int build_layout(Ctx& c, const int32_t* word_ids_dev, const int64_t* doc_off_host)
+int build_layout(Ctx& c, const int32_t* word_ids_dev, const std::vector<int32_t>& doc_off_host, LayoutTemps& temps)
 {
     const int32_t N = (int32_t)c.N, D = (int32_t)c.D, V = c.V;
     cudaStream_t st = c.stream;
@@ -70,88 +70,56 @@ int build_layout(Ctx& c, const int32_t* word_ids_dev, const int64_t* doc_off_hos
     int32_t* word_off = (int32_t*)dev_alloc(c, ((size_t)V + 1) * 4);
     int32_t* doc_off = (int32_t*)dev_alloc(c, ((size_t)D + 1) * 4);
     if (!tok_orig || !inv || !bm_of_tok || !word_off || !doc_off) return LDA_ENOMEM;
-
-    std::vector<int32_t> doc32((size_t)D + 1);
-    for (int64_t d = 0; d <= D; ++d) doc32[(size_t)d] = (int32_t)doc_off_host[d];
-    if (cudaMemcpyAsync(doc_off, doc32.data(), ((size_t)D + 1) * 4, cudaMemcpyHostToDevice, st) !=
-        cudaSuccess)
-        return LDA_ECUDA;
-
-    // transient buffers of the sort
-    int32_t* keys_out = nullptr;
-    uint32_t* iota = nullptr;
-    uint32_t* keys_blk = nullptr;
-    uint32_t* order = nullptr;
-    void* temp = nullptr;
-    void* temp2 = nullptr;
-    size_t temp_bytes = 0, temp2_bytes = 0;
-    int rc = LDA_OK;
-    do {
-        if (!tmp_alloc(c, &keys_out, n1 * 4) || !tmp_alloc(c, &iota, n1 * 4) || !tmp_alloc(c, &keys_blk, n1 * 4) ||
-            !tmp_alloc(c, &order, n1 * 4)) {
-            rc = LDA_ENOMEM;
-            break;
-        }
-        if (N > 0) {
-            k_check_words_iota<<<1184, 256, 0, st>>>(word_ids_dev, iota, N, V, c.v.err);
-            int end_bit = 1;
-            while (end_bit < 31 && (1ll << end_bit) < (long long)V) ++end_bit;
-            if (cub::DeviceRadixSort::SortPairs(nullptr, temp_bytes, word_ids_dev, keys_out, iota,
-                                                tok_orig, N, 0, end_bit, st) != cudaSuccess) {
-                rc = LDA_ECUDA;
-                break;
-            }
-            if (!tmp_alloc(c, &temp, temp_bytes)) {
-                rc = LDA_ENOMEM;
-                break;
-            }
-            if (cub::DeviceRadixSort::SortPairs(temp, temp_bytes, word_ids_dev, keys_out, iota,
-                                                tok_orig, N, 0, end_bit, st) != cudaSuccess) {
-                rc = LDA_ECUDA;
-                break;
-            }
-            // block-major order: tokens sorted by (block of their document-order index, word-sorted
-            // position); a stable sort of the positions by block
-            uint32_t* keys_tmp = reinterpret_cast<uint32_t*>(keys_out);  // the word keys are no longer needed
-            k_block_keys<<<1184, 256, 0, st>>>(tok_orig, N, c.block_shift, keys_blk, iota);
-            int blk_bits = 1;
-            while (blk_bits < 32 && (((long long)N - 1) >> c.block_shift) >= (1ll << blk_bits)) ++blk_bits;
-            if (cub::DeviceRadixSort::SortPairs(nullptr, temp2_bytes, keys_blk, keys_tmp, iota, order, N, 0,
-                                                blk_bits, st) != cudaSuccess) {
-                rc = LDA_ECUDA;
-                break;
-            }
-            if (!tmp_alloc(c, &temp2, temp2_bytes)) {
-                rc = LDA_ENOMEM;
-                break;
-            }
-            // the word offsets are taken from keys_out first: the next sort overwrites it
-            k_word_offsets<<<(V + 1 + 255) / 256, 256, 0, st>>>(keys_out, N, V, word_off);
-            if (cub::DeviceRadixSort::SortPairs(temp2, temp2_bytes, keys_blk, keys_tmp, iota, order, N, 0,
-                                                blk_bits, st) != cudaSuccess) {
-                rc = LDA_ECUDA;
-                break;
-            }
-            k_block_major_maps<<<1184, 256, 0, st>>>(order, tok_orig, N, inv, bm_of_tok);
-        } else {
-            k_word_offsets<<<(V + 1 + 255) / 256, 256, 0, st>>>(keys_out, N, V, word_off);
-        }
-        if (cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess)
-            rc = LDA_ECUDA;
-    } while (0);
-    raw_free(c, keys_out);
-    raw_free(c, iota);
-    raw_free(c, keys_blk);
-    raw_free(c, order);
-    raw_free(c, temp);
-    raw_free(c, temp2);
-    if (rc != LDA_OK) return rc;
     c.v.inv = inv;
     c.v.bm_of_tok = bm_of_tok;
     c.v.tok_orig = tok_orig;
     c.v.word_off = word_off;
     c.v.doc_off = doc_off;
-    return LDA_OK;
+    if (copy_to_device(c, doc_off, doc_off_host.data(), ((size_t)D + 1) * 4) != cudaSuccess) return LDA_ECUDA;
+
+    // transient buffers of the sorts; both sorts share the temporary storage
+    int end_bit = 1, blk_bits = 1;
+    while (end_bit < 31 && (1ll << end_bit) < (long long)V) ++end_bit;
+    while (blk_bits < 32 && (((long long)N - 1) >> c.block_shift) >= (1ll << blk_bits)) ++blk_bits;
+    size_t temp_bytes = 0, temp2_bytes = 0;
+    const int32_t* no_keys = nullptr;
+    const uint32_t* no_values = nullptr;
+    if (N > 0 && (cub::DeviceRadixSort::SortPairs(nullptr, temp_bytes, no_keys, (int32_t*)nullptr, no_values, tok_orig, N, 0, end_bit,
+                                                  st) != cudaSuccess ||
+                  cub::DeviceRadixSort::SortPairs(nullptr, temp2_bytes, no_values, (uint32_t*)nullptr, no_values, tok_orig, N, 0,
+                                                  blk_bits, st) != cudaSuccess))
+        return LDA_ECUDA;
+    auto transient = [&](size_t bytes) -> void* {
+        void* p = nullptr;
+        if (tmp_alloc(c, &p, bytes)) temps.held.push_back(p);
+        return p;
+    };
+    int32_t* keys_out = (int32_t*)transient(n1 * 4);
+    uint32_t* iota = (uint32_t*)transient(n1 * 4);
+    uint32_t* keys_blk = (uint32_t*)transient(n1 * 4);
+    uint32_t* order = (uint32_t*)transient(n1 * 4);
+    void* temp = transient(temp_bytes > temp2_bytes ? temp_bytes : temp2_bytes);
+    if (!keys_out || !iota || !keys_blk || !order || !temp) return LDA_ENOMEM;
+    bool ok = true;
+    if (N > 0) {
+        k_check_words_iota<<<1184, 256, 0, st>>>(word_ids_dev, iota, N, V, c.v.err);
+        ok = cub::DeviceRadixSort::SortPairs(temp, temp_bytes, word_ids_dev, keys_out, iota, tok_orig, N, 0, end_bit, st) == cudaSuccess;
+    }
+    k_word_offsets<<<(V + 1 + 255) / 256, 256, 0, st>>>(keys_out, N, V, word_off);
+    cudaEventRecord(c.ev_chunk, st);
+    if (N > 0 && ok) {
+        // block-major order: tokens sorted by (block of their document-order index, word-sorted
+        // position); a stable sort of the positions by block (one block: the positions themselves)
+        if (((long long)N - 1) >> c.block_shift) {
+            k_block_keys<<<1184, 256, 0, st>>>(tok_orig, N, c.block_shift, keys_blk, iota);
+            uint32_t* keys_tmp = reinterpret_cast<uint32_t*>(keys_out);  // the word keys are no longer needed
+            ok = cub::DeviceRadixSort::SortPairs(temp, temp2_bytes, keys_blk, keys_tmp, iota, order, N, 0, blk_bits, st) == cudaSuccess;
+        } else {
+            order = iota;  // still 0, 1, 2, ...
+        }
+        if (ok) k_block_major_maps<<<1184, 256, 0, st>>>(order, tok_orig, N, inv, bm_of_tok);
+    }
+    return ok && cudaPeekAtLastError() == cudaSuccess ? LDA_OK : LDA_ECUDA;
 }
 
 }  // namespace lda

@@ -298,7 +298,6 @@ struct Ctx {
     // wait for the work queued on `stream` so far, join_streams() makes `stream` wait for theirs.
     cudaStream_t side[2] = {};
     cudaEvent_t ev_fork = nullptr, ev_join[2] = {};
-    bool have_side = false;
     // Assignments travel between host and device in chunks on a stream of their own, so that the copy
     // of one chunk runs beside the kernel that spreads (or collects) its neighbour.  ev_chunk orders a
     // chunk's two halves; ev_export completes when the last chunk of an export has reached the host:
@@ -431,8 +430,12 @@ struct WkCsr {
 int build_wk_csr(Ctx& c, WkCsr& r, bool sizes_only);
 void free_wk_csr(Ctx& c, WkCsr& r);
 
-// load-time layout (sort + offsets); fills c.v token arrays. Returns LDA_* status.
-int build_layout(Ctx& c, const int32_t* word_ids_dev, const int64_t* doc_off_host);
+// load-time layout (sort + offsets), queued; fills c.v token arrays and records ev_chunk when word_off is there.
+// The transient buffers are the caller's to release once the stream is done with them.  LDA_* status.
+struct LayoutTemps {
+    std::vector<void*> held;
+};
+int build_layout(Ctx& c, const int32_t* word_ids_dev, const std::vector<int32_t>& doc_off, LayoutTemps& temps);
 
 void* raw_alloc(Ctx& c, size_t bytes);  // the context's allocator (cudaMalloc by default); nullptr on failure
 void raw_free(Ctx& c, void* p);
