@@ -98,7 +98,7 @@ int lda_set_allocator(lda_ctx* ctx, lda_alloc_fn alloc_fn, lda_free_fn free_fn, 
  *   "dense_frac"   fraction of the vocabulary (by term frequency) whose n_kw rows are dense (Section 5)
  *   "dense_min_tf" words rarer than this (or than K/8) stay sparse even inside dense_frac
  *   "block_log2"   log2 of the tokens per block of documents in the block-major token order that the
- *                  document-side pass of the MH step walks (default 22: the exchange buffers
+ *                  document-side pass of the MH step walks (default: chosen per corpus, 20 or 22: the exchange buffers
  *                  of one block, 20 bytes per token, stay in L2 while the document pass is on it)
  *   "copy_chunk_log2" log2 of the tokens per chunk in which assignments cross the host link (default 25):
  *                  a chunk is copied on the context's copy stream while its neighbour is spread into, or

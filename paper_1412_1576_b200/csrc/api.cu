@@ -524,27 +524,8 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     v.count_bits = cb;
     v.tok_base = (uint32_t)c.shard_first_token;
 
-    // The sorts are queued; the documents' lists are made meanwhile, the words' lists beside the second sort.
-    LayoutTemps temps;
-    struct Release {
-        Ctx& c;
-        LayoutTemps& t;
-        ~Release()
-        {
-            cudaStreamSynchronize(c.stream);
-            for (void* p : t.held) raw_free(c, p);
-        }
-    } release{c, temps};
-    int rc = build_layout(c, words_dev, doc_off, temps);
-    if (rc != LDA_OK) {
-        cudaStreamSynchronize(c.stream);
-        cudaGetLastError();
-        free_corpus(c);
-        return fail(&c, rc, "building the word-sorted layout failed");
-    }
-    // tiles of whole documents: for the MH step, and for the sorted n_kd rows (<= SORT_TILE tokens and <= ROW_TILE_WORDS
-    // documents each)
-    std::vector<int32_t> doc_tiles, long_docs, doc_sort_tiles, doc_sort_long;
+    // shape and form of the document tiles
+    int32_t dense_docs = 0;
     {
         // A document that does not fit a tile takes the long documents' kernels; the shape with the least
         // estimated time is taken, relative costs per token as measured (12 M tokens of 4000-token documents at
@@ -573,6 +554,40 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
         }
         c.doc_tile = DOC_TILE_TOKENS[shape];
         c.doc_threads = DOC_TILE_THREADS[shape];
+        // a counter per topic instead of hashed tables when a tile holds enough documents' worth of them to be
+        // filled (two counters take the room of a slot)
+        const int32_t mean_len = N / std::max(1, D);
+        dense_docs = 2 * DOC_TILE_SLOTS * c.doc_tile / (K + 1);
+        c.doc_dense = D > 0 && dense_docs > 0 && (int64_t)dense_docs * mean_len >= c.doc_tile - mean_len;
+        // Tokens per block of the block-major order: small blocks keep the document pass's scattered accesses in L2, long
+        // ones make the word-order passes' runs longer.  With hashed tables the document pass is bound by
+        // its instructions and 2^22 is best (738 M tokens, K = 10 000: 23.2 ms per sweep, 24.0 with 2^20); with
+        // counters by those accesses, and 2^20 is (99 M tokens, K = 1000: 3.08 ms, 3.35 with 2^22).
+        c.block_shift = c.block_option ? c.block_option : c.doc_dense ? 20 : 22;
+    }
+
+    // The sorts are queued; the documents' lists are made meanwhile, the words' lists beside the second sort.
+    LayoutTemps temps;
+    struct Release {
+        Ctx& c;
+        LayoutTemps& t;
+        ~Release()
+        {
+            cudaStreamSynchronize(c.stream);
+            for (void* p : t.held) raw_free(c, p);
+        }
+    } release{c, temps};
+    int rc = build_layout(c, words_dev, doc_off, temps);
+    if (rc != LDA_OK) {
+        cudaStreamSynchronize(c.stream);
+        cudaGetLastError();
+        free_corpus(c);
+        return fail(&c, rc, "building the word-sorted layout failed");
+    }
+    // tiles of whole documents: for the MH step, and for the sorted n_kd rows (<= SORT_TILE tokens and <= ROW_TILE_WORDS
+    // documents each)
+    std::vector<int32_t> doc_tiles, long_docs, doc_sort_tiles, doc_sort_long;
+    {
         auto pack = [&](int32_t tokens, int32_t documents, std::vector<int32_t>& tiles, std::vector<int32_t>& longer) {
             int32_t s0 = 0, tok = 0;
             auto close = [&](int32_t s1) {
@@ -586,7 +601,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
             }
             close(D);
         };
-        pack(c.doc_tile, c.doc_tile, doc_tiles, long_docs);
+        pack(c.doc_tile, c.doc_dense ? std::min(dense_docs, c.doc_tile) : c.doc_tile, doc_tiles, long_docs);
         pack(SORT_TILE, ROW_TILE_WORDS, doc_sort_tiles, doc_sort_long);
     }
     std::vector<int32_t> word_off((size_t)V + 1);
@@ -994,7 +1009,7 @@ int lda_set_option(lda_ctx* h, const char* key, double value)
     }
     if (!std::strcmp(key, "block_log2")) {
         if (!(value >= 10.0 && value <= 30.0)) return fail(&c, LDA_EINVAL, "block_log2 must be in [10,30]");
-        c.block_shift = (int)value;
+        c.block_option = (int)value;
         return LDA_OK;
     }
     return fail(&c, LDA_EINVAL, "unknown option");

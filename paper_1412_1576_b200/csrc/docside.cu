@@ -13,6 +13,8 @@
 // The current assignments and the word-proposals arrive in block-major order and the results go
 // back in block-major order: a tile's documents lie in one block of that order (two at a block
 // border), so these scattered reads and writes stay in L2.
+#include <type_traits>
+
 #include "lda_device.cuh"
 #include "lda_internal.cuh"
 
@@ -37,20 +39,58 @@ __device__ __forceinline__ void load_topic_pair(const int32_t* zbm, uint32_t bm,
     t1 = w.y;
 }
 
-// The n_kd table of a document in a tile: hashed, in shared memory.
+// --- n_kd of a document in a tile, in shared memory ----------------------------------------------
+// Two forms, chosen per corpus (load_common()):
+//   DENSE   a 16-bit counter per topic (K even or padded): an addition, a read;
+//   hashed  TILE_SLOTS slots per token, as dk_insert in lda_device.cuh has it.  (Probing aligned pairs of slots by
+//           8-byte reads: fewer turns of the loop, more instructions each; 10.6 ms per sweep instead of 10.1 at 738 M
+//           tokens.)
+// Both give (topic << count_bits) | n_kd.
+template <bool DENSE>
 struct TileTable {
-    const uint32_t* tab;      // TILE_SLOTS * doc_len slots
-    const uint32_t* slot_of;  // slot holding the topic of the document's j-th token
-    uint32_t cap;
+    const uint32_t* tab;      // the document's counters, or its slots
+    const uint32_t* tok;      // DENSE: topic of the document's j-th token; hashed: its slot
+    uint32_t cap;             // hashed: slots
     int cb;
-    // (topic << count_bits) | n_kd of topic k, and of the j-th token's topic
+    __device__ __forceinline__ uint32_t counted(uint32_t k) const
+    {
+        return k << cb | reinterpret_cast<const uint16_t*>(tab)[k];
+    }
     __device__ __forceinline__ uint32_t of_topic(uint32_t k) const
     {
+        if (DENSE) return counted(k);
         const uint32_t e = dk_lookup(tab, cap, k, cb);
         return e ? e : k << cb;
     }
-    __device__ __forceinline__ uint32_t of_token(uint32_t j) const { return tab[slot_of[j]]; }
+    // the j-th token's topic (copy), or topic j
+    __device__ __forceinline__ uint32_t drawn(bool copy, uint32_t j) const
+    {
+        if (DENSE) return counted(copy ? tok[j] : j);
+        // the slot to look at first is the token's or the topic's home: one read serves both
+        uint32_t h = copy ? tok[j] : dk_home(j, cap);
+        uint32_t e = tab[h];
+        if (copy) return e;
+        const uint32_t want = j << cb;
+        for (uint32_t n = 0; n < cap; ++n) {
+            if (e == DK_EMPTY) break;
+            if ((e >> cb) == j) return e;
+            if (++h == cap) h = 0;
+            e = tab[h];
+        }
+        return want;
+    }
 };
+
+// Adds one occurrence of topic k; returns what TileTable::tok keeps, or ~0 if there was no room.
+template <bool DENSE>
+__device__ __forceinline__ uint32_t tile_insert(uint32_t* tab, uint32_t cap, uint32_t k, int cb)
+{
+    if (DENSE) {
+        atomicAdd(&tab[k >> 1], (k & 1u) ? 0x10000u : 1u);
+        return k;
+    }
+    return dk_insert(tab, cap, k, cb);
+}
 
 // The table of a document longer than a tile, in device memory or staged: a counter per topic (DENSE) or hashed.
 template <bool DENSE>
@@ -65,7 +105,7 @@ struct LongTable {
         const uint32_t e = dk_lookup(tab, cap, k, cb);
         return e ? e : k << cb;
     }
-    __device__ __forceinline__ uint32_t of_token(uint32_t j) const { return of_topic(topic_of[j]); }
+    __device__ __forceinline__ uint32_t drawn(bool copy, uint32_t j) const { return of_topic(copy ? topic_of[j] : j); }
 };
 
 // Everything pass 3 needs from the document side for one token, written at the token's
@@ -78,7 +118,7 @@ __device__ __forceinline__ void doc_side_token(const View& v, const Table& table
     const T* prop = reinterpret_cast<const T*>(v.prop);
     const size_t N = (size_t)v.N;
     uint32_t* out = v.dside + (size_t)bm * v.side_stride;
-    const double n_d = (double)doc_len;
+    const double n_d = u32_to_double(doc_len);
     // words 0..3 (the whole record when the step count is fixed at compile time) are collected in
     // registers and go out as 16-byte stores at the end, the rest one by one
     constexpr int REGW = (FIXED > 0 && step_record_words<MODE>(FIXED) > 4) ? 8 : 4;
@@ -104,13 +144,8 @@ __device__ __forceinline__ void doc_side_token(const View& v, const Table& table
     // doc-proposal of step st, the di-th of its kind
     auto doc_step = [&](int32_t st, int32_t di) {
         const uint4 r = philox4x32_10(make_uint4(v.tok_base + tok, sweep, (uint32_t)st, 0u), key);
-        const double uu = __dmul_rn((double)r.x, INV_2_32);
-        uint32_t o2;
-        if (__dmul_rn(uu, __dadd_rn(n_d, v.Kalpha)) < n_d) {
-            o2 = table.of_token(scale_to_range(r.y, doc_len));
-        } else {
-            o2 = table.of_topic(scale_to_range(r.y, (uint32_t)v.K));
-        }
+        const bool copy = __dmul_rn(__dmul_rn(u32_to_double(r.x), INV_2_32), __dadd_rn(n_d, v.Kalpha)) < n_d;
+        const uint32_t o2 = table.drawn(copy, scale_to_range(r.y, copy ? doc_len : (uint32_t)v.K));
         put(1 + st, o2);
         put(1 + mh_steps + di, r.w);  // the step's acceptance uniform
     };
@@ -141,7 +176,7 @@ __host__ __device__ constexpr int doc_resident_threads(int mode, int fixed)
 {
     return (fixed == 2 && mode != LDA_PROPOSALS_DOC) ? 2048 : 1536;
 }
-template <typename T, int THREADS, int MODE, int FIXED>
+template <typename T, int THREADS, int MODE, int FIXED, bool DENSE>
 __global__ void __launch_bounds__(THREADS, doc_resident_threads(MODE, FIXED) / THREADS)
 k_doc_tile(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_steps_arg)
 {
@@ -149,18 +184,18 @@ k_doc_tile(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_step
     const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
     constexpr int cap = DOC_TILE_ROUNDS * THREADS;
     extern __shared__ __align__(16) uint32_t doc_smem[];
-    uint32_t* slots = doc_smem;                                  // [TILE_SLOTS * cap] the tile's tables
-    int32_t* soff = reinterpret_cast<int32_t*>(slots + TILE_SLOTS * cap);  // [cap + 1] document offsets
-    uint32_t* slot_s = reinterpret_cast<uint32_t*>(soff + cap + 1);  // [cap] slot (inside its table) of a token's topic
+    uint32_t* area = doc_smem;                                           // [TILE_SLOTS * cap] the tile's tables
+    int32_t* soff = reinterpret_cast<int32_t*>(area + TILE_SLOTS * cap);  // [cap + 1] document offsets
+    uint32_t* tok_s = reinterpret_cast<uint32_t*>(soff + cap + 1);        // [cap] see TileTable::tok
     const int tid = threadIdx.x;
     const int32_t s0 = tiles[2 * blockIdx.x], s1 = tiles[2 * blockIdx.x + 1];
     const int32_t nseg = s1 - s0;
     const int32_t base = v.doc_off[s0];
     const int32_t cnt = v.doc_off[s1] - base;
     if (cnt == 0) return;
+    const int32_t half_k = DENSE ? (v.K + 1) >> 1 : 0;  // words of a document's counters
     const T* zbm = reinterpret_cast<const T*>(v.zbm);
     uint32_t bm[DOC_TILE_ROUNDS], z[DOC_TILE_ROUNDS], t1[DOC_TILE_ROUNDS];
-    int32_t first[DOC_TILE_ROUNDS], len[DOC_TILE_ROUNDS];
 #pragma unroll
     for (int r = 0; r < DOC_TILE_ROUNDS; ++r) {
         const int j = tid + r * THREADS;
@@ -170,34 +205,34 @@ k_doc_tile(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_step
             load_topic_pair(zbm, bm[r], z[r], t1[r]);
         }
     }
-    for (int j = tid; j <= nseg; j += blockDim.x) soff[j] = v.doc_off[s0 + j] - base;
-    const uint4 empty4 = make_uint4(DK_EMPTY, DK_EMPTY, DK_EMPTY, DK_EMPTY);
-    for (int j = tid; j < cnt * (TILE_SLOTS / 4); j += blockDim.x) reinterpret_cast<uint4*>(slots)[j] = empty4;
+    uint32_t doc[DOC_TILE_ROUNDS];  // first token of the token's document | its length << 16: every register counts here
+    for (int j = tid; j <= nseg; j += THREADS) soff[j] = v.doc_off[s0 + j] - base;
+    const uint32_t none = DENSE ? 0u : DK_EMPTY;
+    const int quads = DENSE ? (nseg * half_k + 3) >> 2 : cnt * (TILE_SLOTS / 4);
+    for (int j = tid; j < quads; j += THREADS) reinterpret_cast<uint4*>(area)[j] = make_uint4(none, none, none, none);
     __syncthreads();
-    // every token finds its document, adds itself to the document's table and notes the slot
+    // every token finds its document and adds itself to the document's table
 #pragma unroll
     for (int r = 0; r < DOC_TILE_ROUNDS; ++r) {
         const int j = tid + r * THREADS;
-        first[r] = 0;
-        len[r] = 1;
+        doc[r] = 0;
         if (j < cnt) {
             int lo = 0, hi = nseg;  // last document with soff[doc] <= j
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
                 if (soff[mid] <= j) lo = mid; else hi = mid;
             }
-            first[r] = soff[lo];
-            len[r] = soff[lo + 1] - first[r];
+            const int32_t f = soff[lo], n = soff[lo + 1] - f;
+            doc[r] = (uint32_t)n << 16 | (uint32_t)f;
             uint32_t at = 0xFFFFFFFFu;
             if (z[r] < (uint32_t)v.K)
-                at = dk_insert(slots + TILE_SLOTS * first[r], TILE_SLOTS * (uint32_t)len[r], z[r],
-                               v.count_bits);
+                at = tile_insert<DENSE>(area + (DENSE ? lo * half_k : TILE_SLOTS * f), TILE_SLOTS * (uint32_t)n, z[r], v.count_bits);
             if (at == 0xFFFFFFFFu) {
                 atomicOr(v.err, z[r] < (uint32_t)v.K ? ERR_ROW_OVERFLOW : ERR_TOPIC_RANGE);
                 at = 0;
             }
-            slot_s[j] = at;
-            z[r] = at;  // from here on: the slot
+            tok_s[j] = at;
+            z[r] = DENSE ? (uint32_t)lo << 16 | at : at;  // from here on: the slot, or the topic with its document
         }
     }
     __syncthreads();
@@ -207,9 +242,10 @@ k_doc_tile(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_step
     for (int r = 0; r < DOC_TILE_ROUNDS; ++r) {
         const int j = tid + r * THREADS;
         if (j < cnt) {
-            const TileTable table{slots + TILE_SLOTS * first[r], slot_s + first[r], TILE_SLOTS * (uint32_t)len[r], v.count_bits};
-            doc_side_token<T, MODE, FIXED>(v, table, (uint32_t)(base + j), (uint32_t)len[r], table.tab[z[r]], t1[r], bm[r], key,
-                                           sweep, mh_steps);
+            const uint32_t f = doc[r] & 0xFFFFu, n = doc[r] >> 16;
+            const TileTable<DENSE> table{area + (DENSE ? (z[r] >> 16) * half_k : TILE_SLOTS * f), tok_s + f, TILE_SLOTS * n, v.count_bits};
+            const uint32_t own = DENSE ? table.counted(z[r] & 0xFFFFu) : table.tab[z[r]];
+            doc_side_token<T, MODE, FIXED>(v, table, (uint32_t)(base + j), n, own, t1[r], bm[r], key, sweep, mh_steps);
         }
     }
 }
@@ -325,8 +361,10 @@ size_t doc_tile_smem_bytes(int tile_tokens) { return (size_t)tile_tokens * DOC_T
 template <typename T, int MODE, int FIXED>
 static void set_doc_limit()
 {
-    cudaFuncSetAttribute(k_doc_tile<T, 1024, MODE, FIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)doc_tile_smem_bytes(DOC_TILE_MAX));
+    const int bytes = (int)doc_tile_smem_bytes(DOC_TILE_MAX);
+    cudaFuncSetAttribute(k_doc_tile<T, 1024, MODE, FIXED, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (sizeof(T) == 2)
+        cudaFuncSetAttribute(k_doc_tile<uint16_t, 1024, MODE, FIXED, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 void set_doc_smem_limits()
@@ -355,12 +393,17 @@ static int doc_side_tm(Ctx& c, int mh_steps)
     int launches = 0;
     if (c.n_doc_tiles) {
         const size_t smem = doc_tile_smem_bytes(c.doc_tile);
-        switch (c.doc_threads) {
-            case 128: k_doc_tile<T, 128, MODE, FIXED><<<c.n_doc_tiles, 128, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
-            case 256: k_doc_tile<T, 256, MODE, FIXED><<<c.n_doc_tiles, 256, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
-            case 512: k_doc_tile<T, 512, MODE, FIXED><<<c.n_doc_tiles, 512, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
-            default: k_doc_tile<T, 1024, MODE, FIXED><<<c.n_doc_tiles, 1024, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
-        }
+        auto tiles = [&](auto dense) {
+            constexpr bool DENSE = decltype(dense)::value;
+            switch (c.doc_threads) {
+                case 128: k_doc_tile<T, 128, MODE, FIXED, DENSE><<<c.n_doc_tiles, 128, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
+                case 256: k_doc_tile<T, 256, MODE, FIXED, DENSE><<<c.n_doc_tiles, 256, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
+                case 512: k_doc_tile<T, 512, MODE, FIXED, DENSE><<<c.n_doc_tiles, 512, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
+                default: k_doc_tile<T, 1024, MODE, FIXED, DENSE><<<c.n_doc_tiles, 1024, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
+            }
+        };
+        if (c.doc_dense) tiles(std::integral_constant<bool, sizeof(T) == 2>{});  // never with 32-bit topics
+        else tiles(std::false_type{});
         ++launches;
     }
     if (c.n_long_chunks) {

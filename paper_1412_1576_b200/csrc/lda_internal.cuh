@@ -47,20 +47,14 @@ constexpr int SORT_TILE = 2048;      // tokens per segmented-sort tile (one CTA)
 // Tiles of whole documents (one CTA each) of the document-side kernels: tokens per tile and
 // threads per CTA, chosen per corpus from these shapes; longer documents get a CTA of their own.
 constexpr int DOC_TILE_SHAPES = 4;
-#ifndef LDA_DOC_TILE_ROUNDS
-#define LDA_DOC_TILE_ROUNDS 3
-#endif
-constexpr int DOC_TILE_ROUNDS = LDA_DOC_TILE_ROUNDS;  // tokens per thread: every shape holds this many times its thread count
+constexpr int DOC_TILE_ROUNDS = 3;  // tokens per thread: every shape holds this many times its thread count
 constexpr int DOC_TILE_THREADS[DOC_TILE_SHAPES] = {128, 256, 512, 1024};
 constexpr int DOC_TILE_TOKENS[DOC_TILE_SHAPES] = {DOC_TILE_ROUNDS * 128, DOC_TILE_ROUNDS * 256, DOC_TILE_ROUNDS * 512,
                                                   DOC_TILE_ROUNDS * 1024};
 constexpr int DOC_TILE_MAX = DOC_TILE_ROUNDS * 1024;
-// shared memory per token of a tile: 4 table slots, document offset, topic/slot (4 bytes each)
-#ifndef LDA_DOC_TILE_SLOTS
-#define LDA_DOC_TILE_SLOTS 4
-#endif
-constexpr int DOC_TILE_SLOTS = LDA_DOC_TILE_SLOTS;  // slots per token of a tile's tables in shared memory
+constexpr int DOC_TILE_SLOTS = 4;  // 32-bit words per token of a tile's tables in shared memory
 static_assert(DOC_TILE_SLOTS % 4 == 0, "a tile's tables are cleared 16 bytes at a time");
+// shared memory per token of a tile: table, document offset, topic or slot
 constexpr int DOC_TILE_SMEM_PER_TOKEN = 4 * DOC_TILE_SLOTS + 4 + 4;
 // partial sums of the log-likelihood kernels: word part; document part (tiles + long documents)
 constexpr int LL_WORD_PARTIALS = 592;
@@ -197,8 +191,10 @@ struct Ctx {
     int n_sm = 148;  // multiprocessors of the device
     cudaStream_t stream = nullptr;
     bool wide_topics = false;  // false: 16-bit topic storage, true: 32-bit
+    int block_option = 0;  // option "block_log2", 0: chosen per corpus
     int block_shift = 22;  // log2 of the tokens per block of the block-major order
     int doc_tile = DOC_TILE_TOKENS[0], doc_threads = DOC_TILE_THREADS[0];  // shape of the document tiles
+    bool doc_dense = false;  // their n_kd tables are a counter per topic
     int side_steps = 0;    // number of steps the exchange buffers are allocated for
     int side_mode = 0;     // ... and the proposal schedule they are laid out for
     int proposals = 0;     // LDA_PROPOSALS_*: which proposal each step of a chain draws

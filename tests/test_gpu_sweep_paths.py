@@ -102,3 +102,16 @@ def test_long_documents_by_chunks(K, mode):
     for a, b in zip(g.loglik(), o.loglik()):
         assert a == pytest.approx(b, rel=1e-10)
     assert g.stats()["nnz_dk"] == g.get_csr(binding.LDA_NDK)[1].size
+
+
+@pytest.mark.parametrize("K,length", [(191, 24), (193, 24), (767, 96), (769, 96), (1023, 330), (3_071, 384), (3_073, 384), (3_100, 500)])
+def test_document_tiles_with_counters_and_with_hashed_tables(K, length):
+    """Topic counts on both sides of what a tile's counters hold, odd ones among them."""
+    c = synth.generate(V=900, K=K, D=70, length=("poisson", float(length)), zipf_s=1.05, alpha=0.3, beta=0.01, seed=K)
+    g, o = _pair(c)
+    for steps, mode in ((2, 0), (3, 0), (2, 2), (4, 0)):
+        for e in (g, o):
+            e.set_proposals(mode)
+            e.sweep(2, steps)
+        assert np.array_equal(g.get_assignments(), o.get_assignments()), (steps, mode)
+    _same(g, o)
