@@ -100,7 +100,7 @@ int lda_set_allocator(lda_ctx* ctx, lda_alloc_fn alloc_fn, lda_free_fn free_fn, 
  *   "block_log2"   log2 of the tokens per block of documents in the block-major token order that the
  *                  document-side pass of the MH step walks (default: chosen per corpus, 20 or 22: the exchange buffers
  *                  of one block, 20 bytes per token, stay in L2 while the document pass is on it)
- *   "copy_chunk_log2" log2 of the tokens per chunk in which assignments cross the host link (default 25):
+ *   "copy_chunk_log2" log2 of the tokens per chunk in which assignments cross the host link (default: by corpus):
  *                  a chunk is copied on the context's copy stream while its neighbour is spread into, or
  *                  collected from, the device layout.  Whole number in [10, 30]; no result depends on it.
  *   "alias_slices" number of vocabulary slices (Section 3, Figure 1: the model is visited one slice at a

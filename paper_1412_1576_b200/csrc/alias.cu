@@ -618,13 +618,17 @@ int launch_alias_dense(Ctx& c, bool in_sweep)
 }
 
 // The kernels build the tables of different words: they run side by side, the ones with the longest rows
-// (and the longest tail) first.
-int launch_alias_sparse(Ctx& c, bool all)
+// (and the longest tail) first.  begin_sweep: the sweep's first kernel, the dense table, runs beside them
+// (nothing here reads what it writes).
+int launch_alias_sparse(Ctx& c, bool all, bool begin_sweep)
 {
     const Ctx::Slice& q = c.slices[(size_t)c.cur_slice];
-    if (q.w_hi <= q.w_lo) return 0;
     int launches = 0;
     fork_streams(c);
+    if (begin_sweep) {
+        run_alias_dense(c.v, c.sc_dense, c.side[0]);
+        ++launches;
+    }
     const auto words = [&](int cls) { return c.alias_words[cls] + q.alias_lo[cls]; };
     if (q.alias_n[3]) {
         k_alias_sparse_cluster<<<q.alias_n[3] * ALIAS_ROW_CLUSTER, 512, 0, c.stream>>>(c.v, words(3), c.sc_w, c.sc_de, c.sc_item, all);
@@ -643,6 +647,10 @@ int launch_alias_sparse(Ctx& c, bool all)
     if (q.alias_n[0]) {
         k_alias_sparse_long_warp<<<(q.alias_n[0] + 3) / 4, 128, 0, c.side[0]>>>(c.v, words(0), q.alias_n[0], all, c.sc_w);
         ++launches;
+    }
+    if (q.w_hi <= q.w_lo) {
+        join_streams(c);
+        return launches;
     }
     // words per warp: as many as fill a warp's lanes with the words' sizes, as long as every multiprocessor gets two CTAs
     int per_warp = 32;

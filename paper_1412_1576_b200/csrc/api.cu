@@ -361,8 +361,8 @@ void rebuild_counts(Ctx& c)
 // One sweep, kernel by kernel.  Returns the number of kernels.
 static int queue_sweep(Ctx& c, int mh_steps)
 {
-    int n = launch_alias_dense(c, true);
-    if (c.slices.size() == 1) n += launch_alias_sparse(c, false);  // else slice by slice inside pass 1
+    // several vocabulary slices: the sparse tables are built slice by slice inside pass 1
+    int n = c.slices.size() == 1 ? launch_alias_sparse(c, false, true) : launch_alias_dense(c, true);
     n += launch_sample(c, mh_steps);
     n += launch_count_wk(c);
     n += launch_count_k(c);
@@ -571,11 +571,13 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     struct Release {
         Ctx& c;
         LayoutTemps& t;
-        ~Release()
+        void now()
         {
             cudaStreamSynchronize(c.stream);
             for (void* p : t.held) raw_free(c, p);
+            t.held.clear();
         }
+        ~Release() { now(); }
     } release{c, temps};
     int rc = build_layout(c, words_dev, doc_off, temps);
     if (rc != LDA_OK) {
@@ -800,6 +802,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     }
     const size_t cap_alias = (size_t)slice_rows_max;
 
+    release.now();  // before the large buffers are allocated: they may take over its memory
     const size_t n1 = (size_t)std::max<int64_t>(N, 1), cap1 = (size_t)std::max<int64_t>(cap_total, 1);
     const size_t zt = c.wide_topics ? 4 : 2;
     bool ok = true;
@@ -1086,6 +1089,13 @@ int lda_init(lda_ctx* h, uint64_t seed)
     return LDA_OK;
 }
 
+// Tokens per chunk of a transfer: the kernel's part of the first (or last) chunk runs beside no copy, so chunks
+// are short, but a sixteenth of the corpus is short enough and 2^20 tokens are worth a copy of their own.
+static int64_t transfer_chunk(const Ctx& c)
+{
+    return c.copy_chunk ? c.copy_chunk : std::max<int64_t>((int64_t)1 << 20, c.N / 16);
+}
+
 static int set_assignments(lda_ctx* h, const void* z, bool narrow, uint64_t seed, uint32_t sweep)
 {
     if (!h) return LDA_EINVAL;
@@ -1102,10 +1112,11 @@ static int set_assignments(lda_ctx* h, const void* z, bool narrow, uint64_t seed
     // chunk by chunk on the copy stream, each chunk spread into the block-major order (on the context's
     // stream) while the next one is on its way
     const size_t zt = narrow ? 2 : 4;
+    const int64_t chunk = transfer_chunk(c);
     cudaEventRecord(c.ev_chunk, c.stream);
     cudaStreamWaitEvent(c.copy, c.ev_chunk, 0);  // the staging buffer's earlier users are done
-    for (int64_t first = 0; first < c.N; first += c.copy_chunk) {
-        const int64_t count = std::min<int64_t>(c.copy_chunk, c.N - first);
+    for (int64_t first = 0; first < c.N; first += chunk) {
+        const int64_t count = std::min<int64_t>(chunk, c.N - first);
         if (cudaMemcpyAsync(zdev + (size_t)first * zt, reinterpret_cast<const char*>(z) + (size_t)first * zt,
                             (size_t)count * zt, cudaMemcpyHostToDevice, c.copy) != cudaSuccess)
             return cuda_fail(&c, "copying assignments");
@@ -1367,6 +1378,7 @@ static int get_assignments(lda_ctx* h, void* z_out, bool narrow, bool wait)
     // chunk by chunk: collected into document order on the context's stream, copied out on the copy
     // stream while the next chunk is collected
     const size_t zt = narrow ? 2 : 4;
+    const int64_t chunk = transfer_chunk(c);
     if ((size_t)c.N * zt <= EXPORT_ONE_STREAM_BYTES) {
         // a copy of a few microseconds is not worth the events that would order a second stream
         launch_export_chunk(c, zdev, narrow, 0, c.N);
@@ -1374,8 +1386,8 @@ static int get_assignments(lda_ctx* h, void* z_out, bool narrow, bool wait)
             return cuda_fail(&c, "copying assignments");
         return wait ? wait_all(c) : LDA_OK;
     }
-    for (int64_t first = 0; first < c.N; first += c.copy_chunk) {
-        const int64_t count = std::min<int64_t>(c.copy_chunk, c.N - first);
+    for (int64_t first = 0; first < c.N; first += chunk) {
+        const int64_t count = std::min<int64_t>(chunk, c.N - first);
         launch_export_chunk(c, zdev, narrow, first, count);
         cudaEventRecord(c.ev_chunk, c.stream);
         cudaStreamWaitEvent(c.copy, c.ev_chunk, 0);

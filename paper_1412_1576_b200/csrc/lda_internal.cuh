@@ -298,7 +298,7 @@ struct Ctx {
     // of one chunk runs beside the kernel that spreads (or collects) its neighbour.  ev_chunk orders a
     // chunk's two halves; ev_export completes when the last chunk of an export has reached the host:
     // whatever touches the staging buffer next waits for it on the device (order_after_export()).
-    int64_t copy_chunk = 1 << 25;  // tokens per chunk (option "copy_chunk_log2")
+    int64_t copy_chunk = 0;  // tokens per chunk (option "copy_chunk_log2"; 0: by the size of the corpus)
     cudaStream_t copy = nullptr;
     cudaEvent_t ev_chunk = nullptr, ev_export = nullptr;
     bool export_pending = false;
@@ -378,7 +378,7 @@ void rebuild_counts(Ctx& c);     // n_kw and n_k from the assignments, outside a
 inline void exchange_nk(Ctx& c) { int32_t* t = c.v.nk; c.v.nk = c.v.nk_next; c.v.nk_next = t; }
 int launch_alias_dense(Ctx& c, bool in_sweep);  // in_sweep: as the first kernel of a sweep, see there
 void launch_mix_thresholds(Ctx& c, uint32_t* mix32);  // of the tables last built
-int launch_alias_sparse(Ctx& c, bool all);  // the running slice's tables (all: in every form, for lda_get_tables)
+int launch_alias_sparse(Ctx& c, bool all, bool begin_sweep = false);  // the running slice's tables (all: in every form, for lda_get_tables)
 void set_slice(Ctx& c, int slice);          // makes `slice` the running one (moves the table pointers)
 int launch_sample(Ctx& c, int mh_steps);   // all passes of the MH step; needs ensure_exchange()
 int launch_doc_side(Ctx& c, int mh_steps);  // pass 2 of the MH step
