@@ -12,39 +12,46 @@
 namespace lda {
 
 constexpr int LL_BLOCKS = LL_WORD_PARTIALS;
-// Counts below this take lgamma(count + prior) - lgamma(prior) from a table in shared memory that
-// every CTA fills with the same expression: same values as calling lgamma() per entry.
+// Counts below this take lgamma(count + prior) - lgamma(prior) from a table filled with the same expression: same
+// values as calling lgamma() per entry.
 constexpr int LL_TABLE = 512;
 
-__device__ __forceinline__ void fill_ll_table(double* tab, double prior, double lg_prior)
-{
-    for (int c = threadIdx.x; c < LL_TABLE; c += blockDim.x) tab[c] = lgamma((double)c + prior) - lg_prior;
-    __syncthreads();
-}
-
-__global__ void __launch_bounds__(256) k_ll_word(View v, double lg_beta, int32_t per_warp, double* __restrict__ out)
+// Word part.  A warp takes up to 32 consecutive words, its lanes their sizes at once (rows of a few entries, most of
+// them, would otherwise cost a chain of reads each); rows of more than LL_ROW entries are left and taken in
+// pieces of LL_ROW by all warps: `longer` lists the words that can have one.
+constexpr int LL_ROW = ALIAS_MID_MAX;
+__global__ void __launch_bounds__(256) k_ll_word(View v, double lg_beta, int32_t per_warp, const int32_t* __restrict__ longer,
+                                                 int32_t n_longer, const double* __restrict__ tab, double* __restrict__ out)
 {
     __shared__ double tmp[32];
     __shared__ double small[LL_TABLE];
-    fill_ll_table(small, v.beta, lg_beta);
-    // a warp takes up to 32 consecutive words, its lanes their sizes at once; rows of a few entries (most) would
-    // otherwise cost a chain of reads each
+    for (int c = threadIdx.x; c < LL_TABLE; c += blockDim.x) small[c] = tab[c];
+    __syncthreads();
     const int warps = (gridDim.x * blockDim.x) >> 5, lane = threadIdx.x & 31;
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     double s = 0.0;
-    for (int32_t wb = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per_warp; wb < v.V; wb += warps * per_warp) {
+    auto add = [&](int32_t at) {
+        const uint32_t c = v.wk_count[at];
+        s += c < (uint32_t)LL_TABLE ? small[c] : lgamma((double)c + v.beta) - lg_beta;
+    };
+    for (int32_t wb = warp * per_warp; wb < v.V; wb += warps * per_warp) {
         int32_t n_mine = 0, r_mine = 0;
         if (lane < per_warp && wb + lane < v.V) {
             n_mine = v.wk_nnz[wb + lane];
             r_mine = v.row_start[wb + lane];
         }
-        for (uint32_t some = __ballot_sync(0xFFFFFFFFu, n_mine > 0); some; some &= some - 1) {
+        for (uint32_t some = __ballot_sync(0xFFFFFFFFu, n_mine > 0 && n_mine <= LL_ROW); some; some &= some - 1) {
             const int src = __ffs((int)some) - 1;
             const int32_t n = __shfl_sync(0xFFFFFFFFu, n_mine, src), r0 = __shfl_sync(0xFFFFFFFFu, r_mine, src);
-            for (int32_t j = lane; j < n; j += 32) {
-                const uint32_t c = v.wk_count[r0 + j];
-                s += c < (uint32_t)LL_TABLE ? small[c] : lgamma((double)c + v.beta) - lg_beta;
-            }
+            for (int32_t j = lane; j < n; j += 32) add(r0 + j);
         }
+    }
+    const int32_t pieces = (v.K + LL_ROW - 1) / LL_ROW;
+    for (int64_t i = warp; i < (int64_t)n_longer * pieces; i += warps) {
+        const int32_t w = longer[i / pieces], n = v.wk_nnz[w], j0 = (int32_t)(i % pieces) * LL_ROW;
+        if (n <= LL_ROW || j0 >= n) continue;
+        const int32_t r0 = v.row_start[w], j1 = min(n, j0 + LL_ROW);
+        for (int32_t j = j0 + lane; j < j1; j += 32) add(r0 + j);
     }
     for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < v.K; k += gridDim.x * blockDim.x)
         s -= lgamma((double)v.nk[k] + v.Vbeta);
@@ -62,14 +69,14 @@ __global__ void k_sum_nnz(const int32_t* __restrict__ a, int64_t n, unsigned lon
     if (threadIdx.x == 0 && s) atomicAdd(out, s);
 }
 
-// Tables of the document part in device memory, filled once per corpus: [0, LL_TABLE) holds
-// lgamma(c + alpha) - lgamma(alpha), [LL_TABLE, 2 LL_TABLE) holds lgamma(n + K alpha).
-__global__ void k_ll_fill_tables(View v, double lg_alpha, double* __restrict__ tab)
+// Tables in device memory, filled once per corpus: [0, LL_TABLE) holds lgamma(c + alpha) - lgamma(alpha),
+// [LL_TABLE, 2 LL_TABLE) lgamma(n + K alpha), [2 LL_TABLE, 3 LL_TABLE) lgamma(c + beta) - lgamma(beta).
+__global__ void k_ll_fill_tables(View v, double lg_alpha, double lg_beta, double* __restrict__ tab)
 {
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < LL_TABLE; c += gridDim.x * blockDim.x) {
-        tab[c] = lgamma((double)c + v.alpha) - lg_alpha;
-        tab[LL_TABLE + c] = lgamma((double)c + v.Kalpha);
-    }
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, c = i % LL_TABLE;
+    if (i < LL_TABLE) tab[i] = lgamma((double)c + v.alpha) - lg_alpha;
+    else if (i < 2 * LL_TABLE) tab[i] = lgamma((double)c + v.Kalpha);
+    else if (i < 3 * LL_TABLE) tab[i] = lgamma((double)c + v.beta) - lg_beta;
 }
 
 // lgamma() for the rare count beyond the tables, kept out of line so that the kernel below fits the
@@ -175,11 +182,13 @@ __global__ void __launch_bounds__(256) k_ll_sum_tiles(const double* __restrict__
 
 // Documents longer than a tile, from their tables in device memory (launch_long_tables()): CTAs take them in turns.
 __global__ void __launch_bounds__(512)
-k_ll_doc_long(View v, int32_t n_long, double lg_alpha, double* __restrict__ out, uint32_t* __restrict__ nnz_out)
+k_ll_doc_long(View v, int32_t n_long, double lg_alpha, const double* __restrict__ tab_lg, double* __restrict__ out,
+              uint32_t* __restrict__ nnz_out)
 {
     __shared__ double tmp[32];
     __shared__ double small[LL_TABLE];
-    fill_ll_table(small, v.alpha, lg_alpha);
+    for (int c = threadIdx.x; c < LL_TABLE; c += blockDim.x) small[c] = tab_lg[c];
+    __syncthreads();
     const uint32_t cmask = (1u << v.count_bits) - 1u;
     double s = 0.0;
     unsigned long long filled = 0;
@@ -269,23 +278,28 @@ static void queue_loglik(Ctx& c, bool word_part)
     const uint32_t* nnz_a = nnz;
     double* doc_b = part + LL_BLOCKS + LL_TILE_SUMS;
     uint32_t* nnz_b = nnz + LL_TILE_SUMS;
+    const double lg_beta = std::lgamma(c.beta);
+    if (!c.ll_tables_ready) {
+        k_ll_fill_tables<<<3 * LL_TABLE / 64, 64, 0, c.stream>>>(c.v, lg_alpha, lg_beta, c.ll_tab);
+        c.ll_tables_ready = true;
+    }
     fork_streams(c);
     if (word_part) {
         int per_warp = 32;
-        while (per_warp > 4 && c.V / per_warp < c.n_sm * 16) per_warp /= 2;
+        while (per_warp > 1 && c.V / per_warp < c.n_sm * 16) per_warp /= 2;
         n_word = (int)std::min<int64_t>(LL_BLOCKS, (c.V + 8 * (int64_t)per_warp - 1) / (8 * (int64_t)per_warp));
-        k_ll_word<<<n_word, 256, 0, c.side[0]>>>(c.v, std::lgamma(c.beta), per_warp, part);
+        // a warp per piece of a long row, a thread per topic
+        const int64_t pieces = (int64_t)c.n_alias_words[2] * ((c.K + LL_ROW - 1) / LL_ROW);
+        n_word = (int)std::min<int64_t>(LL_BLOCKS, std::max<int64_t>({(int64_t)n_word, (pieces + 7) / 8, ((int64_t)c.K + 255) / 256}));
+        k_ll_word<<<n_word, 256, 0, c.side[0]>>>(c.v, lg_beta, per_warp, c.alias_words[2], c.n_alias_words[2],
+                                                 c.ll_tab + 2 * LL_TABLE, part);
     }
     if (c.n_long_docs) {
         n_b = long_ll_grid(c);
         launch_long_tables(c, c.side[1], false, -1);
-        k_ll_doc_long<<<n_b, 512, 0, c.side[1]>>>(c.v, c.n_long_docs, lg_alpha, doc_b, nnz_b);
+        k_ll_doc_long<<<n_b, 512, 0, c.side[1]>>>(c.v, c.n_long_docs, lg_alpha, c.ll_tab, doc_b, nnz_b);
     }
     if (c.n_doc_tiles) {
-        if (!c.ll_tables_ready) {
-            k_ll_fill_tables<<<2, 256, 0, c.stream>>>(c.v, lg_alpha, c.ll_tab);
-            c.ll_tables_ready = true;
-        }
         launch_ll_tiles(c, doc_tile_smem_bytes(c.doc_tile), lg_alpha, c.stream);
         if (c.n_doc_tiles <= LL_TILE_DIRECT) {
             doc_a = c.ll_tile_part;
