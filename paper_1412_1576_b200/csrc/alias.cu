@@ -28,7 +28,7 @@ typedef unsigned long long ull;
 
 // The threads that build one row together: a warp, a CTA, or a cluster of CTAs.
 enum GroupKind { WARP, CTA, CLUSTER };
-constexpr int GROUP_SMEM = 99 + 6;  // 64-bit words of shared memory a CTA of a group needs (none for WARP)
+constexpr int GROUP_SMEM = 99 + 6 + 6;  // 64-bit words of shared memory a CTA of a group needs (none for WARP)
 
 template <GroupKind KIND>
 struct Group {
@@ -52,38 +52,48 @@ struct Group {
         else if (KIND == CTA) __syncthreads();
         else cooperative_groups::this_cluster().sync();  // orders global memory between the CTAs too
     }
-    // Sums of three values over the CTAs of the cluster (each thread holds its CTA's values), and over
-    // the CTAs of lower rank.  Through the CTAs' shared memory.
-    __device__ __forceinline__ void cluster_sums(const ull (&mine)[3], ull (&all)[3], ull (&lower)[3]) const
+    // Sums of three values over the CTAs of the cluster (each thread holds its CTA's values), and over the CTAs of
+    // lower rank: one warp reads the other CTAs' shared memory, a lane per CTA.  Two calls in a row use different
+    // slots (`turn` 0 and 1), so the barrier of the second says that everybody has read the first's.
+    __device__ __forceinline__ void cluster_sums(const ull (&mine)[3], ull (&all)[3], ull (&lower)[3], int turn) const
     {
-        ull* slot = smem + 99;
+        ull* slot = smem + 99 + 3 * turn;
+        ull* res = smem + 105;
         if (threadIdx.x == 0) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) slot[q] = mine[q];
         }
         cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
         cl.sync();
-#pragma unroll
-        for (int q = 0; q < 3; ++q) all[q] = lower[q] = 0;
-        for (unsigned r = 0; r < cl.num_blocks(); ++r) {
-            const ull* other = cl.map_shared_rank(slot, r);
+        if (threadIdx.x < 32) {
+            const unsigned r = threadIdx.x;
+            const ull* other = cl.map_shared_rank(slot, r < cl.num_blocks() ? r : 0u);
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-                const ull x = other[q];
-                all[q] += x;
-                if (r < cl.block_rank()) lower[q] += x;
+                const ull x = r < cl.num_blocks() ? other[q] : 0ull;
+                const ull sum = warp_reduce_sum<ull>(x), below = warp_reduce_sum<ull>(r < cl.block_rank() ? x : 0ull);
+                if (r == 0) {
+                    res[q] = sum;
+                    res[3 + q] = below;
+                }
             }
         }
-        cl.sync();  // the slots may be written again
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            all[q] = res[q];
+            lower[q] = res[3 + q];
+        }
+        __syncthreads();
     }
-    __device__ __forceinline__ ull reduce(ull v) const
+    __device__ __forceinline__ ull reduce(ull v, int turn) const
     {
         if (KIND == WARP) return warp_reduce_sum<ull>(v);
         const ull t = block_reduce_sum<ull>(v, smem);
         if (KIND == CTA) return t;
         const ull mine[3] = {t, 0, 0};
         ull all[3], lower[3];
-        cluster_sums(mine, all, lower);
+        cluster_sums(mine, all, lower, turn);
         return all[0];
     }
     // Exclusive scans of three values at once (one pass, one set of barriers); v[] in, prefixes
@@ -126,20 +136,26 @@ struct Group {
         if (KIND == CLUSTER) {
             const ull mine[3] = {tot[0], tot[1], tot[2]};
             ull lower[3];
-            cluster_sums(mine, tot, lower);
+            cluster_sums(mine, tot, lower, 0);  // after reduce() with 0 and 1
 #pragma unroll
             for (int q = 0; q < 3; ++q) v[q] += lower[q];
         }
     }
 };
 
+// What a kernel that finishes the bins needs to know of a row prepared by build_alias_row<.., false>.
+struct RowSums {
+    ull W, d_sum;
+    uint32_t L, H;
+};
+
 // Builds one table of n items.  weight(i) gives the fixed-point weight of item i.
 // sc_w, sc_de, sc_item: scratch of n entries each, private to this row.
 // out.bin(i, split point, alias item) receives every bin.
 // Returns W44 (the sum of the fixed-point weights) to every thread of the group.
-template <GroupKind KIND, class Weight, class Item, class Out>
+template <GroupKind KIND, bool FINISH = true, class Weight, class Item, class Out>
 __device__ ull build_alias_row(const Group<KIND>& g, int32_t n, Weight weight, ull* __restrict__ sc_w, ull* __restrict__ sc_de,
-                               Item* __restrict__ sc_item, const Out& out, int* err)
+                               Item* __restrict__ sc_item, const Out& out, int* err, RowSums* sums = nullptr)
 {
     const int r = g.rank(), gs = g.size();
     // Items are taken four (weights) or two (bins) at a time per thread, their loads issued side by
@@ -160,15 +176,18 @@ __device__ ull build_alias_row(const Group<KIND>& g, int32_t n, Weight weight, u
             s += wt[u];
         }
     }
-    const ull W44 = g.reduce(s);
+    const ull W44 = g.reduce(s, 0);
     int sh = bit_length(W44) + bit_length((ull)n) - 62;
     if (sh < 0) sh = 0;
     s = 0;
 #pragma unroll 4
     for (int32_t i = r; i < n; i += gs) s += sc_w[i] >> sh;
-    const ull W = g.reduce(s);
+    const ull W = g.reduce(s, 1);
     if (W == 0) {
-        if (r == 0) atomicOr(err, ERR_ALIAS);
+        if (r == 0) {
+            atomicOr(err, ERR_ALIAS);
+            if (!FINISH) *sums = RowSums{0, 0, 0, 0};
+        }
         return W44;
     }
     // Every thread takes a run of consecutive items (lights and heavies are numbered in ascending
@@ -208,6 +227,11 @@ __device__ ull build_alias_row(const Group<KIND>& g, int32_t n, Weight weight, u
     }
     const uint32_t L = (uint32_t)tot[0], H = (uint32_t)(tot[0] >> 32);
     const ull d_sum = tot[1];
+    if (!FINISH) {  // the bins are another kernel's work
+        if (r == 0) *sums = RowSums{W, d_sum, L, H};
+        g.sync();  // no CTA of a cluster leaves while another may read its shared memory
+        return W44;
+    }
     g.sync();
     const Frac32 frac(W);
     // The searches below count the entries of a sorted prefix array under a bound, one bit of the
@@ -321,39 +345,96 @@ struct DenseOut {
     }
 };
 
-// First kernel of a sweep: the dense smoothing table.  Also moves the device's sweep counter on and
-// clears the n_k buffer the sweep's rebuild will add into (nothing else of this sweep touches either).
-// One CTA builds a table of up to DENSE_CTA_MAX_K topics; a larger one takes a cluster of DENSE_CLUSTER
-// CTAs, whose passes over the table meet at cluster barriers: what bounds the kernel is the
-// latency of a few dependent passes over K items, so threads, not bytes, are what it is short of.
-constexpr int DENSE_CTA_MAX_K = 2048;
-constexpr int DENSE_CLUSTER = 8;
-template <GroupKind KIND>
-__global__ void __launch_bounds__(1024) k_alias_dense(View v, ull* sc)
+// What the first kernel of a sweep does besides its own work: the device's sweep counter moves on, the n_k
+// buffer the sweep's rebuild will add into is cleared (nothing beside it reads either).
+__device__ __forceinline__ void begin_sweep(const View& v, int rank, int size)
 {
-    __shared__ ull smem[GROUP_SMEM];
-    Group<KIND> g{smem};
-    const int32_t K = v.K;
-    if (v.state && g.rank() == 0) {
+    if (v.state && rank == 0) {
         SweepState& st = *v.state;
         const uint32_t slot = st.next_slot;
         st.sweep = st.next;
         st.next += 1;
         st.slot = slot;
         st.next_slot = slot + 1;
-        st.stamps[slot][STAMP_DENSE] = global_timer();
+        st.stamps[slot][STAMP_DENSE] = st.stamps[slot][STAMP_DENSE_END] = global_timer();
     }
     if (v.nk_next)
-        for (int32_t k = g.rank(); k < v.dense_stride; k += g.size()) v.nk_next[k] = 0;
+        for (int32_t k = rank; k < v.dense_stride; k += size) v.nk_next[k] = 0;
+}
+
+// Doc-proposal chains draw from no word's table: their sweeps begin with this and build none.
+__global__ void __launch_bounds__(1024) k_begin_sweep(View v) { begin_sweep(v, (int)threadIdx.x, (int)blockDim.x); }
+
+int launch_begin_sweep(Ctx& c)
+{
+    k_begin_sweep<<<1, 1024, 0, c.stream>>>(c.v);
+    return 1;
+}
+
+// The dense smoothing table; first kernel of a sweep (unless v.state is null).
+// One CTA builds a table of up to DENSE_CTA_MAX_K topics; a larger one takes a cluster of DENSE_CLUSTER
+// CTAs, whose passes over the table meet at cluster barriers: what bounds the kernel is the
+// latency of a few dependent passes over K items, so threads, not bytes, are what it is short of.
+// The searches of a large table are scattered reads of device memory, too many for eight multiprocessors: its
+// bins are finished by a second kernel, a thread per bin.
+constexpr int DENSE_CTA_MAX_K = 2048;
+constexpr int DENSE_CLUSTER = 8;
+// behind the scratch arrays of K items (20 bytes each)
+__device__ __forceinline__ RowSums* dense_sums(ull* sc, int32_t K)
+{
+    return reinterpret_cast<RowSums*>(sc + 2 * (size_t)K + (K + 1) / 2);
+}
+template <GroupKind KIND>
+__global__ void __launch_bounds__(1024) k_alias_dense(View v, ull* sc)
+{
+    __shared__ ull smem[GROUP_SMEM];
+    Group<KIND> g{smem};
+    const int32_t K = v.K;
+    begin_sweep(v, g.rank(), g.size());
     DenseWeight wf{v.nk, v.beta, v.Vbeta};
-    const ull B = build_alias_row<KIND>(g, K, wf, sc, sc + K, (uint32_t*)(sc + 2 * (size_t)K),
-                                        DenseOut{v.dn_thr, v.dn_idx, v.dn_pk}, v.err);
+    const ull B = build_alias_row<KIND, KIND == CTA>(g, K, wf, sc, sc + K, (uint32_t*)(sc + 2 * (size_t)K),
+                                                     DenseOut{v.dn_thr, v.dn_idx, v.dn_pk}, v.err, dense_sums(sc, K));
     if (g.rank() == 0) {
         *v.dense_mass = B;
         if (v.state) v.state->stamps[v.state->slot][STAMP_DENSE_END] = global_timer();
     }
 }
 
+__global__ void __launch_bounds__(256) k_alias_dense_bins(View v, ull* sc)
+{
+    const uint32_t K = (uint32_t)v.K, i = blockIdx.x * blockDim.x + threadIdx.x;
+    const RowSums t = *dense_sums(sc, v.K);
+    const ull *w = sc, *de = sc + K;
+    const uint32_t* item = (const uint32_t*)(sc + 2 * (size_t)K);
+    if (i >= K || t.W == 0) return;
+    const DenseOut out{v.dn_thr, v.dn_idx, v.dn_pk};
+    const Frac32 frac(t.W);
+    uint32_t pos = 0;
+    if (i < t.L) {
+        const uint32_t k = item[i];
+        const ull a = w[k], D = de[i];
+        for (uint32_t step = t.H ? 1u << (31 - __clz((int)t.H)) : 0u; step; step >>= 1)
+            if (pos + step <= t.H && de[K - pos - step] <= D) pos += step;
+        uint32_t al = k;
+        if (a != t.W) {
+            if (pos < t.H) al = item[K - 1 - pos]; else atomicOr(v.err, ERR_ALIAS);
+        }
+        out.bin(k, frac(a), al);
+    } else {
+        const uint32_t m = i - t.L, k = item[K - 1 - m];
+        const ull E = de[K - 1 - m];
+        for (uint32_t step = t.L ? 1u << (31 - __clz((int)t.L)) : 0u; step; step >>= 1)
+            if (pos + step <= t.L && de[pos + step - 1] < E) pos += step;
+        const ull part = t.W + E - (pos < t.L ? de[pos] : t.d_sum);
+        uint32_t al = k;
+        if (part != t.W) {
+            if (m + 1 < t.H) al = item[K - 2 - m]; else atomicOr(v.err, ERR_ALIAS);
+        }
+        out.bin(k, frac(part), al);
+    }
+}
+
+static int dense_launches(int32_t K) { return K > DENSE_CTA_MAX_K ? 2 : 1; }
 static cudaError_t run_alias_dense(const View& v, ull* scratch, cudaStream_t stream)
 {
     cudaLaunchConfig_t cfg = {};
@@ -370,7 +451,10 @@ static cudaError_t run_alias_dense(const View& v, ull* scratch, cudaStream_t str
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_alias_dense<CLUSTER>, v, scratch);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_alias_dense<CLUSTER>, v, scratch);
+    if (e != cudaSuccess) return e;
+    k_alias_dense_bins<<<(unsigned)((v.K + 255) / 256), 256, 0, stream>>>(v, scratch);
+    return cudaGetLastError();
 }
 
 // Mixture thresholds as lda_get_tables() reports them (the proposal pass works its tiles' out itself).
@@ -614,7 +698,7 @@ int launch_alias_dense(Ctx& c, bool in_sweep)
         v.nk_next = nullptr;
     }
     run_alias_dense(v, c.sc_dense, c.stream);
-    return 1;
+    return dense_launches(c.K);
 }
 
 // The kernels build the tables of different words: they run side by side, the ones with the longest rows
@@ -627,7 +711,7 @@ int launch_alias_sparse(Ctx& c, bool all, bool begin_sweep)
     fork_streams(c);
     if (begin_sweep) {
         run_alias_dense(c.v, c.sc_dense, c.side[0]);
-        ++launches;
+        launches += dense_launches(c.K);
     }
     const auto words = [&](int cls) { return c.alias_words[cls] + q.alias_lo[cls]; };
     if (q.alias_n[3]) {
@@ -639,12 +723,19 @@ int launch_alias_sparse(Ctx& c, bool all, bool begin_sweep)
             <<<q.alias_n[2], 1024, ALIAS_BIG_MAX * ALIAS_SCRATCH_PER_ITEM, c.stream>>>(c.v, words(2), all);
         ++launches;
     }
-    if (q.alias_n[1]) {
+    // a warp takes a row of 257..512 items at the least cost, a CTA in the least time: a CTA if all have room at once
+    const bool few = q.alias_n[0] <= 4 * c.n_sm;
+    if (few && q.alias_n[0]) {
+        k_alias_sparse_cta<256, ALIAS_WARP_MAX, ALIAS_MID_MAX>
+            <<<q.alias_n[0], 256, ALIAS_MID_MAX * ALIAS_SCRATCH_PER_ITEM, c.side[0]>>>(c.v, words(0), all);
+        ++launches;
+    }
+    if (!few && q.alias_n[1]) {
         k_alias_sparse_cta<256, ALIAS_LONG_WARP_MAX, ALIAS_MID_MAX>
             <<<q.alias_n[1], 256, ALIAS_MID_MAX * ALIAS_SCRATCH_PER_ITEM, c.side[0]>>>(c.v, words(1), all);
         ++launches;
     }
-    if (q.alias_n[0]) {
+    if (!few) {
         k_alias_sparse_long_warp<<<(q.alias_n[0] + 3) / 4, 128, 0, c.side[0]>>>(c.v, words(0), q.alias_n[0], all, c.sc_w);
         ++launches;
     }
@@ -654,7 +745,7 @@ int launch_alias_sparse(Ctx& c, bool all, bool begin_sweep)
     }
     // words per warp: as many as fill a warp's lanes with the words' sizes, as long as every multiprocessor gets two CTAs
     int per_warp = 32;
-    while (per_warp > 4 && (int64_t)(q.w_hi - q.w_lo) / per_warp < (int64_t)c.n_sm * 16) per_warp /= 2;
+    while (per_warp > 1 && (int64_t)(q.w_hi - q.w_lo) / per_warp < (int64_t)c.n_sm * 16) per_warp /= 2;
     const int64_t warps = ((int64_t)(q.w_hi - q.w_lo) + per_warp - 1) / per_warp;
     constexpr int WARPS = ALIAS_WARP_THREADS / 32;
     k_alias_sparse_warp<<<(int)std::min<int64_t>((warps + WARPS - 1) / WARPS, (int64_t)c.n_sm * 16), ALIAS_WARP_THREADS,
@@ -668,6 +759,8 @@ void set_alias_smem_limits()
 {
     cudaFuncSetAttribute(k_alias_sparse_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, ALIAS_WARP_SMEM);
     cudaFuncSetAttribute(k_alias_sparse_cta<256, ALIAS_LONG_WARP_MAX, ALIAS_MID_MAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         ALIAS_MID_MAX * ALIAS_SCRATCH_PER_ITEM);
+    cudaFuncSetAttribute(k_alias_sparse_cta<256, ALIAS_WARP_MAX, ALIAS_MID_MAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          ALIAS_MID_MAX * ALIAS_SCRATCH_PER_ITEM);
     cudaFuncSetAttribute(k_alias_sparse_cta<1024, ALIAS_MID_MAX, ALIAS_BIG_MAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          ALIAS_BIG_MAX * ALIAS_SCRATCH_PER_ITEM);
@@ -690,7 +783,7 @@ namespace lda {
 
 constexpr int NOALLOC_MAX_K = LDA_NOALLOC_MAX_K;
 // per topic: one 64-bit mass, one 64-bit prefix sum, one 32-bit item index = 20 bytes
-constexpr size_t NOALLOC_SCRATCH_WORDS = 2 * (size_t)NOALLOC_MAX_K + (size_t)NOALLOC_MAX_K / 2;
+constexpr size_t NOALLOC_SCRATCH_WORDS = 2 * (size_t)NOALLOC_MAX_K + (size_t)NOALLOC_MAX_K / 2 + 4;  // + RowSums
 
 static __device__ __align__(256) unsigned long long g_noalloc_scratch[NOALLOC_SCRATCH_WORDS];
 static __device__ __align__(256) int g_noalloc_status[4];

@@ -361,8 +361,13 @@ void rebuild_counts(Ctx& c)
 // One sweep, kernel by kernel.  Returns the number of kernels.
 static int queue_sweep(Ctx& c, int mh_steps)
 {
-    // several vocabulary slices: the sparse tables are built slice by slice inside pass 1
-    int n = c.slices.size() == 1 ? launch_alias_sparse(c, false, true) : launch_alias_dense(c, true);
+    // several vocabulary slices: the sparse tables are built slice by slice inside pass 1.  The dense table beside
+    // the sparse ones where its 5 to 80 us count (its cluster may have to wait for room among their CTAs).
+    int n = 0;
+    if (c.proposals == LDA_PROPOSALS_DOC) n += launch_begin_sweep(c);  // no word-proposal, no tables
+    else if (c.slices.size() > 1) n += launch_alias_dense(c, true);
+    else if (c.N <= SIDE_BY_SIDE_MAX_TOKENS) n += launch_alias_sparse(c, false, true);
+    else n += launch_alias_dense(c, true) + launch_alias_sparse(c, false);
     n += launch_sample(c, mh_steps);
     n += launch_count_wk(c);
     n += launch_count_k(c);
@@ -666,7 +671,9 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     int32_t k_pow2 = 1;  // a row of K counters: staged by the accept pass, added up by the histograms
     while (k_pow2 < K) k_pow2 *= 2;
     const int32_t hist_run = run_for(t_dense, 8, HIST_RUN_MAX, std::min(std::max(4 * k_pow2, 4096), HIST_RUN_MAX));
-    const int32_t hot_tile = run_for(t_hot, 4, HOT_TILE_MAX, std::min(std::max(k_pow2, 2048), 8192));
+    // a staged row of K counters (and n_k) is worth a quarter of K tokens or more; rows that are not staged
+    // (K > HOT_STAGE_MAX_K: left in device memory, or sorted and no longer than the word's token count) less
+    const int32_t hot_tile = run_for(t_hot, 4, HOT_TILE_MAX, warm_class ? 1024 : std::min(std::max(k_pow2 / 4, 2048), 8192));
     int32_t propose_tile = run_for(t_hot, 4, HOT_TILE_PROPOSE_MAX, 2048);
     if (propose_tile == 2048) propose_tile = 1536;  // one turn of the two-step kernel
     const int32_t cold_tile = run_for(t_cold, 4, COLD_TILE, 256);
@@ -763,7 +770,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.n_word_tiles = (int32_t)(word_tiles.size() / 2);
     c.n_doc_tiles = (int32_t)(doc_tiles.size() / 2);
     c.n_hot_runs = (int32_t)(hot_runs.size() / 4);
-    c.nk_with_rows = K <= NK_WITH_ROWS_MAX_K && c.n_hot_runs + c.n_word_tiles <= NK_WITH_ROWS_MAX_CTAS;
+    choose_nk_mode(c);
     c.n_long_docs = (int32_t)long_docs.size();
     for (int i = 0; i < ALIAS_CLASSES; ++i) c.n_alias_words[i] = (int32_t)alias_words[i].size();
     c.n_hot_tiles = (int32_t)(hot_tiles.size() / 3);
@@ -871,7 +878,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.red = (double*)A(sizeof(double) * (LL_WORD_PARTIALS + LL_DOC_PARTIALS));
     c.red_nnz = (uint32_t*)A(4 * LL_DOC_PARTIALS);
     c.red_i = (int64_t*)A(16);
-    c.ll_tab = (double*)A(sizeof(double) * 2 * 512);
+    c.ll_tab = (double*)A(sizeof(double) * 3 * 512);
     c.ll_tile_part = (double*)A(sizeof(double) * std::max<size_t>((size_t)c.n_doc_tiles, 1));
     c.ll_tile_nnz = (uint32_t*)A(4 * std::max<size_t>((size_t)c.n_doc_tiles, 1));
     c.ll_tables_ready = false;

@@ -27,11 +27,13 @@ struct EmitWord {
     uint32_t* topic;
     uint32_t* count;
     int32_t* nnz;
+    int32_t* nk;  // null: n_k is not added up here
     __device__ __forceinline__ void entry(int32_t seg, int32_t rank, uint32_t k, uint32_t n) const
     {
         const int32_t slot = row_start[seg] + rank;
         topic[slot] = k;
         count[slot] = n;
+        if (nk) atomicAdd(&nk[k], (int32_t)n);
     }
     __device__ __forceinline__ void rows(int32_t seg, int32_t n) const { nnz[seg] = n; }
 };
@@ -129,7 +131,8 @@ k_seg_count_sorted(const int32_t* __restrict__ tiles, const int32_t* __restrict_
 
 // Tail words (K <= WORD_ROWS_BITMAP_MAX_K): one CTA per tile of whole words [s0, s1) holding at most
 // SORT_TILE tokens and ROW_TILE_WORDS words.  The tile's topics are read once, into shared memory; words of
-// up to ROW_WARP_TOKENS are then handed to the CTA's warps one at a time, without a barrier between them:
+// up to ROW_WARP_TOKENS are then handed to the CTA's warps a few at a time, without a barrier between them:
+//   - up to 2 tokens (in a large vocabulary most words): a lane's work;
 //   - up to 32 tokens: a lane holds a token, lanes with the same topic find each other, the lowest of
 //     them writes the entry at the rank of its topic among the word's distinct topics;
 //   - longer: counted in a hash table of the warp's own (load <= 1/2); the token that claims a topic's
@@ -138,12 +141,16 @@ k_seg_count_sorted(const int32_t* __restrict__ tiles, const int32_t* __restrict_
 // Words longer than that take the whole CTA, one after the other, in the same way.
 // What bounds it is latency (a word is a chain of a dozen dependent shared-memory steps): hence many words in
 // flight per multiprocessor, little shared memory per CTA, and no CTA-wide steps for short words.
-// NK: the tile's column sums go to n_k too, through bins in shared memory.
+// NK: the tile's column sums go to n_k too (NkMode).
 constexpr int ROW_WARP_TOKENS = 128;
 constexpr int ROW_WARP_SLOTS = 2 * ROW_WARP_TOKENS;
 constexpr int ROW_CTA_SLOTS = 2 * SORT_TILE;
 constexpr int ROW_COUNT_BITS = 12;  // of a table entry: a tail word has at most SORT_TILE = 2048 tokens
 static_assert(SORT_TILE < (1 << ROW_COUNT_BITS), "count bits");
+
+// How the kernels that write rows add up n_k: not at all (a pass over the rows follows), through bins in shared
+// memory with one global add per bin and CTA, or with one global add per row entry.  Which: choose_nk_mode().
+enum NkMode { NK_NONE, NK_BINS, NK_DIRECT };
 
 struct RowTables {
     const int32_t* row_start;
@@ -182,7 +189,7 @@ __device__ __forceinline__ uint32_t row_count(uint32_t* table, int log2_slots, u
     return 0xFFFFFFFFu;
 }
 
-template <typename T, bool NK>
+template <typename T, NkMode NK>
 __global__ void __launch_bounds__(256, 6)
 k_word_rows(const int32_t* __restrict__ tiles, const int32_t* __restrict__ word_off, const T* __restrict__ z,
             RowTables out, int32_t K, int32_t area_words, int stamp_id)
@@ -209,13 +216,14 @@ k_word_rows(const int32_t* __restrict__ tiles, const int32_t* __restrict__ word_
         if ((uint32_t)k >= (uint32_t)K) atomicOr(err, ERR_TOPIC_RANGE);
         zs[j] = (uint32_t)k < (uint32_t)K ? k : (T)0;
     }
-    if (NK)
+    if (NK == NK_BINS)
         for (int32_t k = tid; k < K; k += 256) bins[k] = 0;
     __syncthreads();
     auto emit = [&](int32_t at, uint32_t k, uint32_t n) {
         out.topic[at] = k;
         out.count[at] = n;
-        if (NK) atomicAdd(&bins[k], (int32_t)n);
+        if (NK == NK_BINS) atomicAdd(&bins[k], (int32_t)n);
+        if (NK == NK_DIRECT) atomicAdd(&out.nk[k], (int32_t)n);
     };
     const int32_t lane_words = row_bitmap_lane_words(K);
     const uint4 empty = make_uint4(DK_EMPTY, DK_EMPTY, DK_EMPTY, DK_EMPTY), zero = make_uint4(0u, 0u, 0u, 0u);
@@ -223,11 +231,31 @@ k_word_rows(const int32_t* __restrict__ tiles, const int32_t* __restrict__ word_
         uint32_t* table = row_area + warp * ROW_WARP_SLOTS;
         uint32_t* bitmap = row_area + 8 * ROW_WARP_SLOTS + warp * 32 * lane_words;
         uint16_t* before = reinterpret_cast<uint16_t*>(row_area + 8 * ROW_WARP_SLOTS + 8 * 32 * lane_words) + warp * 32 * lane_words;
+        const int32_t batch = min(32, max(1, nw >> 4));
+        int32_t wb = 0;
+        uint32_t todo = 0;  // words of the batch that are left for the whole warp
         for (;;) {
-            int32_t w = 0;
-            if (lane == 0) w = atomicAdd(&next_word, 1);
-            w = __shfl_sync(0xFFFFFFFFu, w, 0);
-            if (w >= nw) break;
+            if (!todo) {
+                if (lane == 0) wb = atomicAdd(&next_word, batch);
+                wb = __shfl_sync(0xFFFFFFFFu, wb, 0);
+                if (wb >= nw) break;
+                const int32_t w = wb + lane;
+                const bool mine = lane < batch && w < nw;
+                const int32_t first = mine ? soff[w] : 0, n = mine ? soff[w + 1] - first : 0;
+                if (mine && n <= 2) {
+                    const uint32_t a = n > 0 ? (uint32_t)zs[first] : 0u, b = n > 1 ? (uint32_t)zs[first + 1] : a;
+                    if (n > 0) {
+                        const int32_t out0 = __ldg(out.row_start + s0 + w);
+                        emit(out0, min(a, b), a == b ? (uint32_t)n : 1u);
+                        if (a != b) emit(out0 + 1, max(a, b), 1u);
+                    }
+                    out.nnz[s0 + w] = n == 0 ? 0 : a == b ? 1 : 2;
+                }
+                todo = __ballot_sync(0xFFFFFFFFu, n > 2);
+                continue;
+            }
+            const int32_t w = wb + __ffs((int)todo) - 1;
+            todo &= todo - 1u;
             const int32_t first = soff[w], n = soff[w + 1] - first;
             const int32_t out0 = __ldg(out.row_start + s0 + w);
             if (n <= 32) {
@@ -336,7 +364,7 @@ k_word_rows(const int32_t* __restrict__ tiles, const int32_t* __restrict__ word_
         if (tid == 0) out.nnz[s0 + w] = all;
         __syncthreads();
     }
-    if (NK) {
+    if (NK == NK_BINS) {
         __syncthreads();
         for (int32_t k = tid; k < K; k += 256) {
             const int32_t n = bins[k];
@@ -351,15 +379,16 @@ k_word_rows(const int32_t* __restrict__ tiles, const int32_t* __restrict__ word_
 // are the sorted row: every warp owns a run of consecutive bin pairs, counts its nonzero bins, the
 // warps' totals are scanned, and a second walk writes the entries.
 template <typename T>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(1024)
 k_warm_rows(const int32_t* __restrict__ words, const int32_t* __restrict__ word_off, const T* __restrict__ z,
             const int32_t* __restrict__ row_start, uint32_t* __restrict__ wk_topic, uint32_t* __restrict__ wk_count,
-            int32_t* __restrict__ wk_nnz, int32_t K, int32_t window, SweepState* state)
+            int32_t* __restrict__ wk_nnz, int32_t* __restrict__ nk, int32_t K, int32_t window, SweepState* state)
 {
+    // nk: null if n_k is not added up here
     stamp(state, STAMP_WARM_ROWS);
     int* const err = &state->err;
     extern __shared__ __align__(16) uint32_t bins2[];
-    __shared__ int32_t warp_total[17];
+    __shared__ int32_t warp_total[33];
     const int32_t w = words[blockIdx.x];
     const int32_t first = word_off[w], cnt = word_off[w + 1] - first;
     const int32_t out0 = row_start[w], cap = row_start[w + 1] - out0;
@@ -391,11 +420,11 @@ k_warm_rows(const int32_t* __restrict__ words, const int32_t* __restrict__ word_
         if (threadIdx.x == 0) {
             int32_t run = 0;
             for (int i = 0; i < nwarps; ++i) { const int32_t t = warp_total[i]; warp_total[i] = run; run += t; }
-            warp_total[16] = run;
+            warp_total[32] = run;
         }
         __syncthreads();
         int32_t at = done + warp_total[warp];
-        const int32_t total = warp_total[16];
+        const int32_t total = warp_total[32];
         if (done + total > cap) {
             if (threadIdx.x == 0) atomicOr(err, ERR_ROW_OVERFLOW);
         } else {
@@ -408,11 +437,13 @@ k_warm_rows(const int32_t* __restrict__ words, const int32_t* __restrict__ word_
                 if (lo) {
                     wk_topic[out0 + pos] = (uint32_t)(k0 + 2 * q);
                     wk_count[out0 + pos] = n2 & 0xFFFFu;
+                    if (nk) atomicAdd(&nk[k0 + 2 * q], (int32_t)(n2 & 0xFFFFu));
                     ++pos;
                 }
                 if (hi) {
                     wk_topic[out0 + pos] = (uint32_t)(k0 + 2 * q + 1);
                     wk_count[out0 + pos] = n2 >> 16;
+                    if (nk) atomicAdd(&nk[k0 + 2 * q + 1], (int32_t)(n2 >> 16));
                 }
                 at += __popc(m_lo) + __popc(m_hi);
             }
@@ -429,6 +460,8 @@ k_warm_rows(const int32_t* __restrict__ words, const int32_t* __restrict__ word_
 // n_k.  The runs of a longer word add their nonzero bins to the word's line of `acc`; the last of them to
 // finish takes the line's contents the same way and leaves it zero for the next rebuild.
 // How the tokens are cut: load_common() in api.cu.
+// windows of more topics leave room for one CTA per multiprocessor: it gets twice the threads
+constexpr int HIST_WIDE = 24576;
 struct HotRuns {
     const int4* runs;      // (word, first token, tokens, index of the word among those with several runs or -1)
     const int32_t* dense_slot;
@@ -441,7 +474,7 @@ struct HotRuns {
 
 // Bins [0, nb) of topics k0.. -> dense row and sorted entries from position `done` of the word's row on;
 // returns how many there were.  Every warp owns a run of bins: one walk to count, one to write.
-template <bool NK, class Bin>
+template <NkMode NK, class Bin>
 __device__ __forceinline__ int32_t emit_bins(const Bin& bin, int32_t k0, int32_t nb, int32_t* dense, int32_t out0,
                                              int32_t cap, int32_t done, const RowTables& out, int32_t* warp_total)
 {
@@ -466,7 +499,7 @@ __device__ __forceinline__ int32_t emit_bins(const Bin& bin, int32_t k0, int32_t
             const int32_t slot = out0 + at + __popc(some & ((1u << lane) - 1u));
             out.topic[slot] = (uint32_t)(k0 + q);
             out.count[slot] = (uint32_t)n;
-            if (NK) atomicAdd(&out.nk[k0 + q], n);
+            if (NK != NK_NONE) atomicAdd(&out.nk[k0 + q], n);
         }
         at += __popc(some);
     }
@@ -474,13 +507,13 @@ __device__ __forceinline__ int32_t emit_bins(const Bin& bin, int32_t k0, int32_t
     return total;
 }
 
-template <typename T, bool NK>
-__global__ void __launch_bounds__(512)
+template <typename T, NkMode NK>
+__global__ void __launch_bounds__(1024, 2)
 k_hot_rows(HotRuns h, const T* __restrict__ z, RowTables out, int32_t K, int32_t window)
 {
     stamp(out.state, STAMP_HIST);
     extern __shared__ __align__(16) int32_t hist_bins[];
-    __shared__ int32_t warp_total[16];
+    __shared__ int32_t warp_total[32];
     __shared__ bool last;
     int* const err = &out.state->err;
     const int4 run = h.runs[blockIdx.x];
@@ -659,7 +692,7 @@ void launch_doc_rows_spread(Ctx& c, const int32_t* tiles, int32_t n_tiles, const
 {
     const RowTables out{c.v.doc_off, topic, count, nnz, nullptr, c.v.state};
     const size_t area = row_area_bytes(c.K);
-    k_word_rows<T, false><<<n_tiles, 256, area, c.stream>>>(tiles, c.v.doc_off, z, out, c.K, (int32_t)(area / 4), -1);
+    k_word_rows<T, NK_NONE><<<n_tiles, 256, area, c.stream>>>(tiles, c.v.doc_off, z, out, c.K, (int32_t)(area / 4), -1);
 }
 template void launch_doc_rows_spread<uint16_t>(Ctx&, const int32_t*, int32_t, const uint16_t*, int32_t*, uint32_t*, uint32_t*);
 template void launch_doc_rows_spread<int32_t>(Ctx&, const int32_t*, int32_t, const int32_t*, int32_t*, uint32_t*, uint32_t*);
@@ -668,7 +701,7 @@ template void launch_doc_rows<int32_t>(Ctx&, const int32_t*, int32_t, const int3
 
 static int hist_window(const Ctx& c) { return c.K < HIST_BINS ? c.K : HIST_BINS; }
 
-template <typename T, bool NK>
+template <typename T, NkMode NK>
 static int count_wk_t(Ctx& c)
 {
     View& v = c.v;
@@ -681,16 +714,16 @@ static int count_wk_t(Ctx& c)
         const HotRuns h{reinterpret_cast<const int4*>(c.hot_runs), v.dense_slot, v.dense_rows, v.dense_stride, c.acc,
                         c.acc_done, c.acc_runs};
         const int win = c.K < HIST32_BINS ? c.K : HIST32_BINS;
-        k_hot_rows<T, NK><<<c.n_hot_runs, 512, (size_t)((win + 3) / 4) * 16, c.stream>>>(h, z, out, c.K, win);
+        k_hot_rows<T, NK><<<c.n_hot_runs, win > HIST_WIDE ? 1024 : 512, (size_t)((win + 3) / 4) * 16, c.stream>>>(h, z, out, c.K, win);
         ++launches;
     }
     if (c.n_word_tiles) {
         if (c.K <= WORD_ROWS_BITMAP_MAX_K) {
             const size_t area = row_area_bytes(c.K);
-            k_word_rows<T, NK><<<c.n_word_tiles, 256, area + (NK ? (size_t)c.K * 4 : 0), c.side[0]>>>(
+            k_word_rows<T, NK><<<c.n_word_tiles, 256, area + (NK == NK_BINS ? (size_t)c.K * 4 : 0), c.side[0]>>>(
                 c.word_tiles, v.word_off, z, out, c.K, (int32_t)(area / 4), STAMP_ROWS);
         } else {
-            EmitWord e{v.row_start, v.wk_topic, v.wk_count, v.wk_nnz};
+            EmitWord e{v.row_start, v.wk_topic, v.wk_count, v.wk_nnz, NK == NK_NONE ? nullptr : v.nk_next};
             k_seg_count_sorted<T, EmitWord><<<c.n_word_tiles, 256, 0, c.side[0]>>>(
                 c.word_tiles, v.word_off, z, v.topic_bits, c.K, e, v.state, STAMP_ROWS);
         }
@@ -698,8 +731,9 @@ static int count_wk_t(Ctx& c)
     }
     if (c.n_warm) {
         const int win = c.K < HIST16_BINS ? c.K : HIST16_BINS;
-        k_warm_rows<T><<<c.n_warm, 512, (size_t)((win + 7) / 8) * 16, c.side[1]>>>(
-            c.warm_words, v.word_off, z, v.row_start, v.wk_topic, v.wk_count, v.wk_nnz, c.K, win, v.state);
+        k_warm_rows<T><<<c.n_warm, 1024, (size_t)((win + 7) / 8) * 16, c.side[1]>>>(
+            c.warm_words, v.word_off, z, v.row_start, v.wk_topic, v.wk_count, v.wk_nnz, NK == NK_NONE ? nullptr : v.nk_next, c.K, win,
+            v.state);
         ++launches;
     }
     join_streams(c);
@@ -739,24 +773,39 @@ int launch_count_k_from_rows(Ctx& c)
 
 int launch_count_wk(Ctx& c)
 {
-    if (c.wide_topics) return count_wk_t<int32_t, false>(c);
-    return c.nk_with_rows ? count_wk_t<uint16_t, true>(c) : count_wk_t<uint16_t, false>(c);
+    if (c.wide_topics) return c.nk_mode == NK_NONE ? count_wk_t<int32_t, NK_NONE>(c) : count_wk_t<int32_t, NK_DIRECT>(c);
+    return c.nk_mode == NK_NONE   ? count_wk_t<uint16_t, NK_NONE>(c)
+           : c.nk_mode == NK_BINS ? count_wk_t<uint16_t, NK_BINS>(c)
+                                  : count_wk_t<uint16_t, NK_DIRECT>(c);
 }
-int launch_count_k(Ctx& c) { return c.nk_with_rows ? 0 : launch_count_k_from_rows(c); }
+int launch_count_k(Ctx& c) { return c.nk_mode != NK_NONE ? 0 : launch_count_k_from_rows(c); }
+
+// n_k by the row kernels or by a pass of its own.  Bins: every CTA adds to every topic's counter once, and the adds
+// to one counter queue, so K and the number of CTAs are bounded.  One add per entry: as many adds as nonzeros, fine
+// while they are few (9 M tokens, K = 16 695: 0.36 ms less per rebuild); with more, the pass over the rows (bins again,
+// fewer CTAs) is ahead.
+void choose_nk_mode(Ctx& c)
+{
+    if (c.K <= NK_WITH_ROWS_MAX_K && c.n_hot_runs + c.n_word_tiles <= NK_WITH_ROWS_MAX_CTAS && c.N >= c.K) c.nk_mode = NK_BINS;
+    else c.nk_mode = c.N <= NK_DIRECT_MAX_TOKENS ? NK_DIRECT : NK_NONE;
+}
 
 void set_hist_smem_limits()
 {
     cudaFuncSetAttribute(k_warm_rows<uint16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST16_BINS * 2 + 16);
     cudaFuncSetAttribute(k_warm_rows<int32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST16_BINS * 2 + 16);
-    cudaFuncSetAttribute(k_hot_rows<uint16_t, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST32_BINS * 4);
-    cudaFuncSetAttribute(k_hot_rows<uint16_t, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST32_BINS * 4);
-    cudaFuncSetAttribute(k_hot_rows<int32_t, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST32_BINS * 4);
-    cudaFuncSetAttribute(k_word_rows<uint16_t, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)row_area_bytes(WORD_ROWS_BITMAP_MAX_K));
-    cudaFuncSetAttribute(k_word_rows<int32_t, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)row_area_bytes(WORD_ROWS_BITMAP_MAX_K));
-    cudaFuncSetAttribute(k_word_rows<uint16_t, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)row_area_bytes(NK_WITH_ROWS_MAX_K) + NK_WITH_ROWS_MAX_K * 4);
+    const int hist = HIST32_BINS * 4, rows = (int)row_area_bytes(WORD_ROWS_BITMAP_MAX_K),
+              rows_bins = (int)row_area_bytes(NK_WITH_ROWS_MAX_K) + NK_WITH_ROWS_MAX_K * 4;
+    constexpr auto most = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaFuncSetAttribute(k_hot_rows<uint16_t, NK_NONE>, most, hist);
+    cudaFuncSetAttribute(k_hot_rows<uint16_t, NK_BINS>, most, hist);
+    cudaFuncSetAttribute(k_hot_rows<uint16_t, NK_DIRECT>, most, hist);
+    cudaFuncSetAttribute(k_hot_rows<int32_t, NK_NONE>, most, hist);
+    cudaFuncSetAttribute(k_hot_rows<int32_t, NK_DIRECT>, most, hist);
+    cudaFuncSetAttribute(k_word_rows<uint16_t, NK_NONE>, most, rows);
+    cudaFuncSetAttribute(k_word_rows<uint16_t, NK_DIRECT>, most, rows);
+    cudaFuncSetAttribute(k_word_rows<uint16_t, NK_BINS>, most, rows_bins);
+    cudaFuncSetAttribute(k_word_rows<int32_t, NK_NONE>, most, rows);
     cudaFuncSetAttribute(k_nk_from_sparse, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST_BINS * 4);
 }
 

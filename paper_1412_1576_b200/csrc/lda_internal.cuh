@@ -65,10 +65,10 @@ constexpr int HIST16_BINS = 106496;  // window of a warm word's n_kw histogram (
 constexpr int HIST32_BINS = 49152;   // window of a hot word's n_kw histogram (32-bit bins, 192 KB)
 constexpr int HIST_RUN_MAX = 262144;  // tokens per CTA (one run of a word) in the histogram path, at most
 constexpr int ROW_TILE_WORDS = 512;   // words per tile of the tail words' row kernel
-// n_k is added up by the row kernels themselves up to this K (bins in shared memory) ...
+// n_k added up by the row kernels themselves (choose_nk_mode())
 constexpr int NK_WITH_ROWS_MAX_K = 4096;
-// ... and this many CTAs: each adds to every topic's counter once, and the adds to one counter queue
 constexpr int NK_WITH_ROWS_MAX_CTAS = 16384;
+constexpr int64_t NK_DIRECT_MAX_TOKENS = 1 << 24;
 constexpr int HOT_TILE_MAX = 32768;  // accept pass: tokens of one hot word per CTA (the word's row is staged once per CTA), at most
 constexpr int HOT_TILE_PROPOSE_MAX = 8192;  // propose pass: nothing is staged, shorter runs balance better
 constexpr int COLD_TILE = 2048;      // MH kernel: tokens of a tile of tail words, at most
@@ -219,7 +219,7 @@ struct Ctx {
     int32_t* acc_done = nullptr;     // [...] runs of the word that are done, zero between rebuilds
     int32_t* acc_runs = nullptr;     // [...] runs of the word
     bool cold_direct = false;        // the accept pass keeps the tail tiles' rows as counters
-    bool nk_with_rows = false;       // the row kernels add up n_k too
+    int nk_mode = 0;                 // how the row kernels add up n_k
     int32_t n_long_chunks = 0;
     int32_t* long_chunks = nullptr;  // [n_long_chunks*4] (index into View::long_docs, first token, count, 0)
     int64_t long_slots = 0, long_hashed_slots = 0;  // of View::dk_slots: in all, of the hashed tables
@@ -262,7 +262,7 @@ struct Ctx {
     uint32_t* sc_item = nullptr;          // light items (front) / heavy items (back)
     unsigned long long* sc_dense = nullptr;  // same three for the dense table, [3*K]
     uint32_t* mix32 = nullptr;               // [V] mixture thresholds, for lda_get_tables()
-    double* ll_tab = nullptr;        // [2 * 512] lgamma tables of the log-likelihood's document part
+    double* ll_tab = nullptr;        // [3 * 512] lgamma tables of the log-likelihood
     double* ll_tile_part = nullptr;  // [n_doc_tiles] its partial sums, one per tile of documents
     uint32_t* ll_tile_nnz = nullptr; // [n_doc_tiles] filled table slots of the tile: its share of nnz(n_kd)
     bool ll_tables_ready = false;
@@ -375,7 +375,9 @@ int launch_count_k(Ctx& c);      // n_k of the rows just rebuilt, added to View:
                                  // row kernels have done it
 int launch_count_k_from_rows(Ctx& c);  // ... in any case
 void rebuild_counts(Ctx& c);     // n_kw and n_k from the assignments, outside a sweep
+void choose_nk_mode(Ctx& c);     // after the work lists are made
 inline void exchange_nk(Ctx& c) { int32_t* t = c.v.nk; c.v.nk = c.v.nk_next; c.v.nk_next = t; }
+int launch_begin_sweep(Ctx& c);  // first kernel of a sweep that needs no tables
 int launch_alias_dense(Ctx& c, bool in_sweep);  // in_sweep: as the first kernel of a sweep, see there
 void launch_mix_thresholds(Ctx& c, uint32_t* mix32);  // of the tables last built
 int launch_alias_sparse(Ctx& c, bool all, bool begin_sweep = false);  // the running slice's tables (all: in every form, for lda_get_tables)
