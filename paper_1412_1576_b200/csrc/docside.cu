@@ -119,50 +119,58 @@ __device__ __forceinline__ void doc_side_token(const View& v, const Table& table
     const size_t N = (size_t)v.N;
     uint32_t* out = v.dside + (size_t)bm * v.side_stride;
     const double n_d = u32_to_double(doc_len);
-    // words 0..3 (the whole record when the step count is fixed at compile time) are collected in
-    // registers and go out as 16-byte stores at the end, the rest one by one
+    // The record's words come in order (step_record_at()).  With the step count fixed at compile time they are all
+    // collected in registers; else four at a time, which then go out as one 16-byte store.
     constexpr int REGW = (FIXED > 0 && step_record_words<MODE>(FIXED) > 4) ? 8 : 4;
     static_assert(FIXED == 0 || step_record_words<MODE>(FIXED) <= 8, "the record is kept in eight registers");
     uint32_t wr[REGW];
 #pragma unroll
     for (int q = 0; q < REGW; ++q) wr[q] = 0u;
+    wr[0] = own;
     auto put = [&](int at, uint32_t val) {
         if (FIXED > 0) {
             wr[at] = val;  // the step loops are unrolled: `at` is a constant
         } else {
-            if (at == 1) wr[1] = val;
-            else if (at == 2) wr[2] = val;
-            else if (at == 3) wr[3] = val;
-            else __stcs(out + at, val);
+            const int q = at & 3;
+            wr[0] = q == 0 ? val : wr[0];
+            wr[1] = q == 1 ? val : wr[1];
+            wr[2] = q == 2 ? val : wr[2];
+            wr[3] = q == 3 ? val : wr[3];
+            if (q == 3) __stcs(reinterpret_cast<uint4*>(out + at - 3), make_uint4(wr[0], wr[1], wr[2], wr[3]));
         }
     };
     // word-proposal of step st, the wi-th of its kind: n_kd at the topic pass 1 drew
     auto word_step = [&](int32_t st, int32_t wi) {
         const uint32_t t1 = wi == 0 ? t_first : (uint32_t)__ldcg(prop + (size_t)wi * N + bm);
-        put(1 + st, table.of_topic(t1));
+        put(step_record_at<MODE>(st), table.of_topic(t1));
     };
-    // doc-proposal of step st, the di-th of its kind
-    auto doc_step = [&](int32_t st, int32_t di) {
+    // doc-proposal of step st
+    auto doc_step = [&](int32_t st) {
         const uint4 r = philox4x32_10(make_uint4(v.tok_base + tok, sweep, (uint32_t)st, 0u), key);
         const bool copy = __dmul_rn(__dmul_rn(u32_to_double(r.x), INV_2_32), __dadd_rn(n_d, v.Kalpha)) < n_d;
         const uint32_t o2 = table.drawn(copy, scale_to_range(r.y, copy ? doc_len : (uint32_t)v.K));
-        put(1 + st, o2);
-        put(1 + mh_steps + di, r.w);  // the step's acceptance uniform
+        put(step_record_at<MODE>(st), o2);
+        put(step_record_at<MODE>(st) + 1, r.w);  // the step's acceptance uniform
     };
     if (MODE == LDA_PROPOSALS_CYCLE) {
 #pragma unroll
         for (int32_t st = 0; st < mh_steps; st += 2) {
             word_step(st, st >> 1);
-            if (st + 1 < mh_steps) doc_step(st + 1, st >> 1);
+            if (st + 1 < mh_steps) doc_step(st + 1);
         }
     } else if (MODE == LDA_PROPOSALS_WORD) {
 #pragma unroll
         for (int32_t st = 0; st < mh_steps; ++st) word_step(st, st);
     } else {
 #pragma unroll
-        for (int32_t st = 0; st < mh_steps; ++st) doc_step(st, st);
+        for (int32_t st = 0; st < mh_steps; ++st) doc_step(st);
     }
-    __stcs(reinterpret_cast<uint4*>(out), make_uint4(own, wr[1], wr[2], wr[3]));
+    if (FIXED == 0) {
+        const int words = step_record_words<MODE>(mh_steps);
+        if (words & 3) __stcs(reinterpret_cast<uint4*>(out + (words & ~3)), make_uint4(wr[0], wr[1], wr[2], wr[3]));
+        return;
+    }
+    __stcs(reinterpret_cast<uint4*>(out), make_uint4(wr[0], wr[1], wr[2], wr[3]));
     if (REGW == 8) __stcs(reinterpret_cast<uint4*>(out) + 1, make_uint4(wr[4], wr[5], wr[6], wr[7]));
 }
 

@@ -23,12 +23,19 @@ __host__ __device__ constexpr int step_kind_index(int m)
     return MODE == LDA_PROPOSALS_CYCLE ? m >> 1 : m;
 }
 
-// Words of the record the document side leaves per token for a chain of m steps: the token's own
-// (topic, n_kd) word, one (topic, n_kd) word per step, one acceptance uniform per doc step.
+// The record the document side leaves per token, in the order it is made: the token's own (topic, n_kd) word, then per
+// step a (topic, n_kd) word and, behind a doc step's, its acceptance uniform.  Words of a chain of m steps:
 template <int MODE>
 __host__ __device__ constexpr int step_record_words(int m)
 {
     return 1 + m + (MODE == LDA_PROPOSALS_CYCLE ? m / 2 : MODE == LDA_PROPOSALS_DOC ? m : 0);
+}
+
+// Place of step m's (topic, n_kd) word in it.
+template <int MODE>
+__host__ __device__ constexpr int step_record_at(int m)
+{
+    return step_record_words<MODE>(m);
 }
 
 // Device error word bits (set by kernels, read by the host after a sweep).
@@ -143,7 +150,7 @@ struct View {
     // per-sweep exchange buffers between the word-order and the document-order passes
     void* prop;        // [word steps][N] block-major: topics proposed by the word-proposals after the first
     uint32_t* ua_w;    // [word steps][N] word order: acceptance uniforms of the word-proposal steps
-    uint32_t* dside;   // [N][side_stride] block-major: own record, per step (topic << count_bits) | n_kd,
+    uint32_t* dside;   // [N][side_stride] block-major: step_record_words(): own (topic << count_bits) | n_kd, per step the same,
                        // per doc step its acceptance uniform
     int32_t side_stride;  // words per token in dside, a multiple of 4
     // assignments (topic type: u16 or i32) after the last MH step or initialisation

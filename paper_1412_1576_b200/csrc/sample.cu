@@ -397,7 +397,7 @@ __device__ __forceinline__ void accept_tokens(const View& v, Tile& tile, const i
         const uint32_t* side = v.dside + (size_t)at * v.side_stride;
         auto side_word = [&](int32_t i) {
             if (TWO && i >= 4) return i == 4 ? rec2.x : i == 5 ? rec2.y : i == 6 ? rec2.z : rec2.w;
-            return i == 1 ? rec.y : i == 2 ? rec.z : i == 3 ? rec.w : __ldcs(side + i);
+            return i == 1 ? rec.y : i == 2 ? rec.z : i == 3 ? rec.w : __ldg(side + i);  // its sector's other words come next
         };
         const uint32_t own = rec.x;
         const typename Tile::Ref w = tile.ref(p - p_begin);
@@ -410,10 +410,11 @@ __device__ __forceinline__ void accept_tokens(const View& v, Tile& tile, const i
                 e[i] = 0;
                 ua[i] = 0;
                 if (m0 + i < mh_steps) {
-                    e[i] = side_word(1 + m0 + i);
+                    const int32_t at_word = step_record_at<MODE>(m0 + i);
+                    e[i] = side_word(at_word);
                     // acceptance uniform: word 3 of the step's Philox block, drawn by the pass that made
                     // the proposal (pass 1: word steps, pass 2: doc steps) and left for this one
-                    ua[i] = step_is_doc<MODE>(i) ? side_word(1 + mh_steps + step_kind_index<MODE>(m0 + i))
+                    ua[i] = step_is_doc<MODE>(i) ? side_word(at_word + 1)
                                                  : __ldcs(v.ua_w + (size_t)step_kind_index<MODE>(m0 + i) * N + p);
                 }
             }
