@@ -532,38 +532,45 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     // shape and form of the document tiles
     int32_t dense_docs = 0;
     {
-        // A document that does not fit a tile takes the long documents' kernels; the shape with the least
-        // estimated time is taken, relative costs per token as measured (12 M tokens of 4000-token documents at
-        // K = 777, 99 M of 330 at K = 1000, 200 M of log-normal ones at K = 100 000): a tile of the largest shape leaves few
-        // CTAs per multiprocessor, a table in device memory is the slower the less of it shared memory can stand in for.
-        constexpr double TILE_COST[DOC_TILE_SHAPES] = {1.0, 1.0, 1.02, 1.6};
-        int64_t over[DOC_TILE_SHAPES] = {};
-        double over_cost[DOC_TILE_SHAPES] = {};
-        for (int32_t d = 0; d < D && docs.longest > DOC_TILE_TOKENS[0]; ++d) {
+        // A document that does not fit a tile takes the long documents' kernels.  The tile shape is the one with the
+        // least estimated time, the smaller of two unless the larger is a tenth better; the relative costs per token are
+        // measured (12 M tokens of 4000-token documents at K = 777, 30-70 M of 300 to 1000 at K = 21 to 12 000, 200 M of
+        // log-normal ones at K = 100 000): large tiles leave few CTAs per multiprocessor, a document alone in a tile
+        // leaves part of it empty, a table in device memory is the slower the less shared memory can stand in for it.
+        // Tables of tiles: a counter per topic when a tile holds enough documents' worth of them to be filled (two
+        // counters take the room of a slot), hashed otherwise.
+        constexpr double TILE_COST[2][DOC_TILE_SHAPES] = {{1.0, 1.0, 1.0, 1.05}, {1.0, 1.0, 1.1, 1.2}};
+        const int32_t mean_len = N / std::max(1, D);
+        const auto dense_of = [&](int32_t tile) { return 2 * DOC_TILE_SLOTS * tile / (K + 1); };
+        const auto is_dense = [&](int32_t tile) {
+            return D > 0 && dense_of(tile) > 0 && (int64_t)dense_of(tile) * mean_len >= tile - mean_len;
+        };
+        double cost[DOC_TILE_SHAPES] = {};
+        int64_t inside[DOC_TILE_SHAPES] = {}, rest = N;
+        for (int32_t d = 0; d < D && docs.longest > DOC_TILE_TOKENS[0] / 2; ++d) {
             const int32_t len = doc_off[d + 1] - doc_off[d];
-            if (len <= DOC_TILE_TOKENS[0]) continue;
-            const double cost = (K > DK_SLOTS_PER_TOKEN_HOST * (int64_t)len ? 3.7 : K > LONG_STAGE_MAX_K ? 2.5 : 1.0) * (double)len;
-            for (int sft = 0; sft < DOC_TILE_SHAPES && len > DOC_TILE_TOKENS[sft]; ++sft) {
-                over[sft] += len;
-                over_cost[sft] += cost;
+            if (len <= DOC_TILE_TOKENS[0] / 2) continue;
+            rest -= len;
+            const double outside = K > DK_SLOTS_PER_TOKEN_HOST * (int64_t)len ? 3.7 : K > LONG_STAGE_MAX_K ? 2.8 : 2.6;
+            for (int sft = 0; sft < DOC_TILE_SHAPES; ++sft) {
+                const int32_t tile = DOC_TILE_TOKENS[sft];
+                inside[sft] += len > tile ? 0 : len;
+                cost[sft] += len > tile          ? outside * len
+                             : 2 * len > tile    ? TILE_COST[is_dense(tile)][sft] * std::max((double)len, 0.75 * tile)
+                                                 : TILE_COST[is_dense(tile)][sft] * len;
             }
         }
         int shape = 0;
-        double best = 0;
         for (int sft = 0; sft < DOC_TILE_SHAPES; ++sft) {
-            const double cost = over_cost[sft] + TILE_COST[sft] * (double)(N - over[sft]);
-            if (sft == 0 || cost < best) {
-                best = cost;
-                shape = sft;
-            }
+            cost[sft] += TILE_COST[is_dense(DOC_TILE_TOKENS[sft])][sft] * (double)rest;
+            // (where most tokens are in longer documents anyway, a few large tiles only make a tail: 4000-token documents,
+            // 272 us per pass with the largest shape, 224 with the smallest)
+            if (cost[sft] < 0.9 * cost[shape] && 3 * (inside[sft] + rest) >= N) shape = sft;
         }
         c.doc_tile = DOC_TILE_TOKENS[shape];
         c.doc_threads = DOC_TILE_THREADS[shape];
-        // a counter per topic instead of hashed tables when a tile holds enough documents' worth of them to be
-        // filled (two counters take the room of a slot)
-        const int32_t mean_len = N / std::max(1, D);
-        dense_docs = 2 * DOC_TILE_SLOTS * c.doc_tile / (K + 1);
-        c.doc_dense = D > 0 && dense_docs > 0 && (int64_t)dense_docs * mean_len >= c.doc_tile - mean_len;
+        c.doc_dense = is_dense(c.doc_tile);
+        dense_docs = dense_of(c.doc_tile);
         // Tokens per block of the block-major order: small blocks keep the document pass's scattered accesses in L2, long
         // ones make the word-order passes' runs longer.  With hashed tables the document pass is bound by
         // its instructions and 2^22 is best (738 M tokens, K = 10 000: 23.2 ms per sweep, 24.0 with 2^20); with
@@ -639,11 +646,17 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     int32_t tf_cut = INT32_MAX;
     const int64_t n_top = (int64_t)std::floor(c.dense_frac * (double)V);
     if (n_top > 0) {
-        std::vector<int32_t> tmp(tf);
+        // a dense row of K counters only pays for a word with a fair share of K tokens; only the few words above
+        // that can move the cut
+        tf_cut = std::max((int32_t)std::max(1.0, c.dense_min_tf), K / 8);
+        std::vector<int32_t> above;
+        for (int32_t w = 0; w < V; ++w)
+            if (tf[w] > tf_cut) above.push_back(tf[w]);
         const size_t nth = (size_t)std::min<int64_t>(n_top, V) - 1;
-        std::nth_element(tmp.begin(), tmp.begin() + nth, tmp.end(), std::greater<int32_t>());
-        // a dense row of K counters only pays for a word with a fair share of K tokens
-        tf_cut = std::max<int32_t>({tmp[nth], (int32_t)std::max(1.0, c.dense_min_tf), K / 8});
+        if (nth < above.size()) {
+            std::nth_element(above.begin(), above.begin() + nth, above.end(), std::greater<int32_t>());
+            tf_cut = above[nth];
+        }
     }
     // K above the staging limit: only words with more than WARM_MAX_TF tokens get a dense row, the
     // others with more tokens than a tail tile holds a sorted row built by a CTA of their own

@@ -274,17 +274,29 @@ __device__ __forceinline__ void long_count(const View& v, uint32_t* tab, uint32_
         for (int32_t k = threadIdx.x; k < v.K; k += LONG_THREADS) bins[k] = 0;
         __syncthreads();
     }
-    for (int32_t j = threadIdx.x; j < cnt; j += LONG_THREADS) {
-        const uint32_t k = (uint32_t)__ldcg(zbm + 2 * (size_t)__ldcs(v.bm_of_tok + first + j));
-        if (keep_topics) v.rec[first + j] = min(k, (uint32_t)v.K - 1u);
-        if (k >= (uint32_t)v.K) {
-            atomicOr(v.err, ERR_TOPIC_RANGE);
-        } else if (staged) {
-            atomicAdd(&bins[k], 1u);
-        } else if (DENSE) {
-            atomicAdd(&tab[k], 1u);
-        } else if (dk_insert(tab, cap, k, v.count_bits) == 0xFFFFFFFFu) {
-            atomicOr(v.err, ERR_ROW_OVERFLOW);
+    for (int32_t j0 = threadIdx.x; j0 < cnt; j0 += LONG_AT_ONCE * LONG_THREADS) {
+        uint32_t k[LONG_AT_ONCE];
+#pragma unroll
+        for (int u = 0; u < LONG_AT_ONCE; ++u) {
+            const int32_t j = j0 + u * LONG_THREADS;
+            k[u] = j < cnt ? __ldcs(v.bm_of_tok + first + j) : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < LONG_AT_ONCE; ++u) k[u] = j0 + u * LONG_THREADS < cnt ? (uint32_t)__ldcg(zbm + 2 * (size_t)k[u]) : 0u;
+#pragma unroll
+        for (int u = 0; u < LONG_AT_ONCE; ++u) {
+            const int32_t j = j0 + u * LONG_THREADS;
+            if (j >= cnt) continue;
+            if (keep_topics) v.rec[first + j] = min(k[u], (uint32_t)v.K - 1u);
+            if (k[u] >= (uint32_t)v.K) {
+                atomicOr(v.err, ERR_TOPIC_RANGE);
+            } else if (staged) {
+                atomicAdd(&bins[k[u]], 1u);
+            } else if (DENSE) {
+                atomicAdd(&tab[k[u]], 1u);
+            } else if (dk_insert(tab, cap, k[u], v.count_bits) == 0xFFFFFFFFu) {
+                atomicOr(v.err, ERR_ROW_OVERFLOW);
+            }
         }
     }
     if (staged) {
@@ -316,17 +328,29 @@ __device__ __forceinline__ void long_gather(const View& v, const LongDoc& d, con
     const T* zbm = reinterpret_cast<const T*>(v.zbm);
     const uint32_t sweep = running_sweep(v);
     const LongTable<DENSE> table{tab, v.rec + d.first, DK_SLOTS_PER_TOKEN * (uint32_t)d.len, v.count_bits};
-    for (int32_t j = threadIdx.x; j < cnt; j += LONG_THREADS) {
-        const uint32_t bm = __ldcs(v.bm_of_tok + first + j);
-        uint32_t z, t1;
-        load_topic_pair(zbm, bm, z, t1);
-        doc_side_token<T, MODE, FIXED>(v, table, (uint32_t)(first + j), (uint32_t)d.len, table.of_topic(z), t1, bm, key, sweep,
-                                       mh_steps);
+    for (int32_t j0 = threadIdx.x; j0 < cnt; j0 += LONG_AT_ONCE * LONG_THREADS) {
+        uint32_t bm[LONG_AT_ONCE], z[LONG_AT_ONCE], t1[LONG_AT_ONCE];
+#pragma unroll
+        for (int u = 0; u < LONG_AT_ONCE; ++u) {
+            const int32_t j = j0 + u * LONG_THREADS;
+            bm[u] = z[u] = t1[u] = 0;
+            if (j < cnt) bm[u] = __ldcs(v.bm_of_tok + first + j);
+        }
+#pragma unroll
+        for (int u = 0; u < LONG_AT_ONCE; ++u)
+            if (j0 + u * LONG_THREADS < cnt) load_topic_pair(zbm, bm[u], z[u], t1[u]);
+#pragma unroll
+        for (int u = 0; u < LONG_AT_ONCE; ++u) {
+            const int32_t j = j0 + u * LONG_THREADS;
+            if (j < cnt)
+                doc_side_token<T, MODE, FIXED>(v, table, (uint32_t)(first + j), (uint32_t)d.len, table.of_topic(z[u]), t1[u], bm[u], key,
+                                               sweep, mh_steps);
+        }
     }
 }
 
 template <typename T, int MODE, int FIXED>
-__global__ void __launch_bounds__(LONG_THREADS)
+__global__ void __launch_bounds__(LONG_THREADS, LONG_MIN_CTAS)
 k_long_gather(View v, const int4* __restrict__ chunks, uint2 key, int32_t mh_steps_arg)
 {
     const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;

@@ -131,6 +131,8 @@ struct LongDoc {
     int32_t dense, pad;
 };
 constexpr int LONG_CHUNK = 2048, LONG_THREADS = 256;
+constexpr int LONG_MIN_CTAS = 5;
+constexpr int LONG_AT_ONCE = 4;  // tokens of a thread whose reads are in flight together
 constexpr int LONG_STAGE_MAX_K = 4096;  // counters of a long document staged in shared memory up to this K
 
 // Everything a kernel needs, passed by value.
