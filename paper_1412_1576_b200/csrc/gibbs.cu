@@ -34,11 +34,12 @@ __device__ __forceinline__ ull gibbs_prior_term(double alpha, double beta, doubl
     return __double2ull_rz(__dmul_rn(x, GIBBS_FIXED_ONE));
 }
 
+constexpr int WORD_OF_RUN = 512;
 // word_of[i] = word of the token with document-order index i (the layout keeps tokens by word).  A CTA finds
 // the words of its run of tokens first; a token then searches among those.
 __global__ void __launch_bounds__(256) k_word_of_tokens(View v, int32_t* __restrict__ word_of)
 {
-    constexpr int RUN = 2048;
+    constexpr int RUN = WORD_OF_RUN;
     __shared__ int32_t range[2];
     const int32_t p0 = blockIdx.x * RUN, p1 = min(v.N - p0, RUN) + p0;
     if (threadIdx.x < 2) {
@@ -99,25 +100,26 @@ __device__ __forceinline__ int32_t word_count(const View& v, int32_t row0, int32
     return (lo < nnz && __ldg(v.wk_topic + row0 + lo) == k) ? (int32_t)__ldg(v.wk_count + row0 + lo) : 0;
 }
 
-// One warp per GIBBS_RUN consecutive tokens (of one document or several).  What belongs to a token alone -- its
+// One warp per `run_len` consecutive tokens (of one document or several).  What belongs to a token alone -- its
 // Philox block, the smoothing term's correction and total, a draw from the smoothing term -- is a lane's work for
 // 32 tokens at once; the document term of one token is the whole warp's, a lane per topic of the document: the
 // document's row is read in order, the word's counts lie next to each other in `matrix`, and the running sums
 // the draw needs are a warp scan.  (A lane per token, walking the document's row alone and searching the word's
 // sorted row for every topic of it: 2.15 ms for 2 M tokens of 100-token documents, K = 100.)
+// run_len: up to GIBBS_RUN, shorter where that would leave multiprocessors idle.
 constexpr int GIBBS_RUN = 64;
 template <typename T, bool MATRIX>
 __global__ void __launch_bounds__(256)
 k_gibbs_tokens(View v, const T* __restrict__ z, const int32_t* __restrict__ word_of, const long long* __restrict__ row_off,
                const int32_t* __restrict__ dk_topic, const int32_t* __restrict__ dk_count, const ull* __restrict__ prefix,
-               const int32_t* __restrict__ matrix, int32_t* __restrict__ z_new, uint2 key, uint32_t sweep)
+               const int32_t* __restrict__ matrix, int32_t* __restrict__ z_new, uint2 key, uint32_t sweep, int32_t run_len)
 {
     constexpr uint32_t FULL = 0xFFFFFFFFu;
     const int lane = threadIdx.x & 31;
     const int64_t run = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int32_t K = v.K;
-    int32_t i = (int32_t)min(run * GIBBS_RUN, (int64_t)v.N);
-    const int32_t i_end = (int32_t)min((run + 1) * GIBBS_RUN, (int64_t)v.N);
+    int32_t i = (int32_t)min(run * run_len, (int64_t)v.N);
+    const int32_t i_end = (int32_t)min((run + 1) * run_len, (int64_t)v.N);
     if (i >= i_end) return;
     int32_t d;
     {
@@ -245,16 +247,18 @@ int lda::gibbs_sweep(Ctx& c, int32_t iters)
     // half as much again for n_kw as a matrix; without it the counts are looked up in the sorted rows
     if (rc == LDA_OK && !tmp_alloc(c, &matrix, (size_t)c.V * c.K * 4)) matrix = nullptr;
     const uint2 key = make_uint2((uint32_t)c.seed, (uint32_t)(c.seed >> 32));
-    if (rc == LDA_OK && c.N > 0) k_word_of_tokens<<<(unsigned)((c.N + 2047) / 2048), 256, 0, c.stream>>>(v, word_of);
+    if (rc == LDA_OK && c.N > 0) k_word_of_tokens<<<(unsigned)((c.N + WORD_OF_RUN - 1) / WORD_OF_RUN), 256, 0, c.stream>>>(v, word_of);
     for (int32_t it = 0; rc == LDA_OK && it < iters && c.N > 0; ++it) {
         DkCsr r;
         if ((rc = build_dk_csr(c, r, false))) break;  // also leaves z in document order in the record array
         k_gibbs_prior_prefix<<<c.V, 256, (size_t)c.K * 4, c.stream>>>(v, prefix, matrix);
-        const unsigned grid = (unsigned)((c.N + 8 * GIBBS_RUN - 1) / (8 * GIBBS_RUN));
+        int32_t run_len = GIBBS_RUN;
+        while (run_len > 4 && c.N / run_len < (int64_t)c.n_sm * 32) run_len /= 2;
+        const unsigned grid = (unsigned)((c.N + 8 * run_len - 1) / (8 * run_len));
         auto tokens = [&](auto z) {
             using T = std::remove_const_t<std::remove_pointer_t<decltype(z)>>;
             const auto kernel = matrix ? k_gibbs_tokens<T, true> : k_gibbs_tokens<T, false>;
-            kernel<<<grid, 256, 0, c.stream>>>(v, z, word_of, r.row_off, r.topic, r.count, prefix, matrix, z_new, key, c.sweep);
+            kernel<<<grid, 256, 0, c.stream>>>(v, z, word_of, r.row_off, r.topic, r.count, prefix, matrix, z_new, key, c.sweep, run_len);
         };
         if (c.wide_topics) tokens(reinterpret_cast<const int32_t*>(v.rec));
         else tokens(reinterpret_cast<const uint16_t*>(v.rec));
