@@ -2,8 +2,11 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
+#include <system_error>
+#include <thread>
 #include <utility>
 
 #include "lda_internal.cuh"
@@ -484,25 +487,52 @@ static int scan_documents(Ctx* c, int64_t n_tokens, const int64_t* doc_off, int6
     return LDA_OK;
 }
 
-// Work lists on their way to the device: one allocation and one copy for all of them.
+// Work lists on their way to the device: one allocation and one copy for all of them.  The lists stay where they
+// are until send().
 struct ListPack {
-    std::vector<char> host;
-    std::vector<std::pair<size_t, void**>> lists;
+    struct Entry {
+        const void* list;
+        size_t bytes, at;
+        void** target;
+    };
+    std::vector<Entry> lists;
+    size_t total = 0;
+    std::unique_ptr<char[]> host;  // until the copy is done
     template <typename E, typename P>
     void add(const std::vector<E>& list, P** target)
     {
-        lists.emplace_back(host.size(), const_cast<void**>(reinterpret_cast<const void* const*>(target)));
-        const size_t bytes = list.size() * sizeof(E);
-        host.resize((host.size() + bytes + 15) / 16 * 16);
-        if (bytes) std::memcpy(host.data() + lists.back().first, list.data(), bytes);
+        lists.push_back({list.data(), list.size() * sizeof(E), total, const_cast<void**>(reinterpret_cast<const void* const*>(target))});
+        total = (total + lists.back().bytes + 15) / 16 * 16;
     }
     bool send(Ctx& c)
     {
-        char* dev = (char*)dev_alloc(c, host.size());
-        if (!dev || cudaMemcpyAsync(dev, host.data(), host.size(), cudaMemcpyHostToDevice, c.stream) != cudaSuccess) return false;
-        for (const auto& l : lists) *l.second = dev + l.first;
-        return true;
+        char* dev = (char*)dev_alloc(c, total);
+        host.reset(new char[total]);
+        for (const Entry& l : lists) {
+            if (l.bytes) std::memcpy(host.get() + l.at, l.list, l.bytes);
+            *l.target = dev + l.at;
+        }
+        return dev && cudaMemcpyAsync(dev, host.get(), total, cudaMemcpyHostToDevice, c.stream) == cudaSuccess;
     }
+};
+
+// A task beside the caller, on a thread of its own where it is worth one (and one can be had).
+struct Beside {
+    std::thread thread;
+    template <typename F>
+    Beside(bool worth_it, F f)
+    {
+        if (worth_it) {
+            try {
+                thread = std::thread(f);
+                return;
+            } catch (const std::system_error&) {
+            }
+        }
+        f();
+    }
+    void join() { if (thread.joinable()) thread.join(); }
+    ~Beside() { join(); }
 };
 
 static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const Documents& docs, int64_t n_docs)
@@ -578,7 +608,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
         c.block_shift = c.block_option ? c.block_option : c.doc_dense ? 20 : 22;
     }
 
-    // The sorts are queued; the documents' lists are made meanwhile, the words' lists beside the second sort.
+    // The documents' lists are made on another thread; the sorts are queued, the words' lists made beside the second.
     LayoutTemps temps;
     struct Release {
         Ctx& c;
@@ -591,17 +621,12 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
         }
         ~Release() { now(); }
     } release{c, temps};
-    int rc = build_layout(c, words_dev, doc_off, temps);
-    if (rc != LDA_OK) {
-        cudaStreamSynchronize(c.stream);
-        cudaGetLastError();
-        free_corpus(c);
-        return fail(&c, rc, "building the word-sorted layout failed");
-    }
     // tiles of whole documents: for the MH step, and for the sorted n_kd rows (<= SORT_TILE tokens and <= ROW_TILE_WORDS
-    // documents each)
+    // documents each); made beside all that follows (400 000 documents: 1.6 ms on one core)
     std::vector<int32_t> doc_tiles, long_docs, doc_sort_tiles, doc_sort_long;
-    {
+    bool doc_lists_ok = true;
+    const int32_t tile = c.doc_tile, tile_docs = c.doc_dense ? std::min(dense_docs, tile) : tile;
+    Beside doc_lists(D > 20000, [&, tile, tile_docs] {
         auto pack = [&](int32_t tokens, int32_t documents, std::vector<int32_t>& tiles, std::vector<int32_t>& longer) {
             int32_t s0 = 0, tok = 0;
             auto close = [&](int32_t s1) {
@@ -615,13 +640,24 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
             }
             close(D);
         };
-        pack(c.doc_tile, c.doc_dense ? std::min(dense_docs, c.doc_tile) : c.doc_tile, doc_tiles, long_docs);
-        pack(SORT_TILE, ROW_TILE_WORDS, doc_sort_tiles, doc_sort_long);
+        try {
+            pack(tile, tile_docs, doc_tiles, long_docs);
+            pack(SORT_TILE, ROW_TILE_WORDS, doc_sort_tiles, doc_sort_long);
+        } catch (const std::bad_alloc&) {
+            doc_lists_ok = false;
+        }
+    });
+    int rc = build_layout(c, words_dev, doc_off, temps);
+    if (rc != LDA_OK) {
+        cudaStreamSynchronize(c.stream);
+        cudaGetLastError();
+        free_corpus(c);
+        return fail(&c, rc, "building the word-sorted layout failed");
     }
-    std::vector<int32_t> word_off((size_t)V + 1);
+    std::unique_ptr<int32_t[]> word_off(new int32_t[(size_t)V + 1]);
     int bits = 0;
     cudaStreamWaitEvent(c.side[0], c.ev_chunk, 0);  // word_off is there
-    if (cudaMemcpyAsync(word_off.data(), v.word_off, ((size_t)V + 1) * 4, cudaMemcpyDeviceToHost, c.side[0]) != cudaSuccess ||
+    if (cudaMemcpyAsync(word_off.get(), v.word_off, ((size_t)V + 1) * 4, cudaMemcpyDeviceToHost, c.side[0]) != cudaSuccess ||
         cudaMemcpyAsync(&bits, v.err, sizeof(int), cudaMemcpyDeviceToHost, c.side[0]) != cudaSuccess ||
         cudaStreamSynchronize(c.side[0]) != cudaSuccess) {
         cudaStreamSynchronize(c.stream);
@@ -638,25 +674,32 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     // tf_here: the word's tokens in this corpus (its token range); tf: what the word's row and class
     // are sized for -- the same, unless the corpus is one shard of a larger one (lda_set_shard), in
     // which case the row has to hold the counts of all shards
-    std::vector<int32_t> tf_here((size_t)V), tf((size_t)V);
-    for (int32_t w = 0; w < V; ++w) {
-        tf_here[w] = word_off[w + 1] - word_off[w];
-        tf[w] = c.shard_global_tf.empty() ? tf_here[w] : std::max(tf_here[w], c.shard_global_tf[(size_t)w]);
-    }
+    // The host's lists go over the words present only: a vocabulary may have ten times as many as the corpus uses.
+    const int32_t* global_tf = c.shard_global_tf.empty() ? nullptr : c.shard_global_tf.data();
+    const auto tf_here = [&](int32_t w) { return word_off[w + 1] - word_off[w]; };
+    const auto tf = [&](int32_t w) { return global_tf ? std::max(tf_here(w), global_tf[w]) : tf_here(w); };
+    std::vector<int32_t> present;
+    present.reserve((size_t)std::min<int64_t>(V, global_tf ? V : (int64_t)N));
+    for (int32_t w = 0; w < V; ++w)
+        if (tf(w) > 0) present.push_back(w);
     int32_t tf_cut = INT32_MAX;
-    const int64_t n_top = (int64_t)std::floor(c.dense_frac * (double)V);
+    const int64_t n_top = std::min<int64_t>((int64_t)std::floor(c.dense_frac * (double)V), V);
     if (n_top > 0) {
-        // a dense row of K counters only pays for a word with a fair share of K tokens; only the few words above
-        // that can move the cut
+        // the n_top-th largest frequency -- but a dense row of K counters only pays for a word with a fair share of K
+        // tokens.  Of the words above the cut so far, every 2 n_top-th throws out the lower half.
         tf_cut = std::max((int32_t)std::max(1.0, c.dense_min_tf), K / 8);
         std::vector<int32_t> above;
-        for (int32_t w = 0; w < V; ++w)
-            if (tf[w] > tf_cut) above.push_back(tf[w]);
-        const size_t nth = (size_t)std::min<int64_t>(n_top, V) - 1;
-        if (nth < above.size()) {
-            std::nth_element(above.begin(), above.begin() + nth, above.end(), std::greater<int32_t>());
-            tf_cut = above[nth];
+        const auto cut_to_top = [&] {
+            std::nth_element(above.begin(), above.begin() + (n_top - 1), above.end(), std::greater<int32_t>());
+            above.resize((size_t)n_top);
+            tf_cut = above.back();
+        };
+        for (const int32_t w : present) {
+            if (tf(w) <= tf_cut) continue;
+            above.push_back(tf(w));
+            if ((int64_t)above.size() >= 2 * n_top) cut_to_top();
         }
+        if ((int64_t)above.size() >= n_top) cut_to_top();
     }
     // K above the staging limit: only words with more than WARM_MAX_TF tokens get a dense row, the
     // others with more tokens than a tail tile holds a sorted row built by a CTA of their own
@@ -672,14 +715,14 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
         while (r > shortest && tokens / r < per_sm * c.n_sm) r /= 2;
         return std::max(r, shortest);
     };
-    const auto is_hot = [&](int32_t w) { return tf[w] > COLD_TILE; };
-    const auto has_dense_row = [&](int32_t w) {
-        return !(warm_class && tf[w] > SORT_TILE && tf[w] <= WARM_MAX_TF) && (tf[w] > SORT_TILE || (tf[w] > 0 && tf[w] >= tf_cut));
-    };
-    int64_t t_hot = 0, t_cold = 0, t_dense = 0;
-    for (int32_t w = 0; w < V; ++w) {
-        (is_hot(w) ? t_hot : t_cold) += tf_here[w];
-        if (has_dense_row(w)) t_dense += tf_here[w];
+    const auto is_hot = [&](int32_t w) { return tf(w) > COLD_TILE; };
+    const auto has_warm_row = [&](int32_t w) { return warm_class && tf(w) > SORT_TILE && tf(w) <= WARM_MAX_TF; };
+    const auto has_dense_row = [&](int32_t w) { return !has_warm_row(w) && (tf(w) > SORT_TILE || tf(w) >= tf_cut); };
+    int64_t t_hot = 0, t_cold = 0, t_dense = 0, cap_total = 0;
+    for (const int32_t w : present) {
+        (is_hot(w) ? t_hot : t_cold) += tf_here(w);
+        if (has_dense_row(w)) t_dense += tf_here(w);
+        cap_total += std::min(tf(w), K);
     }
     int32_t k_pow2 = 1;  // a row of K counters: staged by the accept pass, added up by the histograms
     while (k_pow2 < K) k_pow2 *= 2;
@@ -697,87 +740,92 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     const bool sorted_rows = K > WORD_ROWS_BITMAP_MAX_K;
     const int32_t row_tile = run_for(N - t_dense, 4, SORT_TILE, 256), row_tile_words = sorted_rows ? SORT_TILE : ROW_TILE_WORDS;
 
-    std::vector<int32_t> dense_slot((size_t)V, -1), row_start((size_t)V + 1), alias_words[ALIAS_CLASSES];
-    std::vector<uint8_t> hot_word((size_t)V);
-    std::vector<int32_t> hot_runs, acc_runs, word_tiles;
-    int64_t cap_total = 0;
-    c.n_dense = 0;
-    for (int32_t w = 0; w < V; ++w) {
-        row_start[w] = (int32_t)cap_total;
-        const int32_t cap = std::min(tf[w], K);
-        cap_total += cap;
-        hot_word[w] = is_hot(w);
+    std::vector<int32_t> dense_words, alias_words[ALIAS_CLASSES], hot_runs, acc_runs, word_tiles;
+    // vocabulary slices of about equal row capacity; slice_w[s] = first word of slice s, slice_row[s] = room of the words before
+    const int n_slices = std::max(1, c.alias_slices);
+    std::vector<int32_t> slice_w((size_t)n_slices + 1, V);
+    std::vector<int64_t> slice_row((size_t)n_slices + 1, cap_total);
+    slice_w[0] = 0;
+    slice_row[0] = 0;
+    int64_t cap_sum = 0;
+    int32_t end = 0;  // one past the last word seen
+    int sl_next = 1;
+    for (const int32_t w : present) {
+        // (the first word before which there is that much room)
+        for (; sl_next < n_slices && cap_total * sl_next / n_slices <= cap_sum; ++sl_next) {
+            slice_w[(size_t)sl_next] = cap_total * sl_next / n_slices > 0 ? end : 0;
+            slice_row[(size_t)sl_next] = cap_sum;
+        }
+        end = w + 1;
+        const int32_t cap = std::min(tf(w), K);
+        cap_sum += cap;
         for (int i = 0; i < ALIAS_CLASSES && cap > ALIAS_CLASS_MAX[i]; ++i) alias_words[i].push_back(w);
-        if (warm_class && tf[w] > SORT_TILE && tf[w] <= WARM_MAX_TF) {
+        if (has_warm_row(w)) {
             warm_words.push_back(w);
         } else if (has_dense_row(w)) {
-            dense_slot[w] = c.n_dense++;
-            const int32_t runs = std::max(1, (tf_here[w] + hist_run - 1) / hist_run);
+            dense_words.push_back(w);
+            const int32_t runs = std::max(1, (tf_here(w) + hist_run - 1) / hist_run);
             for (int32_t i = 0; i < runs; ++i) {
                 const int32_t o = i * hist_run;
-                hot_runs.insert(hot_runs.end(), {w, word_off[w] + o, std::min(hist_run, tf_here[w] - o),
+                hot_runs.insert(hot_runs.end(), {w, word_off[w] + o, std::min(hist_run, tf_here(w) - o),
                                                  runs > 1 ? (int32_t)acc_runs.size() : -1});
             }
             if (runs > 1) acc_runs.push_back(runs);
         }
     }
-    row_start[V] = (int32_t)cap_total;
-    // vocabulary slices of about equal row capacity; slice_w[s] = first word of slice s
-    const int n_slices = std::max(1, c.alias_slices);
-    std::vector<int32_t> slice_w((size_t)n_slices + 1, V);
-    slice_w[0] = 0;
-    for (int sl = 1; sl < n_slices; ++sl) {
-        const int32_t target = (int32_t)(cap_total * sl / n_slices);
-        slice_w[sl] = (int32_t)(std::lower_bound(row_start.begin(), row_start.begin() + V, target) - row_start.begin());
-    }
-    std::vector<char> slice_starts((size_t)V + 1, 0);
-    for (int sl = 1; sl < n_slices; ++sl) slice_starts[(size_t)slice_w[sl]] = 1;
+    c.n_dense = (int32_t)dense_words.size();
     // tiles of consecutive sparse words: <= row_tile tokens (or one longer word) and <= row_tile_words words each
     {
-        int32_t s0 = 0, tok = 0;
-        auto close = [&](int32_t s1) {
+        int32_t s0 = 0, s1 = 0, tok = 0;
+        auto close = [&] {
             if (s1 > s0) { word_tiles.push_back(s0); word_tiles.push_back(s1); }
         };
-        for (int32_t w = 0; w < V; ++w) {
-            if (dense_slot[w] >= 0 || tf[w] > SORT_TILE) { close(w); s0 = w + 1; tok = 0; continue; }
-            if (tok + tf[w] > row_tile || w - s0 >= row_tile_words) { close(w); s0 = w; tok = 0; }
-            tok += tf[w];
+        for (const int32_t w : present) {
+            const bool other = has_dense_row(w) || tf(w) > SORT_TILE;
+            if (other || tok + tf(w) > row_tile || w - s0 >= row_tile_words) { close(); s0 = s1 = w; tok = 0; }
+            if (other) continue;
+            if (!tok) s0 = w;
+            s1 = w + 1;
+            tok += tf(w);
         }
-        close(V);
+        close();
     }
     // MH kernel work lists: a hot word (more tokens than a tail tile holds; it has a dense row by
     // the rule above) is cut into runs, tail words are packed whole into tiles, one longer than a tile cut
     std::vector<int32_t> hot_tiles, hot_tiles_warm, hot_tiles_propose, cold_tiles;
     {
         static_assert(COLD_TILE >= SORT_TILE, "every word longer than a tail tile must have a dense row or a warm one");
-        int32_t s0 = 0, tok = 0;
-        auto close = [&](int32_t s1) {
+        int32_t s0 = 0, s1 = 0, tok = 0;
+        auto close = [&] {
             if (s1 > s0 && word_off[s1] > word_off[s0])
                 cold_tiles.insert(cold_tiles.end(), {s0, s1, word_off[s0], word_off[s1] - word_off[s0]});
         };
         auto cut = [&](std::vector<int32_t>& list, int32_t w, int32_t run) {
-            for (int32_t o = 0; o < tf_here[w]; o += run)
-                list.insert(list.end(), {w, word_off[w] + o, std::min(run, tf_here[w] - o)});
+            for (int32_t o = 0; o < tf_here(w); o += run)
+                list.insert(list.end(), {w, word_off[w] + o, std::min(run, tf_here(w) - o)});
         };
-        for (int32_t w = 0; w < V; ++w) {
-            if (slice_starts[w]) { close(w); s0 = w; tok = 0; }  // no tile reaches across two slices
+        int sl = 1;
+        for (const int32_t w : present) {
+            bool fresh = false;  // no tile reaches across two slices
+            for (; sl < n_slices && slice_w[(size_t)sl] <= w; ++sl) fresh = true;
+            const bool alone = is_hot(w) || tf(w) > cold_tile;
+            if (fresh || alone || tok + tf(w) > cold_tile || w - s0 >= cold_words) { close(); s0 = s1 = w; tok = 0; }
             if (is_hot(w)) {
-                close(w); s0 = w + 1; tok = 0;
-                cut(dense_slot[w] >= 0 ? hot_tiles : hot_tiles_warm, w, hot_tile);
+                cut(has_dense_row(w) ? hot_tiles : hot_tiles_warm, w, hot_tile);
                 cut(hot_tiles_propose, w, propose_tile);
-                continue;
+            } else if (alone) {
+                for (int32_t o = 0; o < tf_here(w); o += cold_tile)
+                    cold_tiles.insert(cold_tiles.end(), {w, w + 1, word_off[w] + o, std::min(cold_tile, tf_here(w) - o)});
+            } else {
+                if (!tok) s0 = w;
+                s1 = w + 1;
+                tok += tf(w);
             }
-            if (tf[w] > cold_tile) {
-                close(w); s0 = w + 1; tok = 0;
-                for (int32_t o = 0; o < tf_here[w]; o += cold_tile)
-                    cold_tiles.insert(cold_tiles.end(), {w, w + 1, word_off[w] + o, std::min(cold_tile, tf_here[w] - o)});
-                continue;
-            }
-            if (tok + tf[w] > cold_tile || w - s0 >= cold_words) { close(w); s0 = w; tok = 0; }
-            tok += tf[w];
         }
-        close(V);
+        close();
     }
+    doc_lists.join();
+    if (!doc_lists_ok) { free_corpus(c); return fail(&c, LDA_ENOMEM, "host allocation failed"); }
     c.n_doc_sort_tiles = (int32_t)(doc_sort_tiles.size() / 2);
     c.n_doc_sort_long = (int32_t)doc_sort_long.size();
     c.n_word_tiles = (int32_t)(word_tiles.size() / 2);
@@ -807,8 +855,8 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
             Ctx::Slice& q = c.slices[(size_t)sl];
             q.w_lo = slice_w[(size_t)sl];
             q.w_hi = slice_w[(size_t)sl + 1];
-            q.row_lo = row_start[(size_t)q.w_lo];
-            q.row_n = row_start[(size_t)q.w_hi] - q.row_lo;
+            q.row_lo = slice_row[(size_t)sl];
+            q.row_n = slice_row[(size_t)sl + 1] - q.row_lo;
             slice_rows_max = std::max(slice_rows_max, q.row_n);
             for (int i = 0; i < ALIAS_CLASSES; ++i) {
                 q.alias_lo[i] = first_at(alias_words[i], 0, alias_words[i].size(), 1, q.w_lo);
@@ -831,9 +879,8 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     v.zbm = A(2 * n1 * zt);  // (topic, first word-proposal) pairs
     v.rec = (uint32_t*)A(n1 * 4 + 16);  // + one aligned group of four words past the last record
     ListPack lists;
-    lists.add(row_start, &v.row_start);
-    lists.add(dense_slot, &v.dense_slot);
-    lists.add(hot_word, &v.hot_word);
+    const int32_t* dense_words_dev = nullptr;
+    lists.add(dense_words, &dense_words_dev);
     lists.add(word_tiles, &c.word_tiles);
     lists.add(doc_tiles, &c.doc_tiles);
     lists.add(hot_runs, &c.hot_runs);
@@ -897,6 +944,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     c.ll_tables_ready = false;
     if (!ok) { free_corpus(c); return fail(&c, LDA_ENOMEM, "device allocation failed"); }
     set_slice(c, 0);
+    launch_dense_slots(c, dense_words_dev);
     cudaMemsetAsync(v.wk_nnz, 0, ((size_t)V + 1) * 4, c.stream);
     cudaMemsetAsync(v.sp_mass, 0, (size_t)V * 8, c.stream);
     cudaMemsetAsync(c.acc, 0, acc_runs.size() * (size_t)v.dense_stride * 4, c.stream);

@@ -3,7 +3,10 @@
 // contiguous).  Tokens are sorted stably by word id, so inside a word they
 // stay in document order.  The sort itself uses CUB's device radix sort: it
 // runs once per corpus, outside the per-sweep path.
+#include <algorithm>
+
 #include <cub/device/device_radix_sort.cuh>
+#include <cub/device/device_scan.cuh>
 
 #include "lda_device.cuh"
 #include "lda_internal.cuh"
@@ -33,6 +36,36 @@ __global__ void k_word_offsets(const int32_t* __restrict__ sorted_words, int32_t
         if (sorted_words[mid] < w) lo = mid + 1; else hi = mid;
     }
     word_off[w] = lo;
+}
+
+// What the passes need of every word: room for its sparse row (row_len becomes row_start by a prefix sum), whether the
+// MH step treats it as hot, no dense row yet.  `tf` gives the words' frequencies where they are not those of this corpus.
+// (These lists are made here, not on the host: for 944 000 words and 110 000 tokens, the host's copies of
+// them and their pages were 6 of the 12 ms of a load.)
+__global__ void k_word_rooms(const int32_t* __restrict__ word_off, const int32_t* __restrict__ tf, int32_t V, int32_t K,
+                             int32_t* __restrict__ row_len, uint8_t* __restrict__ hot_word, int32_t* __restrict__ dense_slot)
+{
+    const int32_t w = blockIdx.x * blockDim.x + threadIdx.x;
+    if (w > V) return;
+    int32_t n = 0;
+    if (w < V) {
+        n = word_off[w + 1] - word_off[w];
+        if (tf) n = max(n, tf[w]);
+        hot_word[w] = n > COLD_TILE;
+        dense_slot[w] = -1;
+    }
+    row_len[w] = min(n, K);
+}
+
+__global__ void k_dense_slots(const int32_t* __restrict__ dense_words, int32_t n, int32_t* __restrict__ dense_slot)
+{
+    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) dense_slot[dense_words[i]] = i;
+}
+
+void launch_dense_slots(Ctx& c, const int32_t* dense_words)
+{
+    if (c.n_dense) k_dense_slots<<<(c.n_dense + 255) / 256, 256, 0, c.stream>>>(dense_words, c.n_dense, const_cast<int32_t*>(c.v.dense_slot));
 }
 
 // Keys of the block-major order: the block of a token is the high part of its document-order index.
@@ -69,7 +102,13 @@ int build_layout(Ctx& c, const int32_t* word_ids_dev, const std::vector<int32_t>
     uint32_t* bm_of_tok = (uint32_t*)dev_alloc(c, n1 * 4);
     int32_t* word_off = (int32_t*)dev_alloc(c, ((size_t)V + 1) * 4);
     int32_t* doc_off = (int32_t*)dev_alloc(c, ((size_t)D + 1) * 4);
-    if (!tok_orig || !inv || !bm_of_tok || !word_off || !doc_off) return LDA_ENOMEM;
+    int32_t* row_start = (int32_t*)dev_alloc(c, ((size_t)V + 1) * 4);
+    int32_t* dense_slot = (int32_t*)dev_alloc(c, (size_t)V * 4);
+    uint8_t* hot_word = (uint8_t*)dev_alloc(c, (size_t)V);
+    if (!tok_orig || !inv || !bm_of_tok || !word_off || !doc_off || !row_start || !dense_slot || !hot_word) return LDA_ENOMEM;
+    c.v.row_start = row_start;
+    c.v.dense_slot = dense_slot;
+    c.v.hot_word = hot_word;
     c.v.inv = inv;
     c.v.bm_of_tok = bm_of_tok;
     c.v.tok_orig = tok_orig;
@@ -81,7 +120,7 @@ int build_layout(Ctx& c, const int32_t* word_ids_dev, const std::vector<int32_t>
     int end_bit = 1, blk_bits = 1;
     while (end_bit < 31 && (1ll << end_bit) < (long long)V) ++end_bit;
     while (blk_bits < 32 && (((long long)N - 1) >> c.block_shift) >= (1ll << blk_bits)) ++blk_bits;
-    size_t temp_bytes = 0, temp2_bytes = 0;
+    size_t temp_bytes = 0, temp2_bytes = 0, scan_bytes = 0;
     const int32_t* no_keys = nullptr;
     const uint32_t* no_values = nullptr;
     if (N > 0 && (cub::DeviceRadixSort::SortPairs(nullptr, temp_bytes, no_keys, (int32_t*)nullptr, no_values, tok_orig, N, 0, end_bit,
@@ -89,6 +128,7 @@ int build_layout(Ctx& c, const int32_t* word_ids_dev, const std::vector<int32_t>
                   cub::DeviceRadixSort::SortPairs(nullptr, temp2_bytes, no_values, (uint32_t*)nullptr, no_values, tok_orig, N, 0,
                                                   blk_bits, st) != cudaSuccess))
         return LDA_ECUDA;
+    if (cub::DeviceScan::ExclusiveSum(nullptr, scan_bytes, row_start, row_start, V + 1, st) != cudaSuccess) return LDA_ECUDA;
     auto transient = [&](size_t bytes) -> void* {
         void* p = nullptr;
         if (tmp_alloc(c, &p, bytes)) temps.held.push_back(p);
@@ -98,8 +138,9 @@ int build_layout(Ctx& c, const int32_t* word_ids_dev, const std::vector<int32_t>
     uint32_t* iota = (uint32_t*)transient(n1 * 4);
     uint32_t* keys_blk = (uint32_t*)transient(n1 * 4);
     uint32_t* order = (uint32_t*)transient(n1 * 4);
-    void* temp = transient(temp_bytes > temp2_bytes ? temp_bytes : temp2_bytes);
-    if (!keys_out || !iota || !keys_blk || !order || !temp) return LDA_ENOMEM;
+    void* temp = transient(std::max({temp_bytes, temp2_bytes, scan_bytes}));
+    int32_t* tf = c.shard_global_tf.empty() ? nullptr : (int32_t*)transient((size_t)V * 4);
+    if (!keys_out || !iota || !keys_blk || !order || !temp || (!tf && !c.shard_global_tf.empty())) return LDA_ENOMEM;
     bool ok = true;
     if (N > 0) {
         k_check_words_iota<<<1184, 256, 0, st>>>(word_ids_dev, iota, N, V, c.v.err);
@@ -107,6 +148,9 @@ int build_layout(Ctx& c, const int32_t* word_ids_dev, const std::vector<int32_t>
     }
     k_word_offsets<<<(V + 1 + 255) / 256, 256, 0, st>>>(keys_out, N, V, word_off);
     cudaEventRecord(c.ev_chunk, st);
+    if (tf && copy_to_device(c, tf, c.shard_global_tf.data(), (size_t)V * 4) != cudaSuccess) return LDA_ECUDA;
+    k_word_rooms<<<(V + 1 + 255) / 256, 256, 0, st>>>(word_off, tf, V, c.K, row_start, hot_word, dense_slot);
+    ok = ok && cub::DeviceScan::ExclusiveSum(temp, scan_bytes, row_start, row_start, V + 1, st) == cudaSuccess;
     if (N > 0 && ok) {
         // block-major order: tokens sorted by (block of their document-order index, word-sorted
         // position); a stable sort of the positions by block (one block: the positions themselves)

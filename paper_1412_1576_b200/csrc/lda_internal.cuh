@@ -442,6 +442,7 @@ void free_wk_csr(Ctx& c, WkCsr& r);
 struct LayoutTemps {
     std::vector<void*> held;
 };
+void launch_dense_slots(Ctx& c, const int32_t* dense_words);  // slot i to dense_words[i], i < n_dense
 int build_layout(Ctx& c, const int32_t* word_ids_dev, const std::vector<int32_t>& doc_off, LayoutTemps& temps);
 
 void* raw_alloc(Ctx& c, size_t bytes);  // the context's allocator (cudaMalloc by default); nullptr on failure

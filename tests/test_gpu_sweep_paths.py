@@ -115,3 +115,27 @@ def test_document_tiles_with_counters_and_with_hashed_tables(K, length):
             e.sweep(2, steps)
         assert np.array_equal(g.get_assignments(), o.get_assignments()), (steps, mode)
     _same(g, o)
+
+
+@pytest.mark.parametrize("K,slices", [(40, 1), (40, 5), (3_000, 1), (9_000, 4)])
+def test_vocabularies_mostly_empty(K, slices):
+    """Words far apart, gaps wider than any tile, none at the first and last ids; a frequent one among them; gaps in which
+    a slice begins.  20 500 documents, so that their lists are made on another thread."""
+    V = 60_000
+    rng = np.random.default_rng(K)
+    used = np.unique(np.concatenate([rng.integers(5, V - 5, 900), np.arange(30_000, 30_300), [29_000]]))
+    words = rng.permutation(np.concatenate([rng.choice(used, 41_000), np.full(2_500, 29_000)])).astype(np.int32)
+    offsets = np.concatenate([[0], np.sort(rng.integers(0, words.size + 1, 20_500)), [words.size]]).astype(np.int64)
+    g = binding.LightLDA(V, K, 0.05, 0.01)
+    binding.lda_set_option(g._h, "alias_slices", slices)
+    o = ldaref.Oracle(V, K, 0.05, 0.01)
+    for e in (g, o):
+        e.load_corpus(words, offsets)
+        e.init(4)
+        e.sweep(2, 2)
+    for a, b in zip(g.loglik(), o.loglik()):
+        assert a == pytest.approx(b, rel=1e-10)
+    if slices == 1:
+        _same(g, o)
+    else:
+        assert np.array_equal(g.get_assignments(), o.get_assignments())
