@@ -100,22 +100,39 @@ __device__ __forceinline__ int32_t word_count(const View& v, int32_t row0, int32
     return (lo < nnz && __ldg(v.wk_topic + row0 + lo) == k) ? (int32_t)__ldg(v.wk_count + row0 + lo) : 0;
 }
 
-// One warp per `run_len` consecutive tokens (of one document or several).  What belongs to a token alone -- its
-// Philox block, the smoothing term's correction and total, a draw from the smoothing term -- is a lane's work for
-// 32 tokens at once; the document term of one token is the whole warp's, a lane per topic of the document: the
-// document's row is read in order, the word's counts lie next to each other in `matrix`, and the running sums
-// the draw needs are a warp scan.  (A lane per token, walking the document's row alone and searching the word's
-// sorted row for every topic of it: 2.15 ms for 2 M tokens of 100-token documents, K = 100.)
+// a / b for one b and many a: y is 1/b rounded to nearest.  Two steps of Markstein's correction (IBM J. Res. Dev. 34(1),
+// 1990): the first makes the quotient faithful, the second, from a faithful quotient and a correctly rounded
+// reciprocal, the correctly rounded one -- the value of __ddiv_rn(a, b) where nothing over- or underflows.
+__device__ __forceinline__ double div_by(double a, double b, double y)
+{
+    double q = __dmul_rn(a, y);
+    q = __fma_rn(__fma_rn(-b, q, a), y, q);
+    return __fma_rn(__fma_rn(-b, q, a), y, q);
+}
+
+// One warp per `run_len` consecutive tokens (of one document or several), at most 32 of a document at a time.  What
+// belongs to a token alone -- its Philox block, its own topic's mass, the smoothing term's correction and total, a draw
+// from the smoothing term -- is a lane's work for all of them at once.  The document term of a token is the work of LANES
+// lanes, 32 / LANES tokens side by side: each lane adds up its part of the document's row (the first GIBBS_KEPT / LANES
+// topics stay in registers, with the reciprocals of their denominators), a few shuffle steps make the running sums, and
+// the lane in whose part the draw falls finds the topic there.  Bound by the latency of the counts' reads: more
+// registers than three or four CTAs per multiprocessor leave cost more than they save.  16 lanes suit rows that stay in
+// registers, 32 longer ones: 2 M tokens of 100-token documents, K = 100: 517 and 559 us; 1.1 M of 808, rows of
+// 300 topics: 2141 and 1686 us (a warp per token that sums and then scans: 670 and 2199; eight lanes: 615 and 3100; the
+// loads of several topics that are not kept in flight together: slower, by their registers).
 // run_len: up to GIBBS_RUN, shorter where that would leave multiprocessors idle.
 constexpr int GIBBS_RUN = 64;
-template <typename T, bool MATRIX>
-__global__ void __launch_bounds__(256)
+constexpr int GIBBS_KEPT = 64;
+template <typename T, bool MATRIX, int LANES>
+__global__ void __launch_bounds__(256, LANES == 32 ? 4 : 3)
 k_gibbs_tokens(View v, const T* __restrict__ z, const int32_t* __restrict__ word_of, const long long* __restrict__ row_off,
                const int32_t* __restrict__ dk_topic, const int32_t* __restrict__ dk_count, const ull* __restrict__ prefix,
                const int32_t* __restrict__ matrix, int32_t* __restrict__ z_new, uint2 key, uint32_t sweep, int32_t run_len)
 {
     constexpr uint32_t FULL = 0xFFFFFFFFu;
-    const int lane = threadIdx.x & 31;
+    constexpr int TOKENS = 32 / LANES, KEPT = GIBBS_KEPT / LANES;
+    constexpr ull NOT_SMOOTH = ~0ull;
+    const int lane = threadIdx.x & 31, sub = lane % LANES, group = lane / LANES;
     const int64_t run = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int32_t K = v.K;
     int32_t i = (int32_t)min(run * run_len, (int64_t)v.N);
@@ -134,22 +151,25 @@ k_gibbs_tokens(View v, const T* __restrict__ z, const int32_t* __restrict__ word
         while (__ldg(v.doc_off + d + 1) <= i) ++d;
         const long long e0 = row_off[d];
         const int32_t rows = (int32_t)(row_off[d + 1] - e0);
-        const int32_t n = min(32, min(i_end, __ldg(v.doc_off + d + 1)) - i);  // tokens of this turn, a lane each
-        // the first 64 topics of the document stay in registers for all of them
-        uint32_t k_r[2];
-        int32_t c_r[2], n_r[2];
+        const int32_t n = min(32, min(i_end, __ldg(v.doc_off + d + 1)) - i);  // tokens of this turn
+        // this lane's part of the row: entries [e, e + part), fewer at its end
+        const int32_t part = (rows + LANES - 1) / LANES, e = sub * part, mine_n = max(0, min(part, rows - e));
+        uint32_t k_r[KEPT];
+        int32_t c_r[KEPT];
+        double b_r[KEPT], y_r[KEPT];  // denominator of a term in units of 2^-44, and its reciprocal
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int32_t e = 32 * q + lane;
-            k_r[q] = e < rows ? (uint32_t)__ldg(dk_topic + e0 + e) : 0u;
-            c_r[q] = e < rows ? __ldg(dk_count + e0 + e) : 0;
-            n_r[q] = __ldg(v.nk + k_r[q]);
+        for (int q = 0; q < KEPT; ++q) {
+            if (q >= part) break;
+            const bool in = q < mine_n;
+            k_r[q] = in ? (uint32_t)__ldg(dk_topic + e0 + e + q) : 0u;
+            c_r[q] = in ? __ldg(dk_count + e0 + e + q) : 0;
+            b_r[q] = __dmul_rn(__dadd_rn((double)__ldg(v.nk + k_r[q]), v.Vbeta), 1.0 / GIBBS_FIXED_ONE);
+            y_r[q] = __drcp_rn(b_r[q]);
         }
-        uint32_t z_l = 0, r_l = 0, pick_l = (uint32_t)(K - 1);
+        uint32_t z_l = 0, r_l = 0;
         int32_t w_l = 0, row_l = 0, nnz_l = 0;
         long long delta_l = 0;
-        ull prior_l = 0, x_l = 0;
-        bool smooth_l = false;
+        ull prior_l = 0, own_l = 0, x_l = NOT_SMOOTH;
         if (lane < n) {
             z_l = (uint32_t)z[i + lane];
             w_l = word_of[i + lane];
@@ -166,54 +186,75 @@ k_gibbs_tokens(View v, const T* __restrict__ z, const int32_t* __restrict__ word
                       (long long)gibbs_prior_term(v.alpha, v.beta, v.Vbeta, n_zw, n_z);
             prior_l = (ull)((long long)__ldg(prefix + (size_t)w_l * K + K - 1) + delta_l);
             r_l = philox4x32_10(make_uint4(v.tok_base + (uint32_t)(i + lane), sweep, 0u, 2u), key).x;
+            // the token's own topic is in the row; its mass there, the token removed
+            int32_t lo = 0, hi = rows - 1;
+            while (lo < hi) {
+                const int32_t mid = (lo + hi) >> 1;
+                if ((uint32_t)__ldg(dk_topic + e0 + mid) < z_l) lo = mid + 1; else hi = mid;
+            }
+            const int32_t n_zd = __ldg(dk_count + e0 + lo) - 1;
+            if (n_zd > 0) own_l = gibbs_doc_term(v.beta, v.Vbeta, n_zd, n_zw - 1, n_z - 1);
         }
-        for (int t = 0; t < n; ++t) {
+        for (int t0 = 0; t0 < n; t0 += TOKENS) {
+            const int t = min(t0 + group, n - 1);  // the groups past the last token repeat it
             const uint32_t z0 = __shfl_sync(FULL, z_l, t);
+            const ull own = __shfl_sync(FULL, own_l, t), prior = __shfl_sync(FULL, prior_l, t);
+            const uint32_t r = __shfl_sync(FULL, r_l, t);
             const int32_t w = __shfl_sync(FULL, w_l, t);
             const int32_t row0 = MATRIX ? 0 : __shfl_sync(FULL, row_l, t), nnz = MATRIX ? 0 : __shfl_sync(FULL, nnz_l, t);
             const int32_t* line = matrix + (size_t)w * K;
-            // a topic's mass in the document term
-            auto mass = [&](uint32_t k, int32_t c, int32_t n_k) -> ull {
-                const int32_t own = (k == z0), n_kd = c - own;
-                if (n_kd <= 0) return 0ull;
-                const int32_t n_kw = MATRIX ? __ldg(line + k) : word_count(v, row0, nnz, k);
-                return gibbs_doc_term(v.beta, v.Vbeta, n_kd, n_kw - own, n_k - own);
+            auto count_of = [&](uint32_t k) { return MATRIX ? __ldg(line + k) : word_count(v, row0, nnz, k); };
+            auto later = [&](int32_t q) -> ull {  // an entry that is not kept
+                const uint32_t k = (uint32_t)__ldg(dk_topic + e0 + e + q);
+                if (k == z0) return own;
+                return gibbs_doc_term(v.beta, v.Vbeta, __ldg(dk_count + e0 + e + q), count_of(k), __ldg(v.nk + k));
             };
-            auto round_mass = [&](int32_t q) -> ull {
-                const int32_t e = 32 * q + lane;
-                if (e >= rows) return 0ull;
-                const uint32_t k = (uint32_t)__ldg(dk_topic + e0 + e);
-                return mass(k, __ldg(dk_count + e0 + e), __ldg(v.nk + k));
-            };
-            const ull m0 = mass(k_r[0], c_r[0], n_r[0]), m1 = rows > 32 ? mass(k_r[1], c_r[1], n_r[1]) : 0ull;
-            ull mine = m0 + m1;
-            for (int32_t q = 2; 32 * q < rows; ++q) mine += round_mass(q);
-            const ull sum_doc = warp_reduce_sum<ull>(mine);
-            const ull total = sum_doc + __shfl_sync(FULL, prior_l, t);
-            const ull x = __umul64hi(total, (ull)__shfl_sync(FULL, r_l, t) << 32);  // floor(total * r / 2^32)
-            if (x >= sum_doc) {  // from the smoothing term, later
-                if (lane == t) {
-                    smooth_l = true;
-                    x_l = x - sum_doc;
-                }
-                continue;
+            ull m[KEPT];
+            ull mine = 0;
+#pragma unroll
+            for (int q = 0; q < KEPT; ++q) {
+                if (q >= part) break;
+                const double a = __dmul_rn((double)c_r[q], __dadd_rn((double)count_of(k_r[q]), v.beta));
+                const ull term = __double2ull_rz(div_by(a, b_r[q], y_r[q]));
+                m[q] = q >= mine_n ? 0ull : k_r[q] == z0 ? own : term;
+                mine += m[q];
             }
-            ull before = 0;
-            for (int32_t q = 0; 32 * q < rows; ++q) {
-                const ull m = q == 0 ? m0 : q == 1 ? m1 : round_mass(q);
-                const ull cum = before + warp_scan_incl<ull>(m);
-                const uint32_t over = __ballot_sync(FULL, cum > x);
-                if (over) {
-                    const int src = __ffs((int)over) - 1;
-                    const uint32_t k = q == 0 ? k_r[0] : q == 1 ? k_r[1] : (uint32_t)__ldg(dk_topic + e0 + 32 * q + src);
-                    const uint32_t chosen = __shfl_sync(FULL, k, src);
-                    if (lane == t) pick_l = chosen;
-                    break;
+            for (int32_t q = KEPT; q < mine_n; ++q) mine += later(q);
+            ull cum = mine;  // running sum over the group's lanes
+#pragma unroll
+            for (int o = 1; o < LANES; o *= 2) {
+                const ull up = __shfl_up_sync(FULL, cum, o, LANES);
+                if (sub >= o) cum += up;
+            }
+            const ull sum_doc = __shfl_sync(FULL, cum, LANES - 1, LANES);
+            const ull total = sum_doc + prior;
+            const ull x = __umul64hi(total, (ull)r << 32);  // floor(total * r / 2^32)
+            // a draw from the smoothing term is left to the token's lane
+            const ull rest = __shfl_sync(FULL, x >= sum_doc ? x - sum_doc : NOT_SMOOTH, lane % TOKENS * LANES);
+            if (lane / TOKENS * TOKENS == t0) x_l = rest;
+            if (cum > x && cum - mine <= x && t0 + group < n) {
+                ull left = x - (cum - mine);  // the first entry whose running sum exceeds it
+                uint32_t chosen = 0;
+                bool found = false;
+#pragma unroll
+                for (int q = 0; q < KEPT; ++q) {
+                    if (q >= part) break;
+                    if (!found) {
+                        chosen = k_r[q];
+                        found = left < m[q];
+                        left -= found ? 0ull : m[q];
+                    }
                 }
-                before = __shfl_sync(FULL, cum, 31);
+                for (int32_t q = KEPT; !found; ++q) {
+                    const ull mass = later(q);
+                    chosen = (uint32_t)__ldg(dk_topic + e0 + e + q);
+                    found = left < mass || q + 1 >= mine_n;
+                    left -= mass;
+                }
+                z_new[i + t] = (int32_t)chosen;
             }
         }
-        if (smooth_l) {
+        if (lane < n && x_l != NOT_SMOOTH) {
             // running sums of the word, set right at the token's own topic: the first that exceeds x
             const ull* pre = prefix + (size_t)w_l * K;
             int32_t lo = 0, hi = K - 1;
@@ -222,9 +263,8 @@ k_gibbs_tokens(View v, const T* __restrict__ z, const int32_t* __restrict__ word
                 const ull c = (ull)((long long)__ldg(pre + mid) + ((uint32_t)mid >= z_l ? delta_l : 0ll));
                 if (c > x_l) hi = mid; else lo = mid + 1;
             }
-            pick_l = (uint32_t)lo;
+            z_new[i + lane] = lo;
         }
-        if (lane < n) z_new[i + lane] = (int32_t)pick_l;
         i += n;
     }
 }
@@ -257,7 +297,9 @@ int lda::gibbs_sweep(Ctx& c, int32_t iters)
         const unsigned grid = (unsigned)((c.N + 8 * run_len - 1) / (8 * run_len));
         auto tokens = [&](auto z) {
             using T = std::remove_const_t<std::remove_pointer_t<decltype(z)>>;
-            const auto kernel = matrix ? k_gibbs_tokens<T, true> : k_gibbs_tokens<T, false>;
+            const bool long_rows = r.total > c.D * (long long)GIBBS_KEPT;
+            const auto kernel = matrix ? (long_rows ? k_gibbs_tokens<T, true, 32> : k_gibbs_tokens<T, true, 16>)
+                                       : (long_rows ? k_gibbs_tokens<T, false, 32> : k_gibbs_tokens<T, false, 16>);
             kernel<<<grid, 256, 0, c.stream>>>(v, z, word_of, r.row_off, r.topic, r.count, prefix, matrix, z_new, key, c.sweep, run_len);
         };
         if (c.wide_topics) tokens(reinterpret_cast<const int32_t*>(v.rec));

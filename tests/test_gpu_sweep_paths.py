@@ -139,3 +139,22 @@ def test_vocabularies_mostly_empty(K, slices):
         _same(g, o)
     else:
         assert np.array_equal(g.get_assignments(), o.get_assignments())
+
+
+@pytest.mark.parametrize("K,short", [(1, 0), (9, 0), (64, 0), (65, 0), (500, 0), (500, 40)])
+def test_exact_conditional_rows_of_every_length(K, short):
+    """Document rows of one topic to hundreds: parts of a row that are kept in registers and parts that are not, turns
+    of one token and of 32; long rows and, with many short documents, rows that are short on average."""
+    lengths = np.array([1, 2, 3, 7, 8, 9, 31, 32, 33, 63, 64, 65, 66, 127, 0, 200, 700, 1_500, 5] + [1] * short)
+    rng = np.random.default_rng(K)
+    words = rng.integers(0, 80, lengths.sum()).astype(np.int32)
+    offsets = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
+    g = binding.LightLDA(80, K, 0.07, 0.013)
+    o = ldaref.Oracle(80, K, 0.07, 0.013)
+    for e in (g, o):
+        e.load_corpus(words, offsets)
+        e.init(6)
+    for _ in range(3):
+        g.gibbs_sweep(1)
+        o.gibbs_sweep(1)
+        assert np.array_equal(g.get_assignments(), o.get_assignments())
