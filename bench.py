@@ -331,8 +331,8 @@ def run_ours(args):
     rho = rho_sum / args.steps
     b_alg = algorithmic_bytes_per_token(M, topic_bytes, rho)
     per_ms = {k: phases["ms_" + k] / args.steps for k in b_alg}
-    kernels = {"propose": "k_word_hot/k_word_cold (pass 1)", "doc_side": "k_doc_tile",
-               "accept": "k_word_hot/k_word_cold (pass 3)", "count_wk": "n_kw rebuild kernels",
+    kernels = {"propose": "k_word_hot/k_word_cold_propose (pass 1)", "doc_side": "k_doc_tile",
+               "accept": "k_word_hot/k_word_cold_accept (pass 3)", "count_wk": "n_kw rebuild kernels",
                "count_k": "k_nk_from_dense/k_nk_from_sparse", "alias_sparse": "k_alias_sparse_*"}
     top = max(per_ms, key=per_ms.get)          # the dominant kernel of the sweep, by measured time
     top_ms = per_ms[top]
