@@ -590,8 +590,10 @@ __device__ __forceinline__ void alias_row_lanes(const View& v, int32_t w, int32_
 
 constexpr int ALIAS_WARP_THREADS = 256;
 constexpr int ALIAS_WARP_SMEM = ALIAS_WARP_THREADS / 32 * ALIAS_WARP_MAX * ALIAS_SCRATCH_PER_ITEM;
-// Rows of up to ALIAS_WARP_MAX items: a warp takes `per_warp` consecutive words, the short rows several at a time.
-__global__ void __launch_bounds__(ALIAS_WARP_THREADS) k_alias_sparse_warp(View v, int32_t w_lo, int32_t w_hi, int32_t per_warp, bool all)
+// Rows of up to ALIAS_WARP_MAX items: a warp takes `per_warp` consecutive words of the list, the short rows several at a
+// time.  The list holds the words that occur (820 000 words, 300 000 tokens: 38 us over the whole vocabulary).
+__global__ void __launch_bounds__(ALIAS_WARP_THREADS)
+k_alias_sparse_warp(View v, const int32_t* __restrict__ list, int32_t n_list, int32_t per_warp, bool all)
 {
     extern __shared__ __align__(16) unsigned char alias_scratch[];
     constexpr int WARPS = ALIAS_WARP_THREADS / 32;
@@ -599,10 +601,10 @@ __global__ void __launch_bounds__(ALIAS_WARP_THREADS) k_alias_sparse_warp(View v
     const int lane = threadIdx.x & 31, wic = threadIdx.x >> 5;
     const Group<WARP> g{nullptr};
     const int32_t stride = (int32_t)((gridDim.x * blockDim.x) >> 5) * per_warp;
-    for (int32_t wb = w_lo + (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per_warp; wb < w_hi; wb += stride) {
-        const int32_t mine = wb + lane;
-        int32_t n_mine = -1, r_mine = 0;
-        if (lane < per_warp && mine < w_hi) {
+    for (int32_t first = (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per_warp; first < n_list; first += stride) {
+        int32_t n_mine = -1, r_mine = 0, mine = 0;
+        if (lane < per_warp && first + lane < n_list) {
+            mine = __ldg(list + first + lane);
             n_mine = v.wk_nnz[mine];
             r_mine = v.row_start[mine];
             if (n_mine == 0) v.sp_mass[mine] = 0;
@@ -615,7 +617,7 @@ __global__ void __launch_bounds__(ALIAS_WARP_THREADS) k_alias_sparse_warp(View v
                 for (int i = 0; i < lane / WD; ++i) rest &= rest - 1;  // this lane's group takes the (lane / WD)-th
                 const int src = rest ? __ffs((int)rest) - 1 : 0;
                 const int32_t n = __shfl_sync(FULL, n_mine, src), r0 = __shfl_sync(FULL, r_mine, src);
-                alias_row_lanes<WD>(v, wb + src, rest ? n : 0, r0, all);
+                alias_row_lanes<WD>(v, __shfl_sync(FULL, mine, src), rest ? n : 0, r0, all);
                 for (int i = 0; i < 32 / WD; ++i) words &= words - 1;
             }
         };
@@ -625,7 +627,7 @@ __global__ void __launch_bounds__(ALIAS_WARP_THREADS) k_alias_sparse_warp(View v
         for (uint32_t words = __ballot_sync(FULL, n_mine > 32 && n_mine <= ALIAS_WARP_MAX); words; words &= words - 1) {
             const int src = __ffs((int)words) - 1;
             const int32_t n = __shfl_sync(FULL, n_mine, src), r0 = __shfl_sync(FULL, r_mine, src);
-            const int32_t w = wb + src;
+            const int32_t w = __shfl_sync(FULL, mine, src);
             ull* de = reinterpret_cast<ull*>(alias_scratch) + (size_t)wic * ALIAS_WARP_MAX;
             ull* wt = de + WARPS * ALIAS_WARP_MAX;
             uint16_t* item = reinterpret_cast<uint16_t*>(reinterpret_cast<ull*>(alias_scratch) + 2 * WARPS * ALIAS_WARP_MAX) +
@@ -739,17 +741,17 @@ int launch_alias_sparse(Ctx& c, bool all, bool begin_sweep)
         k_alias_sparse_long_warp<<<(q.alias_n[0] + 3) / 4, 128, 0, c.side[0]>>>(c.v, words(0), q.alias_n[0], all, c.sc_w);
         ++launches;
     }
-    if (q.w_hi <= q.w_lo) {
+    if (q.present_n <= 0) {
         join_streams(c);
         return launches;
     }
     // words per warp: as many as fill a warp's lanes with the words' sizes, as long as every multiprocessor gets two CTAs
     int per_warp = 32;
-    while (per_warp > 1 && (int64_t)(q.w_hi - q.w_lo) / per_warp < (int64_t)c.n_sm * 16) per_warp /= 2;
-    const int64_t warps = ((int64_t)(q.w_hi - q.w_lo) + per_warp - 1) / per_warp;
+    while (per_warp > 1 && q.present_n / per_warp < c.n_sm * 16) per_warp /= 2;
+    const int64_t warps = ((int64_t)q.present_n + per_warp - 1) / per_warp;
     constexpr int WARPS = ALIAS_WARP_THREADS / 32;
     k_alias_sparse_warp<<<(int)std::min<int64_t>((warps + WARPS - 1) / WARPS, (int64_t)c.n_sm * 16), ALIAS_WARP_THREADS,
-                          ALIAS_WARP_SMEM, c.side[1]>>>(c.v, q.w_lo, q.w_hi, per_warp, all);
+                          ALIAS_WARP_SMEM, c.side[1]>>>(c.v, c.present + q.present_lo, q.present_n, per_warp, all);
     ++launches;
     join_streams(c);
     return launches;

@@ -862,6 +862,8 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
                 q.alias_lo[i] = first_at(alias_words[i], 0, alias_words[i].size(), 1, q.w_lo);
                 q.alias_n[i] = first_at(alias_words[i], 0, alias_words[i].size(), 1, q.w_hi) - q.alias_lo[i];
             }
+            q.present_lo = first_at(present, 0, present.size(), 1, q.w_lo);
+            q.present_n = first_at(present, 0, present.size(), 1, q.w_hi) - q.present_lo;
             q.hotp_lo = first_at(hot_tiles_propose, 0, (size_t)c.n_hot_tiles_propose, 3, q.w_lo);
             q.hotp_n = first_at(hot_tiles_propose, 0, (size_t)c.n_hot_tiles_propose, 3, q.w_hi) - q.hotp_lo;
             q.cold_lo = first_at(cold_tiles, 0, (size_t)c.n_cold_tiles, 4, q.w_lo);
@@ -881,6 +883,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     ListPack lists;
     const int32_t* dense_words_dev = nullptr;
     lists.add(dense_words, &dense_words_dev);
+    lists.add(present, &c.present);
     lists.add(word_tiles, &c.word_tiles);
     lists.add(doc_tiles, &c.doc_tiles);
     lists.add(hot_runs, &c.hot_runs);

@@ -238,6 +238,7 @@ struct Ctx {
     int32_t* doc_sort_long = nullptr;
     // words whose row can exceed ALIAS_CLASS_MAX[i] (each list is part of the one before it)
     int32_t n_alias_words[ALIAS_CLASSES] = {};
+    int32_t* present = nullptr;  // words that occur, ascending
     int32_t* alias_words[ALIAS_CLASSES] = {};
     int32_t n_warm = 0, n_hot_tiles_warm = 0;
     int32_t* warm_words = nullptr;      // [n_warm] words with a sorted row and more tokens than a tail tile holds
@@ -254,6 +255,7 @@ struct Ctx {
         int32_t w_lo = 0, w_hi = 0;        // words [w_lo, w_hi)
         int64_t row_lo = 0, row_n = 0;     // their row slots [row_lo, row_lo + row_n)
         int32_t alias_lo[ALIAS_CLASSES] = {}, alias_n[ALIAS_CLASSES] = {};  // their part of the lists alias_words
+        int32_t present_lo = 0, present_n = 0;  // ... of present
         int32_t hotp_lo = 0, hotp_n = 0;   // ... of hot_tiles_propose
         int32_t cold_lo = 0, cold_n = 0;   // ... of cold_tiles
     };
