@@ -516,22 +516,35 @@ struct ListPack {
     }
 };
 
-// A task beside the caller, on a thread of its own where it is worth one (and one can be had).
+// A task beside the caller, on a thread of its own where it is worth one (and one can be had).  join() says whether
+// it had the memory it needed.
 struct Beside {
     std::thread thread;
+    bool ok = true;
     template <typename F>
     Beside(bool worth_it, F f)
     {
+        const auto task = [this, f] {
+            try {
+                f();
+            } catch (const std::bad_alloc&) {
+                ok = false;
+            }
+        };
         if (worth_it) {
             try {
-                thread = std::thread(f);
+                thread = std::thread(task);
                 return;
             } catch (const std::system_error&) {
             }
         }
-        f();
+        task();
     }
-    void join() { if (thread.joinable()) thread.join(); }
+    bool join()
+    {
+        if (thread.joinable()) thread.join();
+        return ok;
+    }
     ~Beside() { join(); }
 };
 
@@ -624,29 +637,22 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     // tiles of whole documents: for the MH step, and for the sorted n_kd rows (<= SORT_TILE tokens and <= ROW_TILE_WORDS
     // documents each); made beside all that follows (400 000 documents: 1.6 ms on one core)
     std::vector<int32_t> doc_tiles, long_docs, doc_sort_tiles, doc_sort_long;
-    bool doc_lists_ok = true;
     const int32_t tile = c.doc_tile, tile_docs = c.doc_dense ? std::min(dense_docs, tile) : tile;
-    Beside doc_lists(D > 20000, [&, tile, tile_docs] {
-        auto pack = [&](int32_t tokens, int32_t documents, std::vector<int32_t>& tiles, std::vector<int32_t>& longer) {
-            int32_t s0 = 0, tok = 0;
-            auto close = [&](int32_t s1) {
-                if (s1 > s0) { tiles.push_back(s0); tiles.push_back(s1); }
-            };
-            for (int32_t d = 0; d < D; ++d) {
-                const int32_t len = doc_off[d + 1] - doc_off[d];
-                if (len > tokens) { close(d); s0 = d + 1; tok = 0; longer.push_back(d); continue; }
-                if (tok + len > tokens || d - s0 >= documents) { close(d); s0 = d; tok = 0; }
-                tok += len;
-            }
-            close(D);
+    const auto pack = [&](int32_t tokens, int32_t documents, std::vector<int32_t>& tiles, std::vector<int32_t>& longer) {
+        int32_t s0 = 0, tok = 0;
+        auto close = [&](int32_t s1) {
+            if (s1 > s0) { tiles.push_back(s0); tiles.push_back(s1); }
         };
-        try {
-            pack(tile, tile_docs, doc_tiles, long_docs);
-            pack(SORT_TILE, ROW_TILE_WORDS, doc_sort_tiles, doc_sort_long);
-        } catch (const std::bad_alloc&) {
-            doc_lists_ok = false;
+        for (int32_t d = 0; d < D; ++d) {
+            const int32_t len = doc_off[d + 1] - doc_off[d];
+            if (len > tokens) { close(d); s0 = d + 1; tok = 0; longer.push_back(d); continue; }
+            if (tok + len > tokens || d - s0 >= documents) { close(d); s0 = d; tok = 0; }
+            tok += len;
         }
-    });
+        close(D);
+    };
+    Beside doc_lists(D > 20000, [&, tile, tile_docs] { pack(tile, tile_docs, doc_tiles, long_docs); });
+    Beside doc_sort_lists(D > 20000, [&] { pack(SORT_TILE, ROW_TILE_WORDS, doc_sort_tiles, doc_sort_long); });
     int rc = build_layout(c, words_dev, doc_off, temps);
     if (rc != LDA_OK) {
         cudaStreamSynchronize(c.stream);
@@ -676,8 +682,9 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     // which case the row has to hold the counts of all shards
     // The host's lists go over the words present only: a vocabulary may have ten times as many as the corpus uses.
     const int32_t* global_tf = c.shard_global_tf.empty() ? nullptr : c.shard_global_tf.data();
-    const auto tf_here = [&](int32_t w) { return word_off[w + 1] - word_off[w]; };
-    const auto tf = [&](int32_t w) { return global_tf ? std::max(tf_here(w), global_tf[w]) : tf_here(w); };
+    const int32_t* const off = word_off.get();
+    const auto tf_here = [off](int32_t w) { return off[w + 1] - off[w]; };
+    const auto tf = [=](int32_t w) { return global_tf ? std::max(tf_here(w), global_tf[w]) : tf_here(w); };
     std::vector<int32_t> present;
     present.reserve((size_t)std::min<int64_t>(V, global_tf ? V : (int64_t)N));
     for (int32_t w = 0; w < V; ++w)
@@ -686,20 +693,25 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     const int64_t n_top = std::min<int64_t>((int64_t)std::floor(c.dense_frac * (double)V), V);
     if (n_top > 0) {
         // the n_top-th largest frequency -- but a dense row of K counters only pays for a word with a fair share of K
-        // tokens.  Of the words above the cut so far, every 2 n_top-th throws out the lower half.
+        // tokens.  By a count of each frequency, the few very large ones by themselves.
+        constexpr int32_t COUNTED = 1 << 13;
         tf_cut = std::max((int32_t)std::max(1.0, c.dense_min_tf), K / 8);
-        std::vector<int32_t> above;
-        const auto cut_to_top = [&] {
-            std::nth_element(above.begin(), above.begin() + (n_top - 1), above.end(), std::greater<int32_t>());
-            above.resize((size_t)n_top);
-            tf_cut = above.back();
-        };
+        std::vector<int32_t> words_of(COUNTED), above;
+        int32_t most = 0;
         for (const int32_t w : present) {
-            if (tf(w) <= tf_cut) continue;
-            above.push_back(tf(w));
-            if ((int64_t)above.size() >= 2 * n_top) cut_to_top();
+            const int32_t t = tf(w);
+            if (t <= tf_cut) continue;
+            if (t < COUNTED) { ++words_of[(size_t)t]; most = std::max(most, t); }
+            else above.push_back(t);
         }
-        if ((int64_t)above.size() >= n_top) cut_to_top();
+        if ((int64_t)above.size() >= n_top) {
+            std::nth_element(above.begin(), above.begin() + (n_top - 1), above.end(), std::greater<int32_t>());
+            tf_cut = above[(size_t)n_top - 1];
+        } else {
+            int64_t n = (int64_t)above.size();
+            for (int32_t t = most; t > tf_cut; --t)
+                if ((n += words_of[(size_t)t]) >= n_top) tf_cut = t;  // ends the loop
+        }
     }
     // K above the staging limit: only words with more than WARM_MAX_TF tokens get a dense row, the
     // others with more tokens than a tail tile holds a sorted row built by a CTA of their own
@@ -715,9 +727,9 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
         while (r > shortest && tokens / r < per_sm * c.n_sm) r /= 2;
         return std::max(r, shortest);
     };
-    const auto is_hot = [&](int32_t w) { return tf(w) > COLD_TILE; };
-    const auto has_warm_row = [&](int32_t w) { return warm_class && tf(w) > SORT_TILE && tf(w) <= WARM_MAX_TF; };
-    const auto has_dense_row = [&](int32_t w) { return !has_warm_row(w) && (tf(w) > SORT_TILE || tf(w) >= tf_cut); };
+    const auto is_hot = [tf](int32_t w) { return tf(w) > COLD_TILE; };
+    const auto has_warm_row = [=](int32_t w) { return warm_class && tf(w) > SORT_TILE && tf(w) <= WARM_MAX_TF; };
+    const auto has_dense_row = [=](int32_t w) { return !has_warm_row(w) && (tf(w) > SORT_TILE || tf(w) >= tf_cut); };
     int64_t t_hot = 0, t_cold = 0, t_dense = 0, cap_total = 0;
     for (const int32_t w : present) {
         (is_hot(w) ? t_hot : t_cold) += tf_here(w);
@@ -747,35 +759,42 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     std::vector<int64_t> slice_row((size_t)n_slices + 1, cap_total);
     slice_w[0] = 0;
     slice_row[0] = 0;
-    int64_t cap_sum = 0;
-    int32_t end = 0;  // one past the last word seen
-    int sl_next = 1;
-    for (const int32_t w : present) {
-        // (the first word before which there is that much room)
-        for (; sl_next < n_slices && cap_total * sl_next / n_slices <= cap_sum; ++sl_next) {
-            slice_w[(size_t)sl_next] = cap_total * sl_next / n_slices > 0 ? end : 0;
-            slice_row[(size_t)sl_next] = cap_sum;
-        }
-        end = w + 1;
-        const int32_t cap = std::min(tf(w), K);
-        cap_sum += cap;
-        for (int i = 0; i < ALIAS_CLASSES && cap > ALIAS_CLASS_MAX[i]; ++i) alias_words[i].push_back(w);
-        if (has_warm_row(w)) {
-            warm_words.push_back(w);
-        } else if (has_dense_row(w)) {
-            dense_words.push_back(w);
-            const int32_t runs = std::max(1, (tf_here(w) + hist_run - 1) / hist_run);
-            for (int32_t i = 0; i < runs; ++i) {
-                const int32_t o = i * hist_run;
-                hot_runs.insert(hot_runs.end(), {w, word_off[w] + o, std::min(hist_run, tf_here(w) - o),
-                                                 runs > 1 ? (int32_t)acc_runs.size() : -1});
+    if (n_slices > 1) {
+        int64_t cap_sum = 0;
+        int32_t end = 0;  // one past the last word seen
+        int sl = 1;
+        for (const int32_t w : present) {
+            // (the first word before which there is that much room)
+            for (; sl < n_slices && cap_total * sl / n_slices <= cap_sum; ++sl) {
+                slice_w[(size_t)sl] = cap_total * sl / n_slices > 0 ? end : 0;
+                slice_row[(size_t)sl] = cap_sum;
             }
-            if (runs > 1) acc_runs.push_back(runs);
+            end = w + 1;
+            cap_sum += std::min(tf(w), K);
         }
     }
-    c.n_dense = (int32_t)dense_words.size();
+    // The lists of words do not depend on one another (580 000 words: 1 to 2 ms each on one core).
+    const bool many_words = present.size() > 50000;
+    Beside class_lists(many_words, [&, tf, tf_here, has_warm_row, has_dense_row] {
+        for (const int32_t w : present) {
+            const int32_t cap = std::min(tf(w), K);
+            for (int i = 0; i < ALIAS_CLASSES && cap > ALIAS_CLASS_MAX[i]; ++i) alias_words[i].push_back(w);
+            if (has_warm_row(w)) {
+                warm_words.push_back(w);
+            } else if (has_dense_row(w)) {
+                dense_words.push_back(w);
+                const int32_t runs = std::max(1, (tf_here(w) + hist_run - 1) / hist_run);
+                for (int32_t i = 0; i < runs; ++i) {
+                    const int32_t o = i * hist_run;
+                    hot_runs.insert(hot_runs.end(), {w, word_off[w] + o, std::min(hist_run, tf_here(w) - o),
+                                                     runs > 1 ? (int32_t)acc_runs.size() : -1});
+                }
+                if (runs > 1) acc_runs.push_back(runs);
+            }
+        }
+    });
     // tiles of consecutive sparse words: <= row_tile tokens (or one longer word) and <= row_tile_words words each
-    {
+    Beside word_tile_list(many_words, [&, tf, has_dense_row, row_tile, row_tile_words] {
         int32_t s0 = 0, s1 = 0, tok = 0;
         auto close = [&] {
             if (s1 > s0) { word_tiles.push_back(s0); word_tiles.push_back(s1); }
@@ -789,7 +808,7 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
             tok += tf(w);
         }
         close();
-    }
+    });
     // MH kernel work lists: a hot word (more tokens than a tail tile holds; it has a dense row by
     // the rule above) is cut into runs, tail words are packed whole into tiles, one longer than a tile cut
     std::vector<int32_t> hot_tiles, hot_tiles_warm, hot_tiles_propose, cold_tiles;
@@ -824,8 +843,10 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
         }
         close();
     }
-    doc_lists.join();
-    if (!doc_lists_ok) { free_corpus(c); return fail(&c, LDA_ENOMEM, "host allocation failed"); }
+    bool lists_ok = true;
+    for (Beside* b : {&doc_lists, &doc_sort_lists, &word_tile_list, &class_lists}) lists_ok = b->join() && lists_ok;
+    if (!lists_ok) { free_corpus(c); return fail(&c, LDA_ENOMEM, "host allocation failed"); }
+    c.n_dense = (int32_t)dense_words.size();
     c.n_doc_sort_tiles = (int32_t)(doc_sort_tiles.size() / 2);
     c.n_doc_sort_long = (int32_t)doc_sort_long.size();
     c.n_word_tiles = (int32_t)(word_tiles.size() / 2);
