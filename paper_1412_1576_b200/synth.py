@@ -31,6 +31,7 @@ from __future__ import annotations
 import math
 from dataclasses import dataclass, field
 
+import numpy as np
 import torch
 
 # The five workloads.  "mh_steps" is the number of individual MH proposals per
@@ -112,6 +113,21 @@ def _lengths(kind, D: int, gen: torch.Generator, dev) -> torch.Tensor:
     raise ValueError(f"unknown length law {kind!r}")
 
 
+def _zipf_cdf(V: int, s: float, dev) -> torch.Tensor:
+    """Cumulative Zipf(s) distribution over the ranks 1..V.
+
+    On CUDA a floating-point cumsum adds in an order that changes from call to call, and two calls differ in their
+    last bits: one draw in 5 * 10^9 at V = 10^6 then gives another word.  There the weights are added up on
+    the host, in order and in extended precision, which is as close to the device's sums as those are to each other.
+    """
+    weights = torch.arange(1, V + 1, dtype=torch.float64, device=dev).pow(-s)
+    if dev.type != "cuda":
+        cdf = torch.cumsum(weights, 0)
+        return cdf / cdf[-1]
+    cdf = np.cumsum(weights.cpu().numpy().astype(np.longdouble))
+    return torch.from_numpy((cdf / cdf[-1]).astype(np.float64)).to(dev)
+
+
 def generate(V: int, K: int, D: int, length, zipf_s, alpha: float, beta: float,
              seed: int = 0, device: str = "cpu", **_unused) -> Corpus:
     """Draw a corpus from the collapsed LDA generative process described above."""
@@ -151,12 +167,10 @@ def generate(V: int, K: int, D: int, length, zipf_s, alpha: float, beta: float,
     if zipf_s is None:
         fresh_rank = torch.randint(0, V, (N,), generator=gen, device=dev, dtype=torch.int64)
     else:
-        ranks = torch.arange(1, V + 1, dtype=torch.float64, device=dev)
-        cdf = torch.cumsum(ranks.pow(-float(zipf_s)), 0)
-        cdf = cdf / cdf[-1]
+        cdf = _zipf_cdf(V, float(zipf_s), dev)
         u = torch.rand(N, generator=gen, device=dev, dtype=torch.float64)
         fresh_rank = torch.clamp(torch.searchsorted(cdf, u), max=V - 1)
-        del u, cdf, ranks
+        del u, cdf
     perm = torch.randperm(V, generator=gen, device=dev)
     w_sorted = perm[fresh_rank[root]]
     del fresh_rank, root
