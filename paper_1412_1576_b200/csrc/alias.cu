@@ -188,6 +188,7 @@ __device__ ull build_alias_row(const Group<KIND>& g, int32_t n, Weight weight, u
             atomicOr(err, ERR_ALIAS);
             if (!FINISH) *sums = RowSums{0, 0, 0, 0};
         }
+        g.sync();  // no CTA of a cluster leaves while another may read its shared memory (reduce())
         return W44;
     }
     // Every thread takes a run of consecutive items (lights and heavies are numbered in ascending
@@ -394,6 +395,10 @@ __global__ void __launch_bounds__(1024) k_alias_dense(View v, ull* sc)
     DenseWeight wf{v.nk, v.beta, v.Vbeta};
     const ull B = build_alias_row<KIND, KIND == CTA>(g, K, wf, sc, sc + K, (uint32_t*)(sc + 2 * (size_t)K),
                                                      DenseOut{v.dn_thr, v.dn_idx, v.dn_pk}, v.err, dense_sums(sc, K));
+    // A table without mass (beta so small that every weight is floored to zero) raises the error word and gets no bins;
+    // the proposals that are drawn all the same stay topics of the model.
+    if (B == 0 && v.dn_pk)
+        for (int32_t k = g.rank(); k < K; k += g.size()) v.dn_pk[k] = make_uint2(0xFFFFFFFFu, (uint32_t)k);
     if (g.rank() == 0) {
         *v.dense_mass = B;
         if (v.state) v.state->stamps[v.state->slot][STAMP_DENSE_END] = global_timer();

@@ -1,0 +1,43 @@
+"""Calls at the limits of what the library accepts: priors that leave a table without mass."""
+import numpy as np
+import pytest
+
+from oracle import ldaref
+from paper_1412_1576_b200 import binding, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("K", [16, 2_048, 2_049])
+def test_dense_table_without_mass(K):
+    """beta / (n_k + V beta) below 2^-44 for every topic, on one CTA and on a cluster: an error, and the context can be
+    used again; so can others."""
+    import torch
+    c = synth.generate(V=40, K=K, D=60, length=("fixed", 1_000), zipf_s=None, alpha=0.1, beta=0.01, seed=K)
+    w, off = c.word_ids.numpy(), c.doc_offsets.numpy()
+    g = binding.LightLDA(c.V, c.K, c.alpha, 1e-300)
+    g.load_corpus(w, off)
+    for _ in range(2):
+        g.init(3)
+        assert g.get_nk().min() > 0          # else that topic would have a mass
+        with pytest.raises(binding.LdaError) as e:
+            g.sweep(3, 2)
+        assert e.value.status == binding.LDA_EINTERNAL
+        with pytest.raises(binding.LdaError) as e:
+            g.sweep(1, 2)
+        assert e.value.status == binding.LDA_ESTATE
+    g.init(3)
+    nk = torch.from_numpy(g.get_nk()).cuda()
+    thr, al = torch.zeros(K, dtype=torch.int32, device="cuda"), torch.zeros(K, dtype=torch.int32, device="cuda")
+    mass, status = torch.ones(1, dtype=torch.int64, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    assert binding.lda_dense_table_noalloc(nk.data_ptr(), K, c.V, 1e-300, thr.data_ptr(), al.data_ptr(), mass.data_ptr(),
+                                           status.data_ptr()) == binding.LDA_OK
+    torch.cuda.synchronize()
+    assert int(status) != 0 and int(mass) == 0
+    h, o = binding.LightLDA(c.V, c.K, c.alpha, 0.01), ldaref.Oracle(c.V, c.K, c.alpha, 0.01)
+    for e in (h, o):
+        e.load_corpus(w, off)
+        e.init(3)
+        e.sweep(2, 2)
+    assert np.array_equal(h.get_assignments(), o.get_assignments())
