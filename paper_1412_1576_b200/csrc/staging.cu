@@ -135,7 +135,12 @@ static cudaError_t move_bytes(Ctx& c, void* host, void* dev, size_t bytes)
             return e;
         }
     }
-    return TO_HOST ? cudaMemcpy(host, dev, bytes, cudaMemcpyDeviceToHost) : cudaMemcpy(dev, host, bytes, cudaMemcpyHostToDevice);
+    // on the context's stream: a copy on the default stream may return before the data has arrived, and nothing orders
+    // a non-blocking stream behind that
+    e = TO_HOST ? cudaMemcpyAsync(host, dev, bytes, cudaMemcpyDeviceToHost, c.stream)
+                : cudaMemcpyAsync(dev, host, bytes, cudaMemcpyHostToDevice, c.stream);
+    const cudaError_t done = cudaStreamSynchronize(c.stream);
+    return e != cudaSuccess ? e : done;
 }
 
 cudaError_t copy_to_host(Ctx& c, void* host, const void* dev, size_t bytes)

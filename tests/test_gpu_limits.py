@@ -41,3 +41,42 @@ def test_dense_table_without_mass(K):
         e.init(3)
         e.sweep(2, 2)
     assert np.array_equal(h.get_assignments(), o.get_assignments())
+
+
+def _loaded(c, stream):
+    g = binding.LightLDA(c.V, c.K, c.alpha, c.beta, stream=stream)
+    g.load_corpus(c.word_ids.numpy(), c.doc_offsets.numpy())
+    g.init(5)
+    g.sweep(1, 2)
+    return g
+
+
+def test_host_corpora_on_streams_of_their_own(small_corpus, tiny_corpus):
+    """Loading on a stream that no other is ordered with: corpora small enough for one copy, and larger ones by several
+    threads at once, of which one has the page-locked buffers."""
+    import threading
+
+    import torch
+    want = {}
+    for c in (tiny_corpus, small_corpus):
+        o = ldaref.Oracle(c.V, c.K, c.alpha, c.beta)
+        o.load_corpus(c.word_ids.numpy(), c.doc_offsets.numpy())
+        o.init(5)
+        o.sweep(1, 2)
+        want[id(c)] = o.get_assignments()
+    torch.cuda.synchronize()
+    for _ in range(10):
+        g = _loaded(tiny_corpus, torch.cuda.Stream().cuda_stream)
+        assert np.array_equal(g.get_assignments(), want[id(tiny_corpus)])
+    got, streams = [None] * 4, [torch.cuda.Stream() for _ in range(4)]
+
+    def load(i):
+        torch.cuda.set_device(0)
+        got[i] = [_loaded(small_corpus, streams[i].cuda_stream).get_assignments() for _ in range(3)]
+    threads = [threading.Thread(target=load, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for z in [z for zs in got for z in zs]:
+        assert np.array_equal(z, want[id(small_corpus)])
