@@ -1154,7 +1154,10 @@ int lda_load_corpus_device(lda_ctx* h, const int32_t* word_ids_dev, int64_t n_to
     int rc = check_device(c);
     if (rc) return rc;
     std::vector<int64_t> off((size_t)n_docs + 1);
-    if (copy_to_host(c, off.data(), doc_offsets_dev, ((size_t)n_docs + 1) * 8) != cudaSuccess)
+    // the offsets come after what the default stream has queued, as a copy on that stream does, whatever the
+    // context's stream is
+    if (cudaEventRecord(c.ev_chunk, cudaStreamLegacy) != cudaSuccess || cudaStreamWaitEvent(c.stream, c.ev_chunk, 0) != cudaSuccess ||
+        copy_to_host(c, off.data(), doc_offsets_dev, ((size_t)n_docs + 1) * 8) != cudaSuccess)
         return cuda_fail(&c, "copying doc offsets");
     Documents docs;
     if ((rc = scan_documents(&c, n_tokens, off.data(), n_docs, docs))) return rc;

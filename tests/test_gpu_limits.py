@@ -80,3 +80,20 @@ def test_host_corpora_on_streams_of_their_own(small_corpus, tiny_corpus):
         t.join()
     for z in [z for zs in got for z in zs]:
         assert np.array_equal(z, want[id(small_corpus)])
+
+
+@pytest.mark.parametrize("n_docs", [2_000, 400_000])
+def test_device_offsets_still_on_their_way(n_docs):
+    """Offsets that the default stream is about to write, read by a context on a stream that is not ordered with it."""
+    import torch
+    words = torch.randint(0, 50, (2 * n_docs,), dtype=torch.int32, device="cuda")
+    offsets = torch.zeros(n_docs + 1, dtype=torch.int64, device="cuda")
+    ready = torch.arange(0, 2 * n_docs + 1, 2, dtype=torch.int64, device="cuda")
+    g = binding.LightLDA(50, 20, 0.1, 0.01, stream=torch.cuda.Stream().cuda_stream)
+    torch.cuda.synchronize()
+    torch.cuda._sleep(100_000_000)   # some 50 ms
+    offsets.copy_(ready)
+    assert binding.lda_load_corpus_device(g._h, words.data_ptr(), 2 * n_docs, offsets.data_ptr(), n_docs) == binding.LDA_OK
+    g.N, g.D = 2 * n_docs, n_docs
+    g.init(1)
+    assert int(g.get_nk().sum()) == 2 * n_docs
