@@ -270,7 +270,7 @@ static void free_corpus(Ctx& c)
     nv.state = c.v.state;
     nv.err = &nv.state->err;
     c.v = nv;
-    c.loaded = c.inited = c.tables_valid = false;
+    c.loaded = c.inited = c.tables_valid = c.wide_counts = false;
     c.N = c.D = 0;
     c.side_steps = 0;
     c.slices.clear();
@@ -352,8 +352,15 @@ int lda::ensure_exchange(Ctx& c, int mh_steps)
 
 namespace lda {
 
+void set_wide_counts(Ctx& c, bool wide)
+{
+    if (c.wide_counts != wide && c.cold_direct) drop_graphs(c);  // the accept pass takes another kernel
+    c.wide_counts = wide;
+}
+
 void rebuild_counts(Ctx& c)
 {
+    set_wide_counts(c, false);
     cudaMemsetAsync(c.v.nk_next, 0, (size_t)c.v.dense_stride * 4, c.stream);
     launch_count_wk(c);
     launch_count_k(c);
@@ -1342,7 +1349,8 @@ int lda_word_counts_from_dense(lda_ctx* h, const int32_t* nwk_dev)
     c.tables_valid = false;
     int bits = 0;
     if ((rc = read_err(c, &bits))) { c.inited = false; return rc; }
-    if (bits) {
+    set_wide_counts(c, (bits & NOTE_WIDE_COUNT) != 0);
+    if (bits & ~NOTE_WIDE_COUNT) {
         c.inited = false;
         return fail(&c, LDA_ERANGE,
                     "the matrix has negative entries or more nonzeros in a row than the term frequencies given to lda_set_shard allow");

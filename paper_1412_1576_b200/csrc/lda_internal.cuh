@@ -46,6 +46,7 @@ enum : int {
     ERR_TOPIC_RANGE = 8,  // an assignment outside [0,K)
     ERR_ALIAS = 16,       // alias construction met an impossible state
     ERR_STAGE = 32,       // a bulk copy into shared memory did not complete within its wait limit
+    NOTE_WIDE_COUNT = 64, // no error: an imported count of a tail word does not fit 16 bits (shard.cu)
 };
 
 constexpr uint32_t DK_EMPTY = 0xFFFFFFFFu;  // == DK_EMPTY_SLOT of the device helpers
@@ -227,7 +228,8 @@ struct Ctx {
     int32_t* acc = nullptr;          // [words with several runs][dense_stride], zero between rebuilds
     int32_t* acc_done = nullptr;     // [...] runs of the word that are done, zero between rebuilds
     int32_t* acc_runs = nullptr;     // [...] runs of the word
-    bool cold_direct = false;        // the accept pass keeps the tail tiles' rows as counters
+    bool cold_direct = false;        // the accept pass keeps the tail tiles' rows as 16-bit counters
+    bool wide_counts = false;        // ... unless n_kw was imported with larger counts in tail words
     int nk_mode = 0;                 // how the row kernels add up n_k
     int32_t n_long_chunks = 0;
     int32_t* long_chunks = nullptr;  // [n_long_chunks*4] (index into View::long_docs, first token, count, 0)
@@ -386,6 +388,7 @@ int launch_count_k(Ctx& c);      // n_k of the rows just rebuilt, added to View:
                                  // row kernels have done it
 int launch_count_k_from_rows(Ctx& c);  // ... in any case
 void rebuild_counts(Ctx& c);     // n_kw and n_k from the assignments, outside a sweep
+void set_wide_counts(Ctx& c, bool wide);
 void choose_nk_mode(Ctx& c);     // after the work lists are made
 inline void exchange_nk(Ctx& c) { int32_t* t = c.v.nk; c.v.nk = c.v.nk_next; c.v.nk_next = t; }
 int launch_begin_sweep(Ctx& c);  // first kernel of a sweep that needs no tables

@@ -211,6 +211,7 @@ struct ColdBins {
 //   - otherwise the sorted rows, searched by bisection.  Hashed rows were measured too: what the lookups
 //     gain (2 probes for 5 to 11 steps) the tables' construction costs again, a row of these words having
 //     about as many entries as three tokens have lookups (738 M tokens, K = 10 000: 1.43 against 1.39 ms).
+// (Counts that lda_word_counts_from_dense() brought in may be larger than the word's tokens: Ctx::wide_counts.)
 static_assert(COLD_TILE < 65536, "a tail word's counts fit 16 bits");
 template <bool DIRECT>
 struct ColdRows {
@@ -804,7 +805,8 @@ static int launch_accept(Ctx& c, uint2 key, int mh_steps)
         ++launches;
     }
     if (c.n_cold_tiles) {
-        const auto kernel = c.cold_direct ? k_word_cold_accept<T, CH, MODE, FIXED, true> : k_word_cold_accept<T, CH, MODE, FIXED, false>;
+        const bool direct = c.cold_direct && !c.wide_counts;
+        const auto kernel = direct ? k_word_cold_accept<T, CH, MODE, FIXED, true> : k_word_cold_accept<T, CH, MODE, FIXED, false>;
         kernel<<<c.n_cold_tiles, COLD_THREADS, 0, on[1]>>>(v, reinterpret_cast<const int4*>(c.cold_tiles), mh_steps, STAMP_ACCEPT_COLD);
         ++launches;
     }

@@ -97,3 +97,31 @@ def test_device_offsets_still_on_their_way(n_docs):
     g.N, g.D = 2 * n_docs, n_docs
     g.init(1)
     assert int(g.get_nk().sum()) == 2 * n_docs
+
+
+def test_imported_counts_beyond_16_bits():
+    """Counts of tail words that lda_word_counts_from_dense brings in may be larger than any corpus's: tiles whose rows are
+    otherwise 16-bit counters, sweeps on both sides of the import, replayed ones among them."""
+    import torch
+    c = synth.generate(V=50, K=100, D=60, length=("fixed", 25), zipf_s=None, alpha=0.1, beta=0.01, seed=2)
+    g, o = binding.LightLDA(c.V, c.K, c.alpha, c.beta), ldaref.Oracle(c.V, c.K, c.alpha, c.beta)
+    for e in (g, o):
+        e.load_corpus(c.word_ids.numpy(), c.doc_offsets.numpy())
+        e.init(9)
+    m, m_host = torch.zeros(c.V * c.K, dtype=torch.int32, device="cuda"), np.zeros(c.V * c.K, np.int32)
+    for times in (1, 70_001, 1, 65_535, 70_001):
+        for e in (g, o):
+            e.sweep(4, 2)
+        g.word_counts_to_dense(m)
+        o.word_counts_to_dense(m_host)
+        assert np.array_equal(m.cpu().numpy(), m_host)
+        m *= times
+        m_host *= times
+        torch.cuda.synchronize()
+        g.word_counts_from_dense(m)
+        o.word_counts_from_dense(m_host)
+        assert np.array_equal(g.get_nk(), o.get_nk())
+        for iters in (1, 3):
+            for e in (g, o):
+                e.sweep(iters, 2)
+            assert np.array_equal(g.get_assignments(), o.get_assignments()), (times, iters)
