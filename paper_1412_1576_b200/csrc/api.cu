@@ -482,15 +482,16 @@ static int scan_documents(Ctx* c, int64_t n_tokens, const int64_t* doc_off, int6
     if (doc_off[0] != 0 || doc_off[n_docs] != n_tokens)
         return fail(c, LDA_ERANGE, "doc_offsets must start at 0 and end at n_tokens");
     docs.off.resize((size_t)n_docs + 1);
-    int64_t shortest = 0;
+    bool ordered = true;  // by comparison: the difference of two offsets that are not in order may wrap
     for (int64_t d = 0; d < n_docs; ++d) {
-        const int64_t len = doc_off[d + 1] - doc_off[d];
-        shortest = std::min(shortest, len);
+        const int64_t a = doc_off[d], b = doc_off[d + 1];
+        ordered = ordered && a <= b;
+        const int64_t len = (int64_t)((uint64_t)b - (uint64_t)a);
         docs.longest = std::max(docs.longest, len);
         docs.nonempty += len > 0;
-        docs.off[(size_t)d + 1] = (int32_t)doc_off[d + 1];
+        docs.off[(size_t)d + 1] = (int32_t)b;
     }
-    if (shortest < 0) return fail(c, LDA_ERANGE, "doc_offsets must be non-decreasing");
+    if (!ordered) return fail(c, LDA_ERANGE, "doc_offsets must be non-decreasing");
     return LDA_OK;
 }
 

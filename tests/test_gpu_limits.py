@@ -125,3 +125,14 @@ def test_imported_counts_beyond_16_bits():
             for e in (g, o):
                 e.sweep(iters, 2)
             assert np.array_equal(g.get_assignments(), o.get_assignments()), (times, iters)
+
+
+@pytest.mark.parametrize("offsets", [[0, 2, 1, 4], [0, -1, 4], [0, 5, 4], [0, 2 ** 63 - 1, -2 ** 63, -2 ** 62, 4],
+                                     [0, 2 ** 62, 2 ** 63 - 1, -2 ** 63, -2 ** 62, 0, 4]])
+def test_offsets_out_of_order_are_refused(offsets):
+    """Also those whose differences, taken in 64 bits, are all positive."""
+    words = np.zeros(4, np.int32)
+    g = binding.LightLDA(3, 2, 0.1, 0.01)
+    assert binding.lda_load_corpus(g._h, words, np.array(offsets, np.int64)) == binding.LDA_ERANGE
+    assert "non-decreasing" in binding.lda_last_error(g._h)
+    assert binding.lda_load_corpus(g._h, words, np.array([0, 0, 3, 4, 4], np.int64)) == binding.LDA_OK
