@@ -158,9 +158,27 @@ static int build_dk_csr_t(Ctx& c, DkCsr& r, bool sizes_only)
     if (c.n_doc_sort_long)
         k_long_doc_rows<T, false><<<c.n_doc_sort_long, 512, (size_t)win * 4, c.stream>>>(
             c.doc_sort_long, v.doc_off, z, c.K, win, r.nnz, nullptr, nullptr, nullptr, v.err);
+    // the entries apart are a convenience: without the room for them beside the rest, the sorting kernel makes the rows
+    const auto drop_entries = [&] {
+        cudaStreamSynchronize(c.stream);
+        raw_free(c, topic_at);
+        raw_free(c, count_at);
+        topic_at = count_at = nullptr;
+    };
     int rc = row_offsets(c, r.nnz, r.row_off, D, &r.total);
+    if (rc == LDA_ENOMEM && topic_at) {
+        drop_entries();
+        rc = row_offsets(c, r.nnz, r.row_off, D, &r.total);
+    }
     const size_t cap = (size_t)(r.total > 0 ? r.total : 1);
-    if (rc == LDA_OK && !sizes_only && (!tmp_alloc(c, &r.topic, cap * 4) || !tmp_alloc(c, &r.count, cap * 4))) rc = LDA_ENOMEM;
+    const auto room = [&] { return (r.topic || tmp_alloc(c, &r.topic, cap * 4)) && tmp_alloc(c, &r.count, cap * 4); };
+    if (rc == LDA_OK && !sizes_only && !room()) {
+        rc = LDA_ENOMEM;
+        if (topic_at) {
+            drop_entries();
+            if (room()) rc = LDA_OK;
+        }
+    }
     if (rc == LDA_OK && !sizes_only) {
         if (topic_at) {
             // the rows of the documents longer than a tile are written over below
@@ -172,11 +190,7 @@ static int build_dk_csr_t(Ctx& c, DkCsr& r, bool sizes_only)
             k_long_doc_rows<T, true><<<c.n_doc_sort_long, 512, (size_t)win * 4, c.stream>>>(
                 c.doc_sort_long, v.doc_off, z, c.K, win, nullptr, r.row_off, r.topic, r.count, v.err);
     }
-    if (topic_at) {
-        cudaStreamSynchronize(c.stream);
-        raw_free(c, topic_at);
-        raw_free(c, count_at);
-    }
+    if (topic_at) drop_entries();
     if (rc != LDA_OK) free_dk_csr(c, r);
     return rc;
 }

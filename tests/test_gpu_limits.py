@@ -136,3 +136,61 @@ def test_offsets_out_of_order_are_refused(offsets):
     assert binding.lda_load_corpus(g._h, words, np.array(offsets, np.int64)) == binding.LDA_ERANGE
     assert "non-decreasing" in binding.lda_last_error(g._h)
     assert binding.lda_load_corpus(g._h, words, np.array([0, 0, 3, 4, 4], np.int64)) == binding.LDA_OK
+
+
+class _Budget:
+    """A context's device memory from PyTorch's pool, refused beyond `left` bytes once that is set."""
+
+    def __init__(self):
+        self.left, self.sizes = None, {}
+        alloc, free = binding.torch_caching_allocator(None)
+
+        def take(n, user):
+            if self.left is not None and n > self.left:
+                return None
+            p = alloc(n, user)
+            if p and self.left is not None:
+                self.left -= n
+                self.sizes[p] = n
+            return p
+
+        def give(p, user):
+            if self.left is not None and p:
+                self.left += self.sizes.pop(p, 0)
+            free(p, user)
+        self.functions = binding.ALLOC_FN(take), binding.FREE_FN(give)
+
+    def context(self, c, seed):
+        g = binding.LightLDA(c.V, c.K, c.alpha, c.beta, allocator="cuda")
+        g._allocator = self.functions     # alive as long as the context
+        assert binding.lda_set_allocator(g._h, *self.functions) == 0
+        g.load_corpus(c.word_ids.numpy(), c.doc_offsets.numpy())
+        g.init(seed)
+        return g
+
+
+def _pair_with_budget(K=100, D=1_000):
+    c = synth.generate(V=2_000, K=K, D=D, length=("fixed", 100), zipf_s=1.0, alpha=0.1, beta=0.01, seed=4)
+    b, o = _Budget(), ldaref.Oracle(c.V, c.K, c.alpha, c.beta)
+    o.load_corpus(c.word_ids.numpy(), c.doc_offsets.numpy())
+    o.init(8)
+    return c, b, b.context(c, 8), o
+
+
+SPARE = 64 << 10   # scans' temporary storage
+
+
+def test_document_rows_in_the_room_they_need():
+    """Offsets, sizes and entries are all the device memory that the n_kd rows may insist on."""
+    c, b, g, o = _pair_with_budget()
+    want = o.get_csr(ldaref.NDK)
+    for left in (12 * (c.n_docs + 1) + 8 * want[1].size + SPARE, 12 * (c.n_docs + 1) + 8 * c.n_tokens + SPARE, 1 << 40):
+        b.left = left
+        for x, y in zip(g.get_csr(binding.LDA_NDK), want):
+            assert np.array_equal(x, y)
+        assert b.left == left      # all of it went back
+    b.left = 4 * want[1].size
+    with pytest.raises(binding.LdaError) as e:
+        g.get_csr(binding.LDA_NDK)
+    assert e.value.status == binding.LDA_ENOMEM and b.left == 4 * want[1].size
+    b.left = None
