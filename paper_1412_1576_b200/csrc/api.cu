@@ -1404,6 +1404,34 @@ int lda_loglik(lda_ctx* h, double* total, double* word_ll, double* doc_ll)
     return LDA_OK;
 }
 
+// The n_kw rows without any device memory: they are copied as they lie, room behind them included, and put together here.
+static int word_rows_by_host(Ctx& c, int64_t* row_offsets, int32_t* topics, int32_t* counts, int64_t capacity, int64_t* nnz_out)
+{
+    const View& v = c.v;
+    const size_t V = (size_t)c.V;
+    std::vector<int32_t> nnz(V), start(V + 1), entries;
+    if (copy_to_host(c, nnz.data(), v.wk_nnz, V * 4) != cudaSuccess || copy_to_host(c, start.data(), v.row_start, (V + 1) * 4) != cudaSuccess)
+        return cuda_fail(&c, "copying row sizes");
+    int64_t total = 0;
+    for (const int32_t n : nnz) total += n;
+    if (nnz_out) *nnz_out = total;
+    if (!row_offsets && !topics && !counts) return LDA_OK;
+    if (capacity < total) return fail(&c, LDA_ERANGE, "capacity below the number of nonzeros");
+    if (row_offsets) {
+        row_offsets[0] = 0;
+        for (size_t w = 0; w < V; ++w) row_offsets[w + 1] = row_offsets[w] + nnz[w];
+    }
+    const std::pair<int32_t*, const uint32_t*> columns[2] = {{topics, v.wk_topic}, {counts, v.wk_count}};
+    for (const auto& [to, from] : columns) {
+        if (!to || !total) continue;
+        entries.resize((size_t)start[V]);
+        if (copy_to_host(c, entries.data(), from, entries.size() * 4) != cudaSuccess) return cuda_fail(&c, "copying the n_kw rows");
+        int32_t* out = to;
+        for (size_t w = 0; w < V; ++w) out = std::copy_n(entries.begin() + start[w], nnz[w], out);
+    }
+    return LDA_OK;
+}
+
 int lda_get_counts(lda_ctx* h, int which, int64_t* row_offsets, int32_t* topics, int32_t* counts,
                    int64_t capacity, int64_t* nnz_out)
 {
@@ -1448,7 +1476,9 @@ int lda_get_counts(lda_ctx* h, int which, int64_t* row_offsets, int32_t* topics,
     if (which != LDA_NWK) return fail(&c, LDA_EINVAL, "unknown table");
     const bool sizes_only = !row_offsets && !topics && !counts;
     WkCsr r;
-    if ((rc = build_wk_csr(c, r, sizes_only))) return fail(&c, rc, "building the n_kw rows failed");
+    rc = build_wk_csr(c, r, sizes_only);
+    if (rc == LDA_ENOMEM) return word_rows_by_host(c, row_offsets, topics, counts, capacity, nnz_out);
+    if (rc) return fail(&c, rc, "building the n_kw rows failed");
     const int64_t total = (int64_t)r.total;
     if (nnz_out) *nnz_out = total;
     if (!sizes_only && capacity < total) {

@@ -194,3 +194,24 @@ def test_document_rows_in_the_room_they_need():
         g.get_csr(binding.LDA_NDK)
     assert e.value.status == binding.LDA_ENOMEM and b.left == 4 * want[1].size
     b.left = None
+
+
+def test_word_rows_without_device_memory():
+    """The n_kw rows lie in device memory already: to read them takes no more of it, if there is none."""
+    c, b, g, o = _pair_with_budget()
+    for sweep in range(2):
+        want = o.get_csr(ldaref.NWK)
+        nnz = want[1].size
+        for left in (0, 8 * (c.V + 1), 8 * (c.V + 1) + SPARE + 4 * nnz, 1 << 40):
+            b.left = left
+            for x, y in zip(g.get_csr(binding.LDA_NWK), want):
+                assert np.array_equal(x, y)
+            assert b.left == left
+        b.left = 0
+        column = np.zeros(nnz, np.int32)
+        assert binding.lda_get_counts(g._h, binding.LDA_NWK, None, None, column) == (binding.LDA_OK, nnz)
+        assert np.array_equal(column, want[2])
+        assert binding.lda_get_counts(g._h, binding.LDA_NWK, None, column[1:], None) == (binding.LDA_ERANGE, nnz)
+        b.left = None
+        for e in (g, o):
+            e.sweep(1, 2)
