@@ -290,7 +290,14 @@ int lda::gibbs_sweep(Ctx& c, int32_t iters)
     if (rc == LDA_OK && c.N > 0) k_word_of_tokens<<<(unsigned)((c.N + WORD_OF_RUN - 1) / WORD_OF_RUN), 256, 0, c.stream>>>(v, word_of);
     for (int32_t it = 0; rc == LDA_OK && it < iters && c.N > 0; ++it) {
         DkCsr r;
-        if ((rc = build_dk_csr(c, r, false))) break;  // also leaves z in document order in the record array
+        rc = build_dk_csr(c, r, false);  // also leaves z in document order in the record array
+        if (rc == LDA_ENOMEM && matrix) {  // the rows are needed, the matrix is not
+            cudaStreamSynchronize(c.stream);
+            raw_free(c, matrix);
+            matrix = nullptr;
+            rc = build_dk_csr(c, r, false);
+        }
+        if (rc) break;
         k_gibbs_prior_prefix<<<c.V, 256, (size_t)c.K * 4, c.stream>>>(v, prefix, matrix);
         int32_t run_len = GIBBS_RUN;
         while (run_len > 4 && c.N / run_len < (int64_t)c.n_sm * 32) run_len /= 2;

@@ -215,3 +215,23 @@ def test_word_rows_without_device_memory():
         b.left = None
         for e in (g, o):
             e.sweep(1, 2)
+
+
+def test_exact_conditional_sweep_without_room_for_the_matrix():
+    """Beside the running sums the sweep insists on the documents' rows, not on n_kw as a matrix."""
+    c, b, g, o = _pair_with_budget()
+    rows = 12 * (c.n_docs + 1) + 8 * c.n_tokens
+    matrix = 4 * c.V * c.K
+    assert rows > SPARE and matrix > SPARE
+    needed = 8 * c.n_tokens + 8 * c.V * c.K
+    for left in (needed + max(rows, matrix) + SPARE, needed + rows + matrix + 8 * c.n_tokens + SPARE, 1 << 40):
+        b.left = left
+        g.gibbs_sweep(2)
+        assert b.left == left
+        o.gibbs_sweep(2)
+        assert np.array_equal(g.get_assignments(), o.get_assignments())
+    b.left = needed + rows // 4
+    with pytest.raises(binding.LdaError) as e:
+        g.gibbs_sweep(1)
+    assert e.value.status == binding.LDA_ENOMEM
+    b.left = None
