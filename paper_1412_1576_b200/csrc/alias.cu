@@ -437,6 +437,8 @@ __global__ void __launch_bounds__(256) k_alias_dense_bins(View v, ull* sc)
         }
         out.bin(k, frac(part), al);
     }
+    // all CTAs run at once: the last one's time is the table's
+    if (v.state && blockIdx.x + 1 == gridDim.x && threadIdx.x == 0) v.state->stamps[v.state->slot][STAMP_DENSE_END] = global_timer();
 }
 
 static int dense_launches(int32_t K) { return K > DENSE_CTA_MAX_K ? 2 : 1; }
