@@ -169,6 +169,26 @@ def test_big_shape_sample_against_oracle():
         assert x == pytest.approx(y, rel=1e-9)
 
 
+@pytest.mark.parametrize("workload,scale", [("mid", 0.2), ("big", 0.03)])
+def test_replayed_sweeps_above_the_small_corpora(workload, scale):
+    """Corpora above 2^24 tokens (passes one after the other, n_k by a pass of its own) for five sweeps: the later ones
+    are replayed as a graph.  Every token after each of the two calls, and every count."""
+    if _free_gib() < 12 or _host_gib() < 12:
+        pytest.skip("needs 12 GB of device and of host memory")
+    c = synth.make(workload, seed=1, device="cuda", scale=scale)
+    assert c.n_tokens > 1 << 24
+    g, o, w, off = _gpu_and_oracle(c, 55)
+    del c
+    for iters in (3, 2):
+        g.sweep(iters, 2)
+        o.sweep_threads(iters, 2, CORES)
+        assert np.array_equal(g.get_assignments(), o.get_assignments()), iters
+    assert np.array_equal(g.get_nk(), o.get_nk())
+    for which in (binding.LDA_NWK, binding.LDA_NDK):
+        for x, y in zip(g.get_csr(which), o.get_csr(which)):
+            assert np.array_equal(x, y)
+
+
 def test_big_full_size_invariants_and_sampled_tokens():
     """Config 5 at its full size (~1 G tokens, 105 GB on the device): the counts must be those of the
     library's own assignments, and a sample of tokens must carry the topic the oracle's chain gives them."""

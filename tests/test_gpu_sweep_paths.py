@@ -60,8 +60,8 @@ def test_replayed_sweeps_follow_changes_of_their_arguments(tiny_corpus):
 
 @pytest.mark.parametrize("K,V", [(10_500, 3), (2_500, 40), (600, 400), (40, 3_000)])
 def test_rows_of_every_length(K, V):
-    """Alias rows, count rows and runs on both sides of every class border: words from one token to a few
-    thousand (lengths around powers of two among them), rows from one topic to K."""
+    """Count rows and runs of words from one token to a few thousand, lengths around powers of two among them (the alias
+    rows' classes go by topics: test_alias_rows_at_the_borders_of_their_classes)."""
     rng = np.random.default_rng(K)
     edges = [1, 2, 7, 8, 9, 15, 16, 17, 31, 32, 33, 63, 64, 65, 96, 97, 127, 128, 129, 255, 256, 257, 511, 512, 513, 1023, 2047,
              2048, 2049, 4095, 6000]
@@ -79,6 +79,36 @@ def test_rows_of_every_length(K, V):
     _same(g, o)
     g.sweep(3, 2)
     o.sweep(3, 2)
+    _same(g, o)
+
+
+EDGES = [1, 2, 8, 9, 16, 17, 32, 33, 255, 256, 257, 511, 512, 513, 2_047, 2_048, 2_049]
+
+
+@pytest.mark.parametrize("K,rows", [(10_500, EDGES + [10_239, 10_240, 10_241, 10_500]), (20_000, EDGES + [10_240, 10_241, 15_000]),
+                                    (2_100, EDGES * 45)])
+def test_alias_rows_at_the_borders_of_their_classes(K, rows):
+    """Rows with exactly as many topics as the borders between the kernels that build them, by assignments made for it;
+    and more rows that may be long (765 words, 315 of them above 256 topics) than CTAs are given to at once."""
+    rng = np.random.default_rng(K)
+    many = len(rows) > 100
+    words, z = [], []
+    for w, n in enumerate(rows):
+        topics = rng.permutation(K)[:n]
+        more = rng.choice(topics, max(3, 300 - n if many else 0))     # a word's tokens bound its row
+        words.append(np.full(n + more.size, w))
+        z.append(np.concatenate([topics, more]))
+    mixed = rng.permutation(sum(x.size for x in z))
+    words, z = np.concatenate(words)[mixed].astype(np.int32), np.concatenate(z)[mixed].astype(np.int32)
+    offsets = np.concatenate([[0], np.sort(rng.integers(0, z.size + 1, z.size // 60)), [z.size]]).astype(np.int64)
+    g, o = binding.LightLDA(len(rows), K, 0.05, 0.01), ldaref.Oracle(len(rows), K, 0.05, 0.01)
+    for e in (g, o):
+        e.load_corpus(words, offsets)
+        e.set_assignments(z, 17, 0)
+    assert np.array_equal(np.diff(g.get_csr(binding.LDA_NWK)[0]), rows)
+    _same(g, o)
+    for e in (g, o):
+        e.sweep(3, 2)
     _same(g, o)
 
 
