@@ -189,15 +189,15 @@ __device__ __forceinline__ uint32_t row_count(uint32_t* table, int log2_slots, u
     return 0xFFFFFFFFu;
 }
 
-template <typename T, NkMode NK>
+template <NkMode NK>
 __global__ void __launch_bounds__(256, 6)
-k_word_rows(const int32_t* __restrict__ tiles, const int32_t* __restrict__ word_off, const T* __restrict__ z,
+k_word_rows(const int32_t* __restrict__ tiles, const int32_t* __restrict__ word_off, const uint16_t* __restrict__ z,
             RowTables out, int32_t K, int32_t area_words, int stamp_id)
 {
     stamp(out.state, stamp_id);
     extern __shared__ __align__(16) uint32_t row_area[];  // the warps' tables and bitmaps, then the CTA's; NK: bins behind
     __shared__ int32_t soff[ROW_TILE_WORDS + 1];
-    __shared__ T zs[SORT_TILE];
+    __shared__ uint16_t zs[SORT_TILE];
     __shared__ uint16_t long_words[SORT_TILE / ROW_WARP_TOKENS];
     __shared__ int32_t warp_total[8];
     __shared__ int32_t next_word, n_long;
@@ -212,9 +212,9 @@ k_word_rows(const int32_t* __restrict__ tiles, const int32_t* __restrict__ word_
     }
     for (int32_t j = tid; j <= nw; j += 256) soff[j] = __ldg(word_off + s0 + j) - base;
     for (int32_t j = tid; j < cnt; j += 256) {
-        const T k = __ldcs(z + base + j);
+        const uint16_t k = __ldcs(z + base + j);
         if ((uint32_t)k >= (uint32_t)K) atomicOr(err, ERR_TOPIC_RANGE);
-        zs[j] = (uint32_t)k < (uint32_t)K ? k : (T)0;
+        zs[j] = (uint32_t)k < (uint32_t)K ? k : (uint16_t)0;
     }
     if (NK == NK_BINS)
         for (int32_t k = tid; k < K; k += 256) bins[k] = 0;
@@ -687,15 +687,12 @@ void launch_doc_rows(Ctx& c, const int32_t* tiles, int32_t n_tiles, const T* z, 
 }
 // The same, single pass, for K <= WORD_ROWS_BITMAP_MAX_K: sizes, and entries from the documents' first tokens on (a row
 // has at most as many entries as the document has tokens).
-template <typename T>
-void launch_doc_rows_spread(Ctx& c, const int32_t* tiles, int32_t n_tiles, const T* z, int32_t* nnz, uint32_t* topic, uint32_t* count)
+void launch_doc_rows_spread(Ctx& c, const int32_t* tiles, int32_t n_tiles, const uint16_t* z, int32_t* nnz, uint32_t* topic, uint32_t* count)
 {
     const RowTables out{c.v.doc_off, topic, count, nnz, nullptr, c.v.state};
     const size_t area = row_area_bytes(c.K);
-    k_word_rows<T, NK_NONE><<<n_tiles, 256, area, c.stream>>>(tiles, c.v.doc_off, z, out, c.K, (int32_t)(area / 4), -1);
+    k_word_rows<NK_NONE><<<n_tiles, 256, area, c.stream>>>(tiles, c.v.doc_off, z, out, c.K, (int32_t)(area / 4), -1);
 }
-template void launch_doc_rows_spread<uint16_t>(Ctx&, const int32_t*, int32_t, const uint16_t*, int32_t*, uint32_t*, uint32_t*);
-template void launch_doc_rows_spread<int32_t>(Ctx&, const int32_t*, int32_t, const int32_t*, int32_t*, uint32_t*, uint32_t*);
 template void launch_doc_rows<uint16_t>(Ctx&, const int32_t*, int32_t, const uint16_t*, int32_t*, const long long*, int32_t*, int32_t*);
 template void launch_doc_rows<int32_t>(Ctx&, const int32_t*, int32_t, const int32_t*, int32_t*, const long long*, int32_t*, int32_t*);
 
@@ -720,8 +717,9 @@ static int count_wk_t(Ctx& c)
     if (c.n_word_tiles) {
         if (c.K <= WORD_ROWS_BITMAP_MAX_K) {
             const size_t area = row_area_bytes(c.K);
-            k_word_rows<T, NK><<<c.n_word_tiles, 256, area + (NK == NK_BINS ? (size_t)c.K * 4 : 0), c.side[0]>>>(
-                c.word_tiles, v.word_off, z, out, c.K, (int32_t)(area / 4), STAMP_ROWS);
+            if constexpr (sizeof(T) == 2)  // 32-bit topics mean a larger K
+                k_word_rows<NK><<<c.n_word_tiles, 256, area + (NK == NK_BINS ? (size_t)c.K * 4 : 0), c.side[0]>>>(
+                    c.word_tiles, v.word_off, z, out, c.K, (int32_t)(area / 4), STAMP_ROWS);
         } else {
             EmitWord e{v.row_start, v.wk_topic, v.wk_count, v.wk_nnz, NK == NK_NONE ? nullptr : v.nk_next};
             k_seg_count_sorted<T, EmitWord><<<c.n_word_tiles, 256, 0, c.side[0]>>>(
@@ -802,10 +800,9 @@ void set_hist_smem_limits()
     cudaFuncSetAttribute(k_hot_rows<uint16_t, NK_DIRECT>, most, hist);
     cudaFuncSetAttribute(k_hot_rows<int32_t, NK_NONE>, most, hist);
     cudaFuncSetAttribute(k_hot_rows<int32_t, NK_DIRECT>, most, hist);
-    cudaFuncSetAttribute(k_word_rows<uint16_t, NK_NONE>, most, rows);
-    cudaFuncSetAttribute(k_word_rows<uint16_t, NK_DIRECT>, most, rows);
-    cudaFuncSetAttribute(k_word_rows<uint16_t, NK_BINS>, most, rows_bins);
-    cudaFuncSetAttribute(k_word_rows<int32_t, NK_NONE>, most, rows);
+    cudaFuncSetAttribute(k_word_rows<NK_NONE>, most, rows);
+    cudaFuncSetAttribute(k_word_rows<NK_DIRECT>, most, rows);
+    cudaFuncSetAttribute(k_word_rows<NK_BINS>, most, rows_bins);
     cudaFuncSetAttribute(k_nk_from_sparse, cudaFuncAttributeMaxDynamicSharedMemorySize, HIST_BINS * 4);
 }
 

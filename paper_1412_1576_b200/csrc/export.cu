@@ -125,8 +125,7 @@ static int row_offsets(Ctx& c, const int32_t* nnz, long long* row_off, int64_t n
     return rc;
 }
 
-template <typename T>
-void launch_doc_rows_spread(Ctx& c, const int32_t* tiles, int32_t n_tiles, const T* z, int32_t* nnz, uint32_t* topic,
+void launch_doc_rows_spread(Ctx& c, const int32_t* tiles, int32_t n_tiles, const uint16_t* z, int32_t* nnz, uint32_t* topic,
                             uint32_t* count);  // counts.cu
 
 template <typename T>
@@ -153,7 +152,9 @@ static int build_dk_csr_t(Ctx& c, DkCsr& r, bool sizes_only)
             topic_at = nullptr;
         }
     }
-    if (topic_at) launch_doc_rows_spread<T>(c, c.doc_sort_tiles, c.n_doc_sort_tiles, z, r.nnz, topic_at, count_at);
+    if (topic_at)  // (16-bit topics, by the limit on K)
+        launch_doc_rows_spread(c, c.doc_sort_tiles, c.n_doc_sort_tiles, static_cast<const uint16_t*>(static_cast<void*>(v.rec)), r.nnz,
+                               topic_at, count_at);
     else if (c.n_doc_sort_tiles) launch_doc_rows<T>(c, c.doc_sort_tiles, c.n_doc_sort_tiles, z, r.nnz, nullptr, nullptr, nullptr);
     if (c.n_doc_sort_long)
         k_long_doc_rows<T, false><<<c.n_doc_sort_long, 512, (size_t)win * 4, c.stream>>>(

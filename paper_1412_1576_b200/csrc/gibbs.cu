@@ -12,7 +12,6 @@
 // sweep; the first term walks the document's sorted n_kd row (export.cu) and looks n_kw up in the
 // word's sorted row.  One Philox word per token and sweep: counter (token, sweep, 0, 2).
 #include <algorithm>
-#include <type_traits>
 
 #include "lda_device.cuh"
 #include "lda_internal.cuh"
@@ -123,9 +122,9 @@ __device__ __forceinline__ double div_by(double a, double b, double y)
 // run_len: up to GIBBS_RUN, shorter where that would leave multiprocessors idle.
 constexpr int GIBBS_RUN = 64;
 constexpr int GIBBS_KEPT = 64;
-template <typename T, bool MATRIX, int LANES>
+template <bool MATRIX, int LANES>
 __global__ void __launch_bounds__(256, LANES == 32 ? 4 : 3)
-k_gibbs_tokens(View v, const T* __restrict__ z, const int32_t* __restrict__ word_of, const long long* __restrict__ row_off,
+k_gibbs_tokens(View v, const uint16_t* __restrict__ z, const int32_t* __restrict__ word_of, const long long* __restrict__ row_off,
                const int32_t* __restrict__ dk_topic, const int32_t* __restrict__ dk_count, const ull* __restrict__ prefix,
                const int32_t* __restrict__ matrix, int32_t* __restrict__ z_new, uint2 key, uint32_t sweep, int32_t run_len)
 {
@@ -302,15 +301,11 @@ int lda::gibbs_sweep(Ctx& c, int32_t iters)
         int32_t run_len = GIBBS_RUN;
         while (run_len > 4 && c.N / run_len < (int64_t)c.n_sm * 32) run_len /= 2;
         const unsigned grid = (unsigned)((c.N + 8 * run_len - 1) / (8 * run_len));
-        auto tokens = [&](auto z) {
-            using T = std::remove_const_t<std::remove_pointer_t<decltype(z)>>;
-            const bool long_rows = r.total > c.D * (long long)GIBBS_KEPT;
-            const auto kernel = matrix ? (long_rows ? k_gibbs_tokens<T, true, 32> : k_gibbs_tokens<T, true, 16>)
-                                       : (long_rows ? k_gibbs_tokens<T, false, 32> : k_gibbs_tokens<T, false, 16>);
-            kernel<<<grid, 256, 0, c.stream>>>(v, z, word_of, r.row_off, r.topic, r.count, prefix, matrix, z_new, key, c.sweep, run_len);
-        };
-        if (c.wide_topics) tokens(reinterpret_cast<const int32_t*>(v.rec));
-        else tokens(reinterpret_cast<const uint16_t*>(v.rec));
+        const bool long_rows = r.total > c.D * (long long)GIBBS_KEPT;
+        const auto kernel = matrix ? (long_rows ? k_gibbs_tokens<true, 32> : k_gibbs_tokens<true, 16>)
+                                   : (long_rows ? k_gibbs_tokens<false, 32> : k_gibbs_tokens<false, 16>);
+        kernel<<<grid, 256, 0, c.stream>>>(v, reinterpret_cast<const uint16_t*>(v.rec), word_of, r.row_off, r.topic, r.count, prefix, matrix,
+                                           z_new, key, c.sweep, run_len);
         launch_spread_assignments(c, z_new, false);
         rebuild_counts(c);
         c.sweep += 1;

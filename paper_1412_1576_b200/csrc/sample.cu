@@ -152,7 +152,7 @@ struct HotTile {
         }
         return d;
     }
-    __device__ __forceinline__ void draw_finish(const Ref&, const Draw& d, uint32_t& t, int32_t& n_tw) const
+    __device__ __forceinline__ void draw_finish(const Ref&, const Draw& d, uint32_t& t) const
     {
         if (d.sparse) {
             if (PACKED) t = (d.rz < d.e.x) ? (d.e.y & 0xFFFFu) : (d.e.y >> 16);
@@ -160,7 +160,6 @@ struct HotTile {
         } else {
             t = (d.e.y == d.b || d.rz < d.e.x) ? d.b : d.e.y;
         }
-        n_tw = -1;  // looked up with the other counts
     }
 };
 
@@ -192,7 +191,7 @@ struct ColdBins {
         if (!d.sparse) d.e = __ldg(v.dn_pk + d.b);
         return d;
     }
-    __device__ __forceinline__ void draw_finish(const Ref& w, const Draw& d, uint32_t& t, int32_t& n_tw) const
+    __device__ __forceinline__ void draw_finish(const Ref& w, const Draw& d, uint32_t& t) const
     {
         if (d.sparse) {
             const uint32_t al = idx[w.rs + d.b];
@@ -201,7 +200,6 @@ struct ColdBins {
         } else {
             t = (d.e.y == d.b || d.rz < d.e.x) ? d.b : d.e.y;
         }
-        n_tw = -1;
     }
 };
 
@@ -311,8 +309,7 @@ __device__ __forceinline__ void propose_tokens(const View& v, const Tile& tile, 
             for (int u = 0; u < U; ++u) {
                 const int32_t p = p0 + u * nthreads;
                 uint32_t t;
-                int32_t n_tw;
-                tile.draw_finish(tile.ref((p < p_end ? p : p0) - p_begin), d[u], t, n_tw);
+                tile.draw_finish(tile.ref((p < p_end ? p : p0) - p_begin), d[u], t);
                 if (p < p_end) {
                     __stcs(reinterpret_cast<T*>(v.zbm) + 2 * (size_t)at[u] + 1, (T)t);
                     __stcs(v.ua_w + p, ua[u]);
@@ -329,8 +326,7 @@ __device__ __forceinline__ void propose_tokens(const View& v, const Tile& tile, 
                 const uint4 r = philox4x32_10(make_uint4(tok, running_sweep(v), (uint32_t)m, 0u), key);
                 const Draw d = tile.draw_issue(w, v, r);
                 uint32_t t;
-                int32_t n_tw;
-                tile.draw_finish(w, d, t, n_tw);
+                tile.draw_finish(w, d, t);
                 // the first proposal goes beside the token's topic, the later ones to arrays of their own
                 if (wi == 0) __stcs(reinterpret_cast<T*>(v.zbm) + 2 * (size_t)at + 1, (T)t);
                 else __stcs(prop + (size_t)wi * v.N + at, (T)t);
@@ -491,7 +487,7 @@ __device__ __forceinline__ void accept_tokens(const View& v, Tile& tile, const i
     }
 }
 
-// Hot words: tile = (word, first token, count).  ACCEPT = false: pass 1, true: pass 3.
+// Hot words: tile = (word, first token, count).  ACCEPT = false: pass 1 (CH = 0), true: pass 3.
 // FIXED > 0: the number of steps is this compile-time constant (the argument is ignored), which
 // removes the step loops and their predicates (and, in pass 1, enough registers for a third CTA per SM).
 template <typename T, int CH, bool STAGED, bool ACCEPT, int MODE, int FIXED>
@@ -539,7 +535,7 @@ k_word_hot(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_step
     tile.bar = &bar;
     tile.ready = !(STAGED && ACCEPT);
     tile.gave_up = false;
-    if (ACCEPT) accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, accept_threads(FIXED), mh_steps);
+    if constexpr (ACCEPT) accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, accept_threads(FIXED), mh_steps);
     else propose_tokens<T, MODE, FIXED>(v, tile, p0, p0 + cnt, PROPOSE_THREADS, key, mh_steps);
     // ACCEPT: every thread that had a token waited for the copy; thread 0 always has one.  A thread
     // whose wait ran out waits once more (bounded again) before the CTA may retire: a bulk copy still
@@ -615,7 +611,7 @@ __device__ __forceinline__ void fill_from_marks(uint16_t* a, uint32_t* warp_last
 
 // Tail words: tile = (first word, end word, first token, count): whole words with at most COLD_TILE tokens
 // between them, or a run of one word's tokens (small corpora: see load_common() for where the cuts lie).
-template <typename T, int CH, int MODE, int FIXED>
+template <typename T, int MODE, int FIXED>
 __global__ void __launch_bounds__(COLD_THREADS, 5)
 k_word_cold_propose(View v, const int4* __restrict__ tiles, uint2 key, int32_t mh_steps_arg, int stamp_id)
 {
@@ -813,7 +809,7 @@ static int launch_accept(Ctx& c, uint2 key, int mh_steps)
     return launches;
 }
 
-template <typename T, int CH, int MODE, int FIXED>
+template <typename T, int MODE, int FIXED>
 static int launch_propose(Ctx& c, uint2 key, int mh_steps)
 {
     // the running vocabulary slice's tokens (its tables are the ones in memory)
@@ -823,12 +819,12 @@ static int launch_propose(Ctx& c, uint2 key, int mh_steps)
     const bool noted = c.slices.size() == 1;  // several slices: the pass starts with the first slice's tables
     int launches = 0;
     if (q.hotp_n) {
-        k_word_hot<T, CH, false, false, MODE, FIXED><<<q.hotp_n, PROPOSE_THREADS, 0, on[0]>>>(
+        k_word_hot<T, 0, false, false, MODE, FIXED><<<q.hotp_n, PROPOSE_THREADS, 0, on[0]>>>(
             v, c.hot_tiles_propose + 3 * (size_t)q.hotp_lo, key, mh_steps, noted ? STAMP_PROPOSE_HOT : -1);
         ++launches;
     }
     if (q.cold_n) {
-        k_word_cold_propose<T, CH, MODE, FIXED><<<q.cold_n, COLD_THREADS, 0, on[1]>>>(
+        k_word_cold_propose<T, MODE, FIXED><<<q.cold_n, COLD_THREADS, 0, on[1]>>>(
             v, reinterpret_cast<const int4*>(c.cold_tiles) + q.cold_lo, key, mh_steps, noted ? STAMP_PROPOSE_COLD : -1);
         ++launches;
     }
@@ -850,10 +846,7 @@ static int sample_tc(Ctx& c, int mh_steps)
                 set_slice(c, sl);
                 launches += launch_alias_sparse(c, false);
             }
-            if (CH == 2 && mh_steps == 2)
-                launches += launch_propose<T, 2, MODE, 2>(c, key, mh_steps);
-            else
-                launches += launch_propose<T, CH, MODE, 0>(c, key, mh_steps);
+            launches += mh_steps == 2 ? launch_propose<T, MODE, 2>(c, key, mh_steps) : launch_propose<T, MODE, 0>(c, key, mh_steps);
         }
     }
     // pass 2: document side
