@@ -37,14 +37,15 @@ k_rows_from_dense(View v, const int32_t* __restrict__ in)
     const int32_t* line = in + (size_t)w * K;
     const int32_t out0 = v.row_start[w], cap = v.row_start[w + 1] - out0;
     const int32_t slot = v.dense_slot[w];
-    const bool tail = v.hot_word[w] == 0;
     int32_t* dense = slot >= 0 ? v.dense_rows + (size_t)slot * v.dense_stride : nullptr;
     int32_t done = 0;
     for (int32_t k0 = 0; k0 < K; k0 += blockDim.x) {
         const int32_t k = k0 + (int32_t)threadIdx.x;
         const int32_t n = k < K ? line[k] : 0;
-        if (n < 0) atomicOr(v.err, ERR_COUNT_ZERO);
-        if (tail && n > 0xFFFF) atomicOr(v.err, NOTE_WIDE_COUNT);  // more than its term frequency: only from outside
+        if ((uint32_t)n > 0xFFFFu) {  // negative, or so many that a tail word has them from outside only
+            if (n < 0) atomicOr(v.err, ERR_COUNT_ZERO);
+            else if (v.hot_word[w] == 0) atomicOr(v.err, NOTE_WIDE_COUNT);
+        }
         if (dense && k < K) dense[k] = n;
         int32_t total;
         const int32_t pos = done + block_scan_excl<int32_t>(n > 0 ? 1 : 0, scan_tmp, total);
