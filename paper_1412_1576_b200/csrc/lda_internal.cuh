@@ -431,6 +431,7 @@ void set_gibbs_smem_limits();
 // queued on the context's stream.
 cudaError_t copy_to_host(Ctx& c, void* host, const void* dev, size_t bytes);
 cudaError_t copy_to_device(Ctx& c, void* dev, const void* host, size_t bytes);
+bool page_locked(const void* host);
 
 // n_kw as compact rows in device memory: row offsets [V+1] and the entries (export.cu).  LDA_* status.
 struct WkCsr {

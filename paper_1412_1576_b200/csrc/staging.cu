@@ -65,7 +65,7 @@ struct StagingPool {
     }
 };
 
-static bool page_locked(const void* p)
+bool page_locked(const void* p)
 {
     cudaPointerAttributes a{};
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
