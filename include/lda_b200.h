@@ -13,7 +13,11 @@
  *   - pointers are HOST pointers unless the parameter says DEVICE.
  *   - the caller owns every buffer it passes; inputs are copied, so they may
  *     be freed once the call returns.  The context owns all device memory it
- *     allocates and frees it in lda_destroy().
+ *     allocates for a corpus and frees it in lda_destroy().
+ *   - kept by the process: the streams, events and small state buffers of up to
+ *     four destroyed contexts, for the next ones; and from the first copy of
+ *     2 MiB or more of host memory that is not page-locked on, 32 MiB of
+ *     page-locked memory and eight streams, until the process ends.
  *   - a context is bound to the CUDA device that is current in lda_create()
  *     and to one stream (the legacy default stream unless lda_set_stream() is
  *     called).  One host thread per context.

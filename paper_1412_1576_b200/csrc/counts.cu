@@ -9,7 +9,7 @@
 //   - hot words: shared-memory histogram over a window of topics, written out as
 //     dense row and sorted row.
 // n_k: column sums, added up by the kernels that write the rows when K and the number of CTAs are small
-// enough for that (nk_with_rows), else taken from the rows just written.
+// enough for that (choose_nk_mode()), else taken from the rows just written.
 // n_kd (segments = documents): the MH step builds every document's table itself, per tile, in
 // shared memory (docside.cu), and so does the log-likelihood (loglik.cu); lda_get_counts gets
 // sorted rows from export.cu.

@@ -53,7 +53,7 @@ constexpr uint32_t DK_EMPTY = 0xFFFFFFFFu;  // == DK_EMPTY_SLOT of the device he
 constexpr int DK_SLOTS_PER_TOKEN_HOST = 4;   // == DK_SLOTS_PER_TOKEN of the device helpers
 constexpr int SORT_TILE = 2048;      // tokens per segmented-sort tile (one CTA)
 // Tiles of whole documents (one CTA each) of the document-side kernels: tokens per tile and
-// threads per CTA, chosen per corpus from these shapes; longer documents get a CTA of their own.
+// threads per CTA, chosen per corpus from these shapes; longer documents are cut into chunks (LONG_CHUNK).
 constexpr int DOC_TILE_SHAPES = 4;
 constexpr int DOC_TILE_ROUNDS = 3;  // tokens per thread: every shape holds this many times its thread count
 constexpr int DOC_TILE_THREADS[DOC_TILE_SHAPES] = {128, 256, 512, 1024};
@@ -160,8 +160,8 @@ struct View {
     void* zw;   // word-sorted order: read by the n_kw / n_k rebuild
     void* zbm;  // block-major order, two entries per token: its topic, read (through bm_of_tok) by everything
                 // that works per document, and beside it the first word-proposal of the running MH step
-    // One word per token in document order: scratch (slot indices of long documents during the MH
-    // step, staging of assignments on their way in and out, z in document order for export.cu).
+    // One word per token in document order: scratch (topics of long documents during the MH step,
+    // staging of assignments on their way in and out, z in document order for export.cu).
     uint32_t* rec;
     const uint8_t* hot_word;  // [V] 1: the MH step treats the word as hot (more than COLD_TILE tokens)
     const int32_t* word_off;  // [V+1] token range of each word in word-sorted order

@@ -14,7 +14,8 @@
 namespace lda {
 
 // Every piece costs calls into the driver, which take turns: 160 MB to the device and 320 MB back took 10.0 and 17.5 ms
-// in pieces of 512 KiB, 7.2 and 12.4 in pieces of 2 MiB.  Shorter copies go in shorter pieces, four and more per lane.
+// in pieces of 512 KiB, 7.2 and 12.4 in pieces of 2 MiB.  Shorter copies go in shorter pieces, four per lane as long as
+// those are not below PIECE_MIN (16 MiB; a copy of 2 MiB is four pieces, and four lanes have nothing to do).
 constexpr int LANES = 8;
 constexpr size_t PIECE = 2 << 20, PIECE_MIN = 512 << 10;
 // Below this a copy is over before the threads have started.
