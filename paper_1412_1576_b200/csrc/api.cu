@@ -210,6 +210,17 @@ static int fail(Ctx* c, int code, const char* msg)
     return code;
 }
 
+// Nothing leaves the C entries by an exception: `f` gives the status, or the host had no memory for it.
+template <typename F>
+static int guarded(Ctx& c, F f)
+{
+    try {
+        return f();
+    } catch (const std::bad_alloc&) {
+        return fail(&c, LDA_ENOMEM, "host allocation failed");
+    }
+}
+
 static int cuda_fail(Ctx* c, const char* where)
 {
     cudaError_t e = cudaGetLastError();
@@ -556,7 +567,7 @@ struct Beside {
     ~Beside() { join(); }
 };
 
-static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const Documents& docs, int64_t n_docs)
+static int load_lists(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const Documents& docs, int64_t n_docs)
 {
     free_corpus(c);
     c.N = n_tokens;
@@ -993,6 +1004,16 @@ static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const
     return LDA_OK;
 }
 
+static int load_common(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const Documents& docs, int64_t n_docs)
+{
+    const int rc = guarded(c, [&] { return load_lists(c, words_dev, n_tokens, docs, n_docs); });
+    if (rc != LDA_OK && !c.allocs.empty()) {  // left behind by an exception
+        cudaStreamSynchronize(c.stream);
+        free_corpus(c);
+    }
+    return rc;
+}
+
 }  // namespace lda
 
 using namespace lda;
@@ -1136,7 +1157,7 @@ int lda_load_corpus(lda_ctx* h, const int32_t* word_ids, int64_t n_tokens, const
     if (!doc_offsets || n_tokens < 0 || n_docs < 0 || (n_tokens > 0 && !word_ids))
         return fail(&c, LDA_EINVAL, "null pointer or negative size");
     Documents docs;
-    int rc = scan_documents(&c, n_tokens, doc_offsets, n_docs, docs);
+    int rc = guarded(c, [&] { return scan_documents(&c, n_tokens, doc_offsets, n_docs, docs); });
     if (rc) return rc;
     if ((rc = check_device(c))) return rc;
     int32_t* wd = nullptr;
@@ -1161,14 +1182,15 @@ int lda_load_corpus_device(lda_ctx* h, const int32_t* word_ids_dev, int64_t n_to
     if (n_docs >= 2147483647ll) return fail(&c, LDA_ERANGE, "n_docs must be below 2^31");
     int rc = check_device(c);
     if (rc) return rc;
-    std::vector<int64_t> off((size_t)n_docs + 1);
+    std::vector<int64_t> off;
+    if ((rc = guarded(c, [&] { off.resize((size_t)n_docs + 1); return LDA_OK; }))) return rc;
     // the offsets come after what the default stream has queued, as a copy on that stream does, whatever the
     // context's stream is
     if (cudaEventRecord(c.ev_chunk, cudaStreamLegacy) != cudaSuccess || cudaStreamWaitEvent(c.stream, c.ev_chunk, 0) != cudaSuccess ||
         copy_to_host(c, off.data(), doc_offsets_dev, ((size_t)n_docs + 1) * 8) != cudaSuccess)
         return cuda_fail(&c, "copying doc offsets");
     Documents docs;
-    if ((rc = scan_documents(&c, n_tokens, off.data(), n_docs, docs))) return rc;
+    if ((rc = guarded(c, [&] { return scan_documents(&c, n_tokens, off.data(), n_docs, docs); }))) return rc;
     return load_common(c, word_ids_dev, n_tokens, docs, n_docs);
 }
 
@@ -1321,7 +1343,7 @@ int lda_set_shard(lda_ctx* h, int64_t first_token, const int32_t* global_term_fr
     if (global_term_freq) {
         for (int32_t w = 0; w < c.V; ++w)
             if (global_term_freq[w] < 0) return fail(&c, LDA_ERANGE, "negative term frequency");
-        c.shard_global_tf.assign(global_term_freq, global_term_freq + c.V);
+        return guarded(c, [&] { c.shard_global_tf.assign(global_term_freq, global_term_freq + c.V); return LDA_OK; });
     }
     return LDA_OK;
 }
@@ -1479,7 +1501,8 @@ int lda_get_counts(lda_ctx* h, int which, int64_t* row_offsets, int32_t* topics,
     const bool sizes_only = !row_offsets && !topics && !counts;
     WkCsr r;
     rc = build_wk_csr(c, r, sizes_only);
-    if (rc == LDA_ENOMEM) return word_rows_by_host(c, row_offsets, topics, counts, capacity, nnz_out);
+    if (rc == LDA_ENOMEM)
+        return guarded(c, [&] { return word_rows_by_host(c, row_offsets, topics, counts, capacity, nnz_out); });
     if (rc) return fail(&c, rc, "building the n_kw rows failed");
     const int64_t total = (int64_t)r.total;
     if (nnz_out) *nnz_out = total;
@@ -1556,14 +1579,10 @@ int lda_wait(lda_ctx* h)
     return wait_all(c);
 }
 
-int lda_get_tables(lda_ctx* h, uint32_t* sp_thr32, int32_t* sp_alias, int64_t capacity, uint32_t* mix32,
-                   uint32_t* dn_thr32, int32_t* dn_alias, uint64_t* dense_mass)
+static int get_tables(Ctx& c, uint32_t* sp_thr32, int32_t* sp_alias, int64_t capacity, uint32_t* mix32, uint32_t* dn_thr32,
+                      int32_t* dn_alias, uint64_t* dense_mass)
 {
-    if (!h) return LDA_EINVAL;
-    Ctx& c = h->c;
-    if (!c.inited) return fail(&c, LDA_ESTATE, "lda_get_tables before lda_init");
-    int rc = check_device(c);
-    if (rc) return rc;
+    int rc = LDA_OK;
     const View& v = c.v;
     const size_t V = (size_t)c.V, K = (size_t)c.K;
     const bool want_sparse = sp_thr32 || sp_alias;
@@ -1619,6 +1638,17 @@ int lda_get_tables(lda_ctx* h, uint32_t* sp_thr32, int32_t* sp_alias, int64_t ca
             if (sp_alias) sp_alias[o] = (int32_t)b[(size_t)start[w] + j];
         }
     return LDA_OK;
+}
+
+int lda_get_tables(lda_ctx* h, uint32_t* sp_thr32, int32_t* sp_alias, int64_t capacity, uint32_t* mix32,
+                   uint32_t* dn_thr32, int32_t* dn_alias, uint64_t* dense_mass)
+{
+    if (!h) return LDA_EINVAL;
+    Ctx& c = h->c;
+    if (!c.inited) return fail(&c, LDA_ESTATE, "lda_get_tables before lda_init");
+    int rc = check_device(c);
+    if (rc) return rc;
+    return guarded(c, [&] { return get_tables(c, sp_thr32, sp_alias, capacity, mix32, dn_thr32, dn_alias, dense_mass); });
 }
 
 int lda_get_stats(lda_ctx* h, lda_stats* out)

@@ -235,3 +235,37 @@ def test_exact_conditional_sweep_without_room_for_the_matrix():
         g.gibbs_sweep(1)
     assert e.value.status == binding.LDA_ENOMEM
     b.left = None
+
+
+HOST_MEMORY = """
+import resource
+import numpy as np
+from paper_1412_1576_b200 import binding
+g = binding.LightLDA(5, 4, 0.1, 0.01, allocator="cuda")
+words, few = np.arange(40, dtype=np.int32) % 5, np.array([0, 10, 40], np.int64)
+g.load_corpus(words, few)
+g.init(1)
+g.sweep(1, 2)
+offsets, none = np.zeros(30_000_001, np.int64), np.zeros(0, np.int32)   # documents without a token
+with open("/proc/self/statm") as f:
+    now = int(f.read().split()[0]) * resource.getpagesize()
+soft, hard = resource.getrlimit(resource.RLIMIT_AS)
+resource.setrlimit(resource.RLIMIT_AS, (now + (48 << 20), hard))
+rc = binding.lda_load_corpus(g._h, none, offsets)
+resource.setrlimit(resource.RLIMIT_AS, (soft, hard))
+assert rc == binding.LDA_ENOMEM, rc
+g.sweep(1, 2)                                # the corpus it had is still there
+assert int(g.get_nk().sum()) == 40
+g.load_corpus(none, offsets)
+print("done")
+"""
+
+
+def test_host_memory_that_cannot_be_had_is_an_error():
+    """No exception leaves the library: a list of 120 MB under a limit that does not allow it."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", HOST_MEMORY], cwd=root, capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and r.stdout.strip() == "done", r.stdout + r.stderr
