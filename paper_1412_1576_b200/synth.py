@@ -31,7 +31,6 @@ from __future__ import annotations
 import math
 from dataclasses import dataclass, field
 
-import numpy as np
 import torch
 
 # The five workloads.  "mh_steps" is the number of individual MH proposals per
@@ -117,15 +116,18 @@ def _zipf_cdf(V: int, s: float, dev) -> torch.Tensor:
     """Cumulative Zipf(s) distribution over the ranks 1..V.
 
     On CUDA a floating-point cumsum adds in an order that changes from call to call, and two calls differ in their
-    last bits: one draw in 5 * 10^9 at V = 10^6 then gives another word.  There the weights are added up on
-    the host, in order and in extended precision, which is as close to the device's sums as those are to each other.
+    last bits: one draw in 5 * 10^9 at V = 10^6 then gives another word.  There the sums are made by doubling steps, an
+    order of their own, which leaves them as close to the exact ones as a cumsum's.
     """
-    weights = torch.arange(1, V + 1, dtype=torch.float64, device=dev).pow(-s)
-    if dev.type != "cuda":
-        cdf = torch.cumsum(weights, 0)
-        return cdf / cdf[-1]
-    cdf = np.cumsum(weights.cpu().numpy().astype(np.longdouble))
-    return torch.from_numpy((cdf / cdf[-1]).astype(np.float64)).to(dev)
+    cdf = torch.arange(1, V + 1, dtype=torch.float64, device=dev).pow(-s)
+    if dev.type == "cuda":
+        step = 1
+        while step < V:     # an entry holds the sum of its own weight and the step - 1 before it
+            cdf = torch.cat((cdf[:step], cdf[step:] + cdf[:-step]))
+            step *= 2
+    else:
+        cdf = torch.cumsum(cdf, 0)
+    return cdf / cdf[-1]
 
 
 def generate(V: int, K: int, D: int, length, zipf_s, alpha: float, beta: float,
