@@ -2,6 +2,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <limits>
 #include <memory>
 #include <mutex>
 #include <new>
@@ -277,6 +278,13 @@ static void free_corpus(Ctx& c)
     nv.V = c.V; nv.K = c.K; nv.alpha = c.alpha; nv.beta = c.beta;
     nv.Vbeta = (double)c.V * c.beta;
     nv.Kalpha = (double)c.K * c.alpha;
+    // Rounding errors reach 17 units of 2^-24 on either side: conversions, sums and products of five factors and the uniform.
+    // Priors for which products might underflow leave every step to double precision (an overflow shows by itself).
+    nv.alpha_f = (float)nv.alpha;
+    nv.beta_f = (float)nv.beta;
+    nv.Vbeta_f = (float)nv.Vbeta;
+    const double low = std::min({nv.alpha, nv.beta, nv.Vbeta}), high = std::max({nv.alpha, nv.beta, nv.Vbeta});
+    nv.filter_eps = low >= 0x1p-24 && high <= 0x1p60 ? 0x1p-18f : std::numeric_limits<float>::infinity();
     nv.dense_stride = (c.K + 3) & ~3;
     nv.state = c.v.state;
     nv.err = &nv.state->err;

@@ -140,6 +140,8 @@ constexpr int LONG_STAGE_MAX_K = 4096;  // counters of a long document staged in
 struct View {
     int32_t V, K, N, D;
     double alpha, beta, Vbeta, Kalpha;
+    // for the first look at an acceptance (accept_tokens()): the priors in single precision, and how close its sides may come
+    float alpha_f, beta_f, Vbeta_f, filter_eps;
     uint32_t tok_base;  // Philox token key of the corpus' first token (0 unless the corpus is a shard)
     int topic_bits;  // bits of K-1
     int count_bits;  // low bits of a packed n_kd entry that hold the count

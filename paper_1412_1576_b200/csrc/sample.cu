@@ -44,10 +44,11 @@ constexpr int PROPOSE_TOKENS = LDA_PROPOSE_TOKENS;  // tokens a thread of the tw
 #define LDA_ACCEPT_MIN_CTAS 2
 #endif
 constexpr int PROPOSE_THREADS = LDA_PROPOSE_THREADS;
-// the two-step chain needs few enough registers for two CTAs of 768 threads per SM
-__host__ __device__ constexpr int accept_threads(int fixed)
+// the two-step chain needs few enough registers for two CTAs of 768 threads per SM; with rows left in device memory a few more
+// (200 M tokens, K = 10^5: 5.10 ms with 768 threads, 4.98 with 640, 5.08 with 512)
+__host__ __device__ constexpr int accept_threads(int fixed, bool staged)
 {
-    return fixed == 2 ? LDA_ACCEPT_FIXED2_THREADS : LDA_ACCEPT_THREADS;
+    return fixed != 2 ? LDA_ACCEPT_THREADS : staged ? LDA_ACCEPT_FIXED2_THREADS : 640;
 }
 constexpr int COLD_THREADS = 256;
 constexpr int STAGE_WAIT_LIMIT = 1 << 20;
@@ -434,36 +435,89 @@ __device__ __forceinline__ void accept_tokens(const View& v, Tile& tile, const i
                 n_tw[i] = tile.count(w, t[i]);
                 n_t[i] = tile.nk(t[i]);
             }
-            // Eq. 8 (word steps) / Eq. 11 (doc steps), products taken left to right
+            // Eq. 8 (word steps) / Eq. 11 (doc steps).  With a fixed number of steps first in single precision: terms and products
+            // are positive and right to a few units in the last place, so a step whose two sides differ by more than
+            // filter_eps of their sum goes the way it goes in double precision; a token with a closer one (one in
+            // 10^5) is taken again in that.  Each factor comes without the token itself (a_) and with it (b_).  The double-
+            // precision units are half as wide, and its operands take two registers (738 M tokens, K = 10 000: 6.07 -> 5.61 ms; four
+            // steps, 74 M: 1.33 -> 1.12).  With any number of steps, groups of four, the registers it takes cost more
+            // than that: 1.65 -> 2.14 ms for three steps of 99 M tokens, K = 1000.
+            uint32_t s_new = s, moved_now = 0;
+            bool unsure = true;
+            if constexpr (FIXED > 0) {
+                unsure = false;
+                static_assert(FIXED <= CH, "one group of steps, which starts at z0");
+                const float fa = v.alpha_f, fb = v.beta_f, fV = v.Vbeta_f;
+                float a_sd = __fadd_rn((float)(uint32_t)(n_sd - 1), fa), b_sd = __fadd_rn(a_sd, 1.f);
+                float a_sw = __fadd_rn((float)(uint32_t)(n_sw - 1), fb), b_sw = __fadd_rn(a_sw, 1.f);
+                float a_s = __fadd_rn((float)(uint32_t)(n_s - 1), fV), b_s = __fadd_rn(a_s, 1.f);
 #pragma unroll
-            for (int i = 0; i < CH; ++i) {
-                const bool live = m0 + i < mh_steps && t[i] != s;
-                const int32_t n_td = (int32_t)(e[i] & cmask);
-                const int32_t e_s = (s == z0), e_t = (t[i] == z0);
-                double num = __dadd_rn(u32_to_double((uint32_t)(n_td - e_t)), alpha);
-                num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)(n_tw[i] - e_t)), beta));
-                num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)(n_s - e_s)), Vb));
-                double den = __dadd_rn(u32_to_double((uint32_t)(n_sd - e_s)), alpha);
-                den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)(n_sw - e_s)), beta));
-                den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)(n_t[i] - e_t)), Vb));
-                if (!step_is_doc<MODE>(i)) {
-                    num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)n_sw), beta));
-                    num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)n_t[i]), Vb));
-                    den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)n_tw[i]), beta));
-                    den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)n_s), Vb));
-                } else {
-                    num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)n_sd), alpha));
-                    den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)n_td), alpha));
-                }
-                const double u = __dmul_rn(u32_to_double((uint32_t)ua[i]), INV_2_32);
-                if (live && __dmul_rn(u, den) < num) {
-                    moved += step_is_doc<MODE>(i) ? 0x10000u : 1u;
-                    s = t[i];
-                    n_sd = n_td;
-                    n_sw = n_tw[i];
-                    n_s = n_t[i];
+                for (int i = 0; i < CH; ++i) {
+                    const bool live = m0 + i < mh_steps && t[i] != s_new;
+                    const int32_t e_t = i > 0 && t[i] == z0;  // (z0 proposed at z0 moves nothing)
+                    const float a_td = __fadd_rn((float)((e[i] & cmask) - e_t), fa), b_td = __fadd_rn(a_td, e_t ? 1.f : 0.f);
+                    const float a_tw = __fadd_rn((float)(uint32_t)(n_tw[i] - e_t), fb), b_tw = __fadd_rn(a_tw, e_t ? 1.f : 0.f);
+                    const float a_t = __fadd_rn((float)(uint32_t)(n_t[i] - e_t), fV), b_t = __fadd_rn(a_t, e_t ? 1.f : 0.f);
+                    float num = __fmul_rn(__fmul_rn(a_td, a_tw), a_s), den = __fmul_rn(__fmul_rn(a_sd, a_sw), a_t);
+                    if (!step_is_doc<MODE>(i)) {
+                        num = __fmul_rn(num, __fmul_rn(b_sw, b_t));
+                        den = __fmul_rn(den, __fmul_rn(b_tw, b_s));
+                    } else {
+                        num = __fmul_rn(num, b_sd);
+                        den = __fmul_rn(den, b_td);
+                    }
+                    const float bar = __fmul_rn(__fmul_rn((float)ua[i], (float)INV_2_32), den);
+                    const float over = __fadd_rn(num, -bar);
+                    // (not a comparison the other way round: infinities and what comes of them are unsure)
+                    unsure = unsure || (live && !(fabsf(over) > __fmul_rn(v.filter_eps, __fadd_rn(num, bar))));
+                    if (live && over > 0.f) {
+                        moved_now += step_is_doc<MODE>(i) ? 0x10000u : 1u;
+                        s_new = t[i];
+                        a_sd = a_td; b_sd = b_td;
+                        a_sw = a_tw; b_sw = b_tw;
+                        a_s = a_t; b_s = b_t;
+                    }
                 }
             }
+            if (unsure) {  // products taken left to right
+                s_new = s;
+                moved_now = 0;
+                int32_t x_sd = n_sd, x_sw = n_sw, x_s = n_s;
+#pragma unroll
+                for (int i = 0; i < CH; ++i) {
+                    const bool live = m0 + i < mh_steps && t[i] != s_new;
+                    const int32_t n_td = (int32_t)(e[i] & cmask);
+                    const int32_t e_s = s_new == z0, e_t = t[i] == z0;
+                    double num = __dadd_rn(u32_to_double((uint32_t)(n_td - e_t)), alpha);
+                    num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)(n_tw[i] - e_t)), beta));
+                    num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)(x_s - e_s)), Vb));
+                    double den = __dadd_rn(u32_to_double((uint32_t)(x_sd - e_s)), alpha);
+                    den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)(x_sw - e_s)), beta));
+                    den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)(n_t[i] - e_t)), Vb));
+                    if (!step_is_doc<MODE>(i)) {
+                        num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)x_sw), beta));
+                        num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)n_t[i]), Vb));
+                        den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)n_tw[i]), beta));
+                        den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)x_s), Vb));
+                    } else {
+                        num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)x_sd), alpha));
+                        den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)n_td), alpha));
+                    }
+                    const double u = __dmul_rn(u32_to_double((uint32_t)ua[i]), INV_2_32);
+                    if (live && __dmul_rn(u, den) < num) {
+                        moved_now += step_is_doc<MODE>(i) ? 0x10000u : 1u;
+                        s_new = t[i];
+                        x_sd = n_td;
+                        x_sw = n_tw[i];
+                        x_s = n_t[i];
+                    }
+                }
+                n_sd = x_sd;  // for the next group
+                n_sw = x_sw;
+                n_s = x_s;
+            }
+            s = s_new;
+            moved += moved_now;
         }
         if (!staged_ok) break;
         __stcs(zw + p, (T)s);
@@ -491,7 +545,7 @@ __device__ __forceinline__ void accept_tokens(const View& v, Tile& tile, const i
 // FIXED > 0: the number of steps is this compile-time constant (the argument is ignored), which
 // removes the step loops and their predicates (and, in pass 1, enough registers for a third CTA per SM).
 template <typename T, int CH, bool STAGED, bool ACCEPT, int MODE, int FIXED>
-__global__ void __launch_bounds__(ACCEPT ? accept_threads(FIXED) : PROPOSE_THREADS,
+__global__ void __launch_bounds__(ACCEPT ? accept_threads(FIXED, STAGED) : PROPOSE_THREADS,
                                   ACCEPT      ? LDA_ACCEPT_MIN_CTAS
                                   : FIXED > 0 ? (sizeof(T) == 2 ? 4 : 3)  // 32-bit topics: three table reads per draw, more registers
                                               : LDA_PROPOSE_MIN_CTAS)
@@ -535,7 +589,7 @@ k_word_hot(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_step
     tile.bar = &bar;
     tile.ready = !(STAGED && ACCEPT);
     tile.gave_up = false;
-    if constexpr (ACCEPT) accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, accept_threads(FIXED), mh_steps);
+    if constexpr (ACCEPT) accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, accept_threads(FIXED, STAGED), mh_steps);
     else propose_tokens<T, MODE, FIXED>(v, tile, p0, p0 + cnt, PROPOSE_THREADS, key, mh_steps);
     // ACCEPT: every thread that had a token waited for the copy; thread 0 always has one.  A thread
     // whose wait ran out waits once more (bounded again) before the CTA may retire: a bulk copy still
@@ -546,7 +600,7 @@ k_word_hot(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_step
 // Warm words, accept pass: tile = (word, first token, count) like a hot word's, the sorted row
 // instead of a dense one.
 template <typename T, int CH, int MODE, int FIXED>
-__global__ void __launch_bounds__(accept_threads(FIXED), LDA_ACCEPT_MIN_CTAS)
+__global__ void __launch_bounds__(accept_threads(FIXED, false), LDA_ACCEPT_MIN_CTAS)
 k_word_warm(View v, const int32_t* __restrict__ tiles, int32_t mh_steps_arg, int stamp_id)
 {
     stamp(v, stamp_id);
@@ -576,7 +630,7 @@ k_word_warm(View v, const int32_t* __restrict__ tiles, int32_t mh_steps_arg, int
     }
     __syncthreads();
     WarmTile tile{topic_s, count_s, v.nk, start_s, shift};
-    accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, accept_threads(FIXED), mh_steps);
+    accept_tokens<T, CH, MODE, FIXED>(v, tile, p0, p0 + cnt, accept_threads(FIXED, false), mh_steps);
 }
 
 // `a` holds ascending nonzero marks in some places and zeros elsewhere: every place becomes the last mark at or
@@ -788,15 +842,15 @@ static int launch_accept(Ctx& c, uint2 key, int mh_steps)
     if (c.n_hot_tiles) {
         if (c.K <= HOT_STAGE_MAX_K)
             k_word_hot<T, CH, true, true, MODE, FIXED>
-                <<<c.n_hot_tiles, accept_threads(FIXED), (size_t)v.dense_stride * 8, on[0]>>>(v, c.hot_tiles, key, mh_steps,
+                <<<c.n_hot_tiles, accept_threads(FIXED, true), (size_t)v.dense_stride * 8, on[0]>>>(v, c.hot_tiles, key, mh_steps,
                                                                                           STAMP_ACCEPT_HOT);
         else
             k_word_hot<T, CH, false, true, MODE, FIXED>
-                <<<c.n_hot_tiles, accept_threads(FIXED), 0, on[0]>>>(v, c.hot_tiles, key, mh_steps, STAMP_ACCEPT_HOT);
+                <<<c.n_hot_tiles, accept_threads(FIXED, false), 0, on[0]>>>(v, c.hot_tiles, key, mh_steps, STAMP_ACCEPT_HOT);
         ++launches;
     }
     if (c.n_hot_tiles_warm) {
-        k_word_warm<T, CH, MODE, FIXED><<<c.n_hot_tiles_warm, accept_threads(FIXED), WARM_MAX_TF * 8, on[2]>>>(
+        k_word_warm<T, CH, MODE, FIXED><<<c.n_hot_tiles_warm, accept_threads(FIXED, false), WARM_MAX_TF * 8, on[2]>>>(
             v, c.hot_tiles_warm, mh_steps, STAMP_ACCEPT_WARM);
         ++launches;
     }

@@ -188,3 +188,43 @@ def test_exact_conditional_rows_of_every_length(K, short):
         g.gibbs_sweep(1)
         o.gibbs_sweep(1)
         assert np.array_equal(g.get_assignments(), o.get_assignments())
+
+
+@pytest.mark.parametrize("alpha,beta", [(0.05, 1e-9), (1e-9, 0.01), (2.0, 2.0 ** -24), (2.0 ** -25, 3.0), (1e9, 1e9), (0.05, 1e6)])
+@pytest.mark.parametrize("steps,mode", [(2, 0), (3, 0), (4, 0), (2, 1), (2, 2)])
+def test_acceptances_under_extreme_priors(alpha, beta, steps, mode):
+    """Priors on both sides of those that leave every acceptance to double precision, and such as let single-precision
+    products overflow."""
+    c = synth.generate(V=300, K=40, D=150, length=("poisson", 60.0), zipf_s=1.1, alpha=0.05, beta=0.01, seed=8)
+    w, off = c.word_ids.numpy(), c.doc_offsets.numpy()
+    g, o = binding.LightLDA(c.V, c.K, alpha, beta), ldaref.Oracle(c.V, c.K, alpha, beta)
+    for e in (g, o):
+        e.load_corpus(w, off)
+        e.init(21)
+        e.set_proposals(mode)
+        e.sweep(4, steps)
+    assert np.array_equal(g.get_assignments(), o.get_assignments())
+
+
+@pytest.mark.parametrize("K", [16_384, 16_385, 56_320, 56_321, 115_200, 115_201])
+@pytest.mark.parametrize("steps,mode", [(2, 0), (3, 0), (4, 0), (2, 1)])
+def test_long_words_at_large_topic_counts(K, steps, mode):
+    """Words around the lengths at which a word's rows change their form, and one with more tokens of a topic than 16 bits
+    count, at topic counts around the limits of what shared memory holds of a word."""
+    tf = [66_500, 12_289, 12_288, 2_049, 2_048, 2_047, 300, 1]
+    rng = np.random.default_rng(K)
+    words = np.repeat(np.arange(len(tf)), tf)
+    z = rng.integers(0, K, words.size)
+    z[:66_000] = K - 1                  # of the first word: 65 535 and more
+    z[66_500:68_000] = 0
+    mixed = rng.permutation(words.size)
+    words, z = words[mixed].astype(np.int32), z[mixed].astype(np.int32)
+    offsets = np.concatenate([[0], np.sort(rng.integers(0, z.size + 1, z.size // 80)), [z.size]]).astype(np.int64)
+    g, o = binding.LightLDA(len(tf), K, 0.01, 0.01), ldaref.Oracle(len(tf), K, 0.01, 0.01)
+    for e in (g, o):
+        e.load_corpus(words, offsets)
+        e.set_proposals(mode)
+        e.set_assignments(z, 5, 0)
+        e.sweep(2, steps)
+    assert np.array_equal(g.get_assignments(), o.get_assignments())
+    assert np.array_equal(g.get_nk(), o.get_nk())
