@@ -228,3 +228,22 @@ def test_long_words_at_large_topic_counts(K, steps, mode):
         e.sweep(2, steps)
     assert np.array_equal(g.get_assignments(), o.get_assignments())
     assert np.array_equal(g.get_nk(), o.get_nk())
+
+
+@pytest.mark.parametrize("tokens", [1, 7, 8, 9, 15, 16, 17, 255, 256, 257, 1_023, 1_024, 1_025, 2_047, 2_048])
+def test_sorted_rows_of_tiles_of_every_length(tokens):
+    """Rows of words and of documents at a topic count too large for a bitmap: one word and one document of just so many
+    tokens, then 30 words of about a hundredth as many."""
+    K = 20_000
+    rng = np.random.default_rng(tokens)
+    words = np.concatenate([np.zeros(tokens, np.int32), rng.integers(1, 31, max(tokens // 4, 1)).astype(np.int32)])
+    z = np.where(rng.random(words.size) < 0.5, rng.integers(0, 9, words.size), rng.integers(0, K, words.size)).astype(np.int32)
+    offsets = np.array([0, tokens, tokens, words.size], np.int64)
+    g, o = binding.LightLDA(40, K, 0.05, 0.01), ldaref.Oracle(40, K, 0.05, 0.01)
+    for e in (g, o):
+        e.load_corpus(words, offsets)
+        e.set_assignments(z, 3, 0)
+    _same(g, o)
+    for e in (g, o):
+        e.sweep(2, 2)
+    _same(g, o)
