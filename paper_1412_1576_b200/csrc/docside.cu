@@ -113,7 +113,7 @@ struct LongTable {
 template <typename T, int MODE, int FIXED, class Table>
 __device__ __forceinline__ void doc_side_token(const View& v, const Table& table, uint32_t tok, uint32_t doc_len,
                                                uint32_t own, uint32_t t_first, uint32_t bm,
-                                               uint2 key, uint32_t sweep, int32_t mh_steps)
+                                               const PhiloxKey& key, uint32_t sweep, int32_t mh_steps)
 {
     const T* prop = reinterpret_cast<const T*>(v.prop);
     const size_t N = (size_t)v.N;
@@ -186,7 +186,7 @@ __host__ __device__ constexpr int doc_resident_threads(int mode, int fixed)
 }
 template <typename T, int THREADS, int MODE, int FIXED, bool DENSE>
 __global__ void __launch_bounds__(THREADS, doc_resident_threads(MODE, FIXED) / THREADS)
-k_doc_tile(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_steps_arg)
+k_doc_tile(View v, const int32_t* __restrict__ tiles, PhiloxKey key, int32_t mh_steps_arg)
 {
     stamp(v, STAMP_DOC_TILES);
     const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
@@ -323,7 +323,7 @@ k_long_count(View v, const int4* __restrict__ chunks, bool keep_topics, int stam
 
 template <typename T, int MODE, int FIXED, bool DENSE>
 __device__ __forceinline__ void long_gather(const View& v, const LongDoc& d, const uint32_t* tab, int32_t first, int32_t cnt,
-                                            uint2 key, int32_t mh_steps)
+                                            const PhiloxKey& key, int32_t mh_steps)
 {
     const T* zbm = reinterpret_cast<const T*>(v.zbm);
     const uint32_t sweep = running_sweep(v);
@@ -351,7 +351,7 @@ __device__ __forceinline__ void long_gather(const View& v, const LongDoc& d, con
 
 template <typename T, int MODE, int FIXED>
 __global__ void __launch_bounds__(LONG_THREADS, LONG_MIN_CTAS)
-k_long_gather(View v, const int4* __restrict__ chunks, uint2 key, int32_t mh_steps_arg)
+k_long_gather(View v, const int4* __restrict__ chunks, PhiloxKey key, int32_t mh_steps_arg)
 {
     const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
     extern __shared__ __align__(16) uint32_t long_bins[];
@@ -420,7 +420,7 @@ void set_doc_smem_limits()
 template <typename T, int MODE, int FIXED>
 static int doc_side_tm(Ctx& c, int mh_steps)
 {
-    const uint2 key = make_uint2((uint32_t)c.seed, (uint32_t)(c.seed >> 32));
+    const PhiloxKey key(c.seed);
     const PassStreams on(c, (c.n_doc_tiles > 0) + (c.n_long_chunks > 0));
     int launches = 0;
     if (c.n_doc_tiles) {

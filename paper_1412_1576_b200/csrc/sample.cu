@@ -280,7 +280,7 @@ struct WarmTile {
 // state, so all of them can be drawn before anything is accepted.
 template <typename T, int MODE, int FIXED, class Tile>
 __device__ __forceinline__ void propose_tokens(const View& v, const Tile& tile, const int32_t p_begin,
-                                               const int32_t p_end, const int32_t nthreads, const uint2 key,
+                                               const int32_t p_end, const int32_t nthreads, const PhiloxKey& key,
                                                const int32_t mh_steps)
 {
     T* prop = reinterpret_cast<T*>(v.prop);
@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(ACCEPT ? accept_threads(FIXED, STAGED) : PROPO
                                   ACCEPT      ? LDA_ACCEPT_MIN_CTAS
                                   : FIXED > 0 ? (sizeof(T) == 2 ? 4 : 3)  // 32-bit topics: three table reads per draw, more registers
                                               : LDA_PROPOSE_MIN_CTAS)
-k_word_hot(View v, const int32_t* __restrict__ tiles, uint2 key, int32_t mh_steps_arg, int stamp_id)
+k_word_hot(View v, const int32_t* __restrict__ tiles, PhiloxKey key, int32_t mh_steps_arg, int stamp_id)
 {
     stamp(v, stamp_id);
     const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
@@ -667,7 +667,7 @@ __device__ __forceinline__ void fill_from_marks(uint16_t* a, uint32_t* warp_last
 // between them, or a run of one word's tokens (small corpora: see load_common() for where the cuts lie).
 template <typename T, int MODE, int FIXED>
 __global__ void __launch_bounds__(COLD_THREADS, 5)
-k_word_cold_propose(View v, const int4* __restrict__ tiles, uint2 key, int32_t mh_steps_arg, int stamp_id)
+k_word_cold_propose(View v, const int4* __restrict__ tiles, PhiloxKey key, int32_t mh_steps_arg, int stamp_id)
 {
     stamp(v, stamp_id);
     const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
@@ -774,7 +774,7 @@ k_word_cold_accept(View v, const int4* __restrict__ tiles, int32_t mh_steps_arg,
 
 // z_i uniform on {0..K-1}: Philox counter (token, 0, 0, 1), word 0.
 template <typename T>
-__global__ void k_init(View v, uint2 key)
+__global__ void k_init(View v, PhiloxKey key)
 {
     T* zw = reinterpret_cast<T*>(v.zw);
     T* zbm = reinterpret_cast<T*>(v.zbm);
@@ -834,7 +834,7 @@ static int grid_for(int64_t n, int block)
 }
 
 template <typename T, int CH, int MODE, int FIXED>
-static int launch_accept(Ctx& c, uint2 key, int mh_steps)
+static int launch_accept(Ctx& c, PhiloxKey key, int mh_steps)
 {
     const View& v = c.v;
     const PassStreams on(c, (c.n_hot_tiles > 0) + (c.n_hot_tiles_warm > 0) + (c.n_cold_tiles > 0));
@@ -864,7 +864,7 @@ static int launch_accept(Ctx& c, uint2 key, int mh_steps)
 }
 
 template <typename T, int MODE, int FIXED>
-static int launch_propose(Ctx& c, uint2 key, int mh_steps)
+static int launch_propose(Ctx& c, PhiloxKey key, int mh_steps)
 {
     // the running vocabulary slice's tokens (its tables are the ones in memory)
     const View& v = c.v;
@@ -888,7 +888,7 @@ static int launch_propose(Ctx& c, uint2 key, int mh_steps)
 template <typename T, int CH, int MODE>
 static int sample_tc(Ctx& c, int mh_steps)
 {
-    const uint2 key = make_uint2((uint32_t)c.seed, (uint32_t)(c.seed >> 32));
+    const PhiloxKey key(c.seed);
     int launches = 0;
     // pass 1: word-proposals (none in a doc-proposal-only chain).  With more than one vocabulary
     // slice the sparse alias tables exist for one slice at a time: build a slice's, draw from them,
@@ -972,7 +972,7 @@ void set_sample_smem_limits()
 int launch_init(Ctx& c)
 {
     if (c.N == 0) return 0;
-    const uint2 key = make_uint2((uint32_t)c.seed, (uint32_t)(c.seed >> 32));
+    const PhiloxKey key(c.seed);
     const int g = grid_for(c.N, 256);
     if (c.wide_topics) k_init<int32_t><<<g, 256, 0, c.stream>>>(c.v, key);
     else k_init<uint16_t><<<g, 256, 0, c.stream>>>(c.v, key);
