@@ -646,6 +646,7 @@ static int load_lists(Ctx& c, const int32_t* words_dev, int64_t n_tokens, const 
         // its instructions and 2^22 is best (738 M tokens, K = 10 000: 23.2 ms per sweep, 24.0 with 2^20); with
         // counters by those accesses, and 2^20 is (99 M tokens, K = 1000: 3.08 ms, 3.35 with 2^22).
         c.block_shift = c.block_option ? c.block_option : c.doc_dense ? 20 : 22;
+        v.block_shift = c.block_shift;
     }
 
     // The documents' lists are made on another thread; the sorts are queued, the words' lists made beside the second.

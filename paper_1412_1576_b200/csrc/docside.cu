@@ -174,6 +174,19 @@ __device__ __forceinline__ void doc_side_token(const View& v, const Table& table
     if (REGW == 8) __stcs(reinterpret_cast<uint4*>(out) + 1, make_uint4(wr[4], wr[5], wr[6], wr[7]));
 }
 
+// array[first, first + count) of n elements towards L2, in the 16-byte units that hold it.
+template <typename E>
+__device__ __forceinline__ void prefetch_l2(const E* array, int64_t first, int32_t count, int32_t n)
+{
+    constexpr int64_t UNIT = 16 / sizeof(E);
+    const int64_t a = first & ~(UNIT - 1), b = min((first + count + UNIT - 1) & ~(UNIT - 1), (int64_t)n & ~(UNIT - 1));
+    if (a < b)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(array + a), "r"((uint32_t)((b - a) * sizeof(E))) : "memory");
+}
+template <typename T>
+using PairWord = std::conditional_t<sizeof(T) == 2, uint32_t, uint2>;
+constexpr int64_t PREFETCH_AHEAD = 1 << 20;
+
 // `cap` = tokens a tile can hold (the shared-memory carve-up) = DOC_TILE_ROUNDS x blockDim.x: a
 // thread owns at most DOC_TILE_ROUNDS tokens and keeps what it read about them in registers across
 // the phases.  Small tiles keep many CTAs per SM, which is what hides the gathers of the first phase.
@@ -203,6 +216,14 @@ k_doc_tile(View v, const int32_t* __restrict__ tiles, PhiloxKey key, int32_t mh_
     if (cnt == 0) return;
     const int32_t half_k = DENSE ? (v.K + 1) >> 1 : 0;  // words of a document's counters
     const T* zbm = reinterpret_cast<const T*>(v.zbm);
+    // One thread asks for what later tiles read first: the index of the tokens PREFETCH_AHEAD further on, which is more than the
+    // tiles in flight hold, and the same stretch of the next block's topic pairs (a block's pairs are read all over its
+    // tokens).  A warp's gather is as slow as its slowest read: 738 M tokens, K = 10 000: 9.81 -> 9.71 ms; 99 M, K = 1000:
+    // 1.058 -> 1.038.
+    if (tid == THREADS - 32) {
+        prefetch_l2(v.bm_of_tok, (int64_t)base + PREFETCH_AHEAD, cnt, v.N);
+        prefetch_l2(reinterpret_cast<const PairWord<T>*>(v.zbm), (int64_t)base + ((int64_t)1 << v.block_shift), cnt, v.N);
+    }
     uint32_t bm[DOC_TILE_ROUNDS], z[DOC_TILE_ROUNDS], t1[DOC_TILE_ROUNDS];
 #pragma unroll
     for (int r = 0; r < DOC_TILE_ROUNDS; ++r) {

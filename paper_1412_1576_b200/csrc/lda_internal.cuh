@@ -144,6 +144,7 @@ struct View {
     float alpha_f, beta_f, Vbeta_f, filter_eps;
     uint32_t tok_base;  // Philox token key of the corpus' first token (0 unless the corpus is a shard)
     int topic_bits;  // bits of K-1
+    int block_shift; // log2 of the tokens per block of the block-major order
     int count_bits;  // low bits of a packed n_kd entry that hold the count
     // tokens in word-sorted order (position p)
     const uint32_t* tok_orig;  // index of the token in the caller's document order
