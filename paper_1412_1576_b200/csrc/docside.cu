@@ -170,8 +170,11 @@ __device__ __forceinline__ void doc_side_token(const View& v, const Table& table
         if (words & 3) __stcs(reinterpret_cast<uint4*>(out + (words & ~3)), make_uint4(wr[0], wr[1], wr[2], wr[3]));
         return;
     }
-    __stcs(reinterpret_cast<uint4*>(out), make_uint4(wr[0], wr[1], wr[2], wr[3]));
-    if (REGW == 8) __stcs(reinterpret_cast<uint4*>(out) + 1, make_uint4(wr[4], wr[5], wr[6], wr[7]));
+    if (REGW == 8) {
+        store_32(out, make_uint4(wr[0], wr[1], wr[2], wr[3]), make_uint4(wr[4], wr[5], wr[6], wr[7]));
+    } else {
+        __stcs(reinterpret_cast<uint4*>(out), make_uint4(wr[0], wr[1], wr[2], wr[3]));
+    }
 }
 
 // array[first, first + count) of n elements towards L2, in the 16-byte units that hold it.

@@ -379,18 +379,16 @@ __device__ __forceinline__ void accept_tokens(const View& v, Tile& tile, const i
     uint4 rec_c = make_uint4(0u, 0u, 0u, 0u), rec2_c = make_uint4(0u, 0u, 0u, 0u);
     if (p < p_end) at_c = __ldcs(v.inv + p);
     if (p + nthreads < p_end) at_n = __ldcs(v.inv + p + nthreads);
-    if (p < p_end) {
-        rec_c = __ldcs(side4 + (size_t)at_c * quads);
-        if (TWO) rec2_c = __ldcs(side4 + (size_t)at_c * quads + 1);
-    }
+    auto read_record = [&](uint32_t at) {
+        if (TWO) load_32(side4 + (size_t)at * 2, rec_c, rec2_c);
+        else rec_c = __ldcs(side4 + (size_t)at * quads);
+    };
+    if (p < p_end) read_record(at_c);
     for (; p < p_end; p += nthreads) {
         const uint32_t at = at_c;
         const uint4 rec = rec_c, rec2 = rec2_c;  // own record, then the words pass 2 gathered
         at_c = at_n;
-        if (p + nthreads < p_end) {
-            rec_c = __ldcs(side4 + (size_t)at_c * quads);
-            if (TWO) rec2_c = __ldcs(side4 + (size_t)at_c * quads + 1);
-        }
+        if (p + nthreads < p_end) read_record(at_c);
         if (p + 2 * nthreads < p_end) at_n = __ldcs(v.inv + p + 2 * nthreads);
         const uint32_t* side = v.dside + (size_t)at * v.side_stride;
         auto side_word = [&](int32_t i) {
