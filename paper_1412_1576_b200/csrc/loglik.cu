@@ -5,6 +5,7 @@
 // Each CTA writes one partial sum; a last kernel adds the partials in a fixed order.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "lda_device.cuh"
 #include "lda_internal.cuh"
@@ -20,23 +21,28 @@ constexpr int LL_TABLE = 512;
 // them, would otherwise cost a chain of reads each); rows of more than LL_ROW entries are left and taken in
 // pieces of LL_ROW by all warps: `longer` lists the words that can have one.
 constexpr int LL_ROW = ALIAS_MID_MAX;
-__global__ void __launch_bounds__(256) k_ll_word(View v, double lg_beta, int32_t per_warp, const int32_t* __restrict__ longer,
-                                                 int32_t n_longer, const double* __restrict__ tab, double* __restrict__ out)
+struct LlWords {
+    double lg_beta;
+    int32_t per_warp;          // words a warp takes at a time
+    const int32_t* longer;     // [n_longer]
+    int32_t n_longer;
+    const double* tab;         // [LL_TABLE] lgamma(c + beta) - lgamma(beta)
+};
+// The share of CTA `block` of `blocks`; the CTA's sum, on every thread.
+__device__ __forceinline__ double ll_word_part(const View& v, const LlWords& a, int block, int blocks, double* small, double* tmp)
 {
-    __shared__ double tmp[32];
-    __shared__ double small[LL_TABLE];
-    for (int c = threadIdx.x; c < LL_TABLE; c += blockDim.x) small[c] = tab[c];
+    for (int c = threadIdx.x; c < LL_TABLE; c += blockDim.x) small[c] = a.tab[c];
     __syncthreads();
-    const int warps = (gridDim.x * blockDim.x) >> 5, lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int warps = (blocks * (int)blockDim.x) >> 5, lane = threadIdx.x & 31;
+    const int thread = block * (int)blockDim.x + (int)threadIdx.x, warp = thread >> 5;
     double s = 0.0;
     auto add = [&](int32_t at) {
         const uint32_t c = v.wk_count[at];
-        s += c < (uint32_t)LL_TABLE ? small[c] : lgamma((double)c + v.beta) - lg_beta;
+        s += c < (uint32_t)LL_TABLE ? small[c] : lgamma((double)c + v.beta) - a.lg_beta;
     };
-    for (int32_t wb = warp * per_warp; wb < v.V; wb += warps * per_warp) {
+    for (int32_t wb = warp * a.per_warp; wb < v.V; wb += warps * a.per_warp) {
         int32_t n_mine = 0, r_mine = 0;
-        if (lane < per_warp && wb + lane < v.V) {
+        if (lane < a.per_warp && wb + lane < v.V) {
             n_mine = v.wk_nnz[wb + lane];
             r_mine = v.row_start[wb + lane];
         }
@@ -47,15 +53,21 @@ __global__ void __launch_bounds__(256) k_ll_word(View v, double lg_beta, int32_t
         }
     }
     const int32_t pieces = (v.K + LL_ROW - 1) / LL_ROW;
-    for (int64_t i = warp; i < (int64_t)n_longer * pieces; i += warps) {
-        const int32_t w = longer[i / pieces], n = v.wk_nnz[w], j0 = (int32_t)(i % pieces) * LL_ROW;
+    for (int64_t i = warp; i < (int64_t)a.n_longer * pieces; i += warps) {
+        const int32_t w = a.longer[i / pieces], n = v.wk_nnz[w], j0 = (int32_t)(i % pieces) * LL_ROW;
         if (n <= LL_ROW || j0 >= n) continue;
         const int32_t r0 = v.row_start[w], j1 = min(n, j0 + LL_ROW);
         for (int32_t j = j0 + lane; j < j1; j += 32) add(r0 + j);
     }
-    for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < v.K; k += gridDim.x * blockDim.x)
-        s -= lgamma((double)v.nk[k] + v.Vbeta);
-    s = block_reduce_sum<double>(s, tmp);
+    for (int32_t k = thread; k < v.K; k += blocks * (int)blockDim.x) s -= lgamma((double)v.nk[k] + v.Vbeta);
+    return block_reduce_sum<double>(s, tmp);
+}
+
+__global__ void __launch_bounds__(256) k_ll_word(View v, LlWords a, double* __restrict__ out)
+{
+    __shared__ double tmp[32];
+    __shared__ double small[LL_TABLE];
+    const double s = ll_word_part(v, a, (int)blockIdx.x, (int)gridDim.x, small, tmp);
     if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
@@ -91,17 +103,15 @@ __device__ __noinline__ double lgamma_out_of_line(double x) { return lgamma(x); 
 // One partial sum per tile (a second kernel adds them in a fixed order) and the number of filled
 // slots, nnz(n_kd).
 template <typename T, int THREADS>
-__global__ void __launch_bounds__(THREADS, 1536 / THREADS)
-k_ll_doc_tiles(View v, const int32_t* __restrict__ tiles, double lg_alpha, const double* __restrict__ tab,
-               double* __restrict__ tile_part, uint32_t* __restrict__ tile_nnz)
+__device__ __forceinline__ void ll_doc_tile(const View& v, int tile, const int32_t* __restrict__ tiles, double lg_alpha,
+                                            const double* __restrict__ tab, double* __restrict__ tile_part,
+                                            uint32_t* __restrict__ tile_nnz, uint32_t* doc_smem, double* tmp)
 {
     constexpr int cap = DOC_TILE_ROUNDS * THREADS;
-    extern __shared__ __align__(16) uint32_t doc_smem[];
-    __shared__ double tmp[32];
     uint32_t* slots = doc_smem;                                                            // [DK_SLOTS_PER_TOKEN * cap]
     int32_t* soff = reinterpret_cast<int32_t*>(slots + DK_SLOTS_PER_TOKEN * cap);          // [cap + 1]
     const int tid = threadIdx.x;
-    const int32_t s0 = tiles[2 * blockIdx.x], s1 = tiles[2 * blockIdx.x + 1];
+    const int32_t s0 = tiles[2 * tile], s1 = tiles[2 * tile + 1];
     const int32_t nseg = s1 - s0;
     const int32_t base = v.doc_off[s0];
     const int32_t cnt = v.doc_off[s1] - base;
@@ -154,10 +164,20 @@ k_ll_doc_tiles(View v, const int32_t* __restrict__ tiles, double lg_alpha, const
         if (len > 0) s -= len < LL_TABLE ? __ldg(tab + LL_TABLE + len) : lgamma_out_of_line((double)len + v.Kalpha);
     }
     s = block_reduce_sum<double>(s, tmp);
-    if (tid == 0) tile_part[blockIdx.x] = s;
+    if (tid == 0) tile_part[tile] = s;
     __syncthreads();
     filled = block_reduce_sum<uint32_t>(filled, reinterpret_cast<uint32_t*>(tmp));
-    if (tid == 0) tile_nnz[blockIdx.x] = filled;
+    if (tid == 0) tile_nnz[tile] = filled;
+}
+
+template <typename T, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1536 / THREADS)
+k_ll_doc_tiles(View v, const int32_t* __restrict__ tiles, double lg_alpha, const double* __restrict__ tab,
+               double* __restrict__ tile_part, uint32_t* __restrict__ tile_nnz)
+{
+    extern __shared__ __align__(16) uint32_t doc_smem[];
+    __shared__ double tmp[32];
+    ll_doc_tile<T, THREADS>(v, (int)blockIdx.x, tiles, lg_alpha, tab, tile_part, tile_nnz, doc_smem, tmp);
 }
 
 // Adds the tiles' partial sums: CTA b takes the b-th run of `per` consecutive tiles, always in the same order.
@@ -215,38 +235,82 @@ k_ll_doc_long(View v, int32_t n_long, double lg_alpha, const double* __restrict_
     if (threadIdx.x == 0) nnz_out[blockIdx.x] = (uint32_t)filled;
 }
 
-// Last kernel: the partial sums of both parts, always in the same order, and the error word, to host memory.
-__global__ void __launch_bounds__(512) k_ll_finish(const double* __restrict__ word, int32_t n_word, const double* __restrict__ doc_a,
-                                                   const uint32_t* __restrict__ nnz_a, int32_t n_a, const double* __restrict__ doc_b,
-                                                   const uint32_t* __restrict__ nnz_b, int32_t n_b, const int* __restrict__ err,
-                                                   SweepReport* __restrict__ rep)
+// The partial sums of both parts, always in the same order, and the error word, to host memory.  One CTA.
+struct LlSums {
+    const double* word;
+    int32_t n_word;
+    const double* doc_a;
+    const uint32_t* nnz_a;
+    int32_t n_a;
+    const double* doc_b;
+    const uint32_t* nnz_b;
+    int32_t n_b;
+    const int* err;
+    SweepReport* rep;
+};
+__device__ __forceinline__ void ll_finish(const LlSums& p, double* tmp, unsigned long long* tmp_n)
 {
-    __shared__ double tmp[32];
-    __shared__ unsigned long long tmp_n[32];
     double w = 0.0, d = 0.0;
     unsigned long long nnz = 0;
-    for (int32_t i = threadIdx.x; i < n_word; i += blockDim.x) w += word[i];
-    for (int32_t i = threadIdx.x; i < n_a; i += blockDim.x) {
-        d += doc_a[i];
-        nnz += nnz_a[i];
+    for (int32_t i = threadIdx.x; i < p.n_word; i += blockDim.x) w += __ldcg(p.word + i);
+    for (int32_t i = threadIdx.x; i < p.n_a; i += blockDim.x) {
+        d += __ldcg(p.doc_a + i);
+        nnz += __ldcg(p.nnz_a + i);
     }
-    for (int32_t i = threadIdx.x; i < n_b; i += blockDim.x) {
-        d += doc_b[i];
-        nnz += nnz_b[i];
+    for (int32_t i = threadIdx.x; i < p.n_b; i += blockDim.x) {
+        d += __ldcg(p.doc_b + i);
+        nnz += __ldcg(p.nnz_b + i);
     }
     w = block_reduce_sum<double>(w, tmp);
     __syncthreads();
     d = block_reduce_sum<double>(d, tmp);
     nnz = block_reduce_sum<unsigned long long>(nnz, tmp_n);
     if (threadIdx.x == 0) {
-        rep->ll_word = w;
-        rep->ll_doc = d;
-        rep->nnz_dk = nnz;
-        rep->err = *err;
+        p.rep->ll_word = w;
+        p.rep->ll_doc = d;
+        p.rep->nnz_dk = nnz;
+        p.rep->err = __ldcg(p.err);
     }
+}
+__global__ void __launch_bounds__(512) k_ll_finish(LlSums p)
+{
+    __shared__ double tmp[32];
+    __shared__ unsigned long long tmp_n[32];
+    ll_finish(p, tmp, tmp_n);
+}
+
+// Small corpora: all of it as one kernel.  The first CTAs take a tile of documents each, the others the word part, and
+// the last one to be done adds the partial sums up (`arrived` counts them and is zero between calls).  Three
+// kernels on two streams take the host nine calls, which is longer than a corpus of 10 000 tokens takes the device.
+template <typename T, int THREADS>
+__global__ void __launch_bounds__(THREADS)
+k_ll_all(View v, const int32_t* __restrict__ tiles, int32_t n_tiles, double lg_alpha, const double* __restrict__ tab,
+         double* __restrict__ tile_part, uint32_t* __restrict__ tile_nnz, LlWords words, double* __restrict__ word_part,
+         LlSums sums, unsigned int* __restrict__ arrived)
+{
+    extern __shared__ __align__(16) uint32_t doc_smem[];
+    __shared__ double tmp[32];
+    __shared__ unsigned long long tmp_n[32];
+    __shared__ bool last;
+    const int block = (int)blockIdx.x;
+    if (block < n_tiles) {
+        ll_doc_tile<T, THREADS>(v, block, tiles, lg_alpha, tab, tile_part, tile_nnz, doc_smem, tmp);
+    } else {
+        const double s = ll_word_part(v, words, block - n_tiles, (int)gridDim.x - n_tiles, reinterpret_cast<double*>(doc_smem), tmp);
+        if (threadIdx.x == 0) word_part[block - n_tiles] = s;
+    }
+    if (threadIdx.x == 0) {  // the partial sums are this thread's stores
+        __threadfence();
+        last = atomicAdd(arrived, 1u) + 1u == gridDim.x;
+        if (last) *arrived = 0u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (last) ll_finish(sums, tmp, tmp_n);
 }
 
 constexpr int LL_TILE_SUMS = 1024;  // partial sums the tiles' sums are folded into
+constexpr int LL_ONE_KERNEL_TILES = 1024;  // up to this many tiles everything is one kernel
 constexpr int LL_TILE_DIRECT = 4096;  // up to this many tiles the last kernel adds them up itself
 
 static int long_ll_grid(const Ctx& c) { return std::max(1, std::min<int>(c.n_long_docs, LL_BLOCKS)); }
@@ -267,6 +331,25 @@ static void launch_ll_tiles(Ctx& c, size_t smem, double lg_alpha, cudaStream_t s
     else launch_ll_tiles_t<uint16_t>(c, smem, lg_alpha, stream);
 }
 
+template <typename T>
+static void launch_ll_all_t(Ctx& c, const LlWords& words, int n_word, const LlSums& sums, double lg_alpha, double* word_part)
+{
+    const size_t smem = doc_tile_smem_bytes(c.doc_tile);
+    const int grid = c.n_doc_tiles + n_word;
+    auto go = [&](auto threads) {
+        constexpr int THREADS = decltype(threads)::value;
+        static_assert(LL_TABLE * 8 <= DOC_TILE_ROUNDS * THREADS * DOC_TILE_SMEM_PER_TOKEN, "the word part's table fits in a tile's room");
+        k_ll_all<T, THREADS><<<grid, THREADS, smem, c.stream>>>(c.v, c.doc_tiles, c.n_doc_tiles, lg_alpha, c.ll_tab, c.ll_tile_part,
+                                                                c.ll_tile_nnz, words, word_part, sums, reinterpret_cast<unsigned int*>(c.red_i + 1));
+    };
+    switch (c.doc_threads) {
+        case 128: go(std::integral_constant<int, 128>{}); break;
+        case 256: go(std::integral_constant<int, 256>{}); break;
+        case 512: go(std::integral_constant<int, 512>{}); break;
+        default: go(std::integral_constant<int, 1024>{}); break;
+    }
+}
+
 // Queues the word part (if asked for) and the document part, side by side, and the kernel that reports their sums.
 static void queue_loglik(Ctx& c, bool word_part)
 {
@@ -280,20 +363,27 @@ static void queue_loglik(Ctx& c, bool word_part)
     uint32_t* nnz_b = nnz + LL_TILE_SUMS;
     const double lg_beta = std::lgamma(c.beta);
     if (!c.ll_tables_ready) {
+        cudaMemsetAsync(c.red_i + 1, 0, 8, c.stream);  // k_ll_all's count of CTAs
         k_ll_fill_tables<<<3 * LL_TABLE / 64, 64, 0, c.stream>>>(c.v, lg_alpha, lg_beta, c.ll_tab);
         c.ll_tables_ready = true;
     }
-    fork_streams(c);
+    LlWords words{lg_beta, 32, c.alias_words[2], c.n_alias_words[2], c.ll_tab + 2 * LL_TABLE};
     if (word_part) {
-        int per_warp = 32;
-        while (per_warp > 1 && c.V / per_warp < c.n_sm * 16) per_warp /= 2;
-        n_word = (int)std::min<int64_t>(LL_BLOCKS, (c.V + 8 * (int64_t)per_warp - 1) / (8 * (int64_t)per_warp));
+        while (words.per_warp > 1 && c.V / words.per_warp < c.n_sm * 16) words.per_warp /= 2;
+        n_word = (int)std::min<int64_t>(LL_BLOCKS, (c.V + 8 * (int64_t)words.per_warp - 1) / (8 * (int64_t)words.per_warp));
         // a warp per piece of a long row, a thread per topic
         const int64_t pieces = (int64_t)c.n_alias_words[2] * ((c.K + LL_ROW - 1) / LL_ROW);
         n_word = (int)std::min<int64_t>(LL_BLOCKS, std::max<int64_t>({(int64_t)n_word, (pieces + 7) / 8, ((int64_t)c.K + 255) / 256}));
-        k_ll_word<<<n_word, 256, 0, c.side[0]>>>(c.v, lg_beta, per_warp, c.alias_words[2], c.n_alias_words[2],
-                                                 c.ll_tab + 2 * LL_TABLE, part);
     }
+    if (word_part && !c.n_long_docs && c.n_doc_tiles > 0 && c.n_doc_tiles <= LL_ONE_KERNEL_TILES) {
+        n_word = std::min<int>(LL_BLOCKS, n_word * 256 / c.doc_threads + 1);
+        const LlSums sums{part, n_word, c.ll_tile_part, c.ll_tile_nnz, c.n_doc_tiles, doc_b, nnz_b, 0, c.v.err, c.report};
+        if (c.wide_topics) launch_ll_all_t<int32_t>(c, words, n_word, sums, lg_alpha, part);
+        else launch_ll_all_t<uint16_t>(c, words, n_word, sums, lg_alpha, part);
+        return;
+    }
+    fork_streams(c);
+    if (word_part) k_ll_word<<<n_word, 256, 0, c.side[0]>>>(c.v, words, part);
     if (c.n_long_docs) {
         n_b = long_ll_grid(c);
         launch_long_tables(c, c.side[1], false, -1);
@@ -312,7 +402,7 @@ static void queue_loglik(Ctx& c, bool word_part)
         }
     }
     join_streams(c);
-    k_ll_finish<<<1, 512, 0, c.stream>>>(part, n_word, doc_a, nnz_a, n_a, doc_b, nnz_b, n_b, c.v.err, c.report);
+    k_ll_finish<<<1, 512, 0, c.stream>>>(LlSums{part, n_word, doc_a, nnz_a, n_a, doc_b, nnz_b, n_b, c.v.err, c.report});
 }
 
 int launch_loglik(Ctx& c, double* out3_host)
@@ -348,6 +438,8 @@ void set_loglik_smem_limits()
     const int doc_bytes = (int)doc_tile_smem_bytes(DOC_TILE_MAX);
     cudaFuncSetAttribute(k_ll_doc_tiles<uint16_t, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, doc_bytes);
     cudaFuncSetAttribute(k_ll_doc_tiles<int32_t, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, doc_bytes);
+    cudaFuncSetAttribute(k_ll_all<uint16_t, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, doc_bytes);
+    cudaFuncSetAttribute(k_ll_all<int32_t, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, doc_bytes);
 }
 
 }  // namespace lda

@@ -247,3 +247,24 @@ def test_sorted_rows_of_tiles_of_every_length(tokens):
     for e in (g, o):
         e.sweep(2, 2)
     _same(g, o)
+
+
+@pytest.mark.parametrize("docs,V,K", [(1, 3, 1), (7, 40_000, 50), (1_024, 300, 40), (1_025, 300, 40), (40, 2, 9_000), (40, 50, 70_000)])
+def test_log_likelihood_by_one_kernel_and_by_several(docs, V, K):
+    """As many tiles of documents as one kernel takes and one more; rows longer than a warp's, large vocabularies.  Sums of
+    at most 4 10^5 terms: 1e-10 covers their order."""
+    rng = np.random.default_rng(docs)
+    words = rng.integers(0, V, docs * 384).astype(np.int32)
+    offsets = (np.arange(docs + 1) * 384).astype(np.int64)
+    g, o = binding.LightLDA(V, K, 0.05, 0.01), ldaref.Oracle(V, K, 0.05, 0.01)
+    for e in (g, o):
+        e.load_corpus(words, offsets)
+        e.init(2)
+    first = g.loglik()
+    for a, b in zip(first, o.loglik()):
+        assert a == pytest.approx(b, rel=1e-10)
+    assert g.loglik() == first      # and again
+    for e in (g, o):
+        e.sweep(1, 2)
+    for a, b in zip(g.loglik(), o.loglik()):
+        assert a == pytest.approx(b, rel=1e-10)
