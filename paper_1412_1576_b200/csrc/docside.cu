@@ -21,8 +21,6 @@
 namespace lda {
 
 constexpr double INV_2_32 = 1.0 / 4294967296.0;
-// slots per token of the tables a tile builds in shared memory (DOC_TILE_SLOTS, a multiple of 4)
-constexpr int TILE_SLOTS = DOC_TILE_SLOTS;
 
 // A token's current topic and its first word-proposal sit side by side at its block-major index:
 // one read brings both.
@@ -42,7 +40,7 @@ __device__ __forceinline__ void load_topic_pair(const int32_t* zbm, uint32_t bm,
 // --- n_kd of a document in a tile, in shared memory ----------------------------------------------
 // Two forms, chosen per corpus (load_common()):
 //   DENSE   a 16-bit counter per topic (K even or padded): an addition, a read;
-//   hashed  TILE_SLOTS slots per token, as dk_insert in lda_device.cuh has it.  (Probing aligned pairs of slots by
+//   hashed  tile_slots() slots per token, as dk_insert in lda_device.cuh has it.  (Probing aligned pairs of slots by
 //           8-byte reads: fewer turns of the loop, more instructions each; 10.6 ms per sweep instead of 10.1 at 738 M
 //           tokens.)
 // Both give (topic << count_bits) | n_kd.
@@ -200,13 +198,20 @@ __host__ __device__ constexpr int doc_resident_threads(int mode, int fixed)
 {
     return (fixed == 2 && mode != LDA_PROPOSALS_DOC) ? 2048 : 1536;
 }
+// Slots per token of the hashed tables.  More of them mean shorter searches, but what shared memory takes L1 lacks, and its lines
+// are what the gathers in flight wait in: with 16 CTAs per SM five slots take 10.5 ms and six 13.4 instead of 9.72 (738 M
+// tokens, K = 10 000, two steps); with the twelve of the other forms six are ahead (74 M, four steps: 1.509 -> 1.447 ms).
+__host__ __device__ constexpr int tile_slots(int mode, int fixed, bool dense)
+{
+    return dense ? DOC_TILE_SLOTS : doc_resident_threads(mode, fixed) == 2048 ? DOC_TILE_SLOTS : 6;
+}
 template <typename T, int THREADS, int MODE, int FIXED, bool DENSE>
 __global__ void __launch_bounds__(THREADS, doc_resident_threads(MODE, FIXED) / THREADS)
 k_doc_tile(View v, const int32_t* __restrict__ tiles, PhiloxKey key, int32_t mh_steps_arg)
 {
     stamp(v, STAMP_DOC_TILES);
     const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
-    constexpr int cap = DOC_TILE_ROUNDS * THREADS;
+    constexpr int cap = DOC_TILE_ROUNDS * THREADS, TILE_SLOTS = tile_slots(MODE, FIXED, DENSE);
     extern __shared__ __align__(16) uint32_t doc_smem[];
     uint32_t* area = doc_smem;                                           // [TILE_SLOTS * cap] the tile's tables
     int32_t* soff = reinterpret_cast<int32_t*>(area + TILE_SLOTS * cap);  // [cap + 1] document offsets
@@ -240,7 +245,7 @@ k_doc_tile(View v, const int32_t* __restrict__ tiles, PhiloxKey key, int32_t mh_
     uint32_t doc[DOC_TILE_ROUNDS];  // first token of the token's document | its length << 16: every register counts here
     for (int j = tid; j <= nseg; j += THREADS) soff[j] = v.doc_off[s0 + j] - base;
     const uint32_t none = DENSE ? 0u : DK_EMPTY;
-    const int quads = DENSE ? (nseg * half_k + 3) >> 2 : cnt * (TILE_SLOTS / 4);
+    const int quads = DENSE ? (nseg * half_k + 3) >> 2 : (cnt * TILE_SLOTS + 3) >> 2;
     for (int j = tid; j < quads; j += THREADS) reinterpret_cast<uint4*>(area)[j] = make_uint4(none, none, none, none);
     __syncthreads();
     // every token finds its document and adds itself to the document's table
@@ -412,15 +417,17 @@ int launch_long_tables(Ctx& c, cudaStream_t stream, bool keep_topics, int stamp_
     return 1;
 }
 
-size_t doc_tile_smem_bytes(int tile_tokens) { return (size_t)tile_tokens * DOC_TILE_SMEM_PER_TOKEN + 16; }
+size_t doc_tile_smem_bytes(int tile_tokens, int slots) { return (size_t)tile_tokens * (4 * slots + 4 + 4) + 16; }
 
 template <typename T, int MODE, int FIXED>
 static void set_doc_limit()
 {
-    const int bytes = (int)doc_tile_smem_bytes(DOC_TILE_MAX);
-    cudaFuncSetAttribute(k_doc_tile<T, 1024, MODE, FIXED, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    constexpr auto most = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    constexpr int hashed = tile_slots(MODE, FIXED, false), dense = tile_slots(MODE, FIXED, true);
+    cudaFuncSetAttribute(k_doc_tile<T, 512, MODE, FIXED, false>, most, (int)doc_tile_smem_bytes(DOC_TILE_ROUNDS * 512, hashed));
+    cudaFuncSetAttribute(k_doc_tile<T, 1024, MODE, FIXED, false>, most, (int)doc_tile_smem_bytes(DOC_TILE_MAX, hashed));
     if (sizeof(T) == 2)
-        cudaFuncSetAttribute(k_doc_tile<uint16_t, 1024, MODE, FIXED, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        cudaFuncSetAttribute(k_doc_tile<uint16_t, 1024, MODE, FIXED, true>, most, (int)doc_tile_smem_bytes(DOC_TILE_MAX, dense));
 }
 
 void set_doc_smem_limits()
@@ -448,9 +455,9 @@ static int doc_side_tm(Ctx& c, int mh_steps)
     const PassStreams on(c, (c.n_doc_tiles > 0) + (c.n_long_chunks > 0));
     int launches = 0;
     if (c.n_doc_tiles) {
-        const size_t smem = doc_tile_smem_bytes(c.doc_tile);
         auto tiles = [&](auto dense) {
             constexpr bool DENSE = decltype(dense)::value;
+            const size_t smem = doc_tile_smem_bytes(c.doc_tile, tile_slots(MODE, FIXED, DENSE));
             switch (c.doc_threads) {
                 case 128: k_doc_tile<T, 128, MODE, FIXED, DENSE><<<c.n_doc_tiles, 128, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
                 case 256: k_doc_tile<T, 256, MODE, FIXED, DENSE><<<c.n_doc_tiles, 256, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;

@@ -60,10 +60,7 @@ constexpr int DOC_TILE_THREADS[DOC_TILE_SHAPES] = {128, 256, 512, 1024};
 constexpr int DOC_TILE_TOKENS[DOC_TILE_SHAPES] = {DOC_TILE_ROUNDS * 128, DOC_TILE_ROUNDS * 256, DOC_TILE_ROUNDS * 512,
                                                   DOC_TILE_ROUNDS * 1024};
 constexpr int DOC_TILE_MAX = DOC_TILE_ROUNDS * 1024;
-constexpr int DOC_TILE_SLOTS = 4;  // 32-bit words per token of a tile's tables in shared memory
-static_assert(DOC_TILE_SLOTS % 4 == 0, "a tile's tables are cleared 16 bytes at a time");
-// shared memory per token of a tile: table, document offset, topic or slot
-constexpr int DOC_TILE_SMEM_PER_TOKEN = 4 * DOC_TILE_SLOTS + 4 + 4;
+constexpr int DOC_TILE_SLOTS = 4;  // 32-bit words per token of a tile's counters, and of most hashed tables (tile_slots())
 // partial sums of the log-likelihood kernels: word part; document part (tiles + long documents)
 constexpr int LL_WORD_PARTIALS = 592;
 constexpr int LL_DOC_PARTIALS = 148 * 16 + 592 + 1024;
@@ -402,7 +399,7 @@ void set_slice(Ctx& c, int slice);          // makes `slice` the running one (mo
 int launch_sample(Ctx& c, int mh_steps);   // all passes of the MH step; needs ensure_exchange()
 int launch_doc_side(Ctx& c, int mh_steps);  // pass 2 of the MH step
 int launch_long_tables(Ctx& c, cudaStream_t stream, bool keep_topics, int stamp_id);  // n_kd tables of the documents longer than a tile
-size_t doc_tile_smem_bytes(int tile_tokens);  // dynamic shared memory of the document-tile kernels
+size_t doc_tile_smem_bytes(int tile_tokens, int slots);  // dynamic shared memory of the document-tile kernels, `slots` a token
 int ensure_exchange(Ctx& c, int mh_steps);  // (re)allocates View::prop / View::dside; LDA_* status
 int launch_loglik(Ctx& c, double* out3_host);
 int launch_count_nnz(Ctx& c, int64_t* nnz_wk_host, int64_t* nnz_dk_host);

@@ -334,11 +334,11 @@ static void launch_ll_tiles(Ctx& c, size_t smem, double lg_alpha, cudaStream_t s
 template <typename T>
 static void launch_ll_all_t(Ctx& c, const LlWords& words, int n_word, const LlSums& sums, double lg_alpha, double* word_part)
 {
-    const size_t smem = doc_tile_smem_bytes(c.doc_tile);
+    const size_t smem = doc_tile_smem_bytes(c.doc_tile, DK_SLOTS_PER_TOKEN);
     const int grid = c.n_doc_tiles + n_word;
     auto go = [&](auto threads) {
         constexpr int THREADS = decltype(threads)::value;
-        static_assert(LL_TABLE * 8 <= DOC_TILE_ROUNDS * THREADS * DOC_TILE_SMEM_PER_TOKEN, "the word part's table fits in a tile's room");
+        static_assert(LL_TABLE * 8 <= DOC_TILE_ROUNDS * THREADS * 4 * DK_SLOTS_PER_TOKEN, "the word part's table fits in a tile's room");
         k_ll_all<T, THREADS><<<grid, THREADS, smem, c.stream>>>(c.v, c.doc_tiles, c.n_doc_tiles, lg_alpha, c.ll_tab, c.ll_tile_part,
                                                                 c.ll_tile_nnz, words, word_part, sums, reinterpret_cast<unsigned int*>(c.red_i + 1));
     };
@@ -390,7 +390,7 @@ static void queue_loglik(Ctx& c, bool word_part)
         k_ll_doc_long<<<n_b, 512, 0, c.side[1]>>>(c.v, c.n_long_docs, lg_alpha, c.ll_tab, doc_b, nnz_b);
     }
     if (c.n_doc_tiles) {
-        launch_ll_tiles(c, doc_tile_smem_bytes(c.doc_tile), lg_alpha, c.stream);
+        launch_ll_tiles(c, doc_tile_smem_bytes(c.doc_tile, DK_SLOTS_PER_TOKEN), lg_alpha, c.stream);
         if (c.n_doc_tiles <= LL_TILE_DIRECT) {
             doc_a = c.ll_tile_part;
             nnz_a = c.ll_tile_nnz;
@@ -435,7 +435,7 @@ int launch_count_nnz(Ctx& c, int64_t* nnz_wk_host, int64_t* nnz_dk_host)
 
 void set_loglik_smem_limits()
 {
-    const int doc_bytes = (int)doc_tile_smem_bytes(DOC_TILE_MAX);
+    const int doc_bytes = (int)doc_tile_smem_bytes(DOC_TILE_MAX, DK_SLOTS_PER_TOKEN);
     cudaFuncSetAttribute(k_ll_doc_tiles<uint16_t, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, doc_bytes);
     cudaFuncSetAttribute(k_ll_doc_tiles<int32_t, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, doc_bytes);
     cudaFuncSetAttribute(k_ll_all<uint16_t, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, doc_bytes);
