@@ -67,7 +67,7 @@ constexpr int LL_DOC_PARTIALS = 148 * 16 + 592 + 1024;
 constexpr int HIST_BINS = 32768;     // shared-memory histogram window (32-bit bins)
 constexpr int WORD_ROWS_BITMAP_MAX_K = 16384;  // tail rows: topic bitmap up to this K, key sort above
 constexpr int HIST16_BINS = 106496;  // window of a warm word's n_kw histogram (16-bit bins, 208 KB)
-constexpr int HIST32_BINS = 49152;   // window of a hot word's n_kw histogram (32-bit bins, 192 KB)
+constexpr int HIST32_BINS = 53248;   // window of a hot word's n_kw histogram (32-bit bins, 208 KB)
 constexpr int HIST_RUN_MAX = 262144;  // tokens per CTA (one run of a word) in the histogram path, at most
 constexpr int ROW_TILE_WORDS = 512;   // words per tile of the tail words' row kernel
 // n_k added up by the row kernels themselves (choose_nk_mode())
