@@ -432,6 +432,7 @@ void set_gibbs_smem_limits();
 cudaError_t copy_to_host(Ctx& c, void* host, const void* dev, size_t bytes);
 cudaError_t copy_to_device(Ctx& c, void* dev, const void* host, size_t bytes);
 bool page_locked(const void* host);
+void* device_view(const void* host, size_t bytes);  // address that kernels reach page-locked memory by, or null
 
 // n_kw as compact rows in device memory: row offsets [V+1] and the entries (export.cu).  LDA_* status.
 struct WkCsr {

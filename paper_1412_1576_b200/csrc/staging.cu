@@ -76,6 +76,19 @@ bool page_locked(const void* p)
     return a.type != cudaMemoryTypeUnregistered;
 }
 
+void* device_view(const void* p, size_t bytes)
+{
+    cudaPointerAttributes a{}, b{};
+    const char* const last = static_cast<const char*>(p) + (bytes - 1);
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaPointerGetAttributes(&b, last) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer || !b.devicePointer) return nullptr;
+    const bool one = static_cast<char*>(b.devicePointer) - static_cast<char*>(a.devicePointer) == (ptrdiff_t)(bytes - 1);
+    return one ? a.devicePointer : nullptr;
+}
+
 template <bool TO_HOST>
 static cudaError_t move_lane(Lane& l, int device, int first, char* host, char* dev, size_t bytes, size_t piece)
 {

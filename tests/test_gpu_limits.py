@@ -127,6 +127,29 @@ def test_imported_counts_beyond_16_bits():
             assert np.array_equal(g.get_assignments(), o.get_assignments()), (times, iters)
 
 
+@pytest.mark.parametrize("K,n", [(16, 1), (16, 131_072), (16, 131_073), (70_000, 65_536), (70_000, 65_537)])
+@pytest.mark.parametrize("place", ["pinned", "pinned, behind others", "pageable", "pinned, odd address"])
+def test_snapshots_into_any_host_memory(K, n, place):
+    """As many tokens as the kernel writes to page-locked memory itself, and one more; nothing beside them is touched."""
+    import torch
+    words = (np.arange(n) % 7).astype(np.int32)
+    g, o = binding.LightLDA(7, K, 0.1, 0.01), ldaref.Oracle(7, K, 0.1, 0.01)
+    offsets = np.minimum(np.arange(n // 64 + 2) * 64, n).astype(np.int64)
+    for e in (g, o):
+        e.load_corpus(words, offsets)
+        e.init(3)
+    size = 2 if K <= 65_536 else 4
+    first = {"pinned": 0, "pageable": 0, "pinned, behind others": 6 * size, "pinned, odd address": 6 * size + 1}[place]
+    held = torch.full((first + n * size + 32,), 0x5A, dtype=torch.uint8, pin_memory=place != "pageable")
+    export = binding.lda_get_assignments_u16_async_ptr if size == 2 else binding.lda_get_assignments_async_ptr
+    assert export(g._h, held.data_ptr() + first) == binding.LDA_OK
+    g.wait()
+    raw = held.numpy()
+    z = np.frombuffer(raw[first:first + n * size].tobytes(), np.uint16 if size == 2 else np.int32)
+    assert np.array_equal(z, o.get_assignments())
+    assert (raw[:first] == 0x5A).all() and (raw[first + n * size:] == 0x5A).all()
+
+
 @pytest.mark.parametrize("offsets", [[0, 2, 1, 4], [0, -1, 4], [0, 5, 4], [0, 2 ** 63 - 1, -2 ** 63, -2 ** 62, 4],
                                      [0, 2 ** 62, 2 ** 63 - 1, -2 ** 63, -2 ** 62, 0, 4]])
 def test_offsets_out_of_order_are_refused(offsets):
