@@ -62,7 +62,7 @@ constexpr int DOC_TILE_TOKENS[DOC_TILE_SHAPES] = {DOC_TILE_ROUNDS * 128, DOC_TIL
 constexpr int DOC_TILE_MAX = DOC_TILE_ROUNDS * 1024;
 constexpr int DOC_TILE_SLOTS = 4;  // 32-bit words per token of a tile's counters, and of most hashed tables (tile_slots())
 // partial sums of the log-likelihood kernels: word part; document part (tiles + long documents)
-constexpr int LL_WORD_PARTIALS = 592;
+constexpr int LL_WORD_PARTIALS = 1184;
 constexpr int LL_DOC_PARTIALS = 148 * 16 + 592 + 1024;
 constexpr int HIST_BINS = 32768;     // shared-memory histogram window (32-bit bins)
 constexpr int WORD_ROWS_BITMAP_MAX_K = 16384;  // tail rows: topic bitmap up to this K, key sort above

@@ -12,7 +12,7 @@
 
 namespace lda {
 
-constexpr int LL_BLOCKS = LL_WORD_PARTIALS;
+constexpr int LL_BLOCKS = 592;  // of 256 threads and more
 // Counts below this take lgamma(count + prior) - lgamma(prior) from a table filled with the same expression: same
 // values as calling lgamma() per entry.
 constexpr int LL_TABLE = 512;
@@ -357,9 +357,9 @@ static void queue_loglik(Ctx& c, bool word_part)
     uint32_t* nnz = c.red_nnz;  // [LL_DOC_PARTIALS]
     const double lg_alpha = std::lgamma(c.alpha);
     int n_word = 0, n_a = 0, n_b = 0;
-    const double* doc_a = part + LL_BLOCKS;
+    const double* doc_a = part + LL_WORD_PARTIALS;
     const uint32_t* nnz_a = nnz;
-    double* doc_b = part + LL_BLOCKS + LL_TILE_SUMS;
+    double* doc_b = part + LL_WORD_PARTIALS + LL_TILE_SUMS;
     uint32_t* nnz_b = nnz + LL_TILE_SUMS;
     const double lg_beta = std::lgamma(c.beta);
     if (!c.ll_tables_ready) {
@@ -376,7 +376,7 @@ static void queue_loglik(Ctx& c, bool word_part)
         n_word = (int)std::min<int64_t>(LL_BLOCKS, std::max<int64_t>({(int64_t)n_word, (pieces + 7) / 8, ((int64_t)c.K + 255) / 256}));
     }
     if (word_part && !c.n_long_docs && c.n_doc_tiles > 0 && c.n_doc_tiles <= LL_ONE_KERNEL_TILES) {
-        n_word = std::min<int>(LL_BLOCKS, n_word * 256 / c.doc_threads + 1);
+        n_word = std::min<int>(LL_WORD_PARTIALS, (n_word * 256 + c.doc_threads - 1) / c.doc_threads);  // as many threads
         const LlSums sums{part, n_word, c.ll_tile_part, c.ll_tile_nnz, c.n_doc_tiles, doc_b, nnz_b, 0, c.v.err, c.report};
         if (c.wide_topics) launch_ll_all_t<int32_t>(c, words, n_word, sums, lg_alpha, part);
         else launch_ll_all_t<uint16_t>(c, words, n_word, sums, lg_alpha, part);
@@ -398,7 +398,7 @@ static void queue_loglik(Ctx& c, bool word_part)
         } else {
             const int per = (c.n_doc_tiles + LL_TILE_SUMS - 1) / LL_TILE_SUMS;
             n_a = (c.n_doc_tiles + per - 1) / per;
-            k_ll_sum_tiles<<<n_a, 256, 0, c.stream>>>(c.ll_tile_part, c.ll_tile_nnz, c.n_doc_tiles, per, part + LL_BLOCKS, nnz);
+            k_ll_sum_tiles<<<n_a, 256, 0, c.stream>>>(c.ll_tile_part, c.ll_tile_nnz, c.n_doc_tiles, per, part + LL_WORD_PARTIALS, nnz);
         }
     }
     join_streams(c);
