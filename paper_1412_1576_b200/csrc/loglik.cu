@@ -376,7 +376,9 @@ static void queue_loglik(Ctx& c, bool word_part)
         n_word = (int)std::min<int64_t>(LL_BLOCKS, std::max<int64_t>({(int64_t)n_word, (pieces + 7) / 8, ((int64_t)c.K + 255) / 256}));
     }
     if (word_part && !c.n_long_docs && c.n_doc_tiles > 0 && c.n_doc_tiles <= LL_ONE_KERNEL_TILES) {
-        n_word = std::min<int>(LL_WORD_PARTIALS, (n_word * 256 + c.doc_threads - 1) / c.doc_threads);  // as many threads
+        // as many threads as the word part has by itself (43 000 tokens, V = 435 000, ten sweeps and a look, three kernels against
+        // one: 549.3 and 553.0 us with half as many, on another GPU 554.4 and 552.9 so)
+        n_word = std::min<int>(LL_WORD_PARTIALS, (n_word * 256 + c.doc_threads - 1) / c.doc_threads);
         const LlSums sums{part, n_word, c.ll_tile_part, c.ll_tile_nnz, c.n_doc_tiles, doc_b, nnz_b, 0, c.v.err, c.report};
         if (c.wide_topics) launch_ll_all_t<int32_t>(c, words, n_word, sums, lg_alpha, part);
         else launch_ll_all_t<uint16_t>(c, words, n_word, sums, lg_alpha, part);
