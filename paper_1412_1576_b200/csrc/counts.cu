@@ -19,8 +19,11 @@
 
 #include "lda_device.cuh"
 #include "lda_internal.cuh"
+#include "tile_sort.cuh"
 
 namespace lda {
+
+static_assert(SORT_TILE == SORT_THREADS * SORT_PER, "tiles of documents and of tail words are as large as what is sorted at once");
 
 struct EmitWord {
     const int32_t* row_start;
@@ -38,71 +41,9 @@ struct EmitWord {
     __device__ __forceinline__ void rows(int32_t seg, int32_t n) const { nnz[seg] = n; }
 };
 
-// Ascending sort of the keys of a tile, eight consecutive ones in every thread's registers; what lies past `cnt` has to be
-// the largest value.  Leaves the keys in `keys` [SORT_TILE] as well.  A bitonic network, its steps by the distance of the two
-// keys that they compare: in a thread's registers, in a warp by shuffles, and only the six widest through shared memory.
-// (All 66 steps there, a barrier after each: n_kw of 200 M tokens, V = 10^6, K = 10^5, 3.69 ms; so 2.55.)
-// 256 threads, all of them call it after a barrier; ends with one.
-constexpr int SORT_PER = SORT_TILE / 256;
-static_assert(SORT_PER == 8, "a thread's keys are two 16-byte words");
-__device__ __forceinline__ void sort_tile(uint32_t (&x)[SORT_PER], uint32_t* keys, int32_t cnt)
-{
-    constexpr uint32_t FULL = 0xFFFFFFFFu;
-    const int tid = threadIdx.x;
-    auto order = [](uint32_t& a, uint32_t& b, bool up) {
-        const uint32_t lo = min(a, b), hi = max(a, b);
-        a = up ? lo : hi;
-        b = up ? hi : lo;
-    };
-    auto in_thread = [&](bool up) {  // steps of 4, 2 and 1 in one direction
-#pragma unroll
-        for (int stride = 4; stride > 0; stride >>= 1)
-#pragma unroll
-            for (int q = 0; q < SORT_PER; ++q)
-                if (!(q & stride)) order(x[q], x[q | stride], up);
-    };
-    uint4* area = reinterpret_cast<uint4*>(keys);  // a thread's two words 256 apart: no bank conflicts
-    auto store = [&](int at0, int at1) {
-        area[at0] = make_uint4(x[0], x[1], x[2], x[3]);
-        area[at1] = make_uint4(x[4], x[5], x[6], x[7]);
-    };
-#pragma unroll
-    for (int q = 0; q < SORT_PER; q += 2) order(x[q], x[q + 1], !(q & 2));
-#pragma unroll
-    for (int q = 0; q < SORT_PER; ++q)
-        if (!(q & 2)) order(x[q], x[q | 2], !(q & 4));
-#pragma unroll
-    for (int q = 0; q < SORT_PER; q += 2) order(x[q], x[q + 1], !(q & 4));
-    in_thread(!(tid & 1));
-    // `size`: keys of a sorted run, in threads; a tile of few keys needs only the first of them
-    for (int size = 2; size <= 256 && size * SORT_PER < 2 * cnt; size <<= 1) {
-        const bool up = !(tid & size);
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            const bool keep_low = !(tid & stride) == up;
-            uint32_t y[SORT_PER];
-            if (stride >= 32) {
-                store(tid, tid + 256);
-                __syncthreads();
-                const uint4 a = area[tid ^ stride], b = area[(tid ^ stride) + 256];
-                __syncthreads();
-                y[0] = a.x; y[1] = a.y; y[2] = a.z; y[3] = a.w;
-                y[4] = b.x; y[5] = b.y; y[6] = b.z; y[7] = b.w;
-            } else {
-#pragma unroll
-                for (int q = 0; q < SORT_PER; ++q) y[q] = __shfl_xor_sync(FULL, x[q], stride);
-            }
-#pragma unroll
-            for (int q = 0; q < SORT_PER; ++q) x[q] = keep_low ? min(x[q], y[q]) : max(x[q], y[q]);
-        }
-        in_thread(up);
-    }
-    store(2 * tid, 2 * tid + 1);
-    __syncthreads();
-}
-
 // Tail words when K is large (the bitmap of k_word_rows would cost more than the sort): one CTA per
 // tile of whole words [s0, s1) holding <= SORT_TILE tokens and <= SORT_TILE words sorts the tile's
-// (word, topic) keys in shared memory (bitonic) and run-length encodes them.
+// (word, topic) keys (tile_sort.cuh) and run-length encodes them.
 template <typename T, class Emit>
 __global__ void __launch_bounds__(256)
 k_seg_count_sorted(const int32_t* __restrict__ tiles, const int32_t* __restrict__ seg_off,
@@ -127,28 +68,8 @@ k_seg_count_sorted(const int32_t* __restrict__ tiles, const int32_t* __restrict_
         for (int j = tid; j < nseg; j += blockDim.x) emit.rows(s0 + j, 0);
         return;
     }
-    // every thread takes eight consecutive tokens: the topics are read in order, then picked up from shared memory
-    for (int j = tid; j < SORT_TILE; j += 256) keys[j] = j < cnt ? (uint32_t)z[base + j] : 0xFFFFFFFFu;
-    __syncthreads();
     uint32_t x[SORT_PER];
-    {
-        const uint4 lo4 = reinterpret_cast<const uint4*>(keys)[2 * tid], hi4 = reinterpret_cast<const uint4*>(keys)[2 * tid + 1];
-        const uint32_t k[SORT_PER] = {lo4.x, lo4.y, lo4.z, lo4.w, hi4.x, hi4.y, hi4.z, hi4.w};
-        int seg = 0, hi = nseg;  // last segment with soff[seg] <= j
-        while (hi - seg > 1) {
-            const int mid = (seg + hi) >> 1;
-            if (soff[mid] <= tid * SORT_PER) seg = mid; else hi = mid;
-        }
-#pragma unroll
-        for (int q = 0; q < SORT_PER; ++q) {
-            const int j = tid * SORT_PER + q;
-            x[q] = 0xFFFFFFFFu;
-            if (j >= cnt) continue;
-            while (soff[seg + 1] <= j) ++seg;
-            if (k[q] >= (uint32_t)K) atomicOr(err, ERR_TOPIC_RANGE);
-            x[q] = ((uint32_t)seg << topic_bits) | k[q];
-        }
-    }
+    if (!tile_keys(x, keys, soff, nseg, z + base, cnt, topic_bits, K)) atomicOr(err, ERR_TOPIC_RANGE);
     sort_tile(x, keys, cnt);
     // head flags -> exclusive scan
     uint32_t flags = 0;
