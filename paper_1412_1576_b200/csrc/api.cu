@@ -1548,7 +1548,7 @@ static int get_assignments(lda_ctx* h, void* z_out, bool narrow, bool wait)
     // stream while the next chunk is collected
     const size_t zt = narrow ? 2 : 4;
     if ((size_t)c.N * zt <= EXPORT_ONE_STREAM_BYTES) {
-        // Page-locked memory is written by the kernel that collects the topics: a copy behind it takes as long as one of a
+        // One piece of page-locked memory is written by the kernel that collects the topics: a copy behind it takes as long as one of a
         // sweep's kernels, and what a caller queues next waits for it (a sweep, a snapshot and the log-likelihood of 10 000
         // tokens: 74 -> 71 us, of 60 000: 87 -> 78).
         void* const view = (uintptr_t)z_out % zt == 0 ? device_view(z_out, (size_t)c.N * zt) : nullptr;

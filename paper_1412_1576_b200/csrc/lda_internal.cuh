@@ -432,7 +432,9 @@ void set_gibbs_smem_limits();
 cudaError_t copy_to_host(Ctx& c, void* host, const void* dev, size_t bytes);
 cudaError_t copy_to_device(Ctx& c, void* dev, const void* host, size_t bytes);
 bool page_locked(const void* host);
-void* device_view(const void* host, size_t bytes);  // address that kernels reach page-locked memory by, or null
+// Address that kernels may write [host, host + bytes) by, or null: it has to lie in one allocation or registration of page-locked
+// memory that is not read-only.
+void* device_view(const void* host, size_t bytes);
 
 // n_kw as compact rows in device memory: row offsets [V+1] and the entries (export.cu).  LDA_* status.
 struct WkCsr {

@@ -9,6 +9,8 @@
 #include <mutex>
 #include <thread>
 
+#include <cuda.h>
+
 #include "lda_internal.cuh"
 
 namespace lda {
@@ -76,17 +78,33 @@ bool page_locked(const void* p)
     return a.type != cudaMemoryTypeUnregistered;
 }
 
+// Of the driver's interface, which is not linked: the runtime's own query says nothing about how far page-locked memory
+// reaches.  (Its first and last byte are not enough: two registrations may have other memory between them, and device
+// addresses are host addresses.)
 void* device_view(const void* p, size_t bytes)
 {
-    cudaPointerAttributes a{}, b{};
-    const char* const last = static_cast<const char*>(p) + (bytes - 1);
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaPointerGetAttributes(&b, last) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer || !b.devicePointer) return nullptr;
-    const bool one = static_cast<char*>(b.devicePointer) - static_cast<char*>(a.devicePointer) == (ptrdiff_t)(bytes - 1);
-    return one ? a.devicePointer : nullptr;
+    using Query = CUresult (*)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+    static const Query query = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found{};
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 7000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<Query>(f);
+    }();
+    if (!query) return nullptr;
+    // what a pointer has no value for stays as it is
+    unsigned int type = 0;
+    unsigned long long at = 0, start = 0, size = 0, access = 0;
+    CUpointer_attribute names[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE, CU_POINTER_ATTRIBUTE_ACCESS_FLAGS};
+    void* values[] = {&type, &at, &start, &size, &access};
+    if (query(5, names, values, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return nullptr;
+    if (type != CU_MEMORYTYPE_HOST || access != CU_POINTER_ATTRIBUTE_ACCESS_FLAG_READWRITE) return nullptr;
+    const bool inside = at >= start && at - start <= size && bytes <= size - (at - start);
+    return inside ? reinterpret_cast<void*>((uintptr_t)at) : nullptr;
 }
 
 template <bool TO_HOST>

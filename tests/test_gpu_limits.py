@@ -150,6 +150,39 @@ def test_snapshots_into_any_host_memory(K, n, place):
     assert (raw[:first] == 0x5A).all() and (raw[first + n * size:] == 0x5A).all()
 
 
+def test_which_host_memory_kernels_write():
+    """The look at a snapshot's destination alone, nothing is launched: only what lies in one page-locked piece."""
+    import ctypes
+    import mmap
+
+    import torch
+    torch.cuda.init()
+    view = binding.load_library()._ZN3lda11device_viewEPKvm
+    view.restype, view.argtypes = ctypes.c_void_p, [ctypes.c_void_p, ctypes.c_size_t]
+    page, rt = mmap.PAGESIZE, torch.cuda.cudart()
+    held = mmap.mmap(-1, 12 * page)
+    p = ctypes.addressof(ctypes.c_char.from_buffer(held))
+    pieces = [(p, page), (p + 3 * page, page), (p + 4 * page, page), (p + 6 * page + 100, 5_000)]
+    for at, size in pieces:
+        assert int(rt.cudaHostRegister(at, size, 0)) == 0
+    read_only = p + 10 * page
+    refused = int(rt.cudaHostRegister(read_only, page, 8))  # cudaHostRegisterReadOnly
+    try:
+        for at, size in pieces:
+            assert view(at, size) == at and view(at + 64, size - 64) == at + 64 and view(at + size - 1, 1) == at + size - 1
+            assert view(at, size + 1) is None and view(at + 64, size - 63) is None and view(at + size - 1, 2) is None
+        assert view(p, 4 * page) is None               # first and last page, two between them are not page-locked
+        assert view(p + 3 * page, 2 * page) is None    # two pieces side by side: the copy decides
+        assert view(p + 2 * page, 4) is None and view(p + 2 * page, 2 * page) is None
+        assert view(read_only, 4) is None
+        pinned, on_device = torch.empty(1_000, dtype=torch.int16, pin_memory=True), torch.empty(10, device="cuda")
+        assert view(pinned.data_ptr(), 2_000) == pinned.data_ptr()
+        assert view(on_device.data_ptr(), 4) is None
+    finally:
+        for at, _ in pieces + ([(read_only, 0)] if refused == 0 else []):
+            assert int(rt.cudaHostUnregister(at)) == 0
+
+
 @pytest.mark.parametrize("offsets", [[0, 2, 1, 4], [0, -1, 4], [0, 5, 4], [0, 2 ** 63 - 1, -2 ** 63, -2 ** 62, 4],
                                      [0, 2 ** 62, 2 ** 63 - 1, -2 ** 63, -2 ** 62, 0, 4]])
 def test_offsets_out_of_order_are_refused(offsets):
