@@ -433,17 +433,51 @@ __device__ __forceinline__ void accept_tokens(const View& v, Tile& tile, const i
                 n_tw[i] = tile.count(w, t[i]);
                 n_t[i] = tile.nk(t[i]);
             }
-            // Eq. 8 (word steps) / Eq. 11 (doc steps).  With a fixed number of steps first in single precision: terms and products
+            // Eq. 8 (word steps) / Eq. 11 (doc steps), products taken left to right.  (Works on the chain's own state where nothing
+            // comes before it: by way of copies three steps took 1 % longer, 16 M tokens, K = 300: 302 -> 304 us, so 300.)
+            auto exact_steps = [&](uint32_t& x_at, int32_t& x_sd, int32_t& x_sw, int32_t& x_s, uint32_t& x_moved) {
+#pragma unroll
+                for (int i = 0; i < CH; ++i) {
+                    const bool live = m0 + i < mh_steps && t[i] != x_at;
+                    const int32_t n_td = (int32_t)(e[i] & cmask);
+                    const int32_t e_s = x_at == z0, e_t = t[i] == z0;
+                    double num = __dadd_rn(u32_to_double((uint32_t)(n_td - e_t)), alpha);
+                    num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)(n_tw[i] - e_t)), beta));
+                    num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)(x_s - e_s)), Vb));
+                    double den = __dadd_rn(u32_to_double((uint32_t)(x_sd - e_s)), alpha);
+                    den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)(x_sw - e_s)), beta));
+                    den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)(n_t[i] - e_t)), Vb));
+                    if (!step_is_doc<MODE>(i)) {
+                        num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)x_sw), beta));
+                        num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)n_t[i]), Vb));
+                        den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)n_tw[i]), beta));
+                        den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)x_s), Vb));
+                    } else {
+                        num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)x_sd), alpha));
+                        den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)n_td), alpha));
+                    }
+                    const double u = __dmul_rn(u32_to_double((uint32_t)ua[i]), INV_2_32);
+                    if (live && __dmul_rn(u, den) < num) {
+                        x_moved += step_is_doc<MODE>(i) ? 0x10000u : 1u;
+                        x_at = t[i];
+                        x_sd = n_td;
+                        x_sw = n_tw[i];
+                        x_s = n_t[i];
+                    }
+                }
+            };
+            // With a fixed number of steps first in single precision: terms and products
             // are positive and right to a few units in the last place, so a step whose two sides differ by more than
             // filter_eps of their sum goes the way it goes in double precision; a token with a closer one (one in
             // 10^5) is taken again in that.  Each factor comes without the token itself (a_) and with it (b_).  The double-
             // precision units are half as wide, and its operands take two registers (738 M tokens, K = 10 000: 6.07 -> 5.61 ms; four
             // steps, 74 M: 1.33 -> 1.12).  With any number of steps, groups of four, the registers it takes cost more
             // than that: 1.65 -> 2.14 ms for three steps of 99 M tokens, K = 1000.
-            uint32_t s_new = s, moved_now = 0;
-            bool unsure = true;
-            if constexpr (FIXED > 0) {
-                unsure = false;
+            if constexpr (FIXED == 0) {
+                exact_steps(s, n_sd, n_sw, n_s, moved);
+            } else {
+                uint32_t s_new = s, moved_now = 0;
+                bool unsure = false;
                 static_assert(FIXED <= CH, "one group of steps, which starts at z0");
                 const float fa = v.alpha_f, fb = v.beta_f, fV = v.Vbeta_f;
                 float a_sd = __fadd_rn((float)(uint32_t)(n_sd - 1), fa), b_sd = __fadd_rn(a_sd, 1.f);
@@ -476,46 +510,14 @@ __device__ __forceinline__ void accept_tokens(const View& v, Tile& tile, const i
                         a_s = a_t; b_s = b_t;
                     }
                 }
-            }
-            if (unsure) {  // products taken left to right
-                s_new = s;
-                moved_now = 0;
-                int32_t x_sd = n_sd, x_sw = n_sw, x_s = n_s;
-#pragma unroll
-                for (int i = 0; i < CH; ++i) {
-                    const bool live = m0 + i < mh_steps && t[i] != s_new;
-                    const int32_t n_td = (int32_t)(e[i] & cmask);
-                    const int32_t e_s = s_new == z0, e_t = t[i] == z0;
-                    double num = __dadd_rn(u32_to_double((uint32_t)(n_td - e_t)), alpha);
-                    num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)(n_tw[i] - e_t)), beta));
-                    num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)(x_s - e_s)), Vb));
-                    double den = __dadd_rn(u32_to_double((uint32_t)(x_sd - e_s)), alpha);
-                    den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)(x_sw - e_s)), beta));
-                    den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)(n_t[i] - e_t)), Vb));
-                    if (!step_is_doc<MODE>(i)) {
-                        num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)x_sw), beta));
-                        num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)n_t[i]), Vb));
-                        den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)n_tw[i]), beta));
-                        den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)x_s), Vb));
-                    } else {
-                        num = __dmul_rn(num, __dadd_rn(u32_to_double((uint32_t)x_sd), alpha));
-                        den = __dmul_rn(den, __dadd_rn(u32_to_double((uint32_t)n_td), alpha));
-                    }
-                    const double u = __dmul_rn(u32_to_double((uint32_t)ua[i]), INV_2_32);
-                    if (live && __dmul_rn(u, den) < num) {
-                        moved_now += step_is_doc<MODE>(i) ? 0x10000u : 1u;
-                        s_new = t[i];
-                        x_sd = n_td;
-                        x_sw = n_tw[i];
-                        x_s = n_t[i];
-                    }
+                if (unsure) {
+                    s_new = s;
+                    moved_now = 0;
+                    exact_steps(s_new, n_sd, n_sw, n_s, moved_now);
                 }
-                n_sd = x_sd;  // for the next group
-                n_sw = x_sw;
-                n_s = x_s;
+                s = s_new;
+                moved += moved_now;
             }
-            s = s_new;
-            moved += moved_now;
         }
         if (!staged_ok) break;
         __stcs(zw + p, (T)s);
