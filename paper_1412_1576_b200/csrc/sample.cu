@@ -44,11 +44,13 @@ constexpr int PROPOSE_TOKENS = LDA_PROPOSE_TOKENS;  // tokens a thread of the tw
 #define LDA_ACCEPT_MIN_CTAS 2
 #endif
 constexpr int PROPOSE_THREADS = LDA_PROPOSE_THREADS;
-// the two-step chain needs few enough registers for two CTAs of 768 threads per SM; with rows left in device memory a few more
-// (200 M tokens, K = 10^5: 5.10 ms with 768 threads, 4.98 with 640, 5.08 with 512)
+// Two CTAs per SM share its registers.  The two-step chain needs few enough for 768 threads; with rows left in device memory a few
+// more (200 M tokens, K = 10^5: 5.10 ms with 768 threads, 4.98 with 640, 5.08 with 512).  Four steps with rows in device memory
+// spill under what 512 threads leave (24 M tokens, 512, 448 and 384 threads: V = 10^6, K = 10^5 1.110, 1.091 and 1.040 ms; V = 2000,
+// K = 40 000 1.182, 1.128 and 1.079; before the single-precision look 1.125 and 1.084 with 512).
 __host__ __device__ constexpr int accept_threads(int fixed, bool staged)
 {
-    return fixed != 2 ? LDA_ACCEPT_THREADS : staged ? LDA_ACCEPT_FIXED2_THREADS : 640;
+    return fixed == 2 ? (staged ? LDA_ACCEPT_FIXED2_THREADS : 640) : fixed == 4 && !staged ? 384 : LDA_ACCEPT_THREADS;
 }
 constexpr int COLD_THREADS = 256;
 constexpr int STAGE_WAIT_LIMIT = 1 << 20;
