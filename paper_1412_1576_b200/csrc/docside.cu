@@ -144,7 +144,8 @@ __device__ __forceinline__ void doc_side_token(const View& v, const Table& table
     };
     // doc-proposal of step st
     auto doc_step = [&](int32_t st) {
-        const uint4 r = philox4x32_10(make_uint4(v.tok_base + tok, sweep, (uint32_t)st, 0u), key);
+        const uint4 at = make_uint4(v.tok_base + tok, sweep, (uint32_t)st, 0u);
+        const uint4 r = FIXED > 0 ? philox4x32_10(at, key) : philox4x32_10(at, PhiloxSeed(key));
         const bool copy = __dmul_rn(__dmul_rn(u32_to_double(r.x), INV_2_32), __dadd_rn(n_d, v.Kalpha)) < n_d;
         const uint32_t o2 = table.drawn(copy, scale_to_range(r.y, copy ? doc_len : (uint32_t)v.K));
         put(step_record_at<MODE>(st), o2);
@@ -200,10 +201,13 @@ __host__ __device__ constexpr int doc_resident_threads(int mode, int fixed)
 }
 // Slots per token of the hashed tables.  More of them mean shorter searches, but what shared memory takes L1 lacks, and its lines
 // are what the gathers in flight wait in: with 16 CTAs per SM five slots take 10.5 ms and six 13.4 instead of 9.72 (738 M
-// tokens, K = 10 000, two steps); with the twelve of the other forms six are ahead (74 M, four steps: 1.509 -> 1.447 ms).
+// tokens, K = 10 000, two steps); with the twelve of the other forms with a fixed step count six are ahead (74 M, four steps:
+// 1.509 -> 1.447 ms; doc-proposals alone, two steps, 16 M, K = 3000 and 12 000, documents of 40 and 700: 0.319 -> 0.263 ms,
+// 0.330 -> 0.271).  Loops over any number of steps wait for other things, and lose by it: 24 M, V = 10^6, K = 10^5, four steps of
+// word-proposals 0.805 ms with four slots, 0.834 with six, of doc-proposals 1.121 and 1.139.
 __host__ __device__ constexpr int tile_slots(int mode, int fixed, bool dense)
 {
-    return dense ? DOC_TILE_SLOTS : doc_resident_threads(mode, fixed) == 2048 ? DOC_TILE_SLOTS : 6;
+    return dense || fixed == 0 || doc_resident_threads(mode, fixed) == 2048 ? DOC_TILE_SLOTS : 6;
 }
 template <typename T, int THREADS, int MODE, int FIXED, bool DENSE>
 __global__ void __launch_bounds__(THREADS, doc_resident_threads(MODE, FIXED) / THREADS)

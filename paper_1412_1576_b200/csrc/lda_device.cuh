@@ -7,9 +7,10 @@ namespace lda {
 
 // Philox4x32 with 10 rounds (Salmon et al., SC'11): counter-based, so a random
 // word depends only on (seed, token, sweep, step) and not on which thread asks.
-// The keys of its ten rounds, worked out on the host: a round's exclusive-or takes them from the constant bank.  (The
-// products of a round, 32 bits by 32, run at a quarter of the rate of other operations and bound the generator: 85 cycles per warp
-// and scheduler.  Keys added up in the kernel take issue slots beside them: document pass of 738 M tokens 9.97 ms, 9.81 so.)
+// Its ten rounds' keys come in one of two forms.  (The products of a round, 32 bits by 32, run at a quarter of the rate of other
+// operations and bound the generator: 85 cycles per warp and scheduler.)
+// PhiloxKey: worked out on the host, a round's exclusive-or takes them from the constant bank.  Keys added up in the kernel
+// take issue slots beside the products: document pass of 738 M tokens, two steps, 9.97 ms, 9.81 so.
 struct PhiloxKey {
     uint32_t k[20];
     PhiloxKey() = default;
@@ -20,9 +21,22 @@ struct PhiloxKey {
             k[2 * r + 1] = (uint32_t)(seed >> 32) + (uint32_t)r * 0xBB67AE85u;
         }
     }
+    __device__ __forceinline__ uint2 round(int r) const { return make_uint2(k[2 * r], k[2 * r + 1]); }
+};
+// PhiloxSeed: added up in the kernel.  For loops over steps: the document pass of doc-proposals alone, four steps, 24 M tokens,
+// V = 10^6, K = 10^5 takes 1.121 ms with keys from the constant bank, 1.074 so; three steps of the cycle, 16 M, 404 us and 394.
+struct PhiloxSeed {
+    uint32_t lo, hi;
+    explicit __host__ __device__ PhiloxSeed(unsigned long long seed) : lo((uint32_t)seed), hi((uint32_t)(seed >> 32)) {}
+    explicit __device__ __forceinline__ PhiloxSeed(const PhiloxKey& key) : lo(key.k[0]), hi(key.k[1]) {}
+    __device__ __forceinline__ uint2 round(int r) const
+    {
+        return make_uint2(lo + (uint32_t)r * 0x9E3779B9u, hi + (uint32_t)r * 0xBB67AE85u);
+    }
 };
 
-__device__ __forceinline__ uint4 philox4x32_10(uint4 c, const PhiloxKey& key)
+template <class Key>
+__device__ __forceinline__ uint4 philox4x32_10(uint4 c, const Key& key)
 {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
@@ -30,7 +44,8 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const PhiloxKey& key)
         // costs the kernels at their register limit more than it saves)
         const uint32_t hi0 = __umulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
         const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
-        c = make_uint4(hi1 ^ c.y ^ key.k[2 * r], lo1, hi0 ^ c.w ^ key.k[2 * r + 1], lo0);
+        const uint2 k = key.round(r);
+        c = make_uint4(hi1 ^ c.y ^ k.x, lo1, hi0 ^ c.w ^ k.y, lo0);
     }
     return c;
 }
