@@ -279,11 +279,15 @@ __global__ void __launch_bounds__(512) k_ll_finish(LlSums p)
     ll_finish(p, tmp, tmp_n);
 }
 
-// Small corpora: all of it as one kernel.  The first CTAs take a tile of documents each, the others the word part, and
+// Small corpora: all of it as one kernel.  Some CTAs take a tile of documents each, the others the word part, and
 // the last one to be done adds the partial sums up (`arrived` counts them and is zero between calls).  Three
 // kernels on two streams take the host nine calls, which is longer than a corpus of 10 000 tokens takes the device.
+// The part of fewer CTAs comes first: behind more CTAs of the other than fit the GPU at once it would start late and be alone at
+// the end (10^6 tokens in documents of 800, V = 5000, K = 3000: 51 us with the tiles first, 43.5 so, three kernels 44; in documents
+// of 1400, V = 20 000, K = 12 000: 45.8, 37.3 and 41.6).
+// As many CTAs per multiprocessor as with the tiles first; without the bound the compiler takes registers for one less.
 template <typename T, int THREADS>
-__global__ void __launch_bounds__(THREADS)
+__global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : THREADS == 512 ? 3 : 1280 / THREADS)
 k_ll_all(View v, const int32_t* __restrict__ tiles, int32_t n_tiles, double lg_alpha, const double* __restrict__ tab,
          double* __restrict__ tile_part, uint32_t* __restrict__ tile_nnz, LlWords words, double* __restrict__ word_part,
          LlSums sums, unsigned int* __restrict__ arrived)
@@ -292,12 +296,13 @@ k_ll_all(View v, const int32_t* __restrict__ tiles, int32_t n_tiles, double lg_a
     __shared__ double tmp[32];
     __shared__ unsigned long long tmp_n[32];
     __shared__ bool last;
-    const int block = (int)blockIdx.x;
-    if (block < n_tiles) {
-        ll_doc_tile<T, THREADS>(v, block, tiles, lg_alpha, tab, tile_part, tile_nnz, doc_smem, tmp);
+    const int n_word = (int)gridDim.x - n_tiles, first_tile = n_word < n_tiles ? n_word : 0, first_word = n_word < n_tiles ? 0 : n_tiles;
+    const int tile = (int)blockIdx.x - first_tile, word = (int)blockIdx.x - first_word;
+    if (0 <= tile && tile < n_tiles) {
+        ll_doc_tile<T, THREADS>(v, tile, tiles, lg_alpha, tab, tile_part, tile_nnz, doc_smem, tmp);
     } else {
-        const double s = ll_word_part(v, words, block - n_tiles, (int)gridDim.x - n_tiles, reinterpret_cast<double*>(doc_smem), tmp);
-        if (threadIdx.x == 0) word_part[block - n_tiles] = s;
+        const double s = ll_word_part(v, words, word, n_word, reinterpret_cast<double*>(doc_smem), tmp);
+        if (threadIdx.x == 0) word_part[word] = s;
     }
     if (threadIdx.x == 0) {  // the partial sums are this thread's stores
         __threadfence();
