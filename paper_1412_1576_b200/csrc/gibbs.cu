@@ -126,7 +126,7 @@ template <bool MATRIX, int LANES>
 __global__ void __launch_bounds__(256, LANES == 32 ? 4 : 3)
 k_gibbs_tokens(View v, const uint16_t* __restrict__ z, const int32_t* __restrict__ word_of, const long long* __restrict__ row_off,
                const int32_t* __restrict__ dk_topic, const int32_t* __restrict__ dk_count, const ull* __restrict__ prefix,
-               const int32_t* __restrict__ matrix, int32_t* __restrict__ z_new, PhiloxKey key, uint32_t sweep, int32_t run_len)
+               const int32_t* __restrict__ matrix, int32_t* __restrict__ z_new, PhiloxSeed key, uint32_t sweep, int32_t run_len)
 {
     constexpr uint32_t FULL = 0xFFFFFFFFu;
     constexpr int TOKENS = 32 / LANES, KEPT = GIBBS_KEPT / LANES;
@@ -285,7 +285,7 @@ int lda::gibbs_sweep(Ctx& c, int32_t iters)
         rc = LDA_ENOMEM;
     // half as much again for n_kw as a matrix; without it the counts are looked up in the sorted rows
     if (rc == LDA_OK && !tmp_alloc(c, &matrix, (size_t)c.V * c.K * 4)) matrix = nullptr;
-    const PhiloxKey key(c.seed);
+    const PhiloxSeed key(c.seed);
     if (rc == LDA_OK && c.N > 0) k_word_of_tokens<<<(unsigned)((c.N + WORD_OF_RUN - 1) / WORD_OF_RUN), 256, 0, c.stream>>>(v, word_of);
     for (int32_t it = 0; rc == LDA_OK && it < iters && c.N > 0; ++it) {
         DkCsr r;

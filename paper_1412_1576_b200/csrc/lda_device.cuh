@@ -23,8 +23,9 @@ struct PhiloxKey {
     }
     __device__ __forceinline__ uint2 round(int r) const { return make_uint2(k[2 * r], k[2 * r + 1]); }
 };
-// PhiloxSeed: added up in the kernel.  For loops over steps: the document pass of doc-proposals alone, four steps, 24 M tokens,
-// V = 10^6, K = 10^5 takes 1.121 ms with keys from the constant bank, 1.074 so; three steps of the cycle, 16 M, 404 us and 394.
+// PhiloxSeed: added up in the kernel.  For loops over steps (document pass of doc-proposals alone, four steps, 24 M tokens,
+// V = 10^6, K = 10^5: 1.121 ms with keys from the constant bank, 1.074 so; three steps of the cycle, 16 M: 394 us and 387), and
+// where one block per token is little beside the rest (exact conditional, 2.6 M tokens, K = 1000: 1.298 ms and 1.293).
 struct PhiloxSeed {
     uint32_t lo, hi;
     explicit __host__ __device__ PhiloxSeed(unsigned long long seed) : lo((uint32_t)seed), hi((uint32_t)(seed >> 32)) {}
