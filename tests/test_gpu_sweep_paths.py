@@ -230,6 +230,31 @@ def test_long_words_at_large_topic_counts(K, steps, mode):
     assert np.array_equal(g.get_nk(), o.get_nk())
 
 
+@pytest.mark.parametrize("K", [53_248, 53_249, 106_497])
+@pytest.mark.parametrize("rest", [1, 300, 65_535, 65_536])
+def test_words_of_several_runs_at_large_topic_counts(K, rest):
+    """A word that is counted in two runs, of 262 144 tokens and of `rest`: below 65 536 the second counts in 16 bits where K asks
+    for it, in windows of twice the width, and both add to one line.  Two rebuilds, so that the line is cleared between."""
+    n = 262_144 + rest
+    rng = np.random.default_rng(rest)
+    words = np.zeros(n + 500, np.int32)
+    words[n:] = rng.integers(1, 4, 500)
+    z = rng.integers(0, K, words.size).astype(np.int32)
+    z[:70_000], z[n - rest:n] = K - 1, rng.choice([0, 53_247, K - 1], rest)
+    offsets = np.concatenate([[0], np.sort(rng.integers(0, z.size + 1, z.size // 80)), [z.size]]).astype(np.int64)
+    g, o = binding.LightLDA(4, K, 0.01, 0.01), ldaref.Oracle(4, K, 0.01, 0.01)
+    for e in (g, o):
+        e.load_corpus(words, offsets)
+        e.set_assignments(z, 5, 0)
+    for again in range(2):
+        assert np.array_equal(g.get_nk(), o.get_nk()), again
+        for a, b in zip(g.get_csr(binding.LDA_NWK), o.get_csr(binding.LDA_NWK)):
+            assert np.array_equal(a, b), again
+        for e in (g, o):
+            e.sweep(1, 2)
+        assert np.array_equal(g.get_assignments(), o.get_assignments()), again
+
+
 @pytest.mark.parametrize("tokens", [1, 7, 8, 9, 15, 16, 17, 255, 256, 257, 1_023, 1_024, 1_025, 2_047, 2_048])
 def test_sorted_rows_of_tiles_of_every_length(tokens):
     """Rows of words and of documents at a topic count too large for a bitmap: one word and one document of just so many
