@@ -53,6 +53,7 @@ __host__ __device__ constexpr int accept_threads(int fixed, bool staged)
     return fixed == 2 ? (staged ? LDA_ACCEPT_FIXED2_THREADS : 640) : fixed == 4 && !staged ? 384 : LDA_ACCEPT_THREADS;
 }
 constexpr int COLD_THREADS = 256;
+constexpr int64_t COLD_SIX_MAX_TOKENS = (int64_t)1 << 21;  // cold_propose_room()
 constexpr int STAGE_WAIT_LIMIT = 1 << 20;
 
 // --- shared-memory barrier and bulk-copy primitives ------------------------------------------
@@ -669,8 +670,14 @@ __device__ __forceinline__ void fill_from_marks(uint16_t* a, uint32_t* warp_last
 
 // Tail words: tile = (first word, end word, first token, count): whole words with at most COLD_TILE tokens
 // between them, or a run of one word's tokens (small corpora: see load_common() for where the cuts lie).
+// CTAs per multiprocessor that the registers leave room for; how many there are: cold_propose_room().  The loop over steps of
+// word-proposals alone is slower with more registers where tiles are short (four steps, 60 000 tokens, V = 300 000, K = 1000: 14.3 us
+// with five, 9.9 with six; 16 M tokens, K = 12 000: 350 and 353), the loop of the cycle is not (eight steps, 16 M, K = 1000: 311
+// and 315), and the two-step forms of one proposal alone spill under six.
+template <int MODE, int FIXED>
+constexpr int COLD_PROPOSE_CTAS = (FIXED == 2 && MODE == LDA_PROPOSALS_CYCLE) || (FIXED == 0 && MODE == LDA_PROPOSALS_WORD) ? 6 : 5;
 template <typename T, int MODE, int FIXED>
-__global__ void __launch_bounds__(COLD_THREADS, 5)
+__global__ void __launch_bounds__(COLD_THREADS, (COLD_PROPOSE_CTAS<MODE, FIXED>))
 k_word_cold_propose(View v, const int4* __restrict__ tiles, PhiloxKey key, int32_t mh_steps_arg, int stamp_id)
 {
     stamp(v, stamp_id);
@@ -888,6 +895,18 @@ static int launch_accept(Ctx& c, PhiloxKey key, int mh_steps)
     return launches;
 }
 
+// Dynamic shared memory that nobody uses, so that five CTAs of the tail words' propose kernel share a multiprocessor and not six: L1
+// then has 60 KB instead of 28, and the dense table's bins are gathered through it (two steps, 16 M tokens, K = 1000: 122 us
+// with six, 114 with five; K = 3000: 138, 112; K = 12 000: 168, 127; 24 M, V = 10^6, K = 10^5: 312, 281).  Small corpora wait for
+// the start of each CTA instead, and six are ahead (43 000 tokens, V = 400 000, K = 64: 8.2 us, 9.3 with five; 600 000, K = 600: 11.8,
+// 12.1; 1.5 M, K = 400: 17.2, 17.7).
+template <int MODE, int FIXED>
+static size_t cold_propose_room(const Ctx& c)
+{
+    constexpr size_t SIXTH = 3 << 10;  // 38 KB a CTA: five in 196 KB
+    return COLD_PROPOSE_CTAS<MODE, FIXED> == 6 && (MODE != LDA_PROPOSALS_CYCLE || c.N > COLD_SIX_MAX_TOKENS) ? SIXTH : 0;
+}
+
 template <typename T, int MODE, int FIXED>
 static int launch_propose(Ctx& c, PhiloxKey key, int mh_steps)
 {
@@ -903,7 +922,7 @@ static int launch_propose(Ctx& c, PhiloxKey key, int mh_steps)
         ++launches;
     }
     if (q.cold_n) {
-        k_word_cold_propose<T, MODE, FIXED><<<q.cold_n, COLD_THREADS, 0, on[1]>>>(
+        k_word_cold_propose<T, MODE, FIXED><<<q.cold_n, COLD_THREADS, cold_propose_room<MODE, FIXED>(c), on[1]>>>(
             v, reinterpret_cast<const int4*>(c.cold_tiles) + q.cold_lo, key, mh_steps, noted ? STAMP_PROPOSE_COLD : -1);
         ++launches;
     }
