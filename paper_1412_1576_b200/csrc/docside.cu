@@ -203,22 +203,26 @@ __host__ __device__ constexpr int doc_resident_threads(int mode, int fixed)
 // are what the gathers in flight wait in: with 16 CTAs per SM five slots take 10.5 ms and six 13.4 instead of 9.72 (738 M
 // tokens, K = 10 000, two steps); with the twelve of the other forms with a fixed step count six are ahead (74 M, four steps:
 // 1.509 -> 1.447 ms; doc-proposals alone, two steps, 16 M, K = 3000 and 12 000, documents of 40 and 700: 0.319 -> 0.263 ms,
-// 0.330 -> 0.271).  Loops over any number of steps wait for other things, and lose by it: 24 M, V = 10^6, K = 10^5, four steps of
-// word-proposals 0.805 ms with four slots, 0.834 with six, of doc-proposals 1.121 and 1.139.
-__host__ __device__ constexpr int tile_slots(int mode, int fixed, bool dense)
+// 0.330 -> 0.271).  Loops over any number of steps wait for other things, and lose by six: 24 M, V = 10^6, K = 10^5, four steps of
+// word-proposals 0.805 ms with four slots, 0.834 with six, of doc-proposals 1.121 and 1.139.  `few_tiles`: a multiprocessor has so
+// few that L1 is no matter; with word-proposals six are ahead (65 000 tokens, K = 1812, eight steps of them: 15.2 us with four,
+// 14.4 with six; of the cycle: 12.5 and 12.3; without: 7.6 and 7.8).  As a parameter of the kernel the number costs more than that.
+__host__ __device__ constexpr int tile_slots(int mode, int fixed, bool dense, bool few_tiles)
 {
-    return dense || fixed == 0 || doc_resident_threads(mode, fixed) == 2048 ? DOC_TILE_SLOTS : 6;
+    if (dense || doc_resident_threads(mode, fixed) == 2048) return DOC_TILE_SLOTS;
+    return fixed > 0 || (few_tiles && mode != LDA_PROPOSALS_DOC) ? DOC_TILE_SLOTS_MOST : DOC_TILE_SLOTS;
 }
-template <typename T, int THREADS, int MODE, int FIXED, bool DENSE>
+constexpr int64_t FEW_TILES_TOKENS = (int64_t)1 << 21;
+template <typename T, int THREADS, int MODE, int FIXED, bool DENSE, int SLOTS>
 __global__ void __launch_bounds__(THREADS, doc_resident_threads(MODE, FIXED) / THREADS)
 k_doc_tile(View v, const int32_t* __restrict__ tiles, PhiloxKey key, int32_t mh_steps_arg)
 {
     stamp(v, STAMP_DOC_TILES);
     const int32_t mh_steps = FIXED > 0 ? FIXED : mh_steps_arg;
-    constexpr int cap = DOC_TILE_ROUNDS * THREADS, TILE_SLOTS = tile_slots(MODE, FIXED, DENSE);
+    constexpr int cap = DOC_TILE_ROUNDS * THREADS;
     extern __shared__ __align__(16) uint32_t doc_smem[];
-    uint32_t* area = doc_smem;                                           // [TILE_SLOTS * cap] the tile's tables
-    int32_t* soff = reinterpret_cast<int32_t*>(area + TILE_SLOTS * cap);  // [cap + 1] document offsets
+    uint32_t* area = doc_smem;                                           // [SLOTS * cap] the tile's tables
+    int32_t* soff = reinterpret_cast<int32_t*>(area + SLOTS * cap);  // [cap + 1] document offsets
     uint32_t* tok_s = reinterpret_cast<uint32_t*>(soff + cap + 1);        // [cap] see TileTable::tok
     const int tid = threadIdx.x;
     const int32_t s0 = tiles[2 * blockIdx.x], s1 = tiles[2 * blockIdx.x + 1];
@@ -249,7 +253,7 @@ k_doc_tile(View v, const int32_t* __restrict__ tiles, PhiloxKey key, int32_t mh_
     uint32_t doc[DOC_TILE_ROUNDS];  // first token of the token's document | its length << 16: every register counts here
     for (int j = tid; j <= nseg; j += THREADS) soff[j] = v.doc_off[s0 + j] - base;
     const uint32_t none = DENSE ? 0u : DK_EMPTY;
-    const int quads = DENSE ? (nseg * half_k + 3) >> 2 : (cnt * TILE_SLOTS + 3) >> 2;
+    const int quads = DENSE ? (nseg * half_k + 3) >> 2 : (cnt * SLOTS + 3) >> 2;
     for (int j = tid; j < quads; j += THREADS) reinterpret_cast<uint4*>(area)[j] = make_uint4(none, none, none, none);
     __syncthreads();
     // every token finds its document and adds itself to the document's table
@@ -267,7 +271,7 @@ k_doc_tile(View v, const int32_t* __restrict__ tiles, PhiloxKey key, int32_t mh_
             doc[r] = (uint32_t)n << 16 | (uint32_t)f;
             uint32_t at = 0xFFFFFFFFu;
             if (z[r] < (uint32_t)v.K)
-                at = tile_insert<DENSE>(area + (DENSE ? lo * half_k : TILE_SLOTS * f), TILE_SLOTS * (uint32_t)n, z[r], v.count_bits);
+                at = tile_insert<DENSE>(area + (DENSE ? lo * half_k : SLOTS * f), SLOTS * (uint32_t)n, z[r], v.count_bits);
             if (at == 0xFFFFFFFFu) {
                 atomicOr(v.err, z[r] < (uint32_t)v.K ? ERR_ROW_OVERFLOW : ERR_TOPIC_RANGE);
                 at = 0;
@@ -284,7 +288,7 @@ k_doc_tile(View v, const int32_t* __restrict__ tiles, PhiloxKey key, int32_t mh_
         const int j = tid + r * THREADS;
         if (j < cnt) {
             const uint32_t f = doc[r] & 0xFFFFu, n = doc[r] >> 16;
-            const TileTable<DENSE> table{area + (DENSE ? (z[r] >> 16) * half_k : TILE_SLOTS * f), tok_s + f, TILE_SLOTS * n, v.count_bits};
+            const TileTable<DENSE> table{area + (DENSE ? (z[r] >> 16) * half_k : SLOTS * f), tok_s + f, SLOTS * n, v.count_bits};
             const uint32_t own = DENSE ? table.counted(z[r] & 0xFFFFu) : table.tab[z[r]];
             doc_side_token<T, MODE, FIXED>(v, table, (uint32_t)(base + j), n, own, t1[r], bm[r], key, sweep, mh_steps);
         }
@@ -423,15 +427,20 @@ int launch_long_tables(Ctx& c, cudaStream_t stream, bool keep_topics, int stamp_
 
 size_t doc_tile_smem_bytes(int tile_tokens, int slots) { return (size_t)tile_tokens * (4 * slots + 4 + 4) + 16; }
 
+template <typename T, int MODE, int FIXED, bool DENSE, int SLOTS>
+static void set_tile_limit()
+{
+    constexpr auto most = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaFuncSetAttribute(k_doc_tile<T, 512, MODE, FIXED, DENSE, SLOTS>, most, (int)doc_tile_smem_bytes(DOC_TILE_ROUNDS * 512, SLOTS));
+    cudaFuncSetAttribute(k_doc_tile<T, 1024, MODE, FIXED, DENSE, SLOTS>, most, (int)doc_tile_smem_bytes(DOC_TILE_MAX, SLOTS));
+}
+
 template <typename T, int MODE, int FIXED>
 static void set_doc_limit()
 {
-    constexpr auto most = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    constexpr int hashed = tile_slots(MODE, FIXED, false), dense = tile_slots(MODE, FIXED, true);
-    cudaFuncSetAttribute(k_doc_tile<T, 512, MODE, FIXED, false>, most, (int)doc_tile_smem_bytes(DOC_TILE_ROUNDS * 512, hashed));
-    cudaFuncSetAttribute(k_doc_tile<T, 1024, MODE, FIXED, false>, most, (int)doc_tile_smem_bytes(DOC_TILE_MAX, hashed));
-    if (sizeof(T) == 2)
-        cudaFuncSetAttribute(k_doc_tile<uint16_t, 1024, MODE, FIXED, true>, most, (int)doc_tile_smem_bytes(DOC_TILE_MAX, dense));
+    set_tile_limit<T, MODE, FIXED, false, tile_slots(MODE, FIXED, false, false)>();
+    set_tile_limit<T, MODE, FIXED, false, tile_slots(MODE, FIXED, false, true)>();
+    if constexpr (sizeof(T) == 2) set_tile_limit<T, MODE, FIXED, true, tile_slots(MODE, FIXED, true, false)>();
 }
 
 void set_doc_smem_limits()
@@ -459,18 +468,19 @@ static int doc_side_tm(Ctx& c, int mh_steps)
     const PassStreams on(c, (c.n_doc_tiles > 0) + (c.n_long_chunks > 0));
     int launches = 0;
     if (c.n_doc_tiles) {
-        auto tiles = [&](auto dense) {
+        auto tiles = [&](auto dense, auto few) {
             constexpr bool DENSE = decltype(dense)::value;
-            const size_t smem = doc_tile_smem_bytes(c.doc_tile, tile_slots(MODE, FIXED, DENSE));
-            switch (c.doc_threads) {
-                case 128: k_doc_tile<T, 128, MODE, FIXED, DENSE><<<c.n_doc_tiles, 128, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
-                case 256: k_doc_tile<T, 256, MODE, FIXED, DENSE><<<c.n_doc_tiles, 256, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
-                case 512: k_doc_tile<T, 512, MODE, FIXED, DENSE><<<c.n_doc_tiles, 512, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
-                default: k_doc_tile<T, 1024, MODE, FIXED, DENSE><<<c.n_doc_tiles, 1024, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps); break;
-            }
+            constexpr int SLOTS = tile_slots(MODE, FIXED, DENSE, decltype(few)::value);
+            const size_t smem = doc_tile_smem_bytes(c.doc_tile, SLOTS);
+            const auto kernel = c.doc_threads == 128   ? k_doc_tile<T, 128, MODE, FIXED, DENSE, SLOTS>
+                                : c.doc_threads == 256 ? k_doc_tile<T, 256, MODE, FIXED, DENSE, SLOTS>
+                                : c.doc_threads == 512 ? k_doc_tile<T, 512, MODE, FIXED, DENSE, SLOTS>
+                                                       : k_doc_tile<T, 1024, MODE, FIXED, DENSE, SLOTS>;
+            kernel<<<c.n_doc_tiles, c.doc_threads, smem, on[1]>>>(c.v, c.doc_tiles, key, mh_steps);
         };
-        if (c.doc_dense) tiles(std::integral_constant<bool, sizeof(T) == 2>{});  // never with 32-bit topics
-        else tiles(std::false_type{});
+        if (c.doc_dense) tiles(std::integral_constant<bool, sizeof(T) == 2>{}, std::false_type{});  // never with 32-bit topics
+        else if (c.N <= FEW_TILES_TOKENS) tiles(std::false_type{}, std::true_type{});
+        else tiles(std::false_type{}, std::false_type{});
         ++launches;
     }
     if (c.n_long_chunks) {

@@ -60,7 +60,8 @@ constexpr int DOC_TILE_THREADS[DOC_TILE_SHAPES] = {128, 256, 512, 1024};
 constexpr int DOC_TILE_TOKENS[DOC_TILE_SHAPES] = {DOC_TILE_ROUNDS * 128, DOC_TILE_ROUNDS * 256, DOC_TILE_ROUNDS * 512,
                                                   DOC_TILE_ROUNDS * 1024};
 constexpr int DOC_TILE_MAX = DOC_TILE_ROUNDS * 1024;
-constexpr int DOC_TILE_SLOTS = 4;  // 32-bit words per token of a tile's counters, and of most hashed tables (tile_slots())
+constexpr int DOC_TILE_SLOTS = 4;  // 32-bit words per token of a tile's counters, and of hashed tables at least
+constexpr int DOC_TILE_SLOTS_MOST = 6;  // ... and at most (docside.cu: tile_slots())
 // partial sums of the log-likelihood kernels: word part; document part (tiles + long documents)
 constexpr int LL_WORD_PARTIALS = 1184;
 constexpr int LL_DOC_PARTIALS = 148 * 16 + 592 + 1024;
