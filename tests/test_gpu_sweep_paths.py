@@ -255,6 +255,24 @@ def test_words_of_several_runs_at_large_topic_counts(K, rest):
         assert np.array_equal(g.get_assignments(), o.get_assignments()), again
 
 
+@pytest.mark.parametrize("tokens", [1 << 21, (1 << 21) + 1])
+def test_corpora_around_two_million_tokens(tokens):
+    """As many tokens as let the tail words' kernel have six CTAs per multiprocessor, and loops over steps six slots per token, and
+    one more."""
+    rng = np.random.default_rng(tokens)
+    words = (2_500 * rng.random(tokens) ** 2).astype(np.int32)
+    offsets = np.concatenate([[0], np.sort(rng.integers(0, tokens + 1, tokens // 50)), [tokens]]).astype(np.int64)
+    g, o = binding.LightLDA(2_500, 2_000, 0.05, 0.01), ldaref.Oracle(2_500, 2_000, 0.05, 0.01)
+    for e in (g, o):
+        e.load_corpus(words, offsets)
+        e.init(9)
+    for steps, mode in ((2, 0), (3, 0), (3, 1), (1, 2)):
+        for e in (g, o):
+            e.set_proposals(mode)
+            e.sweep(1, steps)
+        assert np.array_equal(g.get_assignments(), o.get_assignments()), (steps, mode)
+
+
 @pytest.mark.parametrize("tokens", [1, 7, 8, 9, 15, 16, 17, 255, 256, 257, 1_023, 1_024, 1_025, 2_047, 2_048])
 def test_sorted_rows_of_tiles_of_every_length(tokens):
     """Rows of words and of documents at a topic count too large for a bitmap: one word and one document of just so many
