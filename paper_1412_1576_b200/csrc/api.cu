@@ -278,7 +278,9 @@ static void free_corpus(Ctx& c)
     nv.V = c.V; nv.K = c.K; nv.alpha = c.alpha; nv.beta = c.beta;
     nv.Vbeta = (double)c.V * c.beta;
     nv.Kalpha = (double)c.K * c.alpha;
-    // Rounding errors reach 17 units of 2^-24 on either side: conversions, sums and products of five factors and the uniform.
+    // What single precision gets wrong, in units of 2^-24 of the value: 2 for each of a side's three factors without the token
+    // (count and prior as they are converted, then their sum), 3 for each of the two with it put back (one more sum), 4 for the products,
+    // and 2 for the uniform's conversion and product: 18 on its side, 16 on the other, one of the difference.  64 are allowed.
     // Priors for which products might underflow leave every step to double precision (an overflow shows by itself).
     nv.alpha_f = (float)nv.alpha;
     nv.beta_f = (float)nv.beta;

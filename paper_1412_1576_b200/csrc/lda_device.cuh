@@ -99,7 +99,8 @@ __device__ __forceinline__ uint32_t mixture_threshold(unsigned long long S, unsi
 
 // --- n_kd tables --------------------------------------------------------------------------------
 // Section 5's hashed rows (fn. 5 asks for at least twice as many slots as entries), one table per
-// document: `cap` = 4 * (document length) slots, so the load factor stays <= 0.25.  A slot is
+// document: `cap` = DK_SLOTS_PER_TOKEN * (document length) slots, so the load factor stays <= 0.25 (some document tiles have
+// more: tile_slots() in docside.cu).  A slot is
 // (topic << count_bits) | count, or DK_EMPTY_SLOT.  Open addressing with linear probing: topic k
 // starts at slot floor(k * DK_HASH_MULT mod 2^32 * cap / 2^32) and moves up one slot at a time,
 // wrapping; an empty slot met on the way means "absent".  At this load a search takes about 1.2
@@ -143,8 +144,9 @@ __device__ __forceinline__ uint32_t dk_lookup(const uint32_t* tab, uint32_t cap,
     return 0u;
 }
 
-// 32 bytes to an address that is a multiple of 32: a whole sector in one access.  L2 takes scattered whole sectors at more
-// than twice the rate of halves (records written in random order within 2^21 of them: 100 G/s, as two 16-byte stores 52).
+// 32 bytes to an address that is a multiple of 32: a whole sector in one access.  L2 takes scattered whole sectors at a higher
+// rate than halves: records written in random order within 2^20, 2^21 and 2^22 of them 148, 100 and 62 G/s, as two 16-byte
+// stores 61, 52 and 44.
 __device__ __forceinline__ void store_32(void* p, uint4 a, uint4 b)
 {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w),
