@@ -427,19 +427,23 @@ int launch_long_tables(Ctx& c, cudaStream_t stream, bool keep_topics, int stamp_
 
 size_t doc_tile_smem_bytes(int tile_tokens, int slots) { return (size_t)tile_tokens * (4 * slots + 4 + 4) + 16; }
 
+// (A limit that is set loads the kernel: only for what needs more than the 48 KB that every kernel has.)
 template <typename T, int MODE, int FIXED, bool DENSE, int SLOTS>
 static void set_tile_limit()
 {
     constexpr auto most = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaFuncSetAttribute(k_doc_tile<T, 512, MODE, FIXED, DENSE, SLOTS>, most, (int)doc_tile_smem_bytes(DOC_TILE_ROUNDS * 512, SLOTS));
+    if constexpr (SLOTS > DOC_TILE_SLOTS)
+        cudaFuncSetAttribute(k_doc_tile<T, 512, MODE, FIXED, DENSE, SLOTS>, most, (int)doc_tile_smem_bytes(DOC_TILE_ROUNDS * 512, SLOTS));
+    static_assert(DOC_TILE_ROUNDS * 512 * (4 * DOC_TILE_SLOTS + 8) + 16 <= 48 << 10, "tiles of 512 threads with the fewest slots");
     cudaFuncSetAttribute(k_doc_tile<T, 1024, MODE, FIXED, DENSE, SLOTS>, most, (int)doc_tile_smem_bytes(DOC_TILE_MAX, SLOTS));
 }
 
 template <typename T, int MODE, int FIXED>
 static void set_doc_limit()
 {
-    set_tile_limit<T, MODE, FIXED, false, tile_slots(MODE, FIXED, false, false)>();
-    set_tile_limit<T, MODE, FIXED, false, tile_slots(MODE, FIXED, false, true)>();
+    constexpr int many = tile_slots(MODE, FIXED, false, false), few = tile_slots(MODE, FIXED, false, true);
+    set_tile_limit<T, MODE, FIXED, false, many>();
+    if constexpr (few != many) set_tile_limit<T, MODE, FIXED, false, few>();
     if constexpr (sizeof(T) == 2) set_tile_limit<T, MODE, FIXED, true, tile_slots(MODE, FIXED, true, false)>();
 }
 
